@@ -17,6 +17,7 @@
 #include "kernels_conv_tc.cuh"
 #include "kernels_narrow_pack.cuh"
 #include "kernels_elementwise.cuh"
+#include "kernels_stage.cuh"
 
 #include <stdio.h>
 #include <stdlib.h>
@@ -47,7 +48,7 @@ enum PathSwitch : unsigned {
     SW_FORCE_SIMT = 1u << 0, SW_NO_NARROW = 1u << 1, SW_NO_NARROW_RING = 1u << 2, SW_NO_NARROW_TC = 1u << 3,
     SW_NO_NARROW_PACK = 1u << 4, SW_NARROW_PACK_BF16 = 1u << 5, SW_NO_GRAM_Q2 = 1u << 6, SW_NO_T1_TF32 = 1u << 7,
     SW_NO_FUSED_T1 = 1u << 8, SW_NO_GRAM_GROUP = 1u << 9, SW_NO_GRAD_GROUP = 1u << 10, SW_NO_CONV_TC = 1u << 11,
-    SW_NO_CONV_PATCHES = 1u << 12, SW_TILE_M1 = 1u << 13, SW_TILE_M2 = 1u << 14, SW_T1_TWO_LAUNCHES = 1u << 15, SW_NO_PAIR = 1u << 16, SW_LOG = 1u << 17, SW_NO_FACTORS_TAIL = 1u << 18, SW_NO_SM_BUDGET = 1u << 19, SW_NO_OVERLAP = 1u << 20,
+    SW_NO_CONV_PATCHES = 1u << 12, SW_TILE_M1 = 1u << 13, SW_TILE_M2 = 1u << 14, SW_T1_TWO_LAUNCHES = 1u << 15, SW_NO_PAIR = 1u << 16, SW_LOG = 1u << 17, SW_NO_FACTORS_TAIL = 1u << 18, SW_NO_SM_BUDGET = 1u << 19, SW_NO_OVERLAP = 1u << 20, SW_NO_STAGE = 1u << 21,
     SW_LOADED = 1u << 31
 };
 std::atomic<unsigned> g_path_switches{0};
@@ -63,7 +64,7 @@ unsigned read_path_switches() {
         {"DPCLIP_TILE_M", SW_TILE_M2, '2'}, {"DPCLIP_T1_ONE_LAUNCH", SW_T1_TWO_LAUNCHES, '0'},
         {"DPCLIP_NO_PAIR", SW_NO_PAIR, '1'}, {"DPCLIP_LOG", SW_LOG, '1'},
         {"DPCLIP_NO_FACTORS_TAIL", SW_NO_FACTORS_TAIL, '1'}, {"DPCLIP_NO_SM_BUDGET", SW_NO_SM_BUDGET, '1'},
-        {"DPCLIP_NO_OVERLAP", SW_NO_OVERLAP, '1'},
+        {"DPCLIP_NO_OVERLAP", SW_NO_OVERLAP, '1'}, {"DPCLIP_NO_STAGE", SW_NO_STAGE, '1'},
     };
     unsigned v = SW_LOADED;
     for (const auto& e : table) {
@@ -579,7 +580,7 @@ int launch_reduce_partials(const tc::zta::Params& p, int tiles, int ksplit, int 
     r.part = p.part; r.bias_part = p.bias_part;
     r.n_tiles = tiles; r.tiles_n = p.tiles_n; r.ksplit = ksplit; r.BM = BM; r.BN = BN;
     r.d_out = d_out; r.d_in = d_in; r.gW = gW; r.ldg = ldg; r.gb = gb; r.vec_ok = p.vec_ok;
-    if (noise && noise->scale > 0.f && ldg == d_in && d_in % 4 == 0) {
+    if (noise && noise->scale > 0.f && ldg == d_in) {
         r.noise_scale = noise->scale;
         r.k0 = (uint32_t)noise->seed; r.k1 = (uint32_t)(noise->seed >> 32);
         r.sw0 = (uint32_t)noise->sid_w; r.sw1 = (uint32_t)(noise->sid_w >> 32);
@@ -599,13 +600,13 @@ int launch_reduce_partials(const tc::zta::Params& p, int tiles, int ksplit, int 
 
 // Tile shape: 256 x 256 (MT = 2) cuts the L2->SM traffic per flop by a third but has a single
 // accumulator buffer; it pays once d_out spans at least two 128-row sub-tiles.
-template <int MT>
+template <int MT, bool SPLIT = false>
 int launch_zta_tc_mt(const tc::zta::Maps& maps, tc::zta::Params p, int B, bool norm_mode,
                      float* gW, long ldg, float* gb, float* sq, int d_in, int d_out, void* workspace,
                      size_t workspace_bytes, const NoiseSpec* noise, bool* noise_done, cudaStream_t st,
                      bool fit_to_workspace = false, const GradGroup* grp = nullptr) {
     namespace z = tc::zta;
-    constexpr int BM = z::Cfg<MT>::BM;
+    constexpr int BM = z::Cfg<MT, SPLIT>::BM;
     const long R = p.R;
     p.tiles_m_layer = ceil_div(d_out, BM);
     p.tiles_m = p.tiles_m_layer * (grp && grp->n > 0 ? grp->n : 1);
@@ -650,9 +651,9 @@ int launch_zta_tc_mt(const tc::zta::Maps& maps, tc::zta::Params p, int B, bool n
             return DPCLIP_ERR_CUDA;         // single item per tile: direct stores, bias by red.add
         }
     }
-    if (!enable_smem(tc::zta_tc_kernel<MT>, z::SMEM_BYTES)) return DPCLIP_ERR_CUDA;
+    if (!enable_smem(tc::zta_tc_kernel<MT, SPLIT>, z::SMEM_BYTES)) return DPCLIP_ERR_CUDA;
     const int grid = p.n_items < sm_budget() ? p.n_items : sm_budget();
-    tc::zta_tc_kernel<MT><<<grid, z::THREADS, z::SMEM_BYTES, st>>>(maps, p);
+    tc::zta_tc_kernel<MT, SPLIT><<<grid, z::THREADS, z::SMEM_BYTES, st>>>(maps, p);
     int rc = launch_status();
     if (rc || norm_mode || ksplit == 1) return rc;
 
@@ -681,6 +682,7 @@ struct StreamLayer {
     const void* A; long lda; const void* Z; long ldz; int d_in, d_out;
     float* gW; long ldg; float* gb; unsigned long long sid_w, sid_b;
     const float* clip;             // this layer's factors [B], or NULL
+    bool split;                    // scaled operand in two bf16 terms
 };
 
 // Returns DPCLIP_OK, a negative status, or 1 when the workspace cannot hold even one segment per tile (the
@@ -695,7 +697,7 @@ int launch_zta_stream(const StreamLayer* ls, int n, int B, int T, const NoiseSpe
     memset(&p, 0, sizeof(p));
     p.R = (int)R; p.T = T; p.S = (int)ceil_div(R, (long)zp::BK); p.n_layers = n;
     p.status = static_cast<int*>(workspace);
-    bool fuse_noise = noise && noise->scale > 0.f;
+    bool fuse_noise = noise && noise->scale > 0.f, any_split = false;
     int G = 0;
     for (int l = 0; l < n; ++l) {
         const StreamLayer& y = ls[l];
@@ -709,13 +711,15 @@ int launch_zta_stream(const StreamLayer* ls, int n, int B, int T, const NoiseSpe
         G += q.tiles;
         q.do_bias = y.gb ? 1 : 0;
         q.clip = y.clip;
+        q.split = y.split ? 1 : 0;
+        any_split = any_split || y.split;
         q.gW = y.gW; q.gb = y.gb; q.ldg = y.ldg;
         q.vec_ok = aligned_to(y.gW, 16) && y.ldg % 4 == 0;
         q.sw0 = (uint32_t)y.sid_w; q.sw1 = (uint32_t)(y.sid_w >> 32);
         q.sb0 = (uint32_t)y.sid_b; q.sb1 = (uint32_t)(y.sid_b >> 32);
         if (y.gb) p.any_bias = 1;
-        // the noise of element j is indexed by its position in the dense tensor, one Philox block per float4
-        if (y.ldg != y.d_in || y.d_in % 4 != 0) fuse_noise = false;
+        // the noise of element j is indexed by its position in the dense tensor
+        if (y.ldg != y.d_in) fuse_noise = false;
     }
     p.G = G;
     if (G > zp::MAX_TILES) return 1;
@@ -793,7 +797,8 @@ int launch_zta_stream(const StreamLayer* ls, int n, int B, int T, const NoiseSpe
         p.k0 = (uint32_t)noise->seed; p.k1 = (uint32_t)(noise->seed >> 32);
         if (noise_done) *noise_done = true;
     }
-    if (!enable_smem(tc::zta_pair_kernel, zp::SMEM_BYTES)) return DPCLIP_ERR_CUDA;
+    const auto kernel = any_split ? tc::zta_pair_kernel<true> : tc::zta_pair_kernel<false>;
+    if (!enable_smem(kernel, zp::SMEM_BYTES)) return DPCLIP_ERR_CUDA;
     const int pairs = (int)ceil_div(p.total, U) * W;
     DPCLIP_LOGF("clipped sum, CTA pairs: %d layer(s), B*T=%ld, %d tiles of 512x256 in %d super-layer(s) of %d, %d stages per tile, "
                 "%d pairs in gangs of %d, runs of %ld stages, %ld segments, noise %s", n, R, G, n_super, W, p.S, pairs, W, U,
@@ -808,9 +813,9 @@ int launch_zta_stream(const StreamLayer* ls, int n, int B, int T, const NoiseSpe
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr; cfg.numAttrs = 1;
-        if (cudaLaunchKernelEx(&cfg, tc::zta_pair_kernel, maps, p) != cudaSuccess) { cudaGetLastError(); return DPCLIP_ERR_CUDA; }
+        if (cudaLaunchKernelEx(&cfg, kernel, maps, p) != cudaSuccess) { cudaGetLastError(); return DPCLIP_ERR_CUDA; }
     } else {
-        tc::zta_pair_kernel<<<2 * pairs, zp::THREADS, zp::SMEM_BYTES, st>>>(maps, p);
+        kernel<<<2 * pairs, zp::THREADS, zp::SMEM_BYTES, st>>>(maps, p);
     }
     int rc = launch_status();
     if (rc) return rc;
@@ -824,13 +829,14 @@ int launch_zta_stream(const StreamLayer* ls, int n, int B, int T, const NoiseSpe
 int launch_zta_tc(const void* A, long lda, const void* Z, long ldz, int B, int T, int d_in, int d_out,
                   bool norm_mode, int has_bias, const float* clip, float* gW, long ldg, float* gb, float* sq,
                   void* workspace, size_t workspace_bytes, const NoiseSpec* noise, bool* noise_done,
-                  cudaStream_t st, bool fit_to_workspace = false) {
+                  cudaStream_t st, bool fit_to_workspace = false, bool split = false) {
     namespace z = tc::zta;
     const long R = (long)B * T;
     int mt = d_out > 128 ? 2 : 1;
     if (path_switch(SW_TILE_M1)) mt = 1;
     if (path_switch(SW_TILE_M2)) mt = 2;
     const bool pair = !norm_mode && mt == 2 && pair_tile_ok(d_out);
+    if (split && !norm_mode) mt = 1;            // the second operand plane leaves room for the small tile only
     const int bk = mt == 2 ? z::Cfg<2>::BK : z::Cfg<1>::BK;           // rows of a TMA box = rows of a stage
     z::Maps maps;
     if (!make_map_bf16(&maps.a[0], A, R, d_in, lda, 64, bk) || !make_map_bf16(&maps.z[0], Z, R, d_out, ldz, 64, bk))
@@ -849,13 +855,16 @@ int launch_zta_tc(const void* A, long lda, const void* Z, long ldz, int B, int T
         p.vec_ok = aligned_to(gW, 16) && ldg % 4 == 0;
     }
     if (pair) {
-        const StreamLayer one = {A, lda, Z, ldz, d_in, d_out, gW, ldg, gb, noise ? noise->sid_w : 0ull, noise ? noise->sid_b : 0ull, clip};
+        const StreamLayer one = {A, lda, Z, ldz, d_in, d_out, gW, ldg, gb, noise ? noise->sid_w : 0ull, noise ? noise->sid_b : 0ull, clip, split};
         const int rc = launch_zta_stream(&one, 1, B, T, noise, noise_done, workspace, workspace_bytes, st);
         if (rc <= 0) return rc;                 // 1: not even one segment per tile fits -> the single-CTA kernel below
     }
     if (mt == 2)
         return launch_zta_tc_mt<2>(maps, p, B, norm_mode, gW, ldg, gb, sq, d_in, d_out, workspace, workspace_bytes,
                                    noise, noise_done, st, fit_to_workspace);
+    if (split && !norm_mode)
+        return launch_zta_tc_mt<1, true>(maps, p, B, norm_mode, gW, ldg, gb, sq, d_in, d_out, workspace, workspace_bytes,
+                                         noise, noise_done, st, fit_to_workspace);
     return launch_zta_tc_mt<1>(maps, p, B, norm_mode, gW, ldg, gb, sq, d_in, d_out, workspace, workspace_bytes,
                                noise, noise_done, st, fit_to_workspace);
 }
@@ -864,12 +873,12 @@ int launch_zta_tc(const void* A, long lda, const void* Z, long ldz, int B, int T
 // Returns 1 when the group does not qualify (the caller then goes layer by layer).
 int launch_zta_tc_group(const dpclip_layer* const* ls, const int* index, int n, int B, const float* clip,
                         float noise_scale, unsigned long long seed, unsigned long long stream_id0,
-                        void* workspace, size_t workspace_bytes, cudaStream_t st) {
+                        void* workspace, size_t workspace_bytes, cudaStream_t st, bool split = false) {
     namespace z = tc::zta;
     if (n < 2 || n > z::MAX_LAYERS) return 1;
     const dpclip_layer& y0 = *ls[0];
     const long R = (long)B * y0.T;
-    const int bk = y0.d_out > 128 ? z::Cfg<2>::BK : z::Cfg<1>::BK;
+    const int bk = y0.d_out > 128 && !split ? z::Cfg<2>::BK : z::Cfg<1>::BK;
     z::Maps maps;
     GradGroup grp;
     memset(&grp, 0, sizeof(grp));
@@ -896,14 +905,17 @@ int launch_zta_tc_group(const dpclip_layer* const* ls, const int* index, int n, 
     const NoiseSpec ns = {noise_scale, seed, 0, 0};             // the streams come from the group
     bool noise_done = false;
     int rc;
-    if (y0.d_out > 128)
+    if (split)
+        rc = launch_zta_tc_mt<1, true>(maps, p, B, false, y0.gW, y0.d_in, any_gb, nullptr, y0.d_in, y0.d_out, workspace,
+                                       workspace_bytes, &ns, &noise_done, st, false, &grp);
+    else if (y0.d_out > 128)
         rc = launch_zta_tc_mt<2>(maps, p, B, false, y0.gW, y0.d_in, any_gb, nullptr, y0.d_in, y0.d_out, workspace,
                                  workspace_bytes, &ns, &noise_done, st, false, &grp);
     else
         rc = launch_zta_tc_mt<1>(maps, p, B, false, y0.gW, y0.d_in, any_gb, nullptr, y0.d_in, y0.d_out, workspace,
                                  workspace_bytes, &ns, &noise_done, st, false, &grp);
     if (rc) return rc;
-    if (noise_scale > 0.f && !noise_done) return DPCLIP_ERR_UNSUPPORTED;     // the caller checked d_in % 4
+    if (noise_scale > 0.f && !noise_done) return DPCLIP_ERR_UNSUPPORTED;     // the outputs are dense
     return DPCLIP_OK;
 }
 
@@ -994,14 +1006,15 @@ int launch_zta_tf32(const void* A, long lda, const void* Z, long ldz, int B, int
 // clipped sum of one layer, optionally with the noise folded into the last pass over the output
 int clipped_grad_impl(const void* A, long lda, const void* Zbar, long ldz, int B, int T, int d_in, int d_out,
                       dpclip_dtype dtype, const float* clip, float* gW, long ldg, float* gb, void* workspace,
-                      size_t workspace_bytes, const NoiseSpec* noise, bool* noise_done, cudaStream_t st) {
+                      size_t workspace_bytes, const NoiseSpec* noise, bool* noise_done, cudaStream_t st,
+                      bool split = false) {
     DPCLIP_LOGF("clipped_grad B=%d T=%d %d->%d %s: %s", B, T, d_in, d_out, dtype == DPCLIP_F32 ? "f32" : "bf16",
                 tc_eligible(A, lda, Zbar, ldz, dtype) ? "tcgen05 bf16"
                 : (tf32_eligible(A, lda, Zbar, ldz, B, T, d_in, d_out, dtype) && !narrow_layer(T, d_in, d_out, gb != nullptr, lda, ldz))
                       ? "tcgen05 3xtf32" : "fp32-ALU / narrow kernels");
     if (tc_eligible(A, lda, Zbar, ldz, dtype))
         return launch_zta_tc(A, lda, Zbar, ldz, B, T, d_in, d_out, false, 0, clip, gW, ldg, gb, nullptr, workspace,
-                             workspace_bytes, noise, noise_done, st);
+                             workspace_bytes, noise, noise_done, st, false, split);
     if (tf32_eligible(A, lda, Zbar, ldz, B, T, d_in, d_out, dtype) && !narrow_layer(T, d_in, d_out, gb != nullptr, lda, ldz))
         return launch_zta_tf32(A, lda, Zbar, ldz, B, T, d_in, d_out, false, 0, clip, gW, ldg, gb, nullptr, workspace,
                                workspace_bytes, noise, noise_done, st);
@@ -1020,27 +1033,27 @@ inline bool t1_tma_ok(const void* ptr, long ld, dpclip_dtype dtype) {
     return aligned_to(ptr, 16) && ld % (dtype == DPCLIP_BF16 ? 8 : 4) == 0;
 }
 
-template <typename T>
+template <typename T, bool QUADS>
 int launch_fused_t1_tc(tc::f1::Params& q, bool one_launch, int grid, void* workspace, cudaStream_t st) {
     namespace f = tc::f1;
     if (one_launch) {
         // the whole step as one cooperative launch (its CTAs meet at a grid-wide barrier)
         q.grid_counter = reinterpret_cast<unsigned int*>(static_cast<char*>(workspace) + kGridCounterOffset);
-        if (!enable_smem(tc::t1_all_grads_tf32_kernel<true, T>, f::SMEM_BYTES)) return DPCLIP_ERR_CUDA;
+        if (!enable_smem(tc::t1_all_grads_tf32_kernel<true, T, QUADS>, f::SMEM_BYTES)) return DPCLIP_ERR_CUDA;
         cudaLaunchConfig_t cfg;
         memset(&cfg, 0, sizeof(cfg));
         cfg.gridDim = dim3(grid); cfg.blockDim = dim3(f::THREADS); cfg.dynamicSmemBytes = f::SMEM_BYTES; cfg.stream = st;
         cudaLaunchAttribute attr;
         attr.id = cudaLaunchAttributeCooperative; attr.val.cooperative = 1;
         cfg.attrs = &attr; cfg.numAttrs = 1;
-        if (cudaLaunchKernelEx(&cfg, tc::t1_all_grads_tf32_kernel<true, T>, q) != cudaSuccess) {
+        if (cudaLaunchKernelEx(&cfg, tc::t1_all_grads_tf32_kernel<true, T, QUADS>, q) != cudaSuccess) {
             cudaGetLastError();
             return 1;                       // cannot be made resident at once: take the two-launch form
         }
         return launch_status();
     }
-    if (!enable_smem(tc::t1_all_grads_tf32_kernel<false, T>, f::SMEM_BYTES)) return DPCLIP_ERR_CUDA;
-    tc::t1_all_grads_tf32_kernel<false, T><<<grid, f::THREADS, f::SMEM_BYTES, st>>>(q);
+    if (!enable_smem(tc::t1_all_grads_tf32_kernel<false, T, QUADS>, f::SMEM_BYTES)) return DPCLIP_ERR_CUDA;
+    tc::t1_all_grads_tf32_kernel<false, T, QUADS><<<grid, f::THREADS, f::SMEM_BYTES, st>>>(q);
     return launch_status();
 }
 
@@ -1056,8 +1069,10 @@ int launch_fused_t1_tf32(const FusedT1Params& base, bool one_launch, dpclip_dtyp
     q.status = static_cast<int*>(workspace);
     const bool bf16 = dtype == DPCLIP_BF16;
     int items = 0, tc_layers = 0;
+    bool quads = true;
     for (int l = 0; l < base.L; ++l) {
         const FusedT1Layer& y = base.layer[l];
+        quads = quads && y.d_in % 4 == 0;
         const bool thin = y.d_out <= f::THIN_MAX_OUT;
         if (!t1_tma_ok(y.A, y.lda, dtype) || !(t1_tma_ok(y.Z, y.ldz, dtype) || thin)) return 1;
         q.item_begin[l] = items;
@@ -1076,8 +1091,10 @@ int launch_fused_t1_tf32(const FusedT1Params& base, bool one_launch, dpclip_dtyp
     if (!tc_layers) return 1;
     q.total_items = items;
     const int grid = items < kNumSMs ? items : kNumSMs;
-    return bf16 ? launch_fused_t1_tc<__nv_bfloat16>(q, one_launch, grid, workspace, st)
-                : launch_fused_t1_tc<float>(q, one_launch, grid, workspace, st);
+    if (bf16) return quads ? launch_fused_t1_tc<__nv_bfloat16, true>(q, one_launch, grid, workspace, st)
+                           : launch_fused_t1_tc<__nv_bfloat16, false>(q, one_launch, grid, workspace, st);
+    return quads ? launch_fused_t1_tc<float, true>(q, one_launch, grid, workspace, st)
+                 : launch_fused_t1_tc<float, false>(q, one_launch, grid, workspace, st);
 }
 
 // One T = 1 layer of the caller's model as the fused kernels see it.  Returns 0, 1 (the layer does not
@@ -1285,7 +1302,8 @@ size_t dpclip_workspace_bytes(int B, int T, int d_in, int d_out, dpclip_dtype dt
     return (size_t)kHeaderBytes;
 }
 
-size_t dpclip_step_workspace_bytes(const dpclip_layer* layers, int L, int B, dpclip_dtype dtype) {
+// Scratch for a step over these layers (not the staged copies: see stage_plan).
+static size_t step_scratch_bytes(const dpclip_layer* layers, int L, int B, dpclip_dtype dtype) {
     size_t ws = kHeaderBytes;
     if (!layers || L <= 0 || B <= 0) return ws;
     for (int l = 0; l < L; ++l) {
@@ -1314,6 +1332,15 @@ size_t dpclip_step_workspace_bytes(const dpclip_layer* layers, int L, int B, dpc
         if (n >= 2 && kHeaderBytes + pair_scratch_bytes(tiles) > ws) ws = kHeaderBytes + pair_scratch_bytes(tiles);
     }
     return ws;
+}
+
+struct StagePlan;
+static size_t staged_workspace_bytes(const dpclip_layer* layers, const dpclip_model_layer* other, int L, int B, dpclip_dtype dtype);
+
+size_t dpclip_step_workspace_bytes(const dpclip_layer* layers, int L, int B, dpclip_dtype dtype) {
+    const size_t ws = step_scratch_bytes(layers, L, B, dtype);
+    const size_t staged = staged_workspace_bytes(layers, nullptr, L, B, dtype);
+    return staged > ws ? staged : ws;
 }
 
 int dpclip_workspace_init(void* workspace, size_t workspace_bytes, void* stream) {
@@ -1432,7 +1459,7 @@ static int gram_layers_sqnorms(const dpclip_layer* layers, int L, int B, dpclip_
     return DPCLIP_OK;
 }
 
-static int shared_clipped_grad_launches(const dpclip_layer* layers, int L, int B, dpclip_dtype dtype,
+static int shared_clipped_grad_launches(const dpclip_layer* layers, const bool* split, int L, int B, dpclip_dtype dtype,
                                         const float* clip, long clip_ld, float C, float sigma, unsigned long long seed,
                                         unsigned long long stream_id0, int* taken, void* workspace,
                                         size_t workspace_bytes, void* stream);
@@ -1441,13 +1468,13 @@ int dpclip_same_shape_layers_clipped_grad_noise(const dpclip_layer* layers, int 
                                                 const float* clip, float C, float sigma, unsigned long long seed,
                                                 unsigned long long stream_id0, int* taken, void* workspace,
                                                 size_t workspace_bytes, void* stream) {
-    return shared_clipped_grad_launches(layers, L, B, dtype, clip, 0, C, sigma, seed, stream_id0, taken, workspace,
+    return shared_clipped_grad_launches(layers, nullptr, L, B, dtype, clip, 0, C, sigma, seed, stream_id0, taken, workspace,
                                         workspace_bytes, stream);
 }
 
 // clip_ld = 0: one factor vector for all layers (global clipping); clip_ld > 0: layer l's factors are row l of
 // clip[L][clip_ld] (per-layer clipping) -- then only the CTA-pair launches, which take a vector per layer, are made.
-static int shared_clipped_grad_launches(const dpclip_layer* layers, int L, int B, dpclip_dtype dtype,
+static int shared_clipped_grad_launches(const dpclip_layer* layers, const bool* split, int L, int B, dpclip_dtype dtype,
                                         const float* clip, long clip_ld, float C, float sigma, unsigned long long seed,
                                         unsigned long long stream_id0, int* taken, void* workspace,
                                         size_t workspace_bytes, void* stream) {
@@ -1461,7 +1488,7 @@ static int shared_clipped_grad_launches(const dpclip_layer* layers, int L, int B
     if (L > kMaxTracked) return DPCLIP_OK;
     bool done[kMaxTracked] = {false};
     auto candidate = [&](const dpclip_layer& y) {
-        if (y.T <= 1 || !y.gW || y.ldg != y.d_in || y.d_in % 4 != 0 || (y.has_bias && !y.gb)) return false;
+        if (y.T <= 1 || !y.gW || y.ldg != y.d_in || (y.has_bias && !y.gb)) return false;
         if (check_layer_args(y.A, y.lda, y.Zbar, y.ldz, B, y.T, y.d_in, y.d_out, dtype)) return false;
         if (!aligned_to(y.gW, 4) || (y.has_bias && !aligned_to(y.gb, 4))) return false;
         return tc_eligible(y.A, y.lda, y.Zbar, y.ldz, dtype);
@@ -1477,7 +1504,8 @@ static int shared_clipped_grad_launches(const dpclip_layer* layers, int L, int B
             const dpclip_layer& y = layers[l];
             if (done[l] || y.T != layers[l0].T || !pair_tile_ok(y.d_out) || !candidate(y)) continue;
             grp[n] = {y.A, y.lda, y.Zbar, y.ldz, y.d_in, y.d_out, y.gW, y.ldg, y.has_bias ? y.gb : nullptr,
-                      stream_id0 + 2ull * l, stream_id0 + 2ull * l + 1, clip ? clip + (size_t)l * clip_ld : nullptr};
+                      stream_id0 + 2ull * l, stream_id0 + 2ull * l + 1, clip ? clip + (size_t)l * clip_ld : nullptr,
+                      split && split[l]};
             idx[n] = l; ++n;
             tiles += pair_tiles(y.d_in, y.d_out);
         }
@@ -1491,7 +1519,7 @@ static int shared_clipped_grad_launches(const dpclip_layer* layers, int L, int B
                                          (cudaStream_t)stream);
         if (rc < 0) return rc;
         if (rc > 0) continue;
-        if (sigma * C > 0.f && !noise_done) return DPCLIP_ERR_UNSUPPORTED;    // candidate() checked dense rows, d_in % 4
+        if (sigma * C > 0.f && !noise_done) return DPCLIP_ERR_UNSUPPORTED;    // candidate() checked dense rows
         if (!taken) return DPCLIP_ERR_INVALID_ARG;               // without `taken` the caller cannot know
         for (int i = 0; i < n; ++i) { done[idx[i]] = true; taken[idx[i]] = 1; }
     }
@@ -1504,7 +1532,7 @@ static int shared_clipped_grad_launches(const dpclip_layer* layers, int L, int B
         for (int l = l0; l < L && n < z::MAX_LAYERS; ++l) {
             const dpclip_layer& y = layers[l];
             if (done[l] || y.T != layers[l0].T || y.d_in != layers[l0].d_in || y.d_out != layers[l0].d_out) continue;
-            if (!candidate(y)) continue;
+            if (!candidate(y) || (split && split[l] != split[l0])) continue;
             grp[n] = &y; idx[n] = l; ++n;
         }
         for (int i = 0; i < n; ++i) done[idx[i]] = true;
@@ -1515,14 +1543,14 @@ static int shared_clipped_grad_launches(const dpclip_layer* layers, int L, int B
             // whose one-wave split uses the SMs more evenly (measured on two 512 -> 2048 layers at
             // B*T = 32768: 174 us together on 128 CTAs, 2 x 80 us apart on 144).
             const dpclip_layer& y = layers[l0];
-            const int bm = y.d_out > 128 ? 256 : 128;
+            const int bm = y.d_out > 128 && !(split && split[l0]) ? 256 : 128;
             const int tiles = ceil_div(y.d_out, bm) * ceil_div(y.d_in, z::BN);
             const long nkb = ceil_div((long)B * y.T, 64L);          // 64-row blocks
             const int ksplit = tiles < kNumSMs ? kNumSMs / tiles : 1;
             if (nkb / ksplit >= 32) continue;
         }
         const int rc = launch_zta_tc_group(grp, idx, n, B, clip, sigma * C, seed, stream_id0, workspace, workspace_bytes,
-                                           (cudaStream_t)stream);
+                                           (cudaStream_t)stream, split && split[l0]);
         if (rc < 0) return rc;
         if (rc == 0 && taken) for (int i = 0; i < n; ++i) taken[idx[i]] = 1;
         if (rc == 0 && !taken) return DPCLIP_ERR_INVALID_ARG;     // without `taken` the caller cannot know
@@ -2051,6 +2079,216 @@ static int other_kind_clipped_grad_noise(const dpclip_model_layer& m, int B, dpc
     return rc;
 }
 
+// ---------------------------------------------------------------------------
+// Operand staging of a whole step (kernels_stage.cuh): which layers' operands are rewritten, where the copies lie, and
+// the layers as the rest of the step sees them.  The copies lie behind the scratch, in lane 0's workspace, and live
+// from the first launch of the step to its last.
+// ---------------------------------------------------------------------------
+constexpr int kStageMaxLayers = 64;
+// Copies of one step; a layer that no longer fits keeps its fp32-ALU form.  (Every lane of a several-streams step owns
+// a workspace of this size.)
+constexpr size_t kStageCapBytes = (size_t)3 << 30;
+struct StagePlan {
+    bool active = false;
+    dpclip_layer eff[kStageMaxLayers];       // T = 0: a layer of another kind
+    bool other[kStageMaxLayers];             // goes through the entry points of its kind (not staged, not dense)
+    bool split[kStageMaxLayers];             // clipped sum with two-term scaled operands (see zta_tc_kernel)
+    dpclip_dtype t1_dtype;                   // type of the T = 1 layers after staging
+    stage::Job job[2 * kStageMaxLayers];
+    int n_jobs = 0, smem = 0;
+    size_t scratch = 0, bytes = 0;           // bytes before the copies, and with them
+};
+
+// Copying pays once a layer (T > 1) has real contraction work: below 2^25 multiply-adds the fp32-ALU kernels take about as
+// long as the copy's own launch (66 -> 66 features at B = 64, T = 32: 34 us a step either way; 130 -> 130 there, 35 M:
+// 35.1 staged, 41.1 not; 250 -> 250 at T = 128, 512 M: 37 / 119 us).  With few rows the tensor-core kernels fill few SMs: 501
+// -> 501 at B*T = 256 (64 M) 47 / 40 us, 1001 -> 1001 there 53 / 82 us.
+static bool stage_worth_it(double rows, double weights, dpclip_dtype dtype) {
+    const double macs = rows * weights;
+    return macs >= 32.0 * 1024 * 1024 && (dtype == DPCLIP_F32 || rows >= 1024 || macs >= 128e6);
+}
+
+static bool stage_plan(StagePlan& sp, const dpclip_layer* layers, const dpclip_model_layer* other, int L, int B,
+                       dpclip_dtype dtype, char* base, bool t1_too) {
+    sp.active = false;
+    if (L > kStageMaxLayers || path_switch(SW_FORCE_SIMT) || path_switch(SW_NO_STAGE)) return false;
+    const size_t es = elt_size(dtype);
+    const int unit = 16 / (int)es;                                  // elements of 16 bytes
+    sp.n_jobs = 0; sp.smem = 0; sp.t1_dtype = dtype;
+    size_t off = 0;                                                 // within the area of copies
+    bool any = false;
+    struct Take { int job; size_t off; int layer; bool z; };
+    Take takes[2 * kStageMaxLayers];
+    auto add_job = [&](int l, bool z, int kind, const void* src, long src_ld, int dst_ld, int rows, int cols, size_t dst_es) -> stage::Job& {
+        stage::Job& j = sp.job[sp.n_jobs];
+        memset(&j, 0, sizeof(j));
+        j.kind = kind; j.es = (int)es; j.src = src; j.src_ld = src_ld; j.dst_ld = dst_ld; j.rows = rows; j.cols = cols;
+        takes[sp.n_jobs] = {sp.n_jobs, off, l, z};
+        off += round_up((size_t)rows * dst_ld * dst_es, 256);
+        ++sp.n_jobs;
+        return j;
+    };
+    auto misaligned = [&](const void* ptr, long ld) { return !aligned_to(ptr, 16) || ld % unit != 0; };
+    for (int l = 0; l < L; ++l) {
+        sp.eff[l] = layers[l]; sp.split[l] = false;
+        sp.other[l] = other && other[l].kind != DPCLIP_KIND_DENSE;
+        const size_t off0 = off;
+        const int jobs0 = sp.n_jobs;
+        if (sp.other[l]) {
+            if (other[l].kind != DPCLIP_KIND_CONV) continue;
+            const dpclip_layer& y = other[l].layer;
+            const dpclip_conv& g = other[l].conv;
+            SimtParams p;
+            int T = 0;
+            if (conv_setup(p, y.A, y.Zbar, other[l].z_channel_major, B, &g, y.d_out, dtype, y.has_bias, &T)) continue;
+            if (T <= 1 || !y.gW || y.ldg != p.d_in || (y.has_bias && !y.gb)) continue;
+            if (conv_tc_ok(p, y.A, y.Zbar, other[l].z_channel_major, B, T, dtype, base, kHeaderBytes)) continue;
+            // bf16: the gathers of the fp32-ALU convolution kernel cost more than the copy from small sizes on (a CNN with
+            // layers of 4 to 90 M multiply-adds: 80 us, 45 us staged)
+            if ((double)B * T * p.d_in * p.d_out < (dtype == DPCLIP_BF16 ? 4.0 : 32.0) * 1024 * 1024) continue;
+            // narrow fp32 layers go to the kernels that stream dense rows
+            const bool narrow = dtype == DPCLIP_F32 && narrow_layer(T, p.d_in, p.d_out, 1, p.d_in, p.d_out);
+            const long ldp = narrow ? p.d_in : (long)round_up(p.d_in, unit), ldz = narrow ? p.d_out : (long)round_up(p.d_out, unit);
+            const int kk = g.kh * g.kw;
+            int ct = (int)(1152 / (kk * es)) / unit * unit;         // about 36 KB of lines per CTA
+            if (ct < unit) ct = unit;
+            if (ct > (int)round_up(g.C, unit)) ct = (int)round_up(g.C, unit);
+            const int pitch = (int)round_up((size_t)ct * kk * es, 16) + 4;
+            if (stage::IM_ROWS * pitch > stage::SMEM_MAX || (double)B * T * ldp / unit > 4.0e9) continue;
+            {
+                stage::Job& j = add_job(l, false, stage::IM2COL, y.A, 0, (int)ldp, B * T, p.d_in, es);
+                j.T = T; j.C = g.C; j.H = g.H; j.W = g.W; j.kh = g.kh; j.kw = g.kw; j.stride = g.stride; j.pad = g.pad;
+                j.Wo = p.Wo; j.ct = ct; j.pitch = pitch; j.tiles_b = ceil_div(g.C, ct);
+                if (stage::IM_ROWS * pitch > sp.smem) sp.smem = stage::IM_ROWS * pitch;
+            }
+            dpclip_layer& e = sp.eff[l];
+            e = y;
+            e.T = T; e.d_in = p.d_in; e.lda = ldp; e.method = DPCLIP_AUTO; e.ldz = p.d_out;
+            if (other[l].z_channel_major) {
+                stage::Job& j = add_job(l, true, stage::TRANSPOSE, y.Zbar, 0, (int)ldz, B * T, p.d_out, es);
+                j.T = T; j.tiles_a = ceil_div(T, stage::TILE_T); j.tiles_b = ceil_div(p.d_out, stage::TILE_M);
+                const int bytes = stage::TILE_M * (stage::TILE_T + 2) * (int)es;
+                if (bytes > sp.smem) sp.smem = bytes;
+                e.ldz = ldz;
+            } else if (!narrow && misaligned(y.Zbar, p.d_out)) {
+                add_job(l, true, stage::ROWS, y.Zbar, p.d_out, (int)ldz, B * T, p.d_out, es);
+                e.ldz = ldz;
+            }
+        } else {
+            const dpclip_layer& y = layers[l];
+            if (y.T <= 1 || y.method != DPCLIP_AUTO || !y.gW || y.ldg != y.d_in || (y.has_bias && !y.gb)) continue;
+            if (check_layer_args(y.A, y.lda, y.Zbar, y.ldz, B, y.T, y.d_in, y.d_out, dtype)) continue;
+            const bool sa = misaligned(y.A, y.lda), sz = misaligned(y.Zbar, y.ldz);
+            if (!(sa || sz) || narrow_layer(y.T, y.d_in, y.d_out, y.has_bias, y.lda, y.ldz)) continue;
+            if (!stage_worth_it((double)B * y.T, (double)y.d_in * y.d_out, dtype)) continue;
+            if ((double)B * y.T * round_up(y.d_in > y.d_out ? y.d_in : y.d_out, unit) / unit > 4.0e9) continue;
+            const long lda = (long)round_up(y.d_in, unit), ldz = (long)round_up(y.d_out, unit);
+            if (sa) { add_job(l, false, stage::ROWS, y.A, y.lda, (int)lda, B * y.T, y.d_in, es); sp.eff[l].lda = lda; }
+            if (sz) { add_job(l, true, stage::ROWS, y.Zbar, y.ldz, (int)ldz, B * y.T, y.d_out, es); sp.eff[l].ldz = ldz; }
+        }
+        if (off > kStageCapBytes) {                                  // does not fit: this layer stays as it is
+            off = off0; sp.n_jobs = jobs0;
+            sp.eff[l] = layers[l];
+            continue;
+        }
+        sp.other[l] = false;
+        sp.split[l] = dtype == DPCLIP_BF16;
+        any = true;
+    }
+    // T = 1 layers taken together (see prepare_t1_group): one operand that TMA cannot address keeps all of them off the
+    // tensor cores.  fp32: such operands are copied.  bf16: the operands of all of them become fp32 (the fp32-ALU kernel
+    // that these models ran on before applies the factors in fp32; rounding them to bf16 would be a loss).
+    if (t1_too && B <= FUSED_MAX_B && !path_switch(SW_NO_FUSED_T1) && !path_switch(SW_NO_T1_TF32)) {
+        // Worth it from about 2e8 multiply-adds at B >= 64 in bf16, at B >= 256 in fp32 (whole steps, staged / not: B = 256,
+        // 1001 -> 1001: 35 / 39 us, 2001: 64 / 115; B = 64, bf16, 2001: 51 / 58, 1001: 30 / 33; B = 64, fp32, 1001: 30 / 24;
+        // B = 95, fp32, 475 M in five layers: 52 / 48; B = 16, 4001: 163 / 125).
+        int n = 0, wide = 0;
+        bool bad = false, ok = B >= (dtype == DPCLIP_BF16 ? 64 : 256);
+        double macs = 0.0;
+        for (int l = 0; l < L; ++l) {
+            const dpclip_layer& y = layers[l];
+            if (sp.other[l] || y.T != 1 || (other && other[l].kind != DPCLIP_KIND_DENSE)) continue;
+            ++n;
+            if (check_layer_args(y.A, y.lda, y.Zbar, y.ldz, B, 1, y.d_in, y.d_out, dtype)) { ok = false; break; }
+            ok = ok && (y.method == DPCLIP_AUTO || y.method == DPCLIP_T1) && y.ldg == y.d_in && y.gW && aligned_to(y.gW, 16) &&
+                 !(y.has_bias && !y.gb);
+            const bool thin = y.d_out <= tc::f1::THIN_MAX_OUT;
+            wide += !thin;
+            macs += (double)B * y.d_in * y.d_out;
+            bad = bad || misaligned(y.A, y.lda) || (!thin && misaligned(y.Zbar, y.ldz));
+        }
+        if (ok && bad && macs >= 2e8 && n > 0 && n <= FUSED_MAX_LAYERS && wide > 0) {
+            const bool cvt = dtype == DPCLIP_BF16;
+            const size_t off0 = off;
+            const int jobs0 = sp.n_jobs;
+            for (int l = 0; l < L; ++l) {
+                const dpclip_layer& y = layers[l];
+                if (sp.other[l] || y.T != 1 || (other && other[l].kind != DPCLIP_KIND_DENSE)) continue;
+                const bool thin = y.d_out <= tc::f1::THIN_MAX_OUT;
+                const long lda = (long)round_up(y.d_in, 4), ldz = (long)round_up(y.d_out, 4);
+                if (cvt || misaligned(y.A, y.lda)) {
+                    add_job(l, false, cvt ? stage::ROWS_TO_F32 : stage::ROWS, y.A, y.lda, (int)lda, B, y.d_in, 4);
+                    sp.eff[l].lda = lda;
+                }
+                if (cvt || (!thin && misaligned(y.Zbar, y.ldz))) {
+                    add_job(l, true, cvt ? stage::ROWS_TO_F32 : stage::ROWS, y.Zbar, y.ldz, (int)ldz, B, y.d_out, 4);
+                    sp.eff[l].ldz = ldz;
+                }
+            }
+            if (off > kStageCapBytes) {
+                off = off0; sp.n_jobs = jobs0;
+                for (int l = 0; l < L; ++l) if (!sp.other[l] && layers[l].T == 1) sp.eff[l] = layers[l];
+            } else {
+                any = true;
+                sp.t1_dtype = DPCLIP_F32;
+            }
+        }
+    }
+    if (!any) return false;
+    sp.scratch = round_up(step_scratch_bytes(sp.eff, L, B, dtype), 256);
+    if (other) {
+        for (int l = 0; l < L; ++l) {
+            if (!sp.other[l] || other[l].kind != DPCLIP_KIND_CONV) continue;
+            const size_t w = round_up(dpclip_conv_workspace_bytes(B, &other[l].conv, other[l].layer.d_out, dtype, other[l].z_channel_major), 256);
+            if (w > sp.scratch) sp.scratch = w;
+        }
+    }
+    sp.bytes = sp.scratch + off;
+    for (int i = 0; i < sp.n_jobs; ++i) {
+        char* dst = base + sp.scratch + takes[i].off;
+        sp.job[i].dst = dst;
+        (takes[i].z ? sp.eff[takes[i].layer].Zbar : sp.eff[takes[i].layer].A) = dst;
+    }
+    sp.active = true;
+    return true;
+}
+
+static size_t staged_workspace_bytes(const dpclip_layer* layers, const dpclip_model_layer* other, int L, int B, dpclip_dtype dtype) {
+    if (!layers || L <= 0 || B <= 0) return 0;
+    StagePlan sp;
+    return stage_plan(sp, layers, other, L, B, dtype, reinterpret_cast<char*>(256), true) ? sp.bytes : 0;
+}
+
+static int launch_stage(StagePlan& sp, cudaStream_t st) {
+    for (int i0 = 0; i0 < sp.n_jobs; i0 += stage::MAX_JOBS) {
+        stage::Launch q;
+        memset(&q, 0, sizeof(q));
+        q.n = sp.n_jobs - i0 < stage::MAX_JOBS ? sp.n_jobs - i0 : stage::MAX_JOBS;
+        for (int i = 0; i < q.n; ++i) {
+            stage::Job& j = q.job[i] = sp.job[i0 + i];
+            j.blk_begin = q.blocks;
+            if (j.kind == stage::IM2COL) q.blocks += ceil_div(j.rows, stage::IM_ROWS) * j.tiles_b;
+            else if (j.kind == stage::TRANSPOSE) q.blocks += j.rows / j.T * j.tiles_a * j.tiles_b;
+            else q.blocks += ceil_div((long)j.rows * (j.dst_ld / ((j.es == 4 || j.kind == stage::ROWS_TO_F32) ? 4 : 8)),
+                                      (long)stage::ROWS_UNROLL * stage::THREADS);
+        }
+        if (sp.smem > 48 * 1024 && !enable_smem(stage_operands_kernel, sp.smem)) return DPCLIP_ERR_CUDA;
+        stage_operands_kernel<<<q.blocks, stage::THREADS, sp.smem, st>>>(q);
+        if (launch_status()) return DPCLIP_ERR_CUDA;
+    }
+    return DPCLIP_OK;
+}
+
 // The streams a step may spread its layers over.  Lane 0 is the caller's stream: the step starts and ends
 // there.  fork() makes every other lane wait for what lane 0 has enqueued so far, join() makes lane 0 wait for
 // what the other lanes have enqueued; both are event record/wait pairs, which a stream capture records as
@@ -2099,20 +2337,30 @@ struct Lanes {
 // `other`, when given, is the model's own descriptor array: entries of a kind other than dense have a
 // placeholder with T = 0 in `layers`, which every grouping rule below passes over, and go through the two
 // functions above.
-static int step_general(const dpclip_layer* layers, const dpclip_model_layer* other, int L, int B, dpclip_dtype dtype,
+static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer* other, int L, int B, dpclip_dtype dtype,
                         float C, float sigma, unsigned long long seed, unsigned long long stream_id0,
-                        float* sq_layers, float* clip, float* norms, Lanes& lanes) {
+                        float* sq_layers, float* clip, float* norms, Lanes& lanes, StagePlan* sp) {
     int rc;
+    const dpclip_layer* layers = sp ? sp->eff : layers_in;              // the layers with their staged operands
+    dpclip_dtype t1_dtype = sp ? sp->t1_dtype : dtype;
+    const bool* split = sp ? sp->split : nullptr;
+    auto other_kind = [&](int l) { return sp ? sp->other[l] : (other && other[l].kind != DPCLIP_KIND_DENSE); };
+    bool any_other = false;
+    for (int l = 0; l < L; ++l) any_other = any_other || other_kind(l);
     const int last = lanes.n - 1;
     void* const ws0 = lanes.ws[0];
     const size_t workspace_bytes = lanes.ws_bytes;
     T1Group t1;
-    rc = prepare_t1_group(t1, layers, L, B, dtype, C, sigma, seed, stream_id0, sq_layers, clip);
+    rc = prepare_t1_group(t1, layers, L, B, t1_dtype, C, sigma, seed, stream_id0, sq_layers, clip);
     if (rc) return rc;
     if (t1.active && (!lanes.ws[last] || workspace_bytes < (size_t)kHeaderBytes)) t1.active = false;
+    if (!t1.active && sp && t1_dtype != dtype) {                        // not taken together after all: the inputs as given
+        for (int l = 0; l < L; ++l) if (layers_in[l].T == 1) sp->eff[l] = layers_in[l];
+        t1_dtype = dtype;
+    }
     if ((rc = lanes.fork())) return rc;
     if (t1.active) {
-        if (dtype == DPCLIP_F32) t1_all_norms_kernel<float><<<t1.p.L * B, 128, 0, lanes.st[last]>>>(t1.p);
+        if (t1_dtype == DPCLIP_F32) t1_all_norms_kernel<float><<<t1.p.L * B, 128, 0, lanes.st[last]>>>(t1.p);
         else t1_all_norms_kernel<__nv_bfloat16><<<t1.p.L * B, 128, 0, lanes.st[last]>>>(t1.p);
         if (launch_status()) return DPCLIP_ERR_CUDA;
     }
@@ -2124,7 +2372,7 @@ static int step_general(const dpclip_layer* layers, const dpclip_model_layer* ot
         // when one Gram launch takes every layer of the model, its last CTA also computes the factors
         const tc::gram::FactorsTail tail = {sq_layers, L, (long)B, B, C, clip, norms, nullptr};
         rc = gram_layers_sqnorms(layers, L, B, dtype, sq_layers, in_gram_group, ws0, workspace_bytes, lanes.st[0],
-                                 (!t1.active && !other && !path_switch(SW_NO_FACTORS_TAIL)) ? &tail : nullptr, &factors_done);
+                                 (!t1.active && !any_other && !path_switch(SW_NO_FACTORS_TAIL)) ? &tail : nullptr, &factors_done);
         if (rc) return rc;
         for (int l = 0; l < L; ++l) any_gram = any_gram || in_gram_group[l];
     }
@@ -2132,12 +2380,12 @@ static int step_general(const dpclip_layer* layers, const dpclip_model_layer* ot
     // side on different lanes, no launch shared by several layers is in the stage, and the stage is small
     const size_t es = elt_size(dtype);
     auto layer_bytes = [&](int l) -> double {
-        if (other && other[l].kind == DPCLIP_KIND_CONV) {
+        if (other_kind(l) && other[l].kind == DPCLIP_KIND_CONV) {
             const dpclip_conv& g = other[l].conv;
             const double Ho = (g.H + 2 * g.pad - g.kh) / g.stride + 1, Wo = (g.W + 2 * g.pad - g.kw) / g.stride + 1;
             return (double)B * ((double)g.C * g.H * g.W + Ho * Wo * other[l].layer.d_out) * es;
         }
-        const dpclip_layer& y = other && other[l].kind != DPCLIP_KIND_DENSE ? other[l].layer : layers[l];
+        const dpclip_layer& y = other_kind(l) ? other[l].layer : layers[l];
         return (double)B * y.T * ((double)y.d_in + y.d_out) * es;
     };
     auto stage_budgets = [&](const int* skip, bool shared_launch, int* budget) {
@@ -2145,7 +2393,7 @@ static int step_general(const dpclip_layer* layers, const dpclip_model_layer* ot
         double total = 0.0;
         for (int l = 0; l < L; ++l) {
             budget[l] = 0;
-            const bool is_other = other && other[l].kind != DPCLIP_KIND_DENSE;
+            const bool is_other = other_kind(l);
             if (!is_other && ((t1.active && layers[l].T == 1) || (skip && skip[l]))) continue;
             ++n_ent; total += layer_bytes(l);
         }
@@ -2156,7 +2404,7 @@ static int step_general(const dpclip_layer* layers, const dpclip_model_layer* ot
             path_switch(SW_NO_SM_BUDGET)) return;
         const double widen = n_ent > lanes.n ? (double)n_ent / lanes.n : 1.0;      // more launches than lanes: some queue
         for (int l = 0; l < L; ++l) {
-            const bool is_other = other && other[l].kind != DPCLIP_KIND_DENSE;
+            const bool is_other = other_kind(l);
             if (!is_other && ((t1.active && layers[l].T == 1) || (skip && skip[l]))) continue;
             int b = (int)(kNumSMs * layer_bytes(l) / total * widen + 0.5);
             budget[l] = b < 16 ? 16 : (b > kNumSMs ? kNumSMs : b);
@@ -2167,7 +2415,7 @@ static int step_general(const dpclip_layer* layers, const dpclip_model_layer* ot
     int k = any_gram ? 1 : 0;                              // lane 0 already carries the shared Gram launch
     for (int l = 0; l < L; ++l) {
         const dpclip_layer& y = layers[l];
-        const bool is_other = other && other[l].kind != DPCLIP_KIND_DENSE;
+        const bool is_other = other_kind(l);
         if (!is_other && ((t1.active && y.T == 1) || (track && in_gram_group[l]))) continue;
         const SmBudgetScope share(track ? budget[l] : 0);
         const int b = k++ % lanes.n;
@@ -2186,7 +2434,7 @@ static int step_general(const dpclip_layer* layers, const dpclip_model_layer* ot
     }
     if ((rc = lanes.fork())) return rc;
     if (t1.active) {
-        rc = launch_fused_t1_tf32(t1.p, false, dtype, lanes.ws[last], workspace_bytes, lanes.st[last]);
+        rc = launch_fused_t1_tf32(t1.p, false, t1_dtype, lanes.ws[last], workspace_bytes, lanes.st[last]);
         if (rc < 0) return rc;
         if (rc > 0) return DPCLIP_ERR_UNSUPPORTED;           // prepare_t1_group checked the same conditions
     }
@@ -2196,8 +2444,8 @@ static int step_general(const dpclip_layer* layers, const dpclip_model_layer* ot
         // the factors came from the tail of the Gram launch, the last kernel of this stream: the first clipped-sum
         // launch may start loading while that tail runs
         const OverlapPrevScope overlap(factors_done);
-        rc = dpclip_same_shape_layers_clipped_grad_noise(layers, L, B, dtype, clip, C, sigma, seed, stream_id0,
-                                                         in_grad_group, ws0, workspace_bytes, lanes.st[0]);
+        rc = shared_clipped_grad_launches(layers, split, L, B, dtype, clip, 0, C, sigma, seed, stream_id0, in_grad_group, ws0,
+                                          workspace_bytes, lanes.st[0]);
         if (rc) return rc;
         for (int l = 0; l < L; ++l) any_group = any_group || in_grad_group[l];
     }
@@ -2205,7 +2453,7 @@ static int step_general(const dpclip_layer* layers, const dpclip_model_layer* ot
     k = any_group ? 1 : 0;
     for (int l = 0; l < L; ++l) {
         const dpclip_layer& y = layers[l];
-        const bool is_other = other && other[l].kind != DPCLIP_KIND_DENSE;
+        const bool is_other = other_kind(l);
         if (!is_other && ((t1.active && y.T == 1) || (track && in_grad_group[l]))) continue;
         const SmBudgetScope share(track ? budget[l] : 0);
         const int b = k++ % lanes.n;
@@ -2227,7 +2475,7 @@ static int step_general(const dpclip_layer* layers, const dpclip_model_layer* ot
         NoiseSpec ns = {sigma * C, seed, stream_id0 + 2ull * l, stream_id0 + 2ull * l + 1};
         bool noise_done = false;
         rc = clipped_grad_impl(y.A, y.lda, y.Zbar, y.ldz, B, y.T, y.d_in, y.d_out, dtype, clip, y.gW, y.ldg, gb,
-                               workspace, workspace_bytes, &ns, &noise_done, (cudaStream_t)stream);
+                               workspace, workspace_bytes, &ns, &noise_done, (cudaStream_t)stream, split && split[l]);
         if (rc) return rc;
         if (!noise_done) {
             rc = dpclip_add_noise(y.gW, (size_t)y.d_out * y.d_in, sigma, C, seed, ns.sid_w, stream);
@@ -2264,13 +2512,27 @@ static int step_args_ok(const void* layers, int L, int B, dpclip_dtype dtype, fl
     return DPCLIP_OK;
 }
 
+// Plans and launches the staging of a step when the workspace has room for the copies (sp.active says so); the
+// lanes' scratch then ends where the copies begin.
+static int stage_step(StagePlan& sp, const dpclip_layer* layers, const dpclip_model_layer* other, int L, int B,
+                      dpclip_dtype dtype, Lanes& lanes, bool t1_too) {
+    if (!lanes.ws[0] || !stage_plan(sp, layers, other, L, B, dtype, static_cast<char*>(lanes.ws[0]), t1_too)) return DPCLIP_OK;
+    if (lanes.ws_bytes < sp.bytes) { sp.active = false; return DPCLIP_OK; }
+    lanes.ws_bytes = sp.scratch;
+    return launch_stage(sp, lanes.st[0]);
+}
+
 static int step_dense(const dpclip_layer* layers, int L, int B, dpclip_dtype dtype, float C, float sigma,
                       unsigned long long seed, unsigned long long stream_id0, float* sq_layers, float* clip,
                       float* norms, Lanes& lanes) {
-    const int rc = try_fused_t1_step(layers, L, B, dtype, C, sigma, seed, stream_id0, sq_layers, clip, norms, lanes.ws[0],
-                                     lanes.ws_bytes, lanes.st[0]);
+    StagePlan sp;
+    int rc = stage_step(sp, layers, nullptr, L, B, dtype, lanes, true);
+    if (rc) return rc;
+    rc = try_fused_t1_step(sp.active ? sp.eff : layers, L, B, sp.active ? sp.t1_dtype : dtype, C, sigma, seed, stream_id0,
+                           sq_layers, clip, norms, lanes.ws[0], lanes.ws_bytes, lanes.st[0]);
     if (rc <= 0) return rc;                  // done (0) or argument error (< 0); 1 = take the general path
-    return step_general(layers, nullptr, L, B, dtype, C, sigma, seed, stream_id0, sq_layers, clip, norms, lanes);
+    return step_general(layers, nullptr, L, B, dtype, C, sigma, seed, stream_id0, sq_layers, clip, norms, lanes,
+                        sp.active ? &sp : nullptr);
 }
 
 static int step_model(const dpclip_model_layer* layers, int L, int B, dpclip_dtype dtype, float C, float sigma,
@@ -2287,7 +2549,11 @@ static int step_model(const dpclip_model_layer* layers, int L, int B, dpclip_dty
         all_dense = false;
     }
     if (all_dense) return step_dense(dense, L, B, dtype, C, sigma, seed, stream_id0, sq_layers, clip, norms, lanes);
-    return step_general(dense, layers, L, B, dtype, C, sigma, seed, stream_id0, sq_layers, clip, norms, lanes);
+    StagePlan sp;
+    const int rc = stage_step(sp, dense, layers, L, B, dtype, lanes, true);
+    if (rc) return rc;
+    return step_general(dense, layers, L, B, dtype, C, sigma, seed, stream_id0, sq_layers, clip, norms, lanes,
+                        sp.active ? &sp : nullptr);
 }
 
 int dpclip_step(const dpclip_layer* layers, int L, int B, dpclip_dtype dtype, float C, float sigma,
@@ -2339,6 +2605,15 @@ int dpclip_step_per_layer(const dpclip_layer* layers, int L, int B, dpclip_dtype
     constexpr int kMaxTracked = 64;
     int in_gram[kMaxTracked], in_pairs[kMaxTracked];
     const bool track = L <= kMaxTracked;
+    StagePlan sp;
+    {
+        Lanes lanes;
+        one_lane(lanes, workspace, workspace_bytes, stream);
+        if ((rc = stage_step(sp, layers, nullptr, L, B, dtype, lanes, false))) return rc;
+        workspace_bytes = lanes.ws_bytes;
+    }
+    const bool* split = sp.active ? sp.split : nullptr;
+    if (sp.active) layers = sp.eff;
     if (track) {
         rc = dpclip_gram_layers_sqnorms(layers, L, B, dtype, sq_layers, in_gram, workspace, workspace_bytes, stream);
         if (rc) return rc;
@@ -2355,7 +2630,7 @@ int dpclip_step_per_layer(const dpclip_layer* layers, int L, int B, dpclip_dtype
         for (int l = 0; l < L; ++l) th.C[l] = C_layer[l];
         factors_rows_kernel<<<L, 256, 0, (cudaStream_t)stream>>>(sq_layers, (long)B, B, th, clip_layers, norms_layers);
         if (launch_status()) return DPCLIP_ERR_CUDA;
-        rc = shared_clipped_grad_launches(layers, L, B, dtype, clip_layers, (long)B, C_total, sigma, seed, stream_id0,
+        rc = shared_clipped_grad_launches(layers, split, L, B, dtype, clip_layers, (long)B, C_total, sigma, seed, stream_id0,
                                           in_pairs, workspace, workspace_bytes, stream);
         if (rc) return rc;
     } else {
@@ -2372,7 +2647,7 @@ int dpclip_step_per_layer(const dpclip_layer* layers, int L, int B, dpclip_dtype
         NoiseSpec ns = {sigma * C_total, seed, stream_id0 + 2ull * l, stream_id0 + 2ull * l + 1};
         bool noise_done = false;
         rc = clipped_grad_impl(y.A, y.lda, y.Zbar, y.ldz, B, y.T, y.d_in, y.d_out, dtype, clip_layers + (size_t)l * B, y.gW,
-                               y.ldg, gb, workspace, workspace_bytes, &ns, &noise_done, (cudaStream_t)stream);
+                               y.ldg, gb, workspace, workspace_bytes, &ns, &noise_done, (cudaStream_t)stream, split && split[l]);
         if (rc) return rc;
         if (!noise_done) {
             rc = dpclip_add_noise(y.gW, (size_t)y.d_out * y.d_in, sigma, C_total, seed, ns.sid_w, stream);
@@ -2395,7 +2670,9 @@ size_t dpclip_model_workspace_bytes(const dpclip_model_layer* layers, int L, int
             if (layers[l].kind == DPCLIP_KIND_DENSE) dense[l] = layers[l].layer;
             else memset(&dense[l], 0, sizeof(dense[l]));
         }
-        ws = dpclip_step_workspace_bytes(dense, L, B, dtype);
+        ws = step_scratch_bytes(dense, L, B, dtype);
+        const size_t staged = staged_workspace_bytes(dense, layers, L, B, dtype);
+        if (staged > ws) ws = staged;
     }
     for (int l = 0; l < L; ++l) {
         const dpclip_layer& y = layers[l].layer;

@@ -168,7 +168,9 @@ __device__ __forceinline__ bool grid_barrier_arrive_and_wait(unsigned int* ctr, 
 // T = float: error-compensated tf32 as described above.  T = __nv_bfloat16: the same pipeline with one
 // kind::f16 MMA per K = 16 step and no low planes (products of bf16 inputs are exact in fp32; the only
 // rounding is that of c * zb back to bf16); a stage holds 32 rows as two 64-column boxes per operand.
-template <bool ONE_LAUNCH, typename T = float>
+// QUADS: every layer's d_in is a multiple of four, so four outputs of a row are one Philox block.  A kernel of its own:
+// the code of the general case in the same kernel cost the aligned models 3 % (registers).
+template <bool ONE_LAUNCH, typename T, bool QUADS>
 __global__ void __launch_bounds__(f1::THREADS, 1)
 t1_all_grads_tf32_kernel(const __grid_constant__ f1::Params q) {
     using namespace f1;

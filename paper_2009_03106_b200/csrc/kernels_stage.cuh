@@ -1,0 +1,212 @@
+// Operand staging: layer inputs that the tensor-core kernels cannot address (rows that are not 16-byte multiples,
+// convolutions given by their feature map, dL/dZ held channel-major) are rewritten ONCE per step, all of a model's in
+// one launch, as row-major matrices whose rows start on 16-byte boundaries.  The norm and the clipped-sum stage then
+// both read the copies through TMA.
+//
+//   rows       [rows][ld] -> [rows][ld'], same type (or bf16 -> fp32 for T = 1 models, see the dispatch)
+//   transpose  [B][M][T]  -> [B*T][ld'] (M = d_out): dL/dZ of a convolution as back-propagation holds it
+//   im2col     [B][C][H][W] -> [B*T][ld'], columns (c, ky, kx), zeros for the padding: the patch matrix of Sec.
+//              "Convolutional Layers"
+//
+// Bound: bytes.  The copies of one step are a few to a few dozen MB and mostly stay in the 126 MB L2 until the two
+// stages have read them.  Columns between the width and ld' need no value: the tensor maps end at the width.
+#pragma once
+#include "common.cuh"
+
+namespace dpclip {
+namespace stage {
+
+enum Kind : int { ROWS = 0, ROWS_TO_F32 = 1, TRANSPOSE = 2, IM2COL = 3 };
+constexpr int MAX_JOBS = 32;
+constexpr int THREADS = 256;
+constexpr int ROWS_UNROLL = 4;                 // 16-byte output chunks per thread
+constexpr int TILE_T = 64, TILE_M = 64;        // transpose tile
+constexpr int IM_ROWS = 32;                    // im2col: patch rows per CTA (one per lane)
+constexpr int SMEM_MAX = 160 * 1024;
+
+struct Job {
+    int kind, es;                  // es = bytes of an input element
+    const void* src; void* dst;
+    long src_ld; int dst_ld;       // elements (of the input, of the output)
+    int rows, cols;                // output rows and width
+    int blk_begin;
+    // TRANSPOSE / IM2COL
+    int T, tiles_a, tiles_b;       // TRANSPOSE: tiles along T and along M; IM2COL: channel blocks in tiles_b
+    int C, H, W, kh, kw, stride, pad, Wo, ct, pitch;     // IM2COL: ct channels per CTA, pitch = shared-memory row bytes
+};
+struct Launch { Job job[MAX_JOBS]; int n, blocks; };
+
+// eight bf16 elements that start at any 2-byte boundary; reads exactly those sixteen bytes
+__device__ __forceinline__ uint4 load_bf16x8(const uint16_t* p) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(p);
+    uint4 v;
+    if ((a & 7) == 0) {
+        const uint2 lo = __ldg(reinterpret_cast<const uint2*>(p)), hi = __ldg(reinterpret_cast<const uint2*>(p) + 1);
+        v = make_uint4(lo.x, lo.y, hi.x, hi.y);
+    } else if ((a & 3) == 0) {
+        const uint32_t* w = reinterpret_cast<const uint32_t*>(p);
+        v = make_uint4(__ldg(w), __ldg(w + 1), __ldg(w + 2), __ldg(w + 3));
+    } else {
+        const uint32_t* w = reinterpret_cast<const uint32_t*>(p + 1);
+        const uint32_t e0 = __ldg(p), w0 = __ldg(w), w1 = __ldg(w + 1), w2 = __ldg(w + 2), e7 = __ldg(p + 7);
+        v = make_uint4(e0 | (w0 << 16), __funnelshift_l(w0, w1, 16), __funnelshift_l(w1, w2, 16), (w2 >> 16) | (e7 << 16));
+    }
+    return v;
+}
+
+__device__ __forceinline__ void rows_job(const Job& j, int blk) {
+    const bool cvt = j.kind == ROWS_TO_F32;
+    const int per = (j.es == 4 || cvt) ? 4 : 8;              // elements per 16-byte output chunk
+    const uint32_t cpr = (uint32_t)j.dst_ld / per;           // chunks per output row
+    const uint32_t total = (uint32_t)j.rows * cpr;
+    uint4 out[ROWS_UNROLL];
+#pragma unroll
+    for (int u = 0; u < ROWS_UNROLL; ++u) {
+        const uint32_t c = (uint32_t)(blk * ROWS_UNROLL + u) * THREADS + threadIdx.x;
+        out[u] = make_uint4(0, 0, 0, 0);
+        if (c >= total) continue;
+        const uint32_t row = c / cpr;
+        const int col = (int)(c - row * cpr) * per;
+        const int n = min(per, j.cols - col);
+        uint32_t w[4] = {0, 0, 0, 0};
+        if (j.es == 4) {
+            const uint32_t* p = static_cast<const uint32_t*>(j.src) + (size_t)row * j.src_ld + col;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) if (e < n) w[e] = __ldg(p + e);
+        } else {
+            const uint16_t* p = static_cast<const uint16_t*>(j.src) + (size_t)row * j.src_ld + col;
+            if (cvt) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) if (e < n) w[e] = (uint32_t)__ldg(p + e) << 16;
+            } else if (n == 8) {
+                const uint4 v = load_bf16x8(p);
+                w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
+            } else {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) if (e < n) w[e >> 1] |= (uint32_t)__ldg(p + e) << (16 * (e & 1));
+            }
+        }
+        out[u] = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+#pragma unroll
+    for (int u = 0; u < ROWS_UNROLL; ++u) {
+        const uint32_t c = (uint32_t)(blk * ROWS_UNROLL + u) * THREADS + threadIdx.x;
+        if (c < total) static_cast<uint4*>(j.dst)[c] = out[u];
+    }
+}
+
+// 64 positions x 64 channels through shared memory; rows of the tile are 64 + 2 elements (bf16) / 64 + 1 (fp32) long, so
+// that neither the writes along T nor the reads along M fall on one bank
+template <typename E>
+__device__ __forceinline__ void transpose_job(const Job& j, int blk, uint8_t* smem) {
+    constexpr int PITCH = sizeof(E) == 2 ? TILE_T + 2 : TILE_T + 1;
+    E* tile = reinterpret_cast<E*>(smem);
+    const int M = j.cols;
+    const int per_ex = j.tiles_a * j.tiles_b;
+    const int b = blk / per_ex, r = blk - b * per_ex;
+    const int m0 = (r / j.tiles_a) * TILE_M, t0 = (r % j.tiles_a) * TILE_T;
+    const E* src = static_cast<const E*>(j.src) + (size_t)b * M * j.T;
+    const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
+    E v[TILE_M / 4];
+#pragma unroll
+    for (int i = 0; i < TILE_M / 4; ++i) {
+        const int m = m0 + ty + 4 * i, t = t0 + tx;
+        v[i] = (m < M && t < j.T) ? __ldg(src + (size_t)m * j.T + t) : E(0);
+    }
+#pragma unroll
+    for (int i = 0; i < TILE_M / 4; ++i) tile[(ty + 4 * i) * PITCH + tx] = v[i];
+    __syncthreads();
+    constexpr int PER = 16 / sizeof(E), CH = TILE_M / PER;          // chunks of a 64-channel row
+    for (int k = threadIdx.x; k < TILE_T * CH; k += THREADS) {
+        const int c = k % CH, t = k / CH;
+        const int m = m0 + c * PER;
+        if (t0 + t >= j.T || m >= M) continue;
+        union { E e[PER]; uint4 q; } o;
+#pragma unroll
+        for (int i = 0; i < PER; ++i) o.e[i] = tile[(c * PER + i) * PITCH + t];
+        E* dst = static_cast<E*>(j.dst) + ((size_t)b * j.T + t0 + t) * j.dst_ld + m;
+        if ((j.dst_ld % PER) == 0) {
+            *reinterpret_cast<uint4*>(dst) = o.q;
+        } else {
+#pragma unroll
+            for (int i = 0; i < PER; ++i) if (m + i < M) dst[i] = o.e[i];
+        }
+    }
+}
+
+// 32 patch rows (lane = row, so that neighbouring lanes read neighbouring pixels) x ct channels; the window of a (row,
+// channel) goes to kh*kw consecutive elements of the row's line in shared memory, and the lines leave in 16-byte chunks
+template <typename E>
+__device__ __forceinline__ void im2col_job(const Job& j, int blk, uint8_t* smem) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int rb = blk / j.tiles_b, cb = blk - rb * j.tiles_b;
+    const int row0 = rb * IM_ROWS, c0 = cb * j.ct;
+    const int kk = j.kh * j.kw;
+    const int nc = min(j.ct, j.C - c0);
+    const int row = row0 + lane;
+    {
+        const bool ok = row < j.rows;
+        const int b = ok ? row / j.T : 0, t = ok ? row - b * j.T : 0;
+        const int yo = t / j.Wo, xo = t - yo * j.Wo;
+        const int y0 = yo * j.stride - j.pad, x0 = xo * j.stride - j.pad;
+        const E* src = static_cast<const E*>(j.src) + (size_t)b * j.C * j.H * j.W;
+        E* line = reinterpret_cast<E*>(smem + lane * j.pitch);
+        if (kk == 9 && j.kw == 3) {
+            for (int ci = warp; ci < nc; ci += THREADS / 32) {
+                const E* x = src + (size_t)(c0 + ci) * j.H * j.W;
+                E v[9];
+#pragma unroll
+                for (int k = 0; k < 9; ++k) {
+                    const int y = y0 + k / 3, xx = x0 + k % 3;
+                    v[k] = (ok && y >= 0 && y < j.H && xx >= 0 && xx < j.W) ? __ldg(x + y * j.W + xx) : E(0);
+                }
+#pragma unroll
+                for (int k = 0; k < 9; ++k) line[ci * 9 + k] = v[k];
+            }
+        } else {
+            for (int ci = warp; ci < nc; ci += THREADS / 32) {
+                const E* x = src + (size_t)(c0 + ci) * j.H * j.W;
+                for (int ky = 0, k = 0; ky < j.kh; ++ky)
+                    for (int kx = 0; kx < j.kw; ++kx, ++k) {
+                        const int y = y0 + ky, xx = x0 + kx;
+                        line[ci * kk + k] = (ok && y >= 0 && y < j.H && xx >= 0 && xx < j.W) ? __ldg(x + y * j.W + xx) : E(0);
+                    }
+            }
+        }
+    }
+    __syncthreads();
+    constexpr int PER = 16 / sizeof(E);
+    const int width = nc * kk;
+    if ((j.dst_ld % PER) == 0) {
+        const int cpr = (width + PER - 1) / PER;                  // the last chunk may run into the row's padding
+        for (int k = threadIdx.x; k < IM_ROWS * cpr; k += THREADS) {
+            const int r = k / cpr, c = k - r * cpr;
+            if (row0 + r >= j.rows) continue;
+            const uint32_t* s = reinterpret_cast<const uint32_t*>(smem + r * j.pitch + c * 16);
+            const uint4 v = make_uint4(s[0], s[1], s[2], s[3]);
+            *reinterpret_cast<uint4*>(static_cast<E*>(j.dst) + (size_t)(row0 + r) * j.dst_ld + c0 * kk + c * PER) = v;
+        }
+    } else {
+        for (int k = threadIdx.x; k < IM_ROWS * width; k += THREADS) {
+            const int r = k / width, c = k - r * width;
+            if (row0 + r >= j.rows) continue;
+            static_cast<E*>(j.dst)[(size_t)(row0 + r) * j.dst_ld + c0 * kk + c] = reinterpret_cast<const E*>(smem + r * j.pitch)[c];
+        }
+    }
+}
+}  // namespace stage
+
+__global__ void __launch_bounds__(stage::THREADS)
+stage_operands_kernel(const __grid_constant__ stage::Launch q) {
+    using namespace stage;
+    extern __shared__ __align__(16) uint8_t stage_smem[];
+    int k = 0;
+    while (k + 1 < q.n && (int)blockIdx.x >= q.job[k + 1].blk_begin) ++k;
+    const Job& j = q.job[k];
+    const int blk = blockIdx.x - j.blk_begin;
+    if (j.kind == ROWS || j.kind == ROWS_TO_F32) rows_job(j, blk);
+    else if (j.kind == TRANSPOSE) { if (j.es == 2) transpose_job<uint16_t>(j, blk, stage_smem); else transpose_job<uint32_t>(j, blk, stage_smem); }
+    else { if (j.es == 2) im2col_job<uint16_t>(j, blk, stage_smem); else im2col_job<uint32_t>(j, blk, stage_smem); }
+}
+
+}  // namespace dpclip

@@ -140,6 +140,30 @@ __device__ __forceinline__ void box_muller(uint32_t xa, uint32_t xb, float& n0, 
     n1 = -r * s;
 }
 
+__device__ __forceinline__ void normals_block(size_t q, uint32_t s0, uint32_t s1, uint32_t k0, uint32_t k1, float (&z)[4]) {
+    const PhiloxBlock b = philox_block((uint32_t)q, (uint32_t)(q >> 32), s0, s1, k0, k1);
+    box_muller(b.v[0], b.v[1], z[0], z[1]);
+    box_muller(b.v[2], b.v[3], z[2], z[3]);
+}
+// element u of the four that start o elements into e[0..3], y[0..3]
+__device__ __forceinline__ float shifted(const float (&e)[4], const float (&y)[4], int u, int o) {
+    const float a1 = u + 1 < 4 ? e[(u + 1) & 3] : y[(u + 1) & 3], a2 = u + 2 < 4 ? e[(u + 2) & 3] : y[(u + 2) & 3],
+                a3 = u + 3 < 4 ? e[(u + 3) & 3] : y[(u + 3) & 3];
+    return o == 0 ? e[u] : o == 1 ? a1 : o == 2 ? a2 : a3;
+}
+// Elements j .. j + 3 of noise stream (s0, s1): one Philox block when j is a multiple of four, else parts of two.
+__device__ __forceinline__ void normals_at(size_t j, uint32_t s0, uint32_t s1, uint32_t k0, uint32_t k1, float (&z)[4]) {
+    const int o = (int)(j & 3);
+    normals_block(j >> 2, s0, s1, k0, k1, z);
+    if (o) {
+        float y[4];
+        normals_block((j >> 2) + 1, s0, s1, k0, k1, y);
+        const float e[4] = {z[0], z[1], z[2], z[3]};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) z[u] = shifted(e, y, u, o);
+    }
+}
+
 __global__ void __launch_bounds__(256)
 noise_kernel(float* __restrict__ g, size_t n, float scale, uint32_t k0, uint32_t k1,
              uint32_t s0, uint32_t s1, int vec_ok) {

@@ -638,13 +638,18 @@ constexpr int SMEM_BYTES = 192 * 1024 + 256 + OUT_STAGE_BYTES + 1024;
 //           less L2->SM traffic per flop, for layers where that traffic is the limit.
 // Stages are 64 rows: with 32-row stages (twice as many slots) the large tile ran 10-15 % slower, the
 // per-stage cost of the transform warps (barrier round trips, proxy fence) weighing twice.
-template <int MT> struct Cfg {
+// SPLIT (GRAD, MT = 1): the scaled operand c * zb is held as two bf16 terms, hi + lo (relative error 2^-18 instead of
+//           2^-9), and every stage whose rows are not all unscaled runs a second set of MMAs on the lo plane.  For layers
+//           that would otherwise run on the fp32 ALUs, where the product is taken in fp32; 3 stages of 64 KB.
+template <int MT, bool SPLIT = false> struct Cfg {
+    static_assert(!SPLIT || MT == 1, "two planes of a 256-row tile leave room for two stages only");
     static constexpr int BM = 128 * MT;
     static constexpr int BK = 64;                                 // rows per stage
     static constexpr int CHUNK_BYTES = BK * 128;                  // one TMA box: BK rows x 64 bf16 columns
     static constexpr int A_BYTES = (BM / 64) * CHUNK_BYTES;       // Zb tile
     static constexpr int B_BYTES = (BN / 64) * CHUNK_BYTES;       // A tile
-    static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
+    static constexpr int LOAD_BYTES = A_BYTES + B_BYTES;
+    static constexpr int STAGE_BYTES = LOAD_BYTES + (SPLIT ? A_BYTES : 0);
     static constexpr int STAGES = (192 * 1024) / STAGE_BYTES;
     static constexpr int NBUF = MT == 1 ? 2 : 1;
 };
@@ -698,11 +703,35 @@ __device__ __forceinline__ Item decode(const Params& p, int item) {
 }
 }  // namespace zta
 
-template <int MT>
+// Packed bf16 scaling of eight values: f = f_hi + f_lo (two bf16); z*f_lo is tiny, so the fused multiply-add
+// z*f_hi + (z*f_lo) rounds the product once.
+__device__ __forceinline__ void scale_bf16x8(uint4& v, float f) {
+    const __nv_bfloat16 fh = __float2bfloat16_rn(f);
+    const __nv_bfloat16 fl = __float2bfloat16_rn(f - __bfloat162float(fh));
+    const __nv_bfloat162 fh2 = __halves2bfloat162(fh, fh), fl2 = __halves2bfloat162(fl, fl);
+    __nv_bfloat162* z2 = reinterpret_cast<__nv_bfloat162*>(&v);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) z2[u] = __hfma2(z2[u], fh2, __hmul2(z2[u], fl2));
+}
+// The product in two bf16 terms: v becomes round(f*v), lo what is left of the fp32 product.
+__device__ __forceinline__ void scale_bf16x8_split(uint4& v, uint4& lo, float f) {
+    uint32_t* w = reinterpret_cast<uint32_t*>(&v);
+    uint32_t* l = reinterpret_cast<uint32_t*>(&lo);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const float x = __uint_as_float(w[u] << 16) * f, y = __uint_as_float(w[u] & 0xFFFF0000u) * f;
+        const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
+        w[u] = *reinterpret_cast<const uint32_t*>(&h);
+        const __nv_bfloat162 r = __floats2bfloat162_rn(x - __uint_as_float(w[u] << 16), y - __uint_as_float(w[u] & 0xFFFF0000u));
+        l[u] = *reinterpret_cast<const uint32_t*>(&r);
+    }
+}
+
+template <int MT, bool SPLIT>
 __global__ void __launch_bounds__(zta::THREADS, 1)
 zta_tc_kernel(const __grid_constant__ zta::Maps maps, const zta::Params p) {
     using namespace zta;
-    using C = Cfg<MT>;
+    using C = Cfg<MT, SPLIT>;
     constexpr int STAGES = C::STAGES, STAGE_BYTES = C::STAGE_BYTES, A_BYTES = C::A_BYTES, NBUF = C::NBUF;
     constexpr int BK = C::BK, CHUNK_BYTES = C::CHUNK_BYTES;
     extern __shared__ uint8_t smem_raw[];
@@ -714,6 +743,7 @@ zta_tc_kernel(const __grid_constant__ zta::Maps maps, const zta::Params p) {
     uint64_t* acc_empty = acc_full + 2;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    volatile int* has_lo = abort_flag + 1;                                       // SPLIT: [STAGES], the stage's lo plane is in use
     float4* out_stage = reinterpret_cast<float4*>(smem + STAGES * STAGE_BYTES + 256);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -750,7 +780,7 @@ zta_tc_kernel(const __grid_constant__ zta::Maps maps, const zta::Params p) {
                     DPCLIP_TRACE_AT(0, tr); ++tr;
                     uint8_t* dst = smem + stage * STAGE_BYTES;
                     const int y = w.row_begin + kb * BK;
-                    mbar_arrive_expect_tx(&full[stage], STAGE_BYTES);
+                    mbar_arrive_expect_tx(&full[stage], C::LOAD_BYTES);
 #pragma unroll
                     for (int c = 0; c < C::BM / 64; ++c)
                         tma_load_2d(dst + c * CHUNK_BYTES, map_z, &full[stage], w.m0 + c * 64, y);
@@ -793,6 +823,13 @@ zta_tc_kernel(const __grid_constant__ zta::Maps maps, const zta::Params p) {
                             mma_bf16_ss(tmem_base + (buf * MT + h) * BN, da, db, idesc,
                                         (kb == 0 && k4 == 0) ? 0u : 1u);
                         }
+                    }
+                    if (SPLIT && has_lo[stage]) {
+#pragma unroll
+                        for (int k4 = 0; k4 < BK / 16; ++k4)
+                            mma_bf16_ss(tmem_base + buf * BN,
+                                        make_smem_desc_sw128(a_addr + C::LOAD_BYTES + k4 * 2048, CHUNK_BYTES, 1024),
+                                        make_smem_desc_sw128(b_addr + k4 * 2048, CHUNK_BYTES, 1024), idesc, 1u);
                     }
                     mma_commit(&empty[stage]);
                     if (++stage == STAGES) { stage = 0; phase ^= 1; }
@@ -849,16 +886,6 @@ zta_tc_kernel(const __grid_constant__ zta::Maps maps, const zta::Params p) {
                 if (!ok) break;
                 if (t == 0) { DPCLIP_TRACE_AT(1, tr); ++tr; }
                 uint8_t* zt = smem + stage * STAGE_BYTES;
-                // packed bf16 scaling: f = f_hi + f_lo (two bf16); z*f_lo is tiny, so the fused
-                // multiply-add z*f_hi + (z*f_lo) rounds the product once
-                auto scale8 = [](uint4& v, float f) {
-                    const __nv_bfloat16 fh = __float2bfloat16_rn(f);
-                    const __nv_bfloat16 fl = __float2bfloat16_rn(f - __bfloat162float(fh));
-                    const __nv_bfloat162 fh2 = __halves2bfloat162(fh, fh), fl2 = __halves2bfloat162(fl, fl);
-                    __nv_bfloat162* z2 = reinterpret_cast<__nv_bfloat162*>(&v);
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) z2[u] = __hfma2(z2[u], fh2, __hmul2(z2[u], fl2));
-                };
                 auto add8 = [](float* c, const uint4& v) {
                     const uint32_t wds[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
@@ -867,7 +894,30 @@ zta_tc_kernel(const __grid_constant__ zta::Maps maps, const zta::Params p) {
                         c[2 * u + 1] += __uint_as_float(wds[u] & 0xFFFF0000u);
                     }
                 };
-                if (uniform) {
+                if (SPLIT) {
+                    // every warp sees all rows of the stage, so all agree on whether the lo plane is needed
+                    bool any = false;
+#pragma unroll
+                    for (int i = 0; i < NR; ++i) any = any || (uniform ? fr[0] : fr[i]) != 1.f;
+                    any = __any_sync(0xFFFFFFFFu, any);
+                    if (t == 0) has_lo[stage] = any ? 1 : 0;
+                    if (any || bias_here) {
+                        uint4 v[NR];
+#pragma unroll
+                        for (int i = 0; i < NR; ++i) v[i] = *reinterpret_cast<const uint4*>(zt + off + i * 2048);
+#pragma unroll
+                        for (int i = 0; i < NR; ++i) {
+                            const float f = uniform ? fr[0] : fr[i];
+                            uint4 lo = make_uint4(0u, 0u, 0u, 0u);
+                            if (f != 1.f) {
+                                scale_bf16x8_split(v[i], lo, f);
+                                *reinterpret_cast<uint4*>(zt + off + i * 2048) = v[i];
+                            }
+                            if (any) *reinterpret_cast<uint4*>(zt + C::LOAD_BYTES + off + i * 2048) = lo;
+                            if (bias_here) { add8(cs[0], v[i]); if (f != 1.f) add8(cs[0], lo); }
+                        }
+                    }
+                } else if (uniform) {
                     // one factor for the whole stage: all loads are issued before the first store, so the
                     // stage costs one shared-memory round trip instead of one per row
                     const float f = fr[0];
@@ -883,7 +933,7 @@ zta_tc_kernel(const __grid_constant__ zta::Maps maps, const zta::Params p) {
                             for (int h = 0; h < MT; ++h)
 #pragma unroll
                                 for (int i = 0; i < NR; ++i) {
-                                    scale8(v[h][i], f);
+                                    scale_bf16x8(v[h][i], f);
                                     *reinterpret_cast<uint4*>(zt + h * 2 * CHUNK_BYTES + off + i * 2048) = v[h][i];
                                 }
                         }
@@ -912,7 +962,7 @@ zta_tc_kernel(const __grid_constant__ zta::Maps maps, const zta::Params p) {
                             if (fr[i] != 1.f) {
 #pragma unroll
                                 for (int h = 0; h < MT; ++h) {
-                                    scale8(v[h][i], fr[i]);
+                                    scale_bf16x8(v[h][i], fr[i]);
                                     *reinterpret_cast<uint4*>(zt + h * 2 * CHUNK_BYTES + off + i * 2048) = v[h][i];
                                 }
                             }
@@ -1051,8 +1101,7 @@ zta_tc_kernel(const __grid_constant__ zta::Maps maps, const zta::Params p) {
 // Second stage of the split-row clipped sum: adds the partial tiles of every
 // output tile in a fixed order (deterministic, no atomics) and writes gW / gb.
 // When noise_scale > 0 the Gaussian noise of element j = m*d_in + n is added in
-// the same pass (requires dense rows and d_in % 4 == 0, so that a float4 of the
-// output is exactly one Philox block).
+// the same pass (requires dense rows).
 // ---------------------------------------------------------------------------
 struct ReduceParams {
     const float* part; const float* bias_part;
@@ -1133,13 +1182,10 @@ reduce_partials_kernel(const ReduceParams q) {
         }
         if (!live || gy != 0) continue;
         if (p.noise_scale > 0.f) {
-            const size_t q = ((size_t)m * p.d_in + n) >> 2;
-            PhiloxBlock b = philox_block((uint32_t)q, (uint32_t)(q >> 32), p.sw0, p.sw1, p.k0, p.k1);
-            float z0, z1, z2, z3;
-            box_muller(b.v[0], b.v[1], z0, z1);
-            box_muller(b.v[2], b.v[3], z2, z3);
-            acc.x = fmaf(p.noise_scale, z0, acc.x); acc.y = fmaf(p.noise_scale, z1, acc.y);
-            acc.z = fmaf(p.noise_scale, z2, acc.z); acc.w = fmaf(p.noise_scale, z3, acc.w);
+            float z[4];
+            normals_at((size_t)m * p.d_in + n, p.sw0, p.sw1, p.k0, p.k1, z);
+            acc.x = fmaf(p.noise_scale, z[0], acc.x); acc.y = fmaf(p.noise_scale, z[1], acc.y);
+            acc.z = fmaf(p.noise_scale, z[2], acc.z); acc.w = fmaf(p.noise_scale, z[3], acc.w);
         }
         float* dst = p.gW + (size_t)m * p.ldg + n;
         if (p.vec_ok && n + 4 <= p.d_in) {

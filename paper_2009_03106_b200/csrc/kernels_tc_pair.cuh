@@ -63,12 +63,17 @@ constexpr int BK = 64;                         // rows per stage
 constexpr int CHUNK_BYTES = BK * 128;          // one TMA box: BK rows x 64 bf16 columns
 constexpr int Z_BYTES = (BM_CTA / 64) * CHUNK_BYTES;     // 32 KB
 constexpr int A_BYTES = (BN_CTA / 64) * CHUNK_BYTES;     // 16 KB
-constexpr int STAGE_BYTES = Z_BYTES + A_BYTES;           // 48 KB
-constexpr int STAGES = 4;
+constexpr int LOAD_BYTES = Z_BYTES + A_BYTES;            // 48 KB
+// SPLIT: the scaled A half in two bf16 terms, hi + lo (see zta::Cfg), for layers that would otherwise run on the fp32
+// ALUs: 64 KB per stage, three stages instead of four, and a second set of MMAs where a row of the stage is scaled.
+template <bool SPLIT> struct Cfg {
+    static constexpr int STAGE_BYTES = LOAD_BYTES + (SPLIT ? A_BYTES : 0);
+    static constexpr int STAGES = 192 * 1024 / STAGE_BYTES;
+};
 constexpr int N_TRANSFORM_WARPS = 8, N_EPILOGUE_WARPS = 8;
 constexpr int THREADS = 64 + 32 * (N_TRANSFORM_WARPS + N_EPILOGUE_WARPS);
 constexpr int OUT_STAGE_BYTES = N_EPILOGUE_WARPS * 4096;
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 256 + OUT_STAGE_BYTES + 1024;
+constexpr int SMEM_BYTES = 192 * 1024 + 256 + OUT_STAGE_BYTES + 1024;
 constexpr int MAX_LAYERS = zta::MAX_LAYERS;
 constexpr size_t SEG_ELEMS = (size_t)BM * BN;  // fp32 elements of a segment's partial tile
 
@@ -76,7 +81,7 @@ struct Layer {
     int d_in, d_out;
     int tiles_n;                   // pair tiles along d_in
     int tile_base, tiles;          // this layer's tiles are tile_base .. tile_base + tiles - 1 of the launch
-    int do_bias;
+    int do_bias, split;
     const float* clip;             // [B] factors of THIS layer, or NULL (all ones): one vector for the whole model under
                                    // global clipping, one per layer under per-layer clipping
     float* gW; float* gb;          // outputs (dense rows: ldg = d_in for the noise; see ldg)
@@ -140,9 +145,11 @@ __device__ __forceinline__ Seg segment_at(const Params& p, long u, long u_end, i
 }
 }  // namespace ztp
 
+template <bool SPLIT>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(ztp::THREADS, 1)
 zta_pair_kernel(const __grid_constant__ zta::Maps maps, const __grid_constant__ ztp::Params p) {
     using namespace ztp;
+    constexpr int STAGES = Cfg<SPLIT>::STAGES, STAGE_BYTES = Cfg<SPLIT>::STAGE_BYTES;
     extern __shared__ uint8_t smem_raw[];
     // 1024-byte aligned by an OFFSET from the array (keeps the accesses in the shared state space); the offset
     // is the same in both CTAs (same kernel, same static layout), which the pair's descriptors rely on
@@ -155,6 +162,7 @@ zta_pair_kernel(const __grid_constant__ zta::Maps maps, const __grid_constant__ 
     uint64_t* zfree = acc_empty + 1;                                             // bias warps done reading the Zb tile (own)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(zfree + STAGES);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    volatile int* has_lo = abort_flag + 1;                                       // SPLIT: [STAGES], the stage's lo plane is in use
     float4* out_stage = reinterpret_cast<float4*>(smem + STAGES * STAGE_BYTES + 256);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -206,7 +214,7 @@ zta_pair_kernel(const __grid_constant__ zta::Maps maps, const __grid_constant__ 
                     DPCLIP_TRACE_AT(0, tr); ++tr;
                     uint8_t* dst = smem + stage * STAGE_BYTES;
                     const int y = kb * BK;
-                    mbar_arrive_expect_tx(&full[stage], STAGE_BYTES);
+                    mbar_arrive_expect_tx(&full[stage], LOAD_BYTES);
 #pragma unroll
                     for (int c = 0; c < BM_CTA / 64; ++c)
                         tma_load_2d(dst + c * CHUNK_BYTES, map_z, &full[stage], mz + c * 64, y);
@@ -249,6 +257,18 @@ zta_pair_kernel(const __grid_constant__ zta::Maps maps, const __grid_constant__ 
                             const uint64_t da = make_smem_desc_sw128(z_addr + h * 2 * CHUNK_BYTES + k4 * 2048,
                                                                      CHUNK_BYTES, 1024);
                             mma_bf16_ss_pair(tmem_base + h * BN, da, db, idesc, (kb == w.kb0 && k4 == 0) ? 0u : 1u);
+                        }
+                    }
+                    // both CTAs' transform warps see the same rows, so this CTA's flag speaks for the partner's plane too
+                    if (SPLIT && has_lo[stage]) {
+#pragma unroll
+                        for (int k4 = 0; k4 < BK / 16; ++k4) {
+                            const uint64_t db = make_smem_desc_sw128(a_addr + A_BYTES + k4 * 2048, CHUNK_BYTES, 1024);
+#pragma unroll
+                            for (int h = 0; h < 2; ++h)
+                                mma_bf16_ss_pair(tmem_base + h * BN,
+                                                 make_smem_desc_sw128(z_addr + h * 2 * CHUNK_BYTES + k4 * 2048, CHUNK_BYTES, 1024),
+                                                 db, idesc, 1u);
                         }
                     }
                     mma_commit_pair(&empty[stage], 3);          // frees the stage in both CTAs
@@ -302,20 +322,29 @@ zta_pair_kernel(const __grid_constant__ zta::Maps maps, const __grid_constant__ 
                 if (!ok) break;
                 if (t == 0) { DPCLIP_TRACE_AT(1, tr); ++tr; }
                 uint8_t* at = smem + stage * STAGE_BYTES + Z_BYTES;
-                // packed bf16 scaling: f = f_hi + f_lo (two bf16); a*f_lo is tiny, so the fused multiply-add
-                // a*f_hi + (a*f_lo) rounds the product once
-                auto scale8 = [](uint4& v, float f) {
-                    const __nv_bfloat16 fh = __float2bfloat16_rn(f);
-                    const __nv_bfloat16 fl = __float2bfloat16_rn(f - __bfloat162float(fh));
-                    const __nv_bfloat162 fh2 = __halves2bfloat162(fh, fh), fl2 = __halves2bfloat162(fl, fl);
-                    __nv_bfloat162* z2 = reinterpret_cast<__nv_bfloat162*>(&v);
-#pragma unroll
-                    for (int u2 = 0; u2 < 4; ++u2) z2[u2] = __hfma2(z2[u2], fh2, __hmul2(z2[u2], fl2));
-                };
                 bool any = false;
 #pragma unroll
                 for (int i = 0; i < NR; ++i) any = any || fr[i] != 1.f;
-                if (any) {
+                bool split = false;
+                if (SPLIT) {
+                    // every warp sees all rows of the stage, so all warps of both CTAs agree on this
+                    split = __any_sync(0xFFFFFFFFu, any) && p.layer[w.layer].split;
+                    if (t == 0) has_lo[stage] = split ? 1 : 0;
+                }
+                if (SPLIT && split) {
+                    uint4 v[NR];
+#pragma unroll
+                    for (int i = 0; i < NR; ++i) v[i] = *reinterpret_cast<const uint4*>(at + off + i * 2048);
+#pragma unroll
+                    for (int i = 0; i < NR; ++i) {
+                        uint4 lo = make_uint4(0u, 0u, 0u, 0u);
+                        if (fr[i] != 1.f) {
+                            scale_bf16x8_split(v[i], lo, fr[i]);
+                            *reinterpret_cast<uint4*>(at + off + i * 2048) = v[i];
+                        }
+                        *reinterpret_cast<uint4*>(at + A_BYTES + off + i * 2048) = lo;
+                    }
+                } else if (any) {
                     // all loads before the first store: one shared-memory round trip per stage; rows whose
                     // factor is exactly 1 are left as they are
                     uint4 v[NR];
@@ -324,7 +353,7 @@ zta_pair_kernel(const __grid_constant__ zta::Maps maps, const __grid_constant__ 
 #pragma unroll
                     for (int i = 0; i < NR; ++i) {
                         if (fr[i] != 1.f) {
-                            scale8(v[i], fr[i]);
+                            scale_bf16x8(v[i], fr[i]);
                             *reinterpret_cast<uint4*>(at + off + i * 2048) = v[i];
                         }
                     }
@@ -514,10 +543,9 @@ reduce_segments_kernel(const __grid_constant__ ztp::Params p) {
                              : make_float4(0.f, 0.f, 0.f, 0.f);
         float z0 = 0.f, z1 = 0.f, z2 = 0.f, z3 = 0.f;
         if (p.noise_scale > 0.f) {
-            const size_t qd = ((size_t)m * y.d_in + n) >> 2;
-            PhiloxBlock b = philox_block((uint32_t)qd, (uint32_t)(qd >> 32), y.sw0, y.sw1, p.k0, p.k1);
-            box_muller(b.v[0], b.v[1], z0, z1);
-            box_muller(b.v[2], b.v[3], z2, z3);
+            float z[4];
+            normals_at((size_t)m * y.d_in + n, y.sw0, y.sw1, p.k0, p.k1, z);
+            z0 = z[0]; z1 = z[1]; z2 = z[2]; z3 = z[3];
         }
         float4 acc = v[0];                                                  // segment order
 #pragma unroll

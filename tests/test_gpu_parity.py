@@ -1131,3 +1131,76 @@ def test_step_host_matches_device_step(dp):
         assert np.array_equal(hp.gW[l].numpy(), hs.gW[l].numpy())
         assert np.array_equal(hp.gb[l].numpy(), hs.gb[l].numpy())
         assert rel_fro(hs.gb[l].numpy(), dev.gb[l].cpu().numpy()) <= 1e-6
+
+
+# ---------------------------------------------------------------------------
+# staged operands: layers whose rows TMA cannot address, taken to the tensor cores through 16-byte aligned copies
+# ---------------------------------------------------------------------------
+STAGED_MODELS = [
+    # rows of 4-, 2- and odd-element alignment, one wide d_out on the CTA-pair kernel, a T = 1 head of odd width
+    (6, ((77, 300, 300, False), (77, 300, 1100, True), (77, 1100, 302, True), (1, 301, 77, True))),
+    (5, ((300, 130, 70, True), (33, 515, 1030, True))),
+    (9, ((20, 100, 37, True), (20, 512, 300, True), (20, 601, 1001, True))),
+    # all T = 1: odd widths (bf16 goes through fp32 copies)
+    (130, ((1, 783, 301, True), (1, 301, 1003, False), (1, 1003, 10, True))),
+]
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("B,specs", STAGED_MODELS)
+def test_step_staged_operands(dp, B, specs, dtype, path_switch):
+    """Models with unaligned rows: within the fp32 bounds for BOTH types (the scaled bf16 operand is kept in two terms,
+    relative error 2^-18 = 4e-6 a product, on top of the fp32 sums), noise included, and the same clip decisions."""
+    data = [workloads.random_layer(60 + k, B, T, i, o, dtype, scale_z=0.05) for k, (T, i, o, _) in enumerate(specs)]
+    hb = [s[3] for s in specs]
+    sq = np.stack([oracle.layer_sqnorms(A, Z, b) for (A, Z), b in zip(data, hb)])
+    C, sigma, seed = float(np.median(np.sqrt(sq.sum(0)))) * 1.001, 0.02, 5
+    norms_ref, clip_ref = oracle.factors(sq, C)
+    plan = dp.StepPlan([dp.Layer(to_device(A, dtype), to_device(Z, dtype), b) for (A, Z), b in zip(data, hb)])
+    plan.run(C, sigma, seed)
+    assert dp.dpclip_read_status(plan.workspace) == 0
+    assert max_rel(plan.norms.cpu().numpy(), norms_ref) <= TOL["f32"]["norm"]
+    check_saturation(plan.clip.cpu().numpy(), norms_ref, clip_ref, C)
+    for l, ((A, Z), b) in enumerate(zip(data, hb)):
+        W, gb = oracle.clipped_grad(A, Z, clip_ref)
+        for got, ref, sid in ((plan.gW[l], W, 2 * l), (plan.gb[l], gb, 2 * l + 1)):
+            if got is None:
+                continue
+            xi = oracle.normals(ref.size, seed, sid).reshape(ref.shape)
+            # a draw is within 1e-5 of its double-precision value (see dpclip_add_noise)
+            bound = TOL["f32"]["grad"] * np.linalg.norm(ref) + 1e-5 * sigma * C * np.sqrt(ref.size)
+            assert np.linalg.norm(got.cpu().numpy() - sigma * C * xi - ref) <= bound, (l, sid)
+    # without the copies (the fp32-ALU kernels): the same results
+    first = [g.clone() for g in plan.gW]
+    path_switch("DPCLIP_NO_STAGE", "1")
+    plan.run(C, sigma, seed)
+    for g, h in zip(first, plan.gW):
+        assert rel_fro(g.cpu().numpy(), h.cpu().numpy()) <= 2 * TOL["f32"]["grad"]
+
+
+STAGED_CONVS = [  # B, C, H, W, k, pad, stride, d_out, channel-major dL/dZ
+    (5, 3, 28, 28, 3, 1, 1, 16, True), (6, 33, 15, 14, 3, 1, 2, 160, True), (4, 40, 9, 11, (3, 2), 1, 1, 257, False),
+    (3, 9, 14, 14, 5, 2, 2, 30, True), (4, 64, 7, 7, 1, 0, 1, 65, True), (33, 64, 14, 14, 3, 1, 1, 128, True)]
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("case", STAGED_CONVS)
+def test_model_step_staged_convolutions(dp, case, dtype):
+    """Convolutions from their feature maps in a model step: maps and gradients the implicit kernels do not take
+    (strides, odd widths, many channels) are staged as patch matrix and rows; bounds as above."""
+    B, cin, H, W, k, pad, stride, cout, cm = case
+    kh, kw = (k, k) if isinstance(k, int) else k
+    X, Z = workloads.conv_inputs(23, B, cin, H, W, k, pad, stride, cout, dtype, var_z=0.01)
+    A = workloads.im2col(X, k, pad, stride)
+    sq = oracle.layer_sqnorms(A, Z, True)[None]
+    C = float(np.median(np.sqrt(sq))) * 1.001
+    norms_ref, clip_ref = oracle.factors(sq, C)
+    dZ = to_device(Z, dtype)
+    plan = dp.ModelPlan([dp.ModelLayer(dp.DPCLIP_KIND_CONV, to_device(X, dtype), dZ.transpose(1, 2).contiguous() if cm else dZ,
+                                       True, conv=(kh, kw, stride, pad), z_channel_major=cm)])
+    plan.run(C, 0.0, 1)
+    assert dp.dpclip_read_status(plan.workspace) == 0
+    assert max_rel(plan.norms.cpu().numpy(), norms_ref) <= TOL["f32"]["norm"]
+    refW, refb = oracle.clipped_grad(A, Z, clip_ref)
+    assert rel_fro(plan.gW[0].cpu().numpy(), refW) <= TOL["f32"]["grad"]
+    assert rel_fro(plan.gb[0].cpu().numpy(), refb) <= TOL["f32"]["grad"]
