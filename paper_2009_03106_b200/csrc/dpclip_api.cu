@@ -11,6 +11,7 @@
 #include "kernels_tc_pair.cuh"
 #include "kernels_fused_t1_tf32.cuh"
 #include "kernels_tf32.cuh"
+#include "kernels_group.cuh"
 #include "kernels_fused_t1.cuh"
 #include "kernels_narrow.cuh"
 #include "kernels_narrow_tc.cuh"
@@ -48,7 +49,7 @@ enum PathSwitch : unsigned {
     SW_FORCE_SIMT = 1u << 0, SW_NO_NARROW = 1u << 1, SW_NO_NARROW_RING = 1u << 2, SW_NO_NARROW_TC = 1u << 3,
     SW_NO_NARROW_PACK = 1u << 4, SW_NARROW_PACK_BF16 = 1u << 5, SW_NO_GRAM_Q2 = 1u << 6, SW_NO_T1_TF32 = 1u << 7,
     SW_NO_FUSED_T1 = 1u << 8, SW_NO_GRAM_GROUP = 1u << 9, SW_NO_GRAD_GROUP = 1u << 10, SW_NO_CONV_TC = 1u << 11,
-    SW_NO_CONV_PATCHES = 1u << 12, SW_TILE_M1 = 1u << 13, SW_TILE_M2 = 1u << 14, SW_T1_TWO_LAUNCHES = 1u << 15, SW_NO_PAIR = 1u << 16, SW_LOG = 1u << 17, SW_NO_FACTORS_TAIL = 1u << 18, SW_NO_SM_BUDGET = 1u << 19, SW_NO_OVERLAP = 1u << 20, SW_NO_STAGE = 1u << 21,
+    SW_NO_CONV_PATCHES = 1u << 12, SW_TILE_M1 = 1u << 13, SW_TILE_M2 = 1u << 14, SW_T1_TWO_LAUNCHES = 1u << 15, SW_NO_PAIR = 1u << 16, SW_LOG = 1u << 17, SW_NO_FACTORS_TAIL = 1u << 18, SW_NO_SM_BUDGET = 1u << 19, SW_NO_OVERLAP = 1u << 20, SW_NO_STAGE = 1u << 21, SW_GROUP_BF16 = 1u << 22,
     SW_LOADED = 1u << 31
 };
 std::atomic<unsigned> g_path_switches{0};
@@ -65,6 +66,7 @@ unsigned read_path_switches() {
         {"DPCLIP_NO_PAIR", SW_NO_PAIR, '1'}, {"DPCLIP_LOG", SW_LOG, '1'},
         {"DPCLIP_NO_FACTORS_TAIL", SW_NO_FACTORS_TAIL, '1'}, {"DPCLIP_NO_SM_BUDGET", SW_NO_SM_BUDGET, '1'},
         {"DPCLIP_NO_OVERLAP", SW_NO_OVERLAP, '1'}, {"DPCLIP_NO_STAGE", SW_NO_STAGE, '1'},
+        {"DPCLIP_GROUP_BF16", SW_GROUP_BF16, '1'},
     };
     unsigned v = SW_LOADED;
     for (const auto& e : table) {
@@ -929,7 +931,8 @@ inline bool tf32_eligible(const void* A, long lda, const void* Z, long ldz, int 
     return (double)B * T * d_in * d_out >= 32.0 * 1024 * 1024;
 }
 
-bool make_map_f32(CUtensorMap* map, const void* base, long rows, long cols, long ld, int box_cols, int box_rows) {
+bool make_map_f32(CUtensorMap* map, const void* base, long rows, long cols, long ld, int box_cols, int box_rows,
+                  CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B) {
     EncodeTiledFn fn = encode_tiled_fn();
     if (!fn) return false;
     cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
@@ -937,7 +940,7 @@ bool make_map_f32(CUtensorMap* map, const void* base, long rows, long cols, long
     cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(base), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -1003,6 +1006,196 @@ int launch_zta_tf32(const void* A, long lda, const void* Z, long ldz, int B, int
     return launch_reduce_partials(p, tiles, ksplit, t::BM, t::BN, d_in, d_out, gW, ldg, gb, noise, noise_done, st);
 }
 
+// ---------------------------------------------------------------------------
+// Many layers in one launch on CTA pairs (kernels_group.cuh)
+// ---------------------------------------------------------------------------
+struct GroupLayer {
+    const void* A; long lda; const void* Z; long ldz;
+    int T, d_in, d_out;
+    bool bias;
+    float* sq;                                             // norms
+    const float* clip; bool split;                         // clipped sums
+    float* gW; long ldg; float* gb; unsigned long long sid_w, sid_b;
+};
+constexpr size_t kGroupSlotBytes = tc::zg::SLOT_ELEMS * 4 + 256 * 4;
+constexpr int kGroupMinRun = 4;                            // stages of a run, at least: shorter ones are mostly set-up and drain
+
+// Tiling of a layer: which operand the M side is (256-column tiles), and the N side's tile width.
+struct GroupTiling { bool z_on_m; int tiles_m, tiles_n, N; };
+inline GroupTiling group_tiling(int d_in, int d_out) {
+    auto make = [](bool z_on_m, int dm, int dn) {
+        GroupTiling t;
+        t.z_on_m = z_on_m;
+        t.tiles_m = ceil_div(dm, tc::zg::BM);
+        const int parts = ceil_div(dn, tc::zg::BN_MAX);
+        t.N = ceil_div(ceil_div(dn, parts), 64) * 64;
+        t.tiles_n = ceil_div(dn, t.N);
+        return t;
+    };
+    // a stage costs about as much as its columns, 256 + N (bytes through shared memory); A on the M side when equal: its
+    // partial tiles lie the way gW does
+    const GroupTiling a = make(false, d_in, d_out), z = make(true, d_out, d_in);
+    const long ca = (long)a.tiles_m * a.tiles_n * (256 + a.N), cz = (long)z.tiles_m * z.tiles_n * (256 + z.N);
+    return cz < ca ? z : a;
+}
+// fp32: layers with a side of at most 128 leave the 256-column tiles mostly prepared for few products, and are as fast in
+// zta_tf32_kernel (128 x 128 tiles), one or two of them; from three on the shared launch wins (convolutions 288 -> 64 and
+// 576 -> 128 of a CNN, two streams: 139 us a step by layer, 147 together; seven layers of 148 to 592 features, B = 61, T = 48:
+// 252 us a step by layer, 83 together).
+inline bool group_wide(int d_in, int d_out) { return d_in > 128 && d_out > 128; }
+constexpr int kGroupFrom = 3;
+inline int group_tiles(int d_in, int d_out) { const GroupTiling t = group_tiling(d_in, d_out); return t.tiles_m * t.tiles_n; }
+
+// Clears the rows of sq that a launch accumulates into, adjacent rows in one memset.
+inline int clear_rows(float* const* rows, int n, int B, cudaStream_t st) {
+    int order[64];
+    if (n > 64) return DPCLIP_ERR_INVALID_ARG;
+    for (int i = 0; i < n; ++i) {
+        int j = i;
+        for (; j > 0 && rows[order[j - 1]] > rows[i]; --j) order[j] = order[j - 1];
+        order[j] = i;
+    }
+    for (int i = 0; i < n;) {
+        float* begin = rows[order[i]];
+        float* end = begin + B;
+        int j = i + 1;
+        while (j < n && rows[order[j]] == end) { end += B; ++j; }
+        if (cudaMemsetAsync(begin, 0, sizeof(float) * (size_t)(end - begin), st) != cudaSuccess) return DPCLIP_ERR_CUDA;
+        i = j;
+    }
+    return DPCLIP_OK;
+}
+
+template <int MODE, bool NORM>
+int launch_group_kernel(const tc::zg::Maps& maps, const tc::zg::Params& p, cudaStream_t st) {
+    constexpr int smem = tc::zg::Cfg<MODE>::SMEM_BYTES;
+    if (!enable_smem(tc::zta_group_kernel<MODE, NORM>, smem)) return DPCLIP_ERR_CUDA;
+    tc::zta_group_kernel<MODE, NORM><<<2 * p.n_runs, tc::zg::THREADS, smem, st>>>(maps, p);
+    return launch_status();
+}
+
+// Norms (norm = true) or clipped sums with noise of n layers.  Returns DPCLIP_OK, a negative status, or 1 when the
+// workspace cannot hold a few partial tiles (clipped sums only; nothing has been launched then).
+int launch_group(const GroupLayer* ls, int n, int B, dpclip_dtype dtype, bool norm, const NoiseSpec* noise, bool* noise_done,
+                 void* workspace, size_t workspace_bytes, cudaStream_t st, const tc::gram::FactorsTail* tail = nullptr) {
+    namespace g = tc::zg;
+    const bool f32 = dtype == DPCLIP_F32;
+    const int bk = f32 ? g::Cfg<g::F32>::BK : g::Cfg<g::BF16>::BK;
+    const int max_runs = sm_budget() / 2;
+    const size_t room = workspace && workspace_bytes > (size_t)kHeaderBytes ? workspace_bytes - kHeaderBytes : 0;
+    const long cap = (long)(room / kGroupSlotBytes);
+    // norms of long examples keep the sums between two drains in a slot per run
+    bool long_norms = false;
+    for (int l = 0; norm && f32 && l < n; ++l) long_norms = long_norms || ls[l].T > g::FLUSH * bk;
+    if ((!norm || long_norms) && cap < 8) return norm ? DPCLIP_ERR_WORKSPACE : 1;
+    bool fuse_noise = !norm && noise && noise->scale > 0.f;
+    for (int l = 0; l < n && fuse_noise; ++l) fuse_noise = ls[l].ldg == ls[l].d_in;
+    if (norm) {
+        for (int l0 = 0; l0 < n; l0 += 64) {
+            float* rows[64];
+            const int k = n - l0 < 64 ? n - l0 : 64;
+            for (int l = 0; l < k; ++l) rows[l] = ls[l0 + l].sq;
+            const int rc = clear_rows(rows, k, B, st);
+            if (rc) return rc;
+        }
+    }
+    g::Maps maps;
+    g::Params p;
+    int next = 0, next_tile = 0;                            // layer and its tile the next launch begins with
+    while (next < n) {
+        memset(&p, 0, sizeof(p));
+        p.status = static_cast<int*>(workspace);
+        p.first_chunk = p.last_chunk = 1;
+        // the slots of a launch: its tiles and its runs
+        const int runs_cap = (norm && !long_norms) || cap >= 2L * max_runs ? max_runs : (int)(cap / 2);
+        int tiles = 0;
+        bool any_split = false;
+        double cost[g::MAX_LAYERS], total = 0.0;
+        long units[g::MAX_LAYERS], n_units = 0;
+        while (next < n && p.n_layers < g::MAX_LAYERS) {
+            const GroupLayer& y = ls[next];
+            const GroupTiling t = group_tiling(y.d_in, y.d_out);
+            const int all = t.tiles_m * t.tiles_n;
+            int take = all - next_tile;
+            if (!norm && tiles + take > cap - runs_cap) {
+                if (p.n_layers > 0) break;                  // the next launch begins with this layer
+                take = (int)(cap - runs_cap);
+            }
+            const int k = p.n_layers;
+            g::Layer& q = p.layer[k];
+            const long R = (long)B * y.T;
+            const void* pm = t.z_on_m ? y.Z : y.A; const long lm = t.z_on_m ? y.ldz : y.lda;
+            const void* pn = t.z_on_m ? y.A : y.Z; const long ln = t.z_on_m ? y.lda : y.ldz;
+            q.T = y.T; q.R = (int)R;
+            q.d_m = t.z_on_m ? y.d_out : y.d_in; q.d_n = t.z_on_m ? y.d_in : y.d_out; q.z_on_m = t.z_on_m ? 1 : 0;
+            const CUtensorMapSwizzle sw = CU_TENSOR_MAP_SWIZZLE_128B;
+            if (f32 ? !make_map_f32(&maps.m[k], pm, R, q.d_m, lm, 32, bk, sw) || !make_map_f32(&maps.n[k], pn, R, q.d_n, ln, 32, bk, sw)
+                    : !make_map_bf16(&maps.m[k], pm, R, q.d_m, lm, 64, bk) || !make_map_bf16(&maps.n[k], pn, R, q.d_n, ln, 64, bk))
+                return DPCLIP_ERR_CUDA;
+            q.tiles_m = t.tiles_m; q.tiles_n = t.tiles_n; q.N = t.N;
+            q.nkb = ceil_div(norm ? (long)y.T : R, (long)bk);
+            q.tile0 = next_tile; q.tiles = take; q.tile_base = tiles; q.unit_base = (int)n_units;
+            q.do_bias = norm ? y.bias : y.gb != nullptr;
+            q.split = y.split ? 1 : 0; q.clip = y.clip; q.sq = y.sq;
+            q.gW = y.gW; q.gb = y.gb; q.ldg = y.ldg; q.vec_ok = aligned_to(y.gW, 16) && y.ldg % 4 == 0;
+            q.sw0 = (uint32_t)y.sid_w; q.sw1 = (uint32_t)(y.sid_w >> 32);
+            q.sb0 = (uint32_t)y.sid_b; q.sb1 = (uint32_t)(y.sid_b >> 32);
+            q.blk_begin = p.n_blocks;
+            if (!norm) p.n_blocks += take * 8 * (t.N / 32);
+            any_split = any_split || y.split;
+            units[k] = norm ? (long)B * all : (long)take * q.nkb;
+            cost[k] = norm ? (double)q.nkb * (256 + t.N) + 256 : 256 + t.N;
+            total += cost[k] * units[k]; n_units += units[k]; tiles += take;
+            if (n_units > 0x3FFFFFFFL) return DPCLIP_ERR_UNSUPPORTED;
+            ++p.n_layers;
+            if (!norm && next_tile + take < all) {           // a chunk of a layer
+                p.first_chunk = next_tile == 0; p.last_chunk = 0;
+                next_tile += take;
+                break;
+            }
+            if (next_tile > 0) { p.first_chunk = 0; next_tile = 0; ++next; break; }
+            ++next;
+        }
+        long runs = norm ? n_units : n_units / kGroupMinRun;
+        if (runs > runs_cap) runs = runs_cap;
+        if (runs < 1) runs = 1;
+        p.n_runs = (int)runs;
+        // equal shares of the total cost, cut between units
+        {
+            int k = 0;
+            double before = 0.0;                             // cost of the layers before k
+            for (int r = 0; r <= p.n_runs; ++r) {
+                const double at = total * r / p.n_runs;
+                while (k + 1 < p.n_layers && before + cost[k] * units[k] <= at) { before += cost[k] * units[k]; ++k; }
+                long u = p.layer[k].unit_base + (long)((at - before) / cost[k] + 0.5);
+                if (r == p.n_runs || u > n_units) u = n_units;
+                p.run_begin[r] = (int)u;
+            }
+        }
+        p.n_slots = norm ? p.n_runs : tiles + p.n_runs;
+        p.part = reinterpret_cast<float*>(static_cast<char*>(workspace) + kHeaderBytes);
+        p.bias_part = p.part + (size_t)p.n_slots * g::SLOT_ELEMS;
+        if (fuse_noise) { p.noise_scale = noise->scale; p.k0 = (uint32_t)noise->seed; p.k1 = (uint32_t)(noise->seed >> 32); }
+        if (tail && next >= n) {
+            p.tail = *tail;
+            p.tail.done = reinterpret_cast<unsigned int*>(static_cast<char*>(workspace) + kTailCounterOffset);
+        }
+        DPCLIP_LOGF("group %s: %d layer(s) %s, %d tiles, %ld units, %d runs", norm ? "norms" : "clipped sums", p.n_layers,
+                    f32 ? "fp32 in three bf16 terms" : any_split ? "bf16 two-term" : "bf16", tiles, n_units, p.n_runs);
+        int rc;
+        if (norm) rc = f32 ? launch_group_kernel<g::F32, true>(maps, p, st) : launch_group_kernel<g::BF16, true>(maps, p, st);
+        else rc = f32 ? launch_group_kernel<g::F32, false>(maps, p, st)
+                : any_split ? launch_group_kernel<g::BF16_SPLIT, false>(maps, p, st) : launch_group_kernel<g::BF16, false>(maps, p, st);
+        if (rc) return rc;
+        if (norm) continue;
+        const int blocks = p.n_blocks < 8 * kNumSMs ? p.n_blocks : 8 * kNumSMs;
+        tc::reduce_group_kernel<<<blocks, 256, 0, st>>>(p);
+        if ((rc = launch_status())) return rc;
+    }
+    if (fuse_noise && noise_done) *noise_done = true;
+    return DPCLIP_OK;
+}
+
 // clipped sum of one layer, optionally with the noise folded into the last pass over the output
 int clipped_grad_impl(const void* A, long lda, const void* Zbar, long ldz, int B, int T, int d_in, int d_out,
                       dpclip_dtype dtype, const float* clip, float* gW, long ldg, float* gb, void* workspace,
@@ -1015,9 +1208,15 @@ int clipped_grad_impl(const void* A, long lda, const void* Zbar, long ldz, int B
     if (tc_eligible(A, lda, Zbar, ldz, dtype))
         return launch_zta_tc(A, lda, Zbar, ldz, B, T, d_in, d_out, false, 0, clip, gW, ldg, gb, nullptr, workspace,
                              workspace_bytes, noise, noise_done, st, false, split);
-    if (tf32_eligible(A, lda, Zbar, ldz, B, T, d_in, d_out, dtype) && !narrow_layer(T, d_in, d_out, gb != nullptr, lda, ldz))
-        return launch_zta_tf32(A, lda, Zbar, ldz, B, T, d_in, d_out, false, 0, clip, gW, ldg, gb, nullptr, workspace,
-                               workspace_bytes, noise, noise_done, st);
+    if (tf32_eligible(A, lda, Zbar, ldz, B, T, d_in, d_out, dtype) && !narrow_layer(T, d_in, d_out, gb != nullptr, lda, ldz)) {
+        if (!group_wide(d_in, d_out))
+            return launch_zta_tf32(A, lda, Zbar, ldz, B, T, d_in, d_out, false, 0, clip, gW, ldg, gb, nullptr, workspace,
+                                   workspace_bytes, noise, noise_done, st);
+        GroupLayer y = {A, lda, Zbar, ldz, T, d_in, d_out, false, nullptr, clip, false, gW, ldg, gb,
+                        noise ? noise->sid_w : 0ull, noise ? noise->sid_b : 0ull};
+        const int rc = launch_group(&y, 1, B, dtype, false, noise, noise_done, workspace, workspace_bytes, st);
+        return rc > 0 ? DPCLIP_ERR_WORKSPACE : rc;
+    }
     return launch_simt_grad(A, lda, Zbar, ldz, B, T, d_in, d_out, dtype, clip, gW, ldg, gb, st, workspace,
                             workspace_bytes, noise, noise_done);
 }
@@ -1312,6 +1511,17 @@ static size_t step_scratch_bytes(const dpclip_layer* layers, int L, int B, dpcli
         const size_t w = dpclip_workspace_bytes(B, y.T, y.d_in, y.d_out, dtype, (dpclip_method)y.method);
         if (w > ws) ws = w;
     }
+    // the layers that share a clipped-sum launch of launch_group: a slot per tile of all of them and one per run
+    {
+        long tiles = 0;
+        for (int l = 0; l < L; ++l) {
+            const dpclip_layer& y = layers[l];
+            if (y.T > 1 && y.d_in > 0 && y.d_out > 0 && (dtype == DPCLIP_F32 || !pair_tile_ok(y.d_out))) tiles += group_tiles(y.d_in, y.d_out);
+        }
+        if (tiles > 512) tiles = 512;                        // more go in several launches
+        const size_t need = kHeaderBytes + (size_t)(tiles + kNumPairs) * kGroupSlotBytes;
+        if (tiles > 0 && need > ws && (dtype == DPCLIP_BF16 || ws > (size_t)kHeaderBytes)) ws = need;
+    }
     if (dtype != DPCLIP_BF16 || path_switch(SW_NO_GRAD_GROUP)) return ws;
     // layers of one T that share a CTA-pair launch (up to eight): one segment per tile of all of them + one per pair
     for (int l0 = 0; l0 < L; ++l0) {
@@ -1390,8 +1600,11 @@ int dpclip_layer_sqnorms(const void* A, long lda, const void* Zbar, long ldz, in
             if (dtype == DPCLIP_F32) {                    // fp32: materialised tiles via error-compensated tf32
                 if (method != DPCLIP_MATERIALIZE || !aligned_to(A, 16) || !aligned_to(Zbar, 16) || lda % 4 || ldz % 4)
                     return DPCLIP_ERR_UNSUPPORTED;
-                return launch_zta_tf32(A, lda, Zbar, ldz, B, T, d_in, d_out, true, has_bias, nullptr, nullptr, 0,
-                                       nullptr, sq_layer, workspace, workspace_bytes, nullptr, nullptr, st);
+                if (!group_wide(d_in, d_out))
+                    return launch_zta_tf32(A, lda, Zbar, ldz, B, T, d_in, d_out, true, has_bias, nullptr, nullptr, 0,
+                                           nullptr, sq_layer, workspace, workspace_bytes, nullptr, nullptr, st);
+                GroupLayer y = {A, lda, Zbar, ldz, T, d_in, d_out, has_bias != 0, sq_layer};
+                return launch_group(&y, 1, B, dtype, true, nullptr, nullptr, workspace, workspace_bytes, st);
             }
             if (!aligned_to(A, 16) || !aligned_to(Zbar, 16) || lda % 8 || ldz % 8)
                 return DPCLIP_ERR_UNSUPPORTED;
@@ -2289,6 +2502,69 @@ static int launch_stage(StagePlan& sp, cudaStream_t st) {
     return DPCLIP_OK;
 }
 
+// The layers of a step that share the launches of launch_group: T > 1, addressable by TMA, not taken by another shared
+// launch (skip), and -- for the norms -- by the materialised product.  taken[l] is set for them.
+static bool group_candidate(const dpclip_layer& y, int B, dpclip_dtype dtype) {
+    if (y.T <= 1 || check_layer_args(y.A, y.lda, y.Zbar, y.ldz, B, y.T, y.d_in, y.d_out, dtype)) return false;
+    if (dtype == DPCLIP_F32)
+        return tf32_eligible(y.A, y.lda, y.Zbar, y.ldz, B, y.T, y.d_in, y.d_out, dtype) &&
+               !narrow_layer(y.T, y.d_in, y.d_out, y.has_bias, y.lda, y.ldz);
+    return path_switch(SW_GROUP_BF16) && tc_eligible(y.A, y.lda, y.Zbar, y.ldz, dtype);
+}
+// of one or two fp32 layers only the wide ones stay
+static int keep_wide(GroupLayer* g, const dpclip_layer* layers, int L, int* taken) {
+    int k = 0, i = 0;
+    for (int l = 0; l < L; ++l) {
+        if (!taken[l]) continue;
+        if (group_wide(layers[l].d_in, layers[l].d_out)) g[k++] = g[i]; else taken[l] = 0;
+        ++i;
+    }
+    return k;
+}
+static int group_norms(const dpclip_layer* layers, int L, int B, dpclip_dtype dtype, float* sq_layers, const int* skip, int* taken,
+                       void* workspace, size_t workspace_bytes, void* stream, const tc::gram::FactorsTail* tail, bool* tail_done) {
+    GroupLayer g[64];
+    int n = 0;
+    for (int l = 0; l < L; ++l) {
+        taken[l] = 0;
+        const dpclip_layer& y = layers[l];
+        if ((skip && skip[l]) || !group_candidate(y, B, dtype)) continue;
+        int method = y.method;
+        if (method == DPCLIP_AUTO) method = dpclip_pick_method(B, y.T, y.d_in, y.d_out, y.lda, y.ldz, dtype);
+        if (method != DPCLIP_MATERIALIZE) continue;
+        g[n++] = {y.A, y.lda, y.Zbar, y.ldz, y.T, y.d_in, y.d_out, y.has_bias != 0, sq_layers + (size_t)l * B};
+        taken[l] = 1;
+    }
+    if (dtype == DPCLIP_F32 && n < kGroupFrom) n = keep_wide(g, layers, L, taken);
+    if (n == 0) return DPCLIP_OK;
+    if (!workspace || workspace_bytes < (size_t)kHeaderBytes) return DPCLIP_ERR_WORKSPACE;
+    const bool with_tail = tail && n == L;
+    if (tail_done) *tail_done = with_tail;
+    return launch_group(g, n, B, dtype, true, nullptr, nullptr, workspace, workspace_bytes, (cudaStream_t)stream, with_tail ? tail : nullptr);
+}
+// clip_ld as in shared_clipped_grad_launches
+static int group_grads(const dpclip_layer* layers, const bool* split, int L, int B, dpclip_dtype dtype, const float* clip, long clip_ld,
+                       float C, float sigma, unsigned long long seed, unsigned long long stream_id0, const int* skip, int* taken,
+                       void* workspace, size_t workspace_bytes, void* stream) {
+    GroupLayer g[64];
+    int n = 0;
+    for (int l = 0; l < L; ++l) {
+        taken[l] = 0;
+        const dpclip_layer& y = layers[l];
+        if ((skip && skip[l]) || !group_candidate(y, B, dtype) || !y.gW || y.ldg != y.d_in || (y.has_bias && !y.gb)) continue;
+        g[n++] = {y.A, y.lda, y.Zbar, y.ldz, y.T, y.d_in, y.d_out, false, nullptr, clip ? clip + (size_t)l * clip_ld : nullptr,
+                  split && split[l], y.gW, y.ldg, y.has_bias ? y.gb : nullptr, stream_id0 + 2ull * l, stream_id0 + 2ull * l + 1};
+        taken[l] = 1;
+    }
+    if (dtype == DPCLIP_F32 && n < kGroupFrom) n = keep_wide(g, layers, L, taken);
+    if (n == 0) return DPCLIP_OK;
+    const NoiseSpec ns = {sigma * C, seed, 0, 0};
+    bool noise_done = false;
+    const int rc = launch_group(g, n, B, dtype, false, &ns, &noise_done, workspace, workspace_bytes, (cudaStream_t)stream);
+    if (rc > 0) { for (int l = 0; l < L; ++l) taken[l] = 0; return DPCLIP_OK; }         // no room: layer by layer
+    return rc;
+}
+
 // The streams a step may spread its layers over.  Lane 0 is the caller's stream: the step starts and ends
 // there.  fork() makes every other lane wait for what lane 0 has enqueued so far, join() makes lane 0 wait for
 // what the other lanes have enqueued; both are event record/wait pairs, which a stream capture records as
@@ -2366,7 +2642,7 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
     }
     int in_gram_group[64];
     const bool track = L <= 64;
-    bool any_gram = false;
+    bool any_gram = false, any_mat = false;
     bool factors_done = false;
     if (track) {
         // when one Gram launch takes every layer of the model, its last CTA also computes the factors
@@ -2375,6 +2651,18 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
                                  (!t1.active && !any_other && !path_switch(SW_NO_FACTORS_TAIL)) ? &tail : nullptr, &factors_done);
         if (rc) return rc;
         for (int l = 0; l < L; ++l) any_gram = any_gram || in_gram_group[l];
+        // the layers whose norms go by the materialised product, also in one launch
+        int skip[64], taken[64];
+        for (int l = 0; l < L; ++l) skip[l] = in_gram_group[l] || other_kind(l);
+        const int b = any_gram && lanes.n > 1 ? 1 : 0;
+        rc = group_norms(layers, L, B, dtype, sq_layers, skip, taken, lanes.ws[b], workspace_bytes, lanes.st[b],
+                         (!t1.active && !any_other && !any_gram && !path_switch(SW_NO_FACTORS_TAIL)) ? &tail : nullptr,
+                         any_gram ? nullptr : &factors_done);
+        if (rc) return rc;
+        for (int l = 0; l < L; ++l) {
+            any_mat = any_mat || taken[l];
+            if (taken[l]) in_gram_group[l] = 1;                          // nothing left to do for it in this stage
+        }
     }
     // SM shares for the per-layer launches of a stage (see t_sm_budget): only when several of them run side by
     // side on different lanes, no launch shared by several layers is in the stage, and the stage is small
@@ -2411,8 +2699,8 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
         }
     };
     int budget[64] = {0};
-    if (track) stage_budgets(in_gram_group, any_gram, budget);
-    int k = any_gram ? 1 : 0;                              // lane 0 already carries the shared Gram launch
+    if (track) stage_budgets(in_gram_group, any_gram || any_mat, budget);
+    int k = (any_gram ? 1 : 0) + (any_mat ? 1 : 0);        // the first lanes already carry the shared launches
     for (int l = 0; l < L; ++l) {
         const dpclip_layer& y = layers[l];
         const bool is_other = other_kind(l);
@@ -2439,7 +2727,7 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
         if (rc > 0) return DPCLIP_ERR_UNSUPPORTED;           // prepare_t1_group checked the same conditions
     }
     int in_grad_group[64];
-    bool any_group = false;
+    bool any_group = false, any_rest = false;
     if (track) {
         // the factors came from the tail of the Gram launch, the last kernel of this stream: the first clipped-sum
         // launch may start loading while that tail runs
@@ -2448,9 +2736,16 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
                                           workspace_bytes, lanes.st[0]);
         if (rc) return rc;
         for (int l = 0; l < L; ++l) any_group = any_group || in_grad_group[l];
+        int skip[64], taken[64];
+        for (int l = 0; l < L; ++l) skip[l] = in_grad_group[l] || other_kind(l) || (t1.active && layers[l].T == 1);
+        const int b = any_group && lanes.n > 1 ? 1 : 0;
+        rc = group_grads(layers, split, L, B, dtype, clip, 0, C, sigma, seed, stream_id0, skip, taken, lanes.ws[b], workspace_bytes,
+                         lanes.st[b]);
+        if (rc) return rc;
+        for (int l = 0; l < L; ++l) if (taken[l]) { any_rest = true; in_grad_group[l] = 1; }
     }
-    if (track) stage_budgets(in_grad_group, any_group, budget);
-    k = any_group ? 1 : 0;
+    if (track) stage_budgets(in_grad_group, any_group || any_rest, budget);
+    k = (any_group ? 1 : 0) + (any_rest ? 1 : 0);
     for (int l = 0; l < L; ++l) {
         const dpclip_layer& y = layers[l];
         const bool is_other = other_kind(l);
@@ -2617,6 +2912,10 @@ int dpclip_step_per_layer(const dpclip_layer* layers, int L, int B, dpclip_dtype
     if (track) {
         rc = dpclip_gram_layers_sqnorms(layers, L, B, dtype, sq_layers, in_gram, workspace, workspace_bytes, stream);
         if (rc) return rc;
+        int taken[kMaxTracked];
+        rc = group_norms(layers, L, B, dtype, sq_layers, in_gram, taken, workspace, workspace_bytes, stream, nullptr, nullptr);
+        if (rc) return rc;
+        for (int l = 0; l < L; ++l) in_gram[l] = in_gram[l] || taken[l];
     }
     for (int l = 0; l < L; ++l) {
         const dpclip_layer& y = layers[l];
@@ -2633,6 +2932,11 @@ int dpclip_step_per_layer(const dpclip_layer* layers, int L, int B, dpclip_dtype
         rc = shared_clipped_grad_launches(layers, split, L, B, dtype, clip_layers, (long)B, C_total, sigma, seed, stream_id0,
                                           in_pairs, workspace, workspace_bytes, stream);
         if (rc) return rc;
+        int taken[kMaxTracked];
+        rc = group_grads(layers, split, L, B, dtype, clip_layers, (long)B, C_total, sigma, seed, stream_id0, in_pairs, taken, workspace,
+                         workspace_bytes, stream);
+        if (rc) return rc;
+        for (int l = 0; l < L; ++l) in_pairs[l] = in_pairs[l] || taken[l];
     } else {
         for (int l = 0; l < L; ++l) {
             rc = dpclip_factors(sq_layers + (size_t)l * B, 1, B, B, C_layer[l], clip_layers + (size_t)l * B,

@@ -1204,3 +1204,35 @@ def test_model_step_staged_convolutions(dp, case, dtype):
     refW, refb = oracle.clipped_grad(A, Z, clip_ref)
     assert rel_fro(plan.gW[0].cpu().numpy(), refW) <= TOL["f32"]["grad"]
     assert rel_fro(plan.gb[0].cpu().numpy(), refb) <= TOL["f32"]["grad"]
+
+
+# fp32 layers that share the CTA-pair launch: a run boundary inside a tile, items of one stage to several drains (T = 30,
+# 128, 800: one accumulator, two, several windows), N = 64 .. 256 tiles, either operand on the M side, ragged widths
+GROUP_MODELS = [
+    (3, ((30, 516, 64, True), (128, 260, 520, True), (800, 140, 196, False))),
+    (9, ((128, 512, 256, False), (128, 196, 640, True), (33, 100, 300, True), (65, 320, 68, True))),
+    (1, ((1700, 132, 516, True),)),
+]
+
+
+@pytest.mark.parametrize("B,specs", GROUP_MODELS)
+def test_step_fp32_layers_in_one_launch(dp, B, specs):
+    data = [workloads.random_layer(80 + k, B, T, i, o, "f32", scale_z=0.05) for k, (T, i, o, _) in enumerate(specs)]
+    hb = [s[3] for s in specs]
+    sq = np.stack([oracle.layer_sqnorms(A, Z, b) for (A, Z), b in zip(data, hb)])
+    C, sigma, seed = float(np.median(np.sqrt(sq.sum(0)))) * 1.001, 0.02, 6
+    norms_ref, clip_ref = oracle.factors(sq, C)
+    plan = dp.StepPlan([dp.Layer(to_device(A, "f32"), to_device(Z, "f32"), b) for (A, Z), b in zip(data, hb)])
+    for _ in range(2):                                       # the second step reuses every counter and slot
+        plan.run(C, sigma, seed)
+    assert dp.dpclip_read_status(plan.workspace) == 0
+    assert max_rel(np.sqrt(plan.sq_layers.cpu().numpy()), np.sqrt(sq)) <= TOL["f32"]["norm"]
+    check_saturation(plan.clip.cpu().numpy(), norms_ref, clip_ref, C)
+    for l, ((A, Z), b) in enumerate(zip(data, hb)):
+        W, gb = oracle.clipped_grad(A, Z, clip_ref)
+        for got, ref, sid in ((plan.gW[l], W, 2 * l), (plan.gb[l], gb, 2 * l + 1)):
+            if got is None:
+                continue
+            xi = oracle.normals(ref.size, seed, sid).reshape(ref.shape)
+            bound = TOL["f32"]["grad"] * np.linalg.norm(ref) + 1e-5 * sigma * C * np.sqrt(ref.size)
+            assert np.linalg.norm(got.cpu().numpy() - sigma * C * xi - ref) <= bound, (l, sid)
