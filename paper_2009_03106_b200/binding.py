@@ -156,7 +156,8 @@ def _dtype_code(t: torch.Tensor) -> int:
 
 def _stream(stream) -> int:
     if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+        # the raw handle (0.1 us): torch.cuda.current_stream() builds a Stream object, 3 us of a 10 us step
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 

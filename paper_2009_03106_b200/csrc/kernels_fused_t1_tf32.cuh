@@ -176,6 +176,13 @@ t1_all_grads_tf32_kernel(const __grid_constant__ f1::Params q) {
     using namespace f1;
     constexpr bool BF16 = sizeof(T) == 2;
     constexpr int BOXES = BF16 ? 2 : 4, BOX_COLS = BF16 ? 64 : 32;          // TMA boxes per 128-column tile
+    // bf16: a stage is two tiles of 8 KB and no planes, so eight of them fit; with three a wide layer, many tiles per CTA, waited
+    // for its loads (4096 -> 4096 -> 1000, B = 256: see below)
+    constexpr int STAGES = BF16 ? 8 : f1::STAGES, STAGE_BYTES = BF16 ? 2 * BOXES * CHUNK_BYTES : f1::STAGE_BYTES;
+    constexpr int OFF_A = BF16 ? BOXES * CHUNK_BYTES : f1::OFF_A;
+    // stages between two drains of the accumulator: 48 additions either way
+    constexpr int FLUSH = BF16 ? 24 : f1::FLUSH;
+    static_assert(STAGES * STAGE_BYTES <= f1::STAGES * f1::STAGE_BYTES && (3 * STAGES + 4) * 8 + 8 <= 256, "shared memory layout");
     const FusedT1Params& p = q.base;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);   // 1024-byte aligned; an offset from the array keeps the accesses in the shared state space
