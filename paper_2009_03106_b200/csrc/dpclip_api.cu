@@ -2367,20 +2367,26 @@ static bool stage_plan(StagePlan& sp, const dpclip_layer* layers, const dpclip_m
             if (ct < unit) ct = unit;
             if (ct > (int)round_up(g.C, unit)) ct = (int)round_up(g.C, unit);
             const int pitch = (int)round_up((size_t)ct * kk * es, 16) + 4;
-            if (stage::IM_ROWS * pitch > stage::SMEM_MAX || (double)B * T * ldp / unit > 4.0e9) continue;
+            int cta_rows = 32;
+            while (cta_rows * 2 <= stage::IM_MAX_ROWS && cta_rows * 2 * pitch <= 40 * 1024) cta_rows *= 2;
+            const int im_bytes = cta_rows * pitch + stage::IM_MAX_ROWS * (int)sizeof(int2);
+            if (im_bytes > stage::SMEM_MAX || (double)B * T * ldp / unit > 4.0e9 || g.kh > 16 || g.kw > 16) continue;
+            if ((double)(cta_rows / T + 2) * g.C * g.H * g.W > 2.0e9) continue;
             {
                 stage::Job& j = add_job(l, false, stage::IM2COL, y.A, 0, (int)ldp, B * T, p.d_in, es);
                 j.T = T; j.C = g.C; j.H = g.H; j.W = g.W; j.kh = g.kh; j.kw = g.kw; j.stride = g.stride; j.pad = g.pad;
                 j.Wo = p.Wo; j.ct = ct; j.pitch = pitch; j.tiles_b = ceil_div(g.C, ct);
-                if (stage::IM_ROWS * pitch > sp.smem) sp.smem = stage::IM_ROWS * pitch;
+                j.cta_rows = cta_rows;
+                if (im_bytes > sp.smem) sp.smem = im_bytes;
             }
             dpclip_layer& e = sp.eff[l];
             e = y;
             e.T = T; e.d_in = p.d_in; e.lda = ldp; e.method = DPCLIP_AUTO; e.ldz = p.d_out;
             if (other[l].z_channel_major) {
                 stage::Job& j = add_job(l, true, stage::TRANSPOSE, y.Zbar, 0, (int)ldz, B * T, p.d_out, es);
-                j.T = T; j.tiles_a = ceil_div(T, stage::TILE_T); j.tiles_b = ceil_div(p.d_out, stage::TILE_M);
-                const int bytes = stage::TILE_M * (stage::TILE_T + 2) * (int)es;
+                j.ct = p.d_out <= 32 ? 32 : 64;
+                j.T = T; j.tiles_a = ceil_div(T, stage::TILE / j.ct); j.tiles_b = ceil_div(p.d_out, j.ct);
+                const int bytes = j.ct * (stage::TILE / j.ct + 2) * (int)es;
                 if (bytes > sp.smem) sp.smem = bytes;
                 e.ldz = ldz;
             } else if (!narrow && misaligned(y.Zbar, p.d_out)) {
@@ -2490,7 +2496,7 @@ static int launch_stage(StagePlan& sp, cudaStream_t st) {
         for (int i = 0; i < q.n; ++i) {
             stage::Job& j = q.job[i] = sp.job[i0 + i];
             j.blk_begin = q.blocks;
-            if (j.kind == stage::IM2COL) q.blocks += ceil_div(j.rows, stage::IM_ROWS) * j.tiles_b;
+            if (j.kind == stage::IM2COL) q.blocks += ceil_div(j.rows, j.cta_rows) * j.tiles_b;
             else if (j.kind == stage::TRANSPOSE) q.blocks += j.rows / j.T * j.tiles_a * j.tiles_b;
             else q.blocks += ceil_div((long)j.rows * (j.dst_ld / ((j.es == 4 || j.kind == stage::ROWS_TO_F32) ? 4 : 8)),
                                       (long)stage::ROWS_UNROLL * stage::THREADS);

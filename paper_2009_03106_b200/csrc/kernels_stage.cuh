@@ -20,8 +20,8 @@ enum Kind : int { ROWS = 0, ROWS_TO_F32 = 1, TRANSPOSE = 2, IM2COL = 3 };
 constexpr int MAX_JOBS = 32;
 constexpr int THREADS = 256;
 constexpr int ROWS_UNROLL = 4;                 // 16-byte output chunks per thread
-constexpr int TILE_T = 64, TILE_M = 64;        // transpose tile
-constexpr int IM_ROWS = 32;                    // im2col: patch rows per CTA (one per lane)
+constexpr int TILE = 4096;                     // elements of a transpose tile: 64 x 64, or 128 positions x 32 channels
+constexpr int IM_MAX_ROWS = 256;               // im2col: patch rows per CTA, 32 to 256
 constexpr int SMEM_MAX = 160 * 1024;
 
 struct Job {
@@ -31,8 +31,9 @@ struct Job {
     int rows, cols;                // output rows and width
     int blk_begin;
     // TRANSPOSE / IM2COL
-    int T, tiles_a, tiles_b;       // TRANSPOSE: tiles along T and along M; IM2COL: channel blocks in tiles_b
-    int C, H, W, kh, kw, stride, pad, Wo, ct, pitch;     // IM2COL: ct channels per CTA, pitch = shared-memory row bytes
+    int T, tiles_a, tiles_b;       // TRANSPOSE: tiles along T and along M, ct = channels of a tile; IM2COL: channel blocks in tiles_b
+    int C, H, W, kh, kw, stride, pad, Wo, ct, pitch;     // IM2COL: ct channels per CTA, pitch = shared-memory bytes of a patch row
+    int cta_rows;                  // IM2COL: patch rows per CTA
 };
 struct Launch { Job job[MAX_JOBS]; int n, blocks; };
 
@@ -95,29 +96,31 @@ __device__ __forceinline__ void rows_job(const Job& j, int blk) {
     }
 }
 
-// 64 positions x 64 channels through shared memory; rows of the tile are 64 + 2 elements (bf16) / 64 + 1 (fp32) long, so
-// that neither the writes along T nor the reads along M fall on one bank
-template <typename E>
+// A tile of positions x channels through shared memory; its rows are 2 elements (bf16) or 1 (fp32) longer than the
+// tile, so that neither the writes along T nor the reads along M fall on one bank.  32-channel tiles for narrow layers.
+template <typename E, int TM>
 __device__ __forceinline__ void transpose_job(const Job& j, int blk, uint8_t* smem) {
-    constexpr int PITCH = sizeof(E) == 2 ? TILE_T + 2 : TILE_T + 1;
+    constexpr int TT = TILE / TM, PITCH = TT + 4 / sizeof(E);
     E* tile = reinterpret_cast<E*>(smem);
     const int M = j.cols;
     const int per_ex = j.tiles_a * j.tiles_b;
     const int b = blk / per_ex, r = blk - b * per_ex;
-    const int m0 = (r / j.tiles_a) * TILE_M, t0 = (r % j.tiles_a) * TILE_T;
+    const int m0 = (r / j.tiles_a) * TM, t0 = (r % j.tiles_a) * TT;
     const E* src = static_cast<const E*>(j.src) + (size_t)b * M * j.T;
-    const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
-    E v[TILE_M / 4];
+    const int tx = threadIdx.x % TT, ty = threadIdx.x / TT;
+    constexpr int STEP = THREADS / TT, N = TM / STEP;
+    E v[N];
 #pragma unroll
-    for (int i = 0; i < TILE_M / 4; ++i) {
-        const int m = m0 + ty + 4 * i, t = t0 + tx;
+    for (int i = 0; i < N; ++i) {
+        const int m = m0 + ty + STEP * i, t = t0 + tx;
         v[i] = (m < M && t < j.T) ? __ldg(src + (size_t)m * j.T + t) : E(0);
     }
 #pragma unroll
-    for (int i = 0; i < TILE_M / 4; ++i) tile[(ty + 4 * i) * PITCH + tx] = v[i];
+    for (int i = 0; i < N; ++i) tile[(ty + STEP * i) * PITCH + tx] = v[i];
     __syncthreads();
-    constexpr int PER = 16 / sizeof(E), CH = TILE_M / PER;          // chunks of a 64-channel row
-    for (int k = threadIdx.x; k < TILE_T * CH; k += THREADS) {
+    constexpr int PER = 16 / sizeof(E), CH = TM / PER;              // 16-byte chunks of a position's channels
+#pragma unroll
+    for (int k = threadIdx.x; k < TT * CH; k += THREADS) {
         const int c = k % CH, t = k / CH;
         const int m = m0 + c * PER;
         if (t0 + t >= j.T || m >= M) continue;
@@ -134,69 +137,82 @@ __device__ __forceinline__ void transpose_job(const Job& j, int blk, uint8_t* sm
     }
 }
 
-// 32 patch rows (lane = row, so that neighbouring lanes read neighbouring pixels) x ct channels; the window of a (row,
-// channel) goes to kh*kw consecutive elements of the row's line in shared memory, and the lines leave in 16-byte chunks
+// cta_rows patch rows x ct channels.  Where a row's window lies and which of its rows and columns are inside the map is
+// worked out once per row; then a warp takes (32 rows, channel) at a time -- lane = row, so that neighbouring lanes read
+// neighbouring pixels -- and writes the window to kh*kw consecutive elements of the row's line in shared memory; the lines
+// leave in 16-byte chunks.  Rows are added until a CTA holds about 36 KB: CTAs of 32 rows of a 3-channel image were all
+// latency.
 template <typename E>
 __device__ __forceinline__ void im2col_job(const Job& j, int blk, uint8_t* smem) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int rb = blk / j.tiles_b, cb = blk - rb * j.tiles_b;
-    const int row0 = rb * IM_ROWS, c0 = cb * j.ct;
-    const int kk = j.kh * j.kw;
+    const int row0 = rb * j.cta_rows, c0 = cb * j.ct;
+    const int kk = j.kh * j.kw, map = j.H * j.W;
     const int nc = min(j.ct, j.C - c0);
-    const int row = row0 + lane;
-    {
-        const bool ok = row < j.rows;
-        const int b = ok ? row / j.T : 0, t = ok ? row - b * j.T : 0;
-        const int yo = t / j.Wo, xo = t - yo * j.Wo;
-        const int y0 = yo * j.stride - j.pad, x0 = xo * j.stride - j.pad;
-        const E* src = static_cast<const E*>(j.src) + (size_t)b * j.C * j.H * j.W;
-        E* line = reinterpret_cast<E*>(smem + lane * j.pitch);
+    int2* info = reinterpret_cast<int2*>(smem);                   // [cta_rows]: offset of the window, row and column masks
+    uint8_t* lines = smem + IM_MAX_ROWS * sizeof(int2);
+    const int b0 = row0 / j.T;
+    for (int r = threadIdx.x; r < j.cta_rows; r += THREADS) {
+        const int row = row0 + r;
+        int2 v = make_int2(0, 0);
+        if (row < j.rows) {
+            const int b = row / j.T, t = row - b * j.T;
+            const int yo = t / j.Wo, xo = t - yo * j.Wo;
+            const int y0 = yo * j.stride - j.pad, x0 = xo * j.stride - j.pad;
+            uint32_t ym = 0, xm = 0;
+            for (int k = 0; k < j.kh; ++k) ym |= (y0 + k >= 0 && y0 + k < j.H) ? 1u << k : 0u;
+            for (int k = 0; k < j.kw; ++k) xm |= (x0 + k >= 0 && x0 + k < j.W) ? 1u << k : 0u;
+            v = make_int2((b - b0) * j.C * map + y0 * j.W + x0, (int)(ym | xm << 16));
+        }
+        info[r] = v;
+    }
+    __syncthreads();
+    const E* src = static_cast<const E*>(j.src) + ((size_t)b0 * j.C + c0) * map;
+    const int pairs = (j.cta_rows >> 5) * nc;
+    for (int p = warp; p < pairs; p += THREADS / 32) {
+        const int rg = p / nc, ci = p - rg * nc;
+        const int r = rg * 32 + lane;
+        const int2 v = info[r];
+        const E* x = src + (ptrdiff_t)ci * map + v.x;
+        E* line = reinterpret_cast<E*>(lines + r * j.pitch) + ci * kk;
+        const uint32_t ym = (uint32_t)v.y & 0xFFFFu, xm = (uint32_t)v.y >> 16;
         if (kk == 9 && j.kw == 3) {
-            for (int ci = warp; ci < nc; ci += THREADS / 32) {
-                const E* x = src + (size_t)(c0 + ci) * j.H * j.W;
-                E v[9];
+            E e[9];
 #pragma unroll
-                for (int k = 0; k < 9; ++k) {
-                    const int y = y0 + k / 3, xx = x0 + k % 3;
-                    v[k] = (ok && y >= 0 && y < j.H && xx >= 0 && xx < j.W) ? __ldg(x + y * j.W + xx) : E(0);
-                }
+            for (int k = 0; k < 9; ++k) e[k] = (ym >> (k / 3) & xm >> (k % 3) & 1u) ? __ldg(x + (k / 3) * j.W + k % 3) : E(0);
 #pragma unroll
-                for (int k = 0; k < 9; ++k) line[ci * 9 + k] = v[k];
-            }
+            for (int k = 0; k < 9; ++k) line[k] = e[k];
         } else {
-            for (int ci = warp; ci < nc; ci += THREADS / 32) {
-                const E* x = src + (size_t)(c0 + ci) * j.H * j.W;
-                for (int ky = 0, k = 0; ky < j.kh; ++ky)
-                    for (int kx = 0; kx < j.kw; ++kx, ++k) {
-                        const int y = y0 + ky, xx = x0 + kx;
-                        line[ci * kk + k] = (ok && y >= 0 && y < j.H && xx >= 0 && xx < j.W) ? __ldg(x + y * j.W + xx) : E(0);
-                    }
-            }
+            for (int ky = 0, k = 0; ky < j.kh; ++ky)
+                for (int kx = 0; kx < j.kw; ++kx, ++k) line[k] = (ym >> ky & xm >> kx & 1u) ? __ldg(x + ky * j.W + kx) : E(0);
         }
     }
     __syncthreads();
     constexpr int PER = 16 / sizeof(E);
-    const int width = nc * kk;
+    const int width = nc * kk, rows = min(j.cta_rows, j.rows - row0);
+    E* dst = static_cast<E*>(j.dst) + (size_t)row0 * j.dst_ld + c0 * kk;
+    auto chunk = [&](int r, int c) {
+        const uint32_t* s = reinterpret_cast<const uint32_t*>(lines + r * j.pitch + c * 16);
+        *reinterpret_cast<uint4*>(dst + (size_t)r * j.dst_ld + c * PER) = make_uint4(s[0], s[1], s[2], s[3]);
+    };
     if ((j.dst_ld % PER) == 0) {
         const int cpr = (width + PER - 1) / PER;                  // the last chunk may run into the row's padding
-        for (int k = threadIdx.x; k < IM_ROWS * cpr; k += THREADS) {
-            const int r = k / cpr, c = k - r * cpr;
-            if (row0 + r >= j.rows) continue;
-            const uint32_t* s = reinterpret_cast<const uint32_t*>(smem + r * j.pitch + c * 16);
-            const uint4 v = make_uint4(s[0], s[1], s[2], s[3]);
-            *reinterpret_cast<uint4*>(static_cast<E*>(j.dst) + (size_t)(row0 + r) * j.dst_ld + c0 * kk + c * PER) = v;
+        if (cpr >= 16) {
+            for (int r = warp; r < rows; r += THREADS / 32)
+                for (int c = lane; c < cpr; c += 32) chunk(r, c);
+        } else {
+            for (int k = threadIdx.x; k < rows * cpr; k += THREADS) { const int r = k / cpr; chunk(r, k - r * cpr); }
         }
     } else {
-        for (int k = threadIdx.x; k < IM_ROWS * width; k += THREADS) {
+        for (int k = threadIdx.x; k < rows * width; k += THREADS) {
             const int r = k / width, c = k - r * width;
-            if (row0 + r >= j.rows) continue;
-            static_cast<E*>(j.dst)[(size_t)(row0 + r) * j.dst_ld + c0 * kk + c] = reinterpret_cast<const E*>(smem + r * j.pitch)[c];
+            dst[(size_t)r * j.dst_ld + c] = reinterpret_cast<const E*>(lines + r * j.pitch)[c];
         }
     }
 }
 }  // namespace stage
 
-__global__ void __launch_bounds__(stage::THREADS)
+__global__ void __launch_bounds__(stage::THREADS, 6)
 stage_operands_kernel(const __grid_constant__ stage::Launch q) {
     using namespace stage;
     extern __shared__ __align__(16) uint8_t stage_smem[];
@@ -205,7 +221,10 @@ stage_operands_kernel(const __grid_constant__ stage::Launch q) {
     const Job& j = q.job[k];
     const int blk = blockIdx.x - j.blk_begin;
     if (j.kind == ROWS || j.kind == ROWS_TO_F32) rows_job(j, blk);
-    else if (j.kind == TRANSPOSE) { if (j.es == 2) transpose_job<uint16_t>(j, blk, stage_smem); else transpose_job<uint32_t>(j, blk, stage_smem); }
+    else if (j.kind == TRANSPOSE) {
+        if (j.es == 2) { if (j.ct == 32) transpose_job<uint16_t, 32>(j, blk, stage_smem); else transpose_job<uint16_t, 64>(j, blk, stage_smem); }
+        else { if (j.ct == 32) transpose_job<uint32_t, 32>(j, blk, stage_smem); else transpose_job<uint32_t, 64>(j, blk, stage_smem); }
+    }
     else { if (j.es == 2) im2col_job<uint16_t>(j, blk, stage_smem); else im2col_job<uint32_t>(j, blk, stage_smem); }
 }
 
