@@ -49,7 +49,7 @@ enum PathSwitch : unsigned {
     SW_FORCE_SIMT = 1u << 0, SW_NO_NARROW = 1u << 1, SW_NO_NARROW_RING = 1u << 2, SW_NO_NARROW_TC = 1u << 3,
     SW_NO_NARROW_PACK = 1u << 4, SW_NARROW_PACK_BF16 = 1u << 5, SW_NO_GRAM_Q2 = 1u << 6, SW_NO_T1_TF32 = 1u << 7,
     SW_NO_FUSED_T1 = 1u << 8, SW_NO_GRAM_GROUP = 1u << 9, SW_NO_GRAD_GROUP = 1u << 10, SW_NO_CONV_TC = 1u << 11,
-    SW_NO_CONV_PATCHES = 1u << 12, SW_TILE_M1 = 1u << 13, SW_TILE_M2 = 1u << 14, SW_T1_TWO_LAUNCHES = 1u << 15, SW_NO_PAIR = 1u << 16, SW_LOG = 1u << 17, SW_NO_FACTORS_TAIL = 1u << 18, SW_NO_SM_BUDGET = 1u << 19, SW_NO_OVERLAP = 1u << 20, SW_NO_STAGE = 1u << 21, SW_GROUP_BF16 = 1u << 22,
+    SW_NO_CONV_PATCHES = 1u << 12, SW_TILE_M1 = 1u << 13, SW_TILE_M2 = 1u << 14, SW_T1_TWO_LAUNCHES = 1u << 15, SW_NO_PAIR = 1u << 16, SW_LOG = 1u << 17, SW_NO_FACTORS_TAIL = 1u << 18, SW_NO_SM_BUDGET = 1u << 19, SW_NO_OVERLAP = 1u << 20, SW_NO_STAGE = 1u << 21, SW_GROUP_BF16 = 1u << 22, SW_NO_GRAM_PER_EX = 1u << 23,
     SW_LOADED = 1u << 31
 };
 std::atomic<unsigned> g_path_switches{0};
@@ -66,7 +66,7 @@ unsigned read_path_switches() {
         {"DPCLIP_NO_PAIR", SW_NO_PAIR, '1'}, {"DPCLIP_LOG", SW_LOG, '1'},
         {"DPCLIP_NO_FACTORS_TAIL", SW_NO_FACTORS_TAIL, '1'}, {"DPCLIP_NO_SM_BUDGET", SW_NO_SM_BUDGET, '1'},
         {"DPCLIP_NO_OVERLAP", SW_NO_OVERLAP, '1'}, {"DPCLIP_NO_STAGE", SW_NO_STAGE, '1'},
-        {"DPCLIP_GROUP_BF16", SW_GROUP_BF16, '1'},
+        {"DPCLIP_GROUP_BF16", SW_GROUP_BF16, '1'}, {"DPCLIP_NO_GRAM_PER_EX", SW_NO_GRAM_PER_EX, '1'},
     };
     unsigned v = SW_LOADED;
     for (const auto& e : table) {
@@ -424,26 +424,38 @@ struct GramLayer {
     float* sq;
 };
 
+// Examples of two row blocks: their own kernel, one HBM pass per example.
+inline bool gram_two_blocks(int T) {
+    return T == 2 * tc::gram::BM && !path_switch(SW_NO_GRAM_Q2);
+}
+// Row blocks that begin with their example, not with a multiple of 128 rows.  Flattened, a row block of T = 90 meets two column
+// blocks (1.4 blocks of products an example, 1 this way), and long examples were re-read from HBM.  Kernel, flattened / this way:
+// T = 90, 320 + 3296 features, 264 examples: 55 / 47 us; T = 374, 1024, 64: 34 / 21; T = 512, 5120, 256: 608 / 383; T = 2048, 8192,
+// 32: 3813 / 844.  Below 88 rows the empty part of a block costs more (T = 77, six layers of 300 to 1100 features, 50 examples: the
+// step 139 us flattened, 145 this way), and so does a second block of few rows (256 examples of 2048 features, T = 140: 46 / 53;
+// T = 176: 60 / 54).
+inline bool gram_per_ex(int T) {
+    namespace g = tc::gram;
+    return T >= 88 && T != g::BM && !(T > g::BM && T < 168) && !gram_two_blocks(T) && !path_switch(SW_NO_GRAM_PER_EX);
+}
 // every item is on the diagonal when an example spans at most two aligned row blocks
 inline bool gram_diag_only(int T) {
     namespace g = tc::gram;
-    return (T % g::BM == 0 && T <= 2 * g::BM) || (g::BM % T == 0);
+    return (gram_per_ex(T) && T <= 2 * g::BM) || (T % g::BM == 0 && T <= 2 * g::BM) || (g::BM % T == 0);
 }
 
-// Which Gram kernel a layer takes; layers of one class can share a launch.
+// Which Gram kernel a layer takes; layers of one class can share a launch, and the kernel of class 2 takes layers of class 1 too.
 //   0: examples of exactly two row blocks (their own kernel: one HBM pass per example)
 //   1: other layers whose items all sit on the diagonal (stages of two tiles, six of them)
 //   2: the rest
 inline int gram_class(int T) {
-    if (path_switch(SW_NO_GRAM_Q2)) return gram_diag_only(T) ? 1 : 2;
-    if (T == 2 * tc::gram::BM) return 0;
+    if (gram_two_blocks(T)) return 0;
     return gram_diag_only(T) ? 1 : 2;
 }
 
-// Norms of up to gram::MAX_LAYERS layers by the Gram identity in ONE launch.  All layers must agree on
-// gram_class(T).  Layers go in descending order of bytes per group, so that the round-robin deal
+// Norms of up to gram::MAX_LAYERS layers by the Gram identity in ONE launch of kernel class `cls`.  Layers go in descending order of bytes per group, so that the round-robin deal
 // leaves the small items for the end of every CTA's queue.
-int launch_gram_group(const GramLayer* ls, int n, int* status, cudaStream_t st,
+int launch_gram_group(const GramLayer* ls, int n, int cls, int* status, cudaStream_t st,
                       const tc::gram::FactorsTail* tail = nullptr) {
     namespace g = tc::gram;
     if (n <= 0 || n > g::MAX_LAYERS) return DPCLIP_ERR_INVALID_ARG;
@@ -459,11 +471,10 @@ int launch_gram_group(const GramLayer* ls, int n, int* status, cudaStream_t st,
     g::Launch q;
     memset(&q, 0, sizeof(q));
     q.L = n; q.status = status;
-    const int cls = gram_class(ls[0].T);
     int groups = 0;
     for (int k = 0; k < n; ++k) {
         const GramLayer& y = ls[order[k]];
-        if (gram_class(y.T) != cls) return DPCLIP_ERR_INVALID_ARG;
+        if (gram_class(y.T) != cls && !(cls == 2 && gram_class(y.T) == 1)) return DPCLIP_ERR_INVALID_ARG;
         const long R = (long)y.B * y.T;
         if (!make_map_bf16(&q.map_a[k], y.A, R, y.d_in, y.lda, g::BK, g::BM) ||
             !make_map_bf16(&q.map_z[k], y.Z, R, y.d_out, y.ldz, g::BK, g::BM))
@@ -471,7 +482,14 @@ int launch_gram_group(const GramLayer* ls, int n, int* status, cudaStream_t st,
         g::Params& p = q.layer[k];
         p.R = (int)R; p.T = y.T; p.d_in = y.d_in; p.d_out = y.d_out; p.has_bias = y.has_bias ? 1 : 0;
         p.sq = y.sq;
-        if (y.T % g::BM == 0) {
+        if (cls == 0) {
+            p.dense = 1; p.q = 2;
+            p.n_groups = y.B;
+        } else if (gram_per_ex(y.T)) {
+            p.per_ex = 1; p.q = ceil_div(y.T, g::BM); p.subs = g::subs_of(p.q);
+            if ((long)y.B * p.subs > 0x3FFFFFFFL) return DPCLIP_ERR_UNSUPPORTED;
+            p.n_groups = y.B * p.subs;
+        } else if (y.T % g::BM == 0) {
             p.dense = 1; p.q = y.T / g::BM;
             p.n_groups = y.B;                     // one example per group
         } else {
@@ -521,7 +539,7 @@ int launch_gram_group(const GramLayer* ls, int n, int* status, cudaStream_t st,
 int launch_gram_norms(const void* A, long lda, const void* Z, long ldz, int B, int T, int d_in, int d_out,
                       int has_bias, float* sq, int* status, cudaStream_t st) {
     const GramLayer y = {A, lda, Z, ldz, B, T, d_in, d_out, has_bias, sq};
-    return launch_gram_group(&y, 1, status, st);
+    return launch_gram_group(&y, 1, gram_class(T), status, st);
 }
 
 // Largest scratch the split-row clipped sum can ask for: one partial tile per item, at most one
@@ -1638,7 +1656,19 @@ static int gram_layers_sqnorms(const dpclip_layer* layers, int L, int B, dpclip_
     if (dtype != DPCLIP_BF16 || !workspace || workspace_bytes < (size_t)kHeaderBytes) return DPCLIP_OK;
     if (path_switch(SW_NO_GRAM_GROUP)) return DPCLIP_OK;
     namespace g = tc::gram;
-    for (int cls = 0; cls < 3; ++cls) {                    // one launch per kernel class (see gram_class)
+    // One launch per kernel class (see gram_class); layers of class 1 join those of class 2 when there are any: a launch of their own
+    // ends in a wave of its own (convolutions of 784 and 196 positions, 16 examples: two launches 8 and 17 us one after the other,
+    // together 17).
+    auto takes = [&](const dpclip_layer& y) {
+        if (y.T <= 1 || check_layer_args(y.A, y.lda, y.Zbar, y.ldz, B, y.T, y.d_in, y.d_out, dtype)) return false;
+        if (!tc_eligible(y.A, y.lda, y.Zbar, y.ldz, dtype)) return false;
+        const int method = y.method == DPCLIP_AUTO ? dpclip_pick_method(B, y.T, y.d_in, y.d_out, y.lda, y.ldz, dtype) : y.method;
+        return method == DPCLIP_GRAM;
+    };
+    bool any_long = false;
+    for (int l = 0; l < L; ++l) any_long = any_long || (takes(layers[l]) && gram_class(layers[l].T) == 2);
+    auto class_of = [&](int T) { const int c = gram_class(T); return c == 1 && any_long ? 2 : c; };
+    for (int cls = 0; cls < 3; ++cls) {
         GramLayer batch[g::MAX_LAYERS];
         int idx[g::MAX_LAYERS];
         int n = 0;
@@ -1646,7 +1676,7 @@ static int gram_layers_sqnorms(const dpclip_layer* layers, int L, int B, dpclip_
             // a single layer gains nothing from this entry point: leave it to the per-layer call
             if (n >= 2) {
                 const bool with_tail = tail && n == L;             // this launch writes every row of sq
-                const int rc = launch_gram_group(batch, n, (int*)workspace, (cudaStream_t)stream, with_tail ? tail : nullptr);
+                const int rc = launch_gram_group(batch, n, cls, (int*)workspace, (cudaStream_t)stream, with_tail ? tail : nullptr);
                 if (rc) return rc;
                 if (taken) for (int i = 0; i < n; ++i) taken[idx[i]] = 1;
                 if (with_tail && tail_done) *tail_done = true;
@@ -1656,12 +1686,7 @@ static int gram_layers_sqnorms(const dpclip_layer* layers, int L, int B, dpclip_
         };
         for (int l = 0; l < L; ++l) {
             const dpclip_layer& y = layers[l];
-            if (y.T <= 1 || gram_class(y.T) != cls) continue;
-            if (check_layer_args(y.A, y.lda, y.Zbar, y.ldz, B, y.T, y.d_in, y.d_out, dtype)) continue;
-            if (!tc_eligible(y.A, y.lda, y.Zbar, y.ldz, dtype)) continue;
-            int method = y.method;
-            if (method == DPCLIP_AUTO) method = dpclip_pick_method(B, y.T, y.d_in, y.d_out, y.lda, y.ldz, dtype);
-            if (method != DPCLIP_GRAM) continue;
+            if (!takes(y) || class_of(y.T) != cls) continue;
             batch[n] = {y.A, y.lda, y.Zbar, y.ldz, B, y.T, y.d_in, y.d_out, y.has_bias ? 1 : 0, sq_layers + (size_t)l * B};
             idx[n] = l;
             if (++n == g::MAX_LAYERS) { const int rc = flush(); if (rc) return rc; }

@@ -70,6 +70,7 @@ struct Params {            // one layer
     int R, T, d_in, d_out, has_bias;
     int n_groups;          // dense (T % 128 == 0): examples; otherwise: 128-row blocks
     int dense, q;          // q = T / 128 blocks per example in the dense case
+    int per_ex, subs;      // row blocks begin with their example: q = ceil(T / 128), a group is one of the example's `subs` sub-items
     float* sq;
 };
 
@@ -127,12 +128,19 @@ __device__ __forceinline__ int layer_of(const Launch& q, int g) {
     return l;
 }
 
-// One unit of MMA work: row block rb against column blocks cb .. cb + ncb - 1 (ncb = 1 or 2).
-struct Sub { int rb, cb, ncb; };
+// One unit of MMA work: row block rb against column blocks cb .. cb + ncb - 1 (ncb = 1 or 2); rows and columns of the
+// blocks begin at row0 and col0.
+struct Sub { int rb, cb, ncb, row0, col0; };
+
+// Sub-items of an example of q row blocks (per_ex): row block rb takes ceil((q - rb) / 2) of them.
+__host__ __device__ __forceinline__ int subs_of(int q) { int n = 0; for (int rb = 0; rb < q; ++rb) n += (q - rb + 1) >> 1; return n; }
 
 // The sub-items of group g, in a fixed order that every warp role walks identically.
 // Row block rb pairs with column blocks rb .. cb_max(rb) (those that still hold rows of an example
 // that has rows in rb), taken two at a time so that one 128 x 256 MMA covers two of them.
+// With per_ex the row blocks begin with their example and every sub-item is a group of its own, so that neighbouring CTAs
+// stream the same example at the same time and all but the first read of a block hit L2.  One CTA walking an example of
+// 512 rows and 5120 features read it three times from HBM, 148 examples (770 MB) being in flight: 617 us for 256 of them.
 // In the dense case the row blocks of an example are walked from the LAST to the first: row block rb needs
 // the column blocks rb .. q-1, so every pass then fetches exactly one block that has not been read before
 // (its own) and re-reads the others from L2.  Walking upwards, the first pass streams the whole example
@@ -141,12 +149,24 @@ struct Sub { int rb, cb, ncb; };
 // 12.5 us its bytes take).
 struct SubIter {
     int rb, rb_first, rb_last, cb, cb_max;
+    int base;                                   // first row of block 0
     __device__ __forceinline__ static int cbmax(const Params& p, int rb) {
         const long last_row = min((long)rb * BM + BM - 1, (long)p.R - 1);
         const long e_last = last_row / p.T;
         return (int)(min((e_last + 1) * p.T - 1, (long)p.R - 1) / BM);
     }
     __device__ __forceinline__ SubIter(const Params& p, int g) {
+        base = 0;
+        if (p.per_ex) {
+            const int ex = g / p.subs;
+            int i = g - ex * p.subs;
+            rb = 0;
+            while (i >= (p.q - rb + 1) >> 1) { i -= (p.q - rb + 1) >> 1; ++rb; }
+            rb_first = rb_last = rb;
+            cb = rb + 2 * i; cb_max = min(cb + 1, p.q - 1);
+            base = ex * p.T;
+            return;
+        }
         if (p.dense) { rb_first = g * p.q; rb_last = rb_first + p.q - 1; } else { rb_first = g; rb_last = g; }
         rb = rb_last;
         cb = rb; cb_max = cbmax(p, rb);
@@ -154,6 +174,7 @@ struct SubIter {
     __device__ __forceinline__ bool next(const Params& p, Sub& s) {
         if (rb < rb_first) return false;
         s.rb = rb; s.cb = cb; s.ncb = cb + 1 <= cb_max ? 2 : 1;
+        s.row0 = base + rb * BM; s.col0 = base + cb * BM;
         cb += 2;
         if (cb > cb_max) { --rb; if (rb >= rb_first) { cb = rb; cb_max = cbmax(p, rb); } }
         return true;
@@ -217,9 +238,9 @@ gram_norm_kernel(const __grid_constant__ gram::Launch q) {
                         DPCLIP_TRACE_AT(0, tr); ++tr;
                         uint8_t* dst = smem + stage * STAGE_BYTES;
                         mbar_arrive_expect_tx(&full[stage], bytes);
-                        if (!DIAG_ONLY && !diag) tma_load_2d(dst, map, &full[stage], x, s.rb * BM);
-                        tma_load_2d(dst + B_OFF, map, &full[stage], x, s.cb * BM);
-                        if (s.ncb == 2) tma_load_2d(dst + B_OFF + TILE_BYTES, map, &full[stage], x, (s.cb + 1) * BM);
+                        if (!DIAG_ONLY && !diag) tma_load_2d(dst, map, &full[stage], x, s.row0);
+                        tma_load_2d(dst + B_OFF, map, &full[stage], x, s.col0);
+                        if (s.ncb == 2) tma_load_2d(dst + B_OFF + TILE_BYTES, map, &full[stage], x, s.col0 + BM);
                         if (++stage == STAGES) { stage = 0; phase ^= 1; }
                     }
                 }
@@ -295,12 +316,17 @@ gram_norm_kernel(const __grid_constant__ gram::Launch q) {
                 bool valid = false;
                 if (half < s.ncb) {
                     const int cbk = s.cb + half;                 // this warp's column block
-                    const long r = (long)s.rb * BM + row_local;
+                    const long r = (long)s.row0 + row_local, c_first = (long)s.col0 + half * BM;
                     valid = r < p.R;
                     e = valid ? r / p.T : 0;
+                    if (p.per_ex) {                              // rows behind the example's end are the next one's
+                        const long ex = s.row0 / p.T;
+                        valid = valid && e == ex;
+                        e = ex;
+                    }
                     // columns of the block that belong to the same example as row r
-                    int lo = (int)(max(e * p.T, (long)cbk * BM) - (long)cbk * BM);
-                    int hi = (int)(min(min((e + 1) * p.T, (long)p.R), (long)cbk * BM + BM) - (long)cbk * BM);
+                    int lo = (int)(max(e * p.T, c_first) - c_first);
+                    int hi = (int)(min(min((e + 1) * p.T, (long)p.R), c_first + BM) - c_first);
                     if (!valid) { lo = 0; hi = 0; }
                     float sa = 0.f, sb = 0.f;
                     const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + half * BM;
@@ -332,6 +358,7 @@ gram_norm_kernel(const __grid_constant__ gram::Launch q) {
                     // blocks above the diagonal stand for their mirror image too
                     val = (cbk > s.rb ? 2.f : 1.f) * (sa + (p.has_bias ? sb : 0.f));
                     if (hi <= lo) valid = false;
+                    if (p.per_ex && !valid) { val = 0.f; valid = true; }     // one example for the whole warp: one atomic
                 }
                 tc_fence_before_sync();
                 __syncwarp();

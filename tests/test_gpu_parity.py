@@ -1236,3 +1236,23 @@ def test_step_fp32_layers_in_one_launch(dp, B, specs):
             xi = oracle.normals(ref.size, seed, sid).reshape(ref.shape)
             bound = TOL["f32"]["grad"] * np.linalg.norm(ref) + 1e-5 * sigma * C * np.sqrt(ref.size)
             assert np.linalg.norm(got.cpu().numpy() - sigma * C * xi - ref) <= bound, (l, sid)
+
+
+# Gram norms with row blocks that begin with their example (65 rows on, more than two blocks) and the two-block kernel with
+# masked rows and columns: one row behind a block's edge, one short of it, several layers with and without a bias in one launch
+GRAM_ROWS = [(5, (65, 127)), (3, (129, 159, 255)), (2, (257, 300, 383)), (2, (513, 640)), (4, (192, 256))]
+
+
+@pytest.mark.parametrize("B,Ts", GRAM_ROWS)
+def test_gram_norms_row_blocks_of_an_example(dp, B, Ts):
+    specs = [(T, i, o, k % 2 == 0) for k, T in enumerate(Ts) for i, o in ((136, 72), (64, 200))]
+    data = [workloads.random_layer(90 + k, B, T, i, o, "bf16", scale_z=0.05) for k, (T, i, o, _) in enumerate(specs)]
+    plan = dp.StepPlan([dp.Layer(to_device(A, "bf16"), to_device(Z, "bf16"), s[3], dp.DPCLIP_GRAM) for (A, Z), s in zip(data, specs)])
+    taken = dp.dpclip_gram_layers_sqnorms(plan)
+    assert all(taken) or len(Ts) == 1
+    got = plan.sq_layers.cpu().numpy()
+    assert dp.dpclip_read_status(plan.workspace) == 0
+    for l, ((A, Z), s) in enumerate(zip(data, specs)):
+        ref = oracle.layer_sqnorms(A, Z, s[3])
+        # products of bf16 inputs are exact in fp32; sums of T^2 of them: 1e-4 is two orders above what fp32 sums give
+        assert max_rel(np.sqrt(got[l]), np.sqrt(ref)) <= 1e-4, s
