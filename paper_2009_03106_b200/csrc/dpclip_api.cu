@@ -49,7 +49,7 @@ enum PathSwitch : unsigned {
     SW_FORCE_SIMT = 1u << 0, SW_NO_NARROW = 1u << 1, SW_NO_NARROW_RING = 1u << 2, SW_NO_NARROW_TC = 1u << 3,
     SW_NO_NARROW_PACK = 1u << 4, SW_NARROW_PACK_BF16 = 1u << 5, SW_NO_GRAM_Q2 = 1u << 6, SW_NO_T1_TF32 = 1u << 7,
     SW_NO_FUSED_T1 = 1u << 8, SW_NO_GRAM_GROUP = 1u << 9, SW_NO_GRAD_GROUP = 1u << 10, SW_NO_CONV_TC = 1u << 11,
-    SW_NO_CONV_PATCHES = 1u << 12, SW_TILE_M1 = 1u << 13, SW_TILE_M2 = 1u << 14, SW_T1_TWO_LAUNCHES = 1u << 15, SW_NO_PAIR = 1u << 16, SW_LOG = 1u << 17, SW_NO_FACTORS_TAIL = 1u << 18, SW_NO_SM_BUDGET = 1u << 19, SW_NO_OVERLAP = 1u << 20, SW_NO_STAGE = 1u << 21, SW_GROUP_BF16 = 1u << 22, SW_NO_GRAM_PER_EX = 1u << 23,
+    SW_NO_CONV_PATCHES = 1u << 12, SW_TILE_M1 = 1u << 13, SW_TILE_M2 = 1u << 14, SW_T1_TWO_LAUNCHES = 1u << 15, SW_NO_PAIR = 1u << 16, SW_LOG = 1u << 17, SW_NO_FACTORS_TAIL = 1u << 18, SW_NO_SM_BUDGET = 1u << 19, SW_NO_OVERLAP = 1u << 20, SW_NO_STAGE = 1u << 21, SW_GROUP_BF16 = 1u << 22, SW_NO_GRAM_PER_EX = 1u << 23, SW_NO_PAIR_JOIN = 1u << 24,
     SW_LOADED = 1u << 31
 };
 std::atomic<unsigned> g_path_switches{0};
@@ -66,7 +66,7 @@ unsigned read_path_switches() {
         {"DPCLIP_NO_PAIR", SW_NO_PAIR, '1'}, {"DPCLIP_LOG", SW_LOG, '1'},
         {"DPCLIP_NO_FACTORS_TAIL", SW_NO_FACTORS_TAIL, '1'}, {"DPCLIP_NO_SM_BUDGET", SW_NO_SM_BUDGET, '1'},
         {"DPCLIP_NO_OVERLAP", SW_NO_OVERLAP, '1'}, {"DPCLIP_NO_STAGE", SW_NO_STAGE, '1'},
-        {"DPCLIP_GROUP_BF16", SW_GROUP_BF16, '1'}, {"DPCLIP_NO_GRAM_PER_EX", SW_NO_GRAM_PER_EX, '1'},
+        {"DPCLIP_GROUP_BF16", SW_GROUP_BF16, '1'}, {"DPCLIP_NO_GRAM_PER_EX", SW_NO_GRAM_PER_EX, '1'}, {"DPCLIP_NO_PAIR_JOIN", SW_NO_PAIR_JOIN, '1'},
     };
     unsigned v = SW_LOADED;
     for (const auto& e : table) {
@@ -690,6 +690,20 @@ inline bool pair_tile_ok(int d_out) {
     return pad_pair <= 1.1 * pad_single;
 }
 inline int pair_tiles(int d_in, int d_out) { return ceil_div(d_out, tc::ztp::BM) * ceil_div(d_in, tc::ztp::BN); }
+// Layers of a step that share a pair launch: besides the above, those whose padding costs a pair at most twelve stages (0.9 us
+// each), because every launch of its own costs about 25 us (set-up, a short row slice per CTA, drain, reduce).  Sequence model of
+// four projections d -> d, d -> f -> d and gates, in a graph, apart / shared: 2048 rows, d = 136, f = 400: 76 / 36 us (per-layer
+// clipping, which had no shared launch for them: 111 / 35); 16384: 123 / 79; 32000, d = 300, f = 1100 (ten stages): 515 / 428; but
+// 32000, d = 640, f = 2048 (fifteen): 557 / 572.  Not below eight stages of rows: the two kernels round a different operand to bf16
+// (c a here, c zb there), and on so few rows a step's sums are held to those of the single-layer calls.
+inline bool pair_shared_ok(int d_in, int d_out, long rows) {
+    if (path_switch(SW_NO_PAIR)) return false;
+    if (pair_tile_ok(d_out)) return true;
+    const long stages = ceil_div(rows, (long)tc::ztp::BK);
+    if (path_switch(SW_NO_PAIR_JOIN) || stages < 8) return false;
+    const double waste = pair_tiles(d_in, d_out) - 0.25 * ceil_div(d_out, 128) * ceil_div(d_in, 256);
+    return waste * stages <= 12.0 * kNumPairs;
+}
 inline size_t pair_segment_bytes(bool bias) {
     return tc::ztp::SEG_ELEMS * 4 + (bias ? (size_t)tc::ztp::BM * 4 : 0);
 }
@@ -1544,13 +1558,13 @@ static size_t step_scratch_bytes(const dpclip_layer* layers, int L, int B, dpcli
     // layers of one T that share a CTA-pair launch (up to eight): one segment per tile of all of them + one per pair
     for (int l0 = 0; l0 < L; ++l0) {
         const dpclip_layer& y0 = layers[l0];
-        if (y0.T <= 1 || !pair_tile_ok(y0.d_out)) continue;
+        if (y0.T <= 1 || !pair_shared_ok(y0.d_in, y0.d_out, (long)B * y0.T)) continue;
         bool first = true;
-        for (int l = 0; l < l0; ++l) first = first && !(layers[l].T == y0.T && pair_tile_ok(layers[l].d_out));
+        for (int l = 0; l < l0; ++l) first = first && !(layers[l].T == y0.T && pair_shared_ok(layers[l].d_in, layers[l].d_out, (long)B * y0.T));
         if (!first) continue;
         int n = 0, tiles = 0;
         for (int l = l0; l < L; ++l) {
-            if (layers[l].T != y0.T || !pair_tile_ok(layers[l].d_out)) continue;
+            if (layers[l].T != y0.T || !pair_shared_ok(layers[l].d_in, layers[l].d_out, (long)B * y0.T)) continue;
             tiles += pair_tiles(layers[l].d_in, layers[l].d_out);
             if (++n == tc::ztp::MAX_LAYERS) {
                 if (kHeaderBytes + pair_scratch_bytes(tiles) > ws) ws = kHeaderBytes + pair_scratch_bytes(tiles);
@@ -1697,7 +1711,7 @@ static int gram_layers_sqnorms(const dpclip_layer* layers, int L, int B, dpclip_
     return DPCLIP_OK;
 }
 
-static int shared_clipped_grad_launches(const dpclip_layer* layers, const bool* split, int L, int B, dpclip_dtype dtype,
+static int shared_clipped_grad_launches(const dpclip_layer* layers, const bool* split, bool join, int L, int B, dpclip_dtype dtype,
                                         const float* clip, long clip_ld, float C, float sigma, unsigned long long seed,
                                         unsigned long long stream_id0, int* taken, void* workspace,
                                         size_t workspace_bytes, void* stream);
@@ -1706,13 +1720,14 @@ int dpclip_same_shape_layers_clipped_grad_noise(const dpclip_layer* layers, int 
                                                 const float* clip, float C, float sigma, unsigned long long seed,
                                                 unsigned long long stream_id0, int* taken, void* workspace,
                                                 size_t workspace_bytes, void* stream) {
-    return shared_clipped_grad_launches(layers, nullptr, L, B, dtype, clip, 0, C, sigma, seed, stream_id0, taken, workspace,
+    return shared_clipped_grad_launches(layers, nullptr, false, L, B, dtype, clip, 0, C, sigma, seed, stream_id0, taken, workspace,
                                         workspace_bytes, stream);
 }
 
+// join: take the layers of pair_shared_ok, not only those wide enough for the pair kernel by themselves.
 // clip_ld = 0: one factor vector for all layers (global clipping); clip_ld > 0: layer l's factors are row l of
 // clip[L][clip_ld] (per-layer clipping) -- then only the CTA-pair launches, which take a vector per layer, are made.
-static int shared_clipped_grad_launches(const dpclip_layer* layers, const bool* split, int L, int B, dpclip_dtype dtype,
+static int shared_clipped_grad_launches(const dpclip_layer* layers, const bool* split, bool join, int L, int B, dpclip_dtype dtype,
                                         const float* clip, long clip_ld, float C, float sigma, unsigned long long seed,
                                         unsigned long long stream_id0, int* taken, void* workspace,
                                         size_t workspace_bytes, void* stream) {
@@ -1734,13 +1749,14 @@ static int shared_clipped_grad_launches(const dpclip_layer* layers, const bool* 
     // Layers wide enough for the CTA-pair kernel need not have one shape: all that have one T (hence the same
     // rows B*T) go into one stream-K launch, up to eight at a time.
     for (int l0 = 0; l0 < L; ++l0) {
-        if (done[l0] || !candidate(layers[l0]) || !pair_tile_ok(layers[l0].d_out)) continue;
+        auto on_pairs = [&](const dpclip_layer& y) { return join ? pair_shared_ok(y.d_in, y.d_out, (long)B * y.T) : pair_tile_ok(y.d_out); };
+        if (done[l0] || !candidate(layers[l0]) || !on_pairs(layers[l0])) continue;
         StreamLayer grp[tc::ztp::MAX_LAYERS];
         int idx[tc::ztp::MAX_LAYERS];
         int n = 0, tiles = 0;
         for (int l = l0; l < L && n < tc::ztp::MAX_LAYERS; ++l) {
             const dpclip_layer& y = layers[l];
-            if (done[l] || y.T != layers[l0].T || !pair_tile_ok(y.d_out) || !candidate(y)) continue;
+            if (done[l] || y.T != layers[l0].T || !on_pairs(y) || !candidate(y)) continue;
             grp[n] = {y.A, y.lda, y.Zbar, y.ldz, y.d_in, y.d_out, y.gW, y.ldg, y.has_bias ? y.gb : nullptr,
                       stream_id0 + 2ull * l, stream_id0 + 2ull * l + 1, clip ? clip + (size_t)l * clip_ld : nullptr,
                       split && split[l]};
@@ -2763,7 +2779,16 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
         // the factors came from the tail of the Gram launch, the last kernel of this stream: the first clipped-sum
         // launch may start loading while that tail runs
         const OverlapPrevScope overlap(factors_done);
-        rc = shared_clipped_grad_launches(layers, split, L, B, dtype, clip, 0, C, sigma, seed, stream_id0, in_grad_group, ws0,
+        // layers of several T would share several launches, one after the other on lane 0, where side by side on the lanes they
+        // are faster (four convolutions of 49 and 16 positions, 78 examples, four lanes: 97 us, 80 apart)
+        bool join = true;
+        int T_dense = 0;
+        for (int l = 0; l < L && lanes.n > 1; ++l) {
+            if (other_kind(l) || layers[l].T <= 1) continue;
+            join = join && (T_dense == 0 || layers[l].T == T_dense);
+            T_dense = layers[l].T;
+        }
+        rc = shared_clipped_grad_launches(layers, split, join, L, B, dtype, clip, 0, C, sigma, seed, stream_id0, in_grad_group, ws0,
                                           workspace_bytes, lanes.st[0]);
         if (rc) return rc;
         for (int l = 0; l < L; ++l) any_group = any_group || in_grad_group[l];
@@ -2960,7 +2985,7 @@ int dpclip_step_per_layer(const dpclip_layer* layers, int L, int B, dpclip_dtype
         for (int l = 0; l < L; ++l) th.C[l] = C_layer[l];
         factors_rows_kernel<<<L, 256, 0, (cudaStream_t)stream>>>(sq_layers, (long)B, B, th, clip_layers, norms_layers);
         if (launch_status()) return DPCLIP_ERR_CUDA;
-        rc = shared_clipped_grad_launches(layers, split, L, B, dtype, clip_layers, (long)B, C_total, sigma, seed, stream_id0,
+        rc = shared_clipped_grad_launches(layers, split, true, L, B, dtype, clip_layers, (long)B, C_total, sigma, seed, stream_id0,
                                           in_pairs, workspace, workspace_bytes, stream);
         if (rc) return rc;
         int taken[kMaxTracked];

@@ -1256,3 +1256,40 @@ def test_gram_norms_row_blocks_of_an_example(dp, B, Ts):
         ref = oracle.layer_sqnorms(A, Z, s[3])
         # products of bf16 inputs are exact in fp32; sums of T^2 of them: 1e-4 is two orders above what fp32 sums give
         assert max_rel(np.sqrt(got[l]), np.sqrt(ref)) <= 1e-4, s
+
+
+# Layers that are not wide enough for a CTA-pair launch of their own share one: outputs of less than a tile, a tile and one
+# column, rows that end inside a stage; the fewest rows that share (eight stages of 64)
+PAIR_JOIN = [(8, 64, (72, 24, 136)), (31, 17, (264, 1048, 64)), (8, 100, (304, 520, 136))]
+
+
+@pytest.mark.parametrize("clip", ["global", "per_layer"])
+@pytest.mark.parametrize("B,T,widths", PAIR_JOIN)
+def test_step_narrow_layers_share_a_pair_launch(dp, path_switch, B, T, widths, clip):
+    L = workloads.LayerSpec
+    a, b, c = widths
+    specs = (L("p", T, a, a, True, "normal"), L("i", T, a, b, True, "normal"), L("o", T, b, c, False, "relu"))
+    w = workloads.Workload("narrow", B, "bf16", specs, 1.0, 0.0, 1.0 / (B * T))
+    cal = _calibrate(w, workloads.generate(w, 11), 11, w.C)
+    mk = lambda: dp.StepPlan([dp.Layer(to_device(A, "bf16"), to_device(Z, "bf16"), s.has_bias)   # noqa: E731
+                              for (A, Z), s in zip(cal, w.layers)])
+    def step():
+        plan = mk()
+        n0 = dp.dpclip_launch_count()
+        if clip == "global":
+            plan.run(w.C, 0.0, 3)
+            factors = [plan.clip] * 3
+        else:
+            factors = list(dp.dpclip_step_per_layer(plan, [0.5, 0.6, 0.5], 0.0, 3))
+        n1 = dp.dpclip_launch_count()
+        torch.cuda.synchronize()
+        assert dp.dpclip_read_status(plan.workspace) == 0
+        return plan, factors, n1 - n0
+    plan, factors, launches = step()
+    for l, ((A, Z), s) in enumerate(zip(cal, w.layers)):
+        gW, gb = oracle.clipped_grad(A, Z, factors[l].cpu().numpy())
+        assert rel_fro(plan.gW[l].cpu().numpy(), gW) <= TOL["bf16"]["grad"]
+        if s.has_bias:
+            assert rel_fro(plan.gb[l].cpu().numpy(), gb) <= TOL["bf16"]["grad"]
+    path_switch("DPCLIP_NO_PAIR_JOIN", "1")
+    assert launches < step()[2]
