@@ -182,7 +182,9 @@ t1_all_grads_tf32_kernel(const __grid_constant__ f1::Params q) {
     constexpr int OFF_A = BF16 ? BOXES * CHUNK_BYTES : f1::OFF_A;
     // stages between two drains of the accumulator: 48 additions either way
     constexpr int FLUSH = BF16 ? 24 : f1::FLUSH;
-    static_assert(STAGES * STAGE_BYTES <= f1::STAGES * f1::STAGE_BYTES && (3 * STAGES + 4) * 8 + 8 <= 256, "shared memory layout");
+    static_assert(STAGES * STAGE_BYTES + (BF16 ? 4 * 128 * 4 : 0) <= f1::STAGES * f1::STAGE_BYTES && (3 * STAGES + 6) * 8 + 8 <= 256,
+                  "shared memory layout");
+    static_assert(!BF16 || (STAGES & (STAGES - 1)) == 0, "stage of a running number");
     const FusedT1Params& p = q.base;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);   // 1024-byte aligned; an offset from the array keeps the accesses in the shared state space
@@ -191,7 +193,9 @@ t1_all_grads_tf32_kernel(const __grid_constant__ f1::Params q) {
     uint64_t* empty = ready + STAGES;                                            // MMA done with the stage
     uint64_t* acc_full = empty + STAGES;
     uint64_t* acc_empty = acc_full + 2;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
+    uint64_t* bias_full = acc_empty + 2;                                         // bf16: the groups' bias sums are written
+    uint64_t* bias_free = bias_full + 1;                                         // ... and read
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bias_free + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     float4* out_stage = reinterpret_cast<float4*>(smem + STAGES * STAGE_BYTES + 256);
     float* clip_s = reinterpret_cast<float*>(smem + STAGES * STAGE_BYTES + 256 + OUT_STAGE_BYTES);
@@ -200,10 +204,11 @@ t1_all_grads_tf32_kernel(const __grid_constant__ f1::Params q) {
     if (threadIdx.x == 0) {
         DPCLIP_TRACE_AT(0, 255);
         for (int s = 0; s < STAGES; ++s) {
-            mbar_init(&full[s], 1); mbar_init(&ready[s], BF16 ? N_TRANSFORM_WARPS : N_TRANSFORM_WARPS + N_EPILOGUE_WARPS);
+            mbar_init(&full[s], 1); mbar_init(&ready[s], BF16 ? N_TRANSFORM_WARPS / 4 : N_TRANSFORM_WARPS + N_EPILOGUE_WARPS);
             mbar_init(&empty[s], 1);
         }
         for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], N_EPILOGUE_WARPS); }
+        mbar_init(bias_full, N_TRANSFORM_WARPS); mbar_init(bias_free, N_TRANSFORM_WARPS / 4);
         *abort_flag = 0;
         mbar_fence_init();
     }

@@ -1293,3 +1293,27 @@ def test_step_narrow_layers_share_a_pair_launch(dp, path_switch, B, T, widths, c
             assert rel_fro(plan.gb[l].cpu().numpy(), gb) <= TOL["bf16"]["grad"]
     path_switch("DPCLIP_NO_PAIR_JOIN", "1")
     assert launches < step()[2]
+
+
+# bf16 T = 1 models: the transform warps take the 32-row stages of a tile in four groups.  Fewer stages than groups, a number
+# that is no multiple of four (with several tiles per CTA, so that a tile starts at any group), and bias sums in every tile
+T1_GROUPS = [(5, (136, 72)), (33, (264, 1048)), (97, (128, 37896)), (160, (4104, 1304)), (289, (72, 19000, 10))]
+
+
+@pytest.mark.parametrize("B,widths", T1_GROUPS)
+def test_step_t1_bf16_stage_groups(dp, B, widths):
+    L = workloads.LayerSpec
+    specs = tuple(L(f"l{k}", 1, i, o, True, "normal") for k, (i, o) in enumerate(zip(widths, widths[1:])))
+    w = workloads.Workload("t1_groups", B, "bf16", specs, 1.0, 0.0, 1.0 / B)
+    cal = _calibrate(w, workloads.generate(w, 13), 13, w.C)
+    plan = dp.StepPlan([dp.Layer(to_device(A, "bf16"), to_device(Z, "bf16"), True) for A, Z in cal])
+    for _ in range(2):
+        plan.run(w.C, 0.0, 3)
+    torch.cuda.synchronize()
+    assert dp.dpclip_read_status(plan.workspace) == 0
+    clip = plan.clip.cpu().numpy()
+    for l, (A, Z) in enumerate(cal):
+        # products of c zb rounded to bf16 (2^-9 each, independent) with exact sums otherwise
+        a, z = A.reshape(B, -1).astype(np.float64), Z.reshape(B, -1).astype(np.float64)
+        assert rel_fro(plan.gW[l].cpu().numpy(), (z * clip[:, None]).T @ a) <= TOL["bf16"]["grad"]
+        assert rel_fro(plan.gb[l].cpu().numpy(), (z * clip[:, None]).sum(0)) <= TOL["bf16"]["grad"]
