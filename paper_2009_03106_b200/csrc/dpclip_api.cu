@@ -293,6 +293,16 @@ int launch_simt_norms(const void* A, long lda, const void* Z, long ldz, int B, i
 
 struct NoiseSpec { float scale; unsigned long long seed, sid_w, sid_b; };
 
+// noise in the epilogue of the fp32-ALU kernel; it indexes the dense tensor
+void simt_noise(SimtParams& p, const NoiseSpec* noise, bool* noise_done) {
+    if (!noise || !(noise->scale > 0.f) || p.ldg != p.d_in) return;
+    p.noise_scale = noise->scale;
+    p.k0 = (uint32_t)noise->seed; p.k1 = (uint32_t)(noise->seed >> 32);
+    p.sw0 = (uint32_t)noise->sid_w; p.sw1 = (uint32_t)(noise->sid_w >> 32);
+    p.sb0 = (uint32_t)noise->sid_b; p.sb1 = (uint32_t)(noise->sid_b >> 32);
+    if (noise_done) *noise_done = true;
+}
+
 int launch_simt_grad(const void* A, long lda, const void* Z, long ldz, int B, int T, int d_in, int d_out,
                      dpclip_dtype dtype, const float* clip, float* gW, long ldg, float* gb, cudaStream_t st,
                      void* workspace = nullptr, size_t workspace_bytes = 0, const NoiseSpec* noise = nullptr,
@@ -363,6 +373,7 @@ int launch_simt_grad(const void* A, long lda, const void* Z, long ldz, int B, in
         if (gb && cudaMemsetAsync(gb, 0, sizeof(float) * (size_t)d_out, st) != cudaSuccess)
             return DPCLIP_ERR_CUDA;
     }
+    simt_noise(p, noise, noise_done);
     dim3 grid(n_tiles, (unsigned)ksplit);
     if (dtype == DPCLIP_F32) zta_simt_kernel<float, true><<<grid, SIMT_THREADS, 0, st>>>(p);
     else zta_simt_kernel<__nv_bfloat16, true><<<grid, SIMT_THREADS, 0, st>>>(p);
@@ -1946,7 +1957,7 @@ extern "C++" {
 template <bool GRAD>
 static int launch_conv_tc(const SimtParams& sp, const void* X, const void* Zbar, int B, int T, int has_bias,
                           const float* clip, float* sq, float* gW, long ldg, float* gb, void* workspace,
-                          size_t workspace_bytes, cudaStream_t st) {
+                          size_t workspace_bytes, cudaStream_t st, const NoiseSpec* noise = nullptr, bool* noise_done = nullptr) {
     namespace c = tc::ctc;
     CUtensorMap mz;
     // dL/dZ as [B][T][d_out]: boxes of 64 rows t x 64 columns; as [B][d_out][T]: one box of d_out rows x 64 t
@@ -1995,6 +2006,13 @@ static int launch_conv_tc(const SimtParams& sp, const void* X, const void* Zbar,
     r.part = p.part; r.n_tiles = p.tiles_n; r.tiles_n = p.tiles_n; r.ksplit = slices; r.BM = 128; r.BN = c::BN;
     r.d_out = sp.d_out; r.d_in = sp.d_in; r.gW = gW; r.ldg = ldg; r.gb = gb; r.vec_ok = zp.vec_ok;
     r.bias_col = 1;
+    if (noise && noise->scale > 0.f && ldg == sp.d_in) {
+        r.noise_scale = noise->scale;
+        r.k0 = (uint32_t)noise->seed; r.k1 = (uint32_t)(noise->seed >> 32);
+        r.sw0 = (uint32_t)noise->sid_w; r.sw1 = (uint32_t)(noise->sid_w >> 32);
+        r.sb0 = (uint32_t)noise->sid_b; r.sb1 = (uint32_t)(noise->sid_b >> 32);
+        if (noise_done) *noise_done = true;
+    }
     const long n_vec = (long)sp.d_out * ((sp.d_in + 3) / 4);
     int lanes = 1;
     while (lanes < 8 && lanes * 2 <= slices && n_vec * lanes < 2L * kNumSMs * 256) lanes *= 2;
@@ -2106,9 +2124,10 @@ int dpclip_conv_sqnorms(const void* X, const void* Zbar, int z_channel_major, in
     return launch_status();
 }
 
-int dpclip_conv_clipped_grad(const void* X, const void* Zbar, int z_channel_major, int B, const dpclip_conv* geom,
-                             int d_out, dpclip_dtype dtype, const float* clip, float* gW, long ldg, float* gb,
-                             void* workspace, size_t workspace_bytes, void* stream) {
+static int conv_clipped_grad_impl(const void* X, const void* Zbar, int z_channel_major, int B, const dpclip_conv* geom,
+                                  int d_out, dpclip_dtype dtype, const float* clip, float* gW, long ldg, float* gb,
+                                  void* workspace, size_t workspace_bytes, const NoiseSpec* noise, bool* noise_done,
+                                  void* stream) {
     SimtParams p;
     int T = 0;
     int rc = conv_setup(p, X, Zbar, z_channel_major, B, geom, d_out, dtype, gb != nullptr, &T);
@@ -2118,7 +2137,8 @@ int dpclip_conv_clipped_grad(const void* X, const void* Zbar, int z_channel_majo
     cudaStream_t st = (cudaStream_t)stream;
     tc::ConvGather cg;
     if (conv_tc_ok(p, X, Zbar, z_channel_major, B, T, dtype, workspace, workspace_bytes)) {
-        rc = launch_conv_tc<true>(p, X, Zbar, B, T, gb != nullptr, clip, nullptr, gW, ldg, gb, workspace, workspace_bytes, st);
+        rc = launch_conv_tc<true>(p, X, Zbar, B, T, gb != nullptr, clip, nullptr, gW, ldg, gb, workspace, workspace_bytes, st, noise,
+                                  noise_done);
         if (rc <= 0) return rc;
     }
     int z_cm = z_channel_major;
@@ -2126,13 +2146,13 @@ int dpclip_conv_clipped_grad(const void* X, const void* Zbar, int z_channel_majo
     if (rc) return rc;
     if (const float* patches = conv_f32_narrow_patches(p, X, z_rows, z_cm, B, T, dtype, gb != nullptr, workspace,
                                                        workspace_bytes, st, &rc))
-        return dpclip_clipped_grad(patches, p.d_in, z_rows, d_out, B, T, p.d_in, d_out, dtype, clip, gW, ldg, gb, workspace,
-                                   (size_t)kHeaderBytes + kTcScratchBytes, stream);
+        return clipped_grad_impl(patches, p.d_in, z_rows, d_out, B, T, p.d_in, d_out, dtype, clip, gW, ldg, gb, workspace,
+                                 (size_t)kHeaderBytes + kTcScratchBytes, noise, noise_done, st);
     if (rc) return rc;
     if (conv_tf32_ok(p, X, z_rows, z_cm, B, T, dtype, workspace, workspace_bytes, &cg) &&
         workspace_bytes >= (size_t)kHeaderBytes + kTcScratchBytes)
         return launch_zta_tf32(nullptr, p.d_in, z_rows, d_out, B, T, p.d_in, d_out, false, 0, clip, gW, ldg, gb, nullptr,
-                               workspace, workspace_bytes, nullptr, nullptr, st, &cg);
+                               workspace, workspace_bytes, noise, noise_done, st, &cg);
     const int n_tiles = p.tiles_m * p.tiles_n;
     const long rows = (long)B * T;
     long ksplit = ceil_div(4 * kNumSMs, n_tiles);
@@ -2151,10 +2171,18 @@ int dpclip_conv_clipped_grad(const void* X, const void* Zbar, int z_channel_majo
             return DPCLIP_ERR_CUDA;
         if (gb && cudaMemsetAsync(gb, 0, sizeof(float) * (size_t)d_out, st) != cudaSuccess) return DPCLIP_ERR_CUDA;
     }
+    simt_noise(p, noise, noise_done);
     dim3 grid(n_tiles, (unsigned)ksplit);
     if (dtype == DPCLIP_F32) zta_simt_kernel<float, true, true><<<grid, SIMT_THREADS, 0, st>>>(p);
     else zta_simt_kernel<__nv_bfloat16, true, true><<<grid, SIMT_THREADS, 0, st>>>(p);
     return launch_status();
+}
+
+int dpclip_conv_clipped_grad(const void* X, const void* Zbar, int z_channel_major, int B, const dpclip_conv* geom,
+                             int d_out, dpclip_dtype dtype, const float* clip, float* gW, long ldg, float* gb,
+                             void* workspace, size_t workspace_bytes, void* stream) {
+    return conv_clipped_grad_impl(X, Zbar, z_channel_major, B, geom, d_out, dtype, clip, gW, ldg, gb, workspace, workspace_bytes,
+                                  nullptr, nullptr, stream);
 }
 
 int dpclip_step_noise(const dpclip_layer* layers, int L, float C, float sigma, unsigned long long seed,
@@ -2319,8 +2347,11 @@ static int other_kind_clipped_grad_noise(const dpclip_model_layer& m, int B, dpc
     } else if (m.kind == DPCLIP_KIND_CONV) {
         const long d_in = (long)m.conv.C * m.conv.kh * m.conv.kw;
         if (y.ldg != d_in) return DPCLIP_ERR_UNSUPPORTED;        // noise indexes the dense tensor
-        rc = dpclip_conv_clipped_grad(y.A, y.Zbar, m.z_channel_major, B, &m.conv, y.d_out, dtype, clip, y.gW, y.ldg, gb,
-                                      workspace, workspace_bytes, stream);
+        const NoiseSpec ns = {sigma * C, seed, sid_w, sid_b};
+        bool noise_done = false;
+        rc = conv_clipped_grad_impl(y.A, y.Zbar, m.z_channel_major, B, &m.conv, y.d_out, dtype, clip, y.gW, y.ldg, gb,
+                                    workspace, workspace_bytes, &ns, &noise_done, stream);
+        if (rc || noise_done) return rc;
         n_w = (size_t)y.d_out * (size_t)d_in;
     } else {
         return DPCLIP_ERR_INVALID_ARG;

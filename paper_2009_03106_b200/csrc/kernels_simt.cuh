@@ -20,9 +20,12 @@
 //   GRAD mode: rows = one slice of all B*T rows; each Zbar row is multiplied by
 //              its example's clip factor as it is loaded (diag(c) fused into
 //              the operand load); tiles are stored, or added atomically when
-//              the rows are split over several CTAs.
+//              the rows are split over several CTAs.  The CTAs of the first slice add
+//              the noise of their outputs: as launches of their own behind the kernel
+//              the two tensors' noise took 3 us of a 124 us step (16384 -> 10, B = 64).
 #pragma once
 #include "common.cuh"
+#include "kernels_stream.cuh"
 
 namespace dpclip {
 
@@ -39,6 +42,7 @@ struct SimtParams {
     // GRAD
     const float* clip; float* gW; long ldg; float* gb;
     long rows_total; long rows_per_split;
+    float noise_scale; uint32_t k0, k1, sw0, sw1, sb0, sb1;       // 0: no noise
     // CONV (implicit im2col): A is the feature map [B][C][H][W]; row (i, y', x') and column (c, ky, kx) of the
     // patch matrix are gathered on the fly; Z may be channel-major [B][d_out][T]
     int cC, cH, cW, kh, kw, stride, pad, Wo, z_cm;
@@ -190,6 +194,20 @@ zta_simt_kernel(SimtParams p) {
             for (int i = 0; i < 4; ++i) {
                 const int m = m0 + (ty << 2) + i;
                 if (m >= p.d_out) continue;
+                if (p.noise_scale > 0.f && blockIdx.y == 0) {
+                    const int n = n0 + (tx << 2);
+                    float z[4];
+                    if (n < p.d_in) {
+                        normals_at((size_t)m * p.d_in + n, p.sw0, p.sw1, p.k0, p.k1, z);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) if (n + j < p.d_in) acc[i][j] = fmaf(p.noise_scale, z[j], acc[i][j]);
+                    }
+                    if (n <= p.d_in && p.d_in < n + 4 && p.has_bias && p.gb) {
+                        normals_at((size_t)m, p.sb0, p.sb1, p.k0, p.k1, z);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) if (n + j == p.d_in) acc[i][j] = fmaf(p.noise_scale, z[0], acc[i][j]);
+                    }
+                }
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int n = n0 + (tx << 2) + j;
