@@ -49,7 +49,7 @@ enum PathSwitch : unsigned {
     SW_FORCE_SIMT = 1u << 0, SW_NO_NARROW = 1u << 1, SW_NO_NARROW_RING = 1u << 2, SW_NO_NARROW_TC = 1u << 3,
     SW_NO_NARROW_PACK = 1u << 4, SW_NARROW_PACK_BF16 = 1u << 5, SW_NO_GRAM_Q2 = 1u << 6, SW_NO_T1_TF32 = 1u << 7,
     SW_NO_FUSED_T1 = 1u << 8, SW_NO_GRAM_GROUP = 1u << 9, SW_NO_GRAD_GROUP = 1u << 10, SW_NO_CONV_TC = 1u << 11,
-    SW_NO_CONV_PATCHES = 1u << 12, SW_TILE_M1 = 1u << 13, SW_TILE_M2 = 1u << 14, SW_T1_TWO_LAUNCHES = 1u << 15, SW_NO_PAIR = 1u << 16, SW_LOG = 1u << 17, SW_NO_FACTORS_TAIL = 1u << 18, SW_NO_SM_BUDGET = 1u << 19, SW_NO_OVERLAP = 1u << 20, SW_NO_STAGE = 1u << 21, SW_GROUP_BF16 = 1u << 22, SW_NO_GRAM_PER_EX = 1u << 23, SW_NO_PAIR_JOIN = 1u << 24,
+    SW_NO_CONV_PATCHES = 1u << 12, SW_TILE_M1 = 1u << 13, SW_TILE_M2 = 1u << 14, SW_T1_TWO_LAUNCHES = 1u << 15, SW_NO_PAIR = 1u << 16, SW_LOG = 1u << 17, SW_NO_FACTORS_TAIL = 1u << 18, SW_NO_SM_BUDGET = 1u << 19, SW_NO_OVERLAP = 1u << 20, SW_NO_STAGE = 1u << 21, SW_NO_GRAM_PER_EX = 1u << 22, SW_NO_PAIR_JOIN = 1u << 23,
     SW_LOADED = 1u << 31
 };
 std::atomic<unsigned> g_path_switches{0};
@@ -66,7 +66,7 @@ unsigned read_path_switches() {
         {"DPCLIP_NO_PAIR", SW_NO_PAIR, '1'}, {"DPCLIP_LOG", SW_LOG, '1'},
         {"DPCLIP_NO_FACTORS_TAIL", SW_NO_FACTORS_TAIL, '1'}, {"DPCLIP_NO_SM_BUDGET", SW_NO_SM_BUDGET, '1'},
         {"DPCLIP_NO_OVERLAP", SW_NO_OVERLAP, '1'}, {"DPCLIP_NO_STAGE", SW_NO_STAGE, '1'},
-        {"DPCLIP_GROUP_BF16", SW_GROUP_BF16, '1'}, {"DPCLIP_NO_GRAM_PER_EX", SW_NO_GRAM_PER_EX, '1'}, {"DPCLIP_NO_PAIR_JOIN", SW_NO_PAIR_JOIN, '1'},
+        {"DPCLIP_NO_GRAM_PER_EX", SW_NO_GRAM_PER_EX, '1'}, {"DPCLIP_NO_PAIR_JOIN", SW_NO_PAIR_JOIN, '1'},
     };
     unsigned v = SW_LOADED;
     for (const auto& e : table) {
@@ -1057,7 +1057,7 @@ struct GroupLayer {
     int T, d_in, d_out;
     bool bias;
     float* sq;                                             // norms
-    const float* clip; bool split;                         // clipped sums
+    const float* clip;                                     // clipped sums
     float* gW; long ldg; float* gb; unsigned long long sid_w, sid_b;
 };
 constexpr size_t kGroupSlotBytes = tc::zg::SLOT_ELEMS * 4 + 256 * 4;
@@ -1109,27 +1109,26 @@ inline int clear_rows(float* const* rows, int n, int B, cudaStream_t st) {
     return DPCLIP_OK;
 }
 
-template <int MODE, bool NORM>
+template <bool NORM>
 int launch_group_kernel(const tc::zg::Maps& maps, const tc::zg::Params& p, cudaStream_t st) {
-    constexpr int smem = tc::zg::Cfg<MODE>::SMEM_BYTES;
-    if (!enable_smem(tc::zta_group_kernel<MODE, NORM>, smem)) return DPCLIP_ERR_CUDA;
-    tc::zta_group_kernel<MODE, NORM><<<2 * p.n_runs, tc::zg::THREADS, smem, st>>>(maps, p);
+    constexpr int smem = tc::zg::Cfg::SMEM_BYTES;
+    if (!enable_smem(tc::zta_group_kernel<NORM>, smem)) return DPCLIP_ERR_CUDA;
+    tc::zta_group_kernel<NORM><<<2 * p.n_runs, tc::zg::THREADS, smem, st>>>(maps, p);
     return launch_status();
 }
 
-// Norms (norm = true) or clipped sums with noise of n layers.  Returns DPCLIP_OK, a negative status, or 1 when the
+// Norms (norm = true) or clipped sums with noise of n fp32 layers.  Returns DPCLIP_OK, a negative status, or 1 when the
 // workspace cannot hold a few partial tiles (clipped sums only; nothing has been launched then).
-int launch_group(const GroupLayer* ls, int n, int B, dpclip_dtype dtype, bool norm, const NoiseSpec* noise, bool* noise_done,
+int launch_group(const GroupLayer* ls, int n, int B, bool norm, const NoiseSpec* noise, bool* noise_done,
                  void* workspace, size_t workspace_bytes, cudaStream_t st, const tc::gram::FactorsTail* tail = nullptr) {
     namespace g = tc::zg;
-    const bool f32 = dtype == DPCLIP_F32;
-    const int bk = f32 ? g::Cfg<g::F32>::BK : g::Cfg<g::BF16>::BK;
+    constexpr int bk = g::Cfg::BK;
     const int max_runs = sm_budget() / 2;
     const size_t room = workspace && workspace_bytes > (size_t)kHeaderBytes ? workspace_bytes - kHeaderBytes : 0;
     const long cap = (long)(room / kGroupSlotBytes);
     // norms of long examples keep the sums between two drains in a slot per run
     bool long_norms = false;
-    for (int l = 0; norm && f32 && l < n; ++l) long_norms = long_norms || ls[l].T > g::FLUSH * bk;
+    for (int l = 0; norm && l < n; ++l) long_norms = long_norms || ls[l].T > g::FLUSH * bk;
     if ((!norm || long_norms) && cap < 8) return norm ? DPCLIP_ERR_WORKSPACE : 1;
     bool fuse_noise = !norm && noise && noise->scale > 0.f;
     for (int l = 0; l < n && fuse_noise; ++l) fuse_noise = ls[l].ldg == ls[l].d_in;
@@ -1152,7 +1151,6 @@ int launch_group(const GroupLayer* ls, int n, int B, dpclip_dtype dtype, bool no
         // the slots of a launch: its tiles and its runs
         const int runs_cap = (norm && !long_norms) || cap >= 2L * max_runs ? max_runs : (int)(cap / 2);
         int tiles = 0;
-        bool any_split = false;
         double cost[g::MAX_LAYERS], total = 0.0;
         long units[g::MAX_LAYERS], n_units = 0;
         while (next < n && p.n_layers < g::MAX_LAYERS) {
@@ -1172,20 +1170,18 @@ int launch_group(const GroupLayer* ls, int n, int B, dpclip_dtype dtype, bool no
             q.T = y.T; q.R = (int)R;
             q.d_m = t.z_on_m ? y.d_out : y.d_in; q.d_n = t.z_on_m ? y.d_in : y.d_out; q.z_on_m = t.z_on_m ? 1 : 0;
             const CUtensorMapSwizzle sw = CU_TENSOR_MAP_SWIZZLE_128B;
-            if (f32 ? !make_map_f32(&maps.m[k], pm, R, q.d_m, lm, 32, bk, sw) || !make_map_f32(&maps.n[k], pn, R, q.d_n, ln, 32, bk, sw)
-                    : !make_map_bf16(&maps.m[k], pm, R, q.d_m, lm, 64, bk) || !make_map_bf16(&maps.n[k], pn, R, q.d_n, ln, 64, bk))
+            if (!make_map_f32(&maps.m[k], pm, R, q.d_m, lm, 32, bk, sw) || !make_map_f32(&maps.n[k], pn, R, q.d_n, ln, 32, bk, sw))
                 return DPCLIP_ERR_CUDA;
             q.tiles_m = t.tiles_m; q.tiles_n = t.tiles_n; q.N = t.N;
             q.nkb = ceil_div(norm ? (long)y.T : R, (long)bk);
             q.tile0 = next_tile; q.tiles = take; q.tile_base = tiles; q.unit_base = (int)n_units;
             q.do_bias = norm ? y.bias : y.gb != nullptr;
-            q.split = y.split ? 1 : 0; q.clip = y.clip; q.sq = y.sq;
+            q.clip = y.clip; q.sq = y.sq;
             q.gW = y.gW; q.gb = y.gb; q.ldg = y.ldg; q.vec_ok = aligned_to(y.gW, 16) && y.ldg % 4 == 0;
             q.sw0 = (uint32_t)y.sid_w; q.sw1 = (uint32_t)(y.sid_w >> 32);
             q.sb0 = (uint32_t)y.sid_b; q.sb1 = (uint32_t)(y.sid_b >> 32);
             q.blk_begin = p.n_blocks;
             if (!norm) p.n_blocks += take * 8 * (t.N / 32);
-            any_split = any_split || y.split;
             units[k] = norm ? (long)B * all : (long)take * q.nkb;
             cost[k] = norm ? (double)q.nkb * (256 + t.N) + 256 : 256 + t.N;
             total += cost[k] * units[k]; n_units += units[k]; tiles += take;
@@ -1223,12 +1219,9 @@ int launch_group(const GroupLayer* ls, int n, int B, dpclip_dtype dtype, bool no
             p.tail = *tail;
             p.tail.done = reinterpret_cast<unsigned int*>(static_cast<char*>(workspace) + kTailCounterOffset);
         }
-        DPCLIP_LOGF("group %s: %d layer(s) %s, %d tiles, %ld units, %d runs", norm ? "norms" : "clipped sums", p.n_layers,
-                    f32 ? "fp32 in three bf16 terms" : any_split ? "bf16 two-term" : "bf16", tiles, n_units, p.n_runs);
-        int rc;
-        if (norm) rc = f32 ? launch_group_kernel<g::F32, true>(maps, p, st) : launch_group_kernel<g::BF16, true>(maps, p, st);
-        else rc = f32 ? launch_group_kernel<g::F32, false>(maps, p, st)
-                : any_split ? launch_group_kernel<g::BF16_SPLIT, false>(maps, p, st) : launch_group_kernel<g::BF16, false>(maps, p, st);
+        DPCLIP_LOGF("group %s: %d layer(s), %d tiles, %ld units, %d runs", norm ? "norms" : "clipped sums", p.n_layers, tiles,
+                    n_units, p.n_runs);
+        int rc = norm ? launch_group_kernel<true>(maps, p, st) : launch_group_kernel<false>(maps, p, st);
         if (rc) return rc;
         if (norm) continue;
         const int blocks = p.n_blocks < 8 * kNumSMs ? p.n_blocks : 8 * kNumSMs;
@@ -1255,9 +1248,9 @@ int clipped_grad_impl(const void* A, long lda, const void* Zbar, long ldz, int B
         if (!group_wide(d_in, d_out))
             return launch_zta_tf32(A, lda, Zbar, ldz, B, T, d_in, d_out, false, 0, clip, gW, ldg, gb, nullptr, workspace,
                                    workspace_bytes, noise, noise_done, st);
-        GroupLayer y = {A, lda, Zbar, ldz, T, d_in, d_out, false, nullptr, clip, false, gW, ldg, gb,
+        GroupLayer y = {A, lda, Zbar, ldz, T, d_in, d_out, false, nullptr, clip, gW, ldg, gb,
                         noise ? noise->sid_w : 0ull, noise ? noise->sid_b : 0ull};
-        const int rc = launch_group(&y, 1, B, dtype, false, noise, noise_done, workspace, workspace_bytes, st);
+        const int rc = launch_group(&y, 1, B, false, noise, noise_done, workspace, workspace_bytes, st);
         return rc > 0 ? DPCLIP_ERR_WORKSPACE : rc;
     }
     return launch_simt_grad(A, lda, Zbar, ldz, B, T, d_in, d_out, dtype, clip, gW, ldg, gb, st, workspace,
@@ -1559,11 +1552,11 @@ static size_t step_scratch_bytes(const dpclip_layer* layers, int L, int B, dpcli
         long tiles = 0;
         for (int l = 0; l < L; ++l) {
             const dpclip_layer& y = layers[l];
-            if (y.T > 1 && y.d_in > 0 && y.d_out > 0 && (dtype == DPCLIP_F32 || !pair_tile_ok(y.d_out))) tiles += group_tiles(y.d_in, y.d_out);
+            if (y.T > 1 && y.d_in > 0 && y.d_out > 0 && dtype == DPCLIP_F32) tiles += group_tiles(y.d_in, y.d_out);
         }
         if (tiles > 512) tiles = 512;                        // more go in several launches
         const size_t need = kHeaderBytes + (size_t)(tiles + kNumPairs) * kGroupSlotBytes;
-        if (tiles > 0 && need > ws && (dtype == DPCLIP_BF16 || ws > (size_t)kHeaderBytes)) ws = need;
+        if (tiles > 0 && need > ws && ws > (size_t)kHeaderBytes) ws = need;
     }
     if (dtype != DPCLIP_BF16 || path_switch(SW_NO_GRAD_GROUP)) return ws;
     // layers of one T that share a CTA-pair launch (up to eight): one segment per tile of all of them + one per pair
@@ -1647,7 +1640,7 @@ int dpclip_layer_sqnorms(const void* A, long lda, const void* Zbar, long ldz, in
                     return launch_zta_tf32(A, lda, Zbar, ldz, B, T, d_in, d_out, true, has_bias, nullptr, nullptr, 0,
                                            nullptr, sq_layer, workspace, workspace_bytes, nullptr, nullptr, st);
                 GroupLayer y = {A, lda, Zbar, ldz, T, d_in, d_out, has_bias != 0, sq_layer};
-                return launch_group(&y, 1, B, dtype, true, nullptr, nullptr, workspace, workspace_bytes, st);
+                return launch_group(&y, 1, B, true, nullptr, nullptr, workspace, workspace_bytes, st);
             }
             if (!aligned_to(A, 16) || !aligned_to(Zbar, 16) || lda % 8 || ldz % 8)
                 return DPCLIP_ERR_UNSUPPORTED;
@@ -2584,10 +2577,8 @@ static int launch_stage(StagePlan& sp, cudaStream_t st) {
 // launch (skip), and -- for the norms -- by the materialised product.  taken[l] is set for them.
 static bool group_candidate(const dpclip_layer& y, int B, dpclip_dtype dtype) {
     if (y.T <= 1 || check_layer_args(y.A, y.lda, y.Zbar, y.ldz, B, y.T, y.d_in, y.d_out, dtype)) return false;
-    if (dtype == DPCLIP_F32)
-        return tf32_eligible(y.A, y.lda, y.Zbar, y.ldz, B, y.T, y.d_in, y.d_out, dtype) &&
-               !narrow_layer(y.T, y.d_in, y.d_out, y.has_bias, y.lda, y.ldz);
-    return path_switch(SW_GROUP_BF16) && tc_eligible(y.A, y.lda, y.Zbar, y.ldz, dtype);
+    return dtype == DPCLIP_F32 && tf32_eligible(y.A, y.lda, y.Zbar, y.ldz, B, y.T, y.d_in, y.d_out, dtype) &&
+           !narrow_layer(y.T, y.d_in, y.d_out, y.has_bias, y.lda, y.ldz);
 }
 // of one or two fp32 layers only the wide ones stay
 static int keep_wide(GroupLayer* g, const dpclip_layer* layers, int L, int* taken) {
@@ -2613,15 +2604,15 @@ static int group_norms(const dpclip_layer* layers, int L, int B, dpclip_dtype dt
         g[n++] = {y.A, y.lda, y.Zbar, y.ldz, y.T, y.d_in, y.d_out, y.has_bias != 0, sq_layers + (size_t)l * B};
         taken[l] = 1;
     }
-    if (dtype == DPCLIP_F32 && n < kGroupFrom) n = keep_wide(g, layers, L, taken);
+    if (n < kGroupFrom) n = keep_wide(g, layers, L, taken);
     if (n == 0) return DPCLIP_OK;
     if (!workspace || workspace_bytes < (size_t)kHeaderBytes) return DPCLIP_ERR_WORKSPACE;
     const bool with_tail = tail && n == L;
     if (tail_done) *tail_done = with_tail;
-    return launch_group(g, n, B, dtype, true, nullptr, nullptr, workspace, workspace_bytes, (cudaStream_t)stream, with_tail ? tail : nullptr);
+    return launch_group(g, n, B, true, nullptr, nullptr, workspace, workspace_bytes, (cudaStream_t)stream, with_tail ? tail : nullptr);
 }
 // clip_ld as in shared_clipped_grad_launches
-static int group_grads(const dpclip_layer* layers, const bool* split, int L, int B, dpclip_dtype dtype, const float* clip, long clip_ld,
+static int group_grads(const dpclip_layer* layers, int L, int B, dpclip_dtype dtype, const float* clip, long clip_ld,
                        float C, float sigma, unsigned long long seed, unsigned long long stream_id0, const int* skip, int* taken,
                        void* workspace, size_t workspace_bytes, void* stream) {
     GroupLayer g[64];
@@ -2631,14 +2622,14 @@ static int group_grads(const dpclip_layer* layers, const bool* split, int L, int
         const dpclip_layer& y = layers[l];
         if ((skip && skip[l]) || !group_candidate(y, B, dtype) || !y.gW || y.ldg != y.d_in || (y.has_bias && !y.gb)) continue;
         g[n++] = {y.A, y.lda, y.Zbar, y.ldz, y.T, y.d_in, y.d_out, false, nullptr, clip ? clip + (size_t)l * clip_ld : nullptr,
-                  split && split[l], y.gW, y.ldg, y.has_bias ? y.gb : nullptr, stream_id0 + 2ull * l, stream_id0 + 2ull * l + 1};
+                  y.gW, y.ldg, y.has_bias ? y.gb : nullptr, stream_id0 + 2ull * l, stream_id0 + 2ull * l + 1};
         taken[l] = 1;
     }
-    if (dtype == DPCLIP_F32 && n < kGroupFrom) n = keep_wide(g, layers, L, taken);
+    if (n < kGroupFrom) n = keep_wide(g, layers, L, taken);
     if (n == 0) return DPCLIP_OK;
     const NoiseSpec ns = {sigma * C, seed, 0, 0};
     bool noise_done = false;
-    const int rc = launch_group(g, n, B, dtype, false, &ns, &noise_done, workspace, workspace_bytes, (cudaStream_t)stream);
+    const int rc = launch_group(g, n, B, false, &ns, &noise_done, workspace, workspace_bytes, (cudaStream_t)stream);
     if (rc > 0) { for (int l = 0; l < L; ++l) taken[l] = 0; return DPCLIP_OK; }         // no room: layer by layer
     return rc;
 }
@@ -2826,7 +2817,7 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
         int skip[64], taken[64];
         for (int l = 0; l < L; ++l) skip[l] = in_grad_group[l] || other_kind(l) || (t1.active && layers[l].T == 1);
         const int b = any_group && lanes.n > 1 ? 1 : 0;
-        rc = group_grads(layers, split, L, B, dtype, clip, 0, C, sigma, seed, stream_id0, skip, taken, lanes.ws[b], workspace_bytes,
+        rc = group_grads(layers, L, B, dtype, clip, 0, C, sigma, seed, stream_id0, skip, taken, lanes.ws[b], workspace_bytes,
                          lanes.st[b]);
         if (rc) return rc;
         for (int l = 0; l < L; ++l) if (taken[l]) { any_rest = true; in_grad_group[l] = 1; }
@@ -3020,7 +3011,7 @@ int dpclip_step_per_layer(const dpclip_layer* layers, int L, int B, dpclip_dtype
                                           in_pairs, workspace, workspace_bytes, stream);
         if (rc) return rc;
         int taken[kMaxTracked];
-        rc = group_grads(layers, split, L, B, dtype, clip_layers, (long)B, C_total, sigma, seed, stream_id0, in_pairs, taken, workspace,
+        rc = group_grads(layers, L, B, dtype, clip_layers, (long)B, C_total, sigma, seed, stream_id0, in_pairs, taken, workspace,
                          workspace_bytes, stream);
         if (rc) return rc;
         for (int l = 0; l < L; ++l) in_pairs[l] = in_pairs[l] || taken[l];

@@ -1,5 +1,5 @@
 // Zb^T diag(f) A of MANY layers in one launch, on CTA pairs (tcgen05.mma.cta_group::2): the per-example norms by the
-// materialised product and the clipped sums of the layers that have no kernel of their own -- the fp32 layers above all.
+// materialised product and the clipped sums of fp32 layers.
 //
 // Why one launch.  A small model's layers are each a chain of latencies (set-up, first loads, drain) that fills few
 // SMs, and launched one after the other they add up: seven fp32 layers of 148 to 592 features (B = 61, T = 48) were 7
@@ -20,7 +20,7 @@
 //              grow along the sequence, so no slot is used twice), and reduce_group_kernel adds a tile's slots in order.
 //       NORM: unit = one (example, tile); runs end between units; squares are summed into sq with atomics.
 //
-// Types (MODE): F32       x = b0 + b1 + b2, three bf16 terms cut off the top of the fp32 word: 3 x 8 bits, exact.  Six products,
+// Numbers.      fp32 inputs: x = b0 + b1 + b2, three bf16 terms cut off the top of the fp32 word: 3 x 8 bits, exact.  Six products,
 //                         b0 b0, b0 b1, b1 b0, b1 b1, b0 b2, b2 b0; what is dropped is below 2^-22 of a product, 2^-24 on
 //                         average.  The tensor core needs as long for them as for three tf32 products (which drop as much),
 //                         but 16-bit operands come out of the MN-major layout at full rate: the twelve tf32 MMAs of a 256 x
@@ -30,8 +30,6 @@
 //                         a stage instead of twelve, and every FLUSH stages (48 additions) both are added up outside.  (Draining
 //                         one accumulator every four stages into registers of the warps that also prepare the stages took 2 us
 //                         each time, a quarter of the kernel.)
-//               BF16      one MMA per product; c * zb rounded once to bf16.
-//               BF16_SPLIT  c * zb in two bf16 terms (see zta::Cfg).
 //
 // Measured (fp32): the clipped-sum loop of 256 x 256 tiles takes 1.15 us a stage, 1.6 PFLOP/s of bf16 products, the tensor
 // core's rate (two plane stages and four raw ones, or three and two: the same).  Seven layers of 512 and 2048 features, B = 32,
@@ -46,32 +44,28 @@
 namespace dpclip {
 namespace tc {
 namespace zg {
-enum Mode : int { F32 = 0, BF16 = 1, BF16_SPLIT = 2 };
 constexpr int BM = 256, BM_CTA = 128, BN_MAX = 256;
 constexpr int PITCH = 256;                           // fp32 elements between two N-side columns of a partial tile
 constexpr size_t SLOT_ELEMS = (size_t)BN_MAX * PITCH;
 constexpr int PREP = 16, EPI = 8, THREADS = 64 + 32 * (PREP + EPI);
 constexpr int MAX_LAYERS = 16, MAX_RUNS = kNumSMs / 2;
-constexpr int FLUSH = 24;                            // F32: stages between two drains of a tile's accumulators ...
+constexpr int FLUSH = 24;                            // stages between two drains of a tile's accumulators ...
 constexpr int FLUSH_ONE = 4;                         // ... and in a segment of at most so many, one accumulator takes all products
 
-// A stage = BK rows.  BF16: one ring of stages, prepared in place.  F32: TMA fills a ring of raw stages, the planes of a
-// stage are written into a second ring.
-template <int MODE> struct Cfg {
-    static constexpr int BK = MODE == F32 ? 32 : 64;               // rows per stage
-    static constexpr int BOX = MODE == F32 ? 32 : 64;              // columns per TMA box (128 bytes)
+// A stage = BK rows.  TMA fills a ring of raw stages, the planes of a stage are written into a second ring.
+struct Cfg {
+    static constexpr int BK = 32;                                  // rows per stage
+    static constexpr int BOX = 32;                                 // columns per TMA box (128 bytes)
     static constexpr int BOX_BYTES = BK * 128;
     static constexpr int RAW_SIDE = (BM_CTA / BOX) * BOX_BYTES;    // 128 columns as loaded: 16 KB
     static constexpr int CHUNK_BYTES = BK * 128;                   // 64 bf16 columns of an operand plane
-    static constexpr int SIDE_BYTES = 2 * CHUNK_BYTES;             // 128 columns of a plane: 8 KB (F32), 16 KB
-    static constexpr int PLANES = MODE == F32 ? 3 : 1;
-    static constexpr int OFF_M = 0, OFF_N = PLANES * SIDE_BYTES, OFF_LO = 2 * SIDE_BYTES;      // OFF_LO: BF16_SPLIT
-    static constexpr int STAGE_BYTES = MODE == F32 ? 2 * PLANES * SIDE_BYTES : MODE == BF16 ? 2 * SIDE_BYTES : 3 * SIDE_BYTES;
-    static constexpr int STAGES = MODE == F32 ? 2 : 192 * 1024 / STAGE_BYTES;           // 2, 6, 4
-    static constexpr int RAW_STAGES = MODE == F32 ? 4 : STAGES;
-    static constexpr int OFF_RAW = MODE == F32 ? STAGES * STAGE_BYTES : 0;              // raw ring behind the planes
-    static constexpr int RAW_BYTES = MODE == F32 ? 2 * RAW_SIDE : STAGE_BYTES;
-    static constexpr int RING_BYTES = STAGES * STAGE_BYTES + (MODE == F32 ? RAW_STAGES * RAW_BYTES : 0);
+    static constexpr int SIDE_BYTES = 2 * CHUNK_BYTES;             // 128 columns of a plane: 8 KB
+    static constexpr int PLANES = 3;
+    static constexpr int OFF_M = 0, OFF_N = PLANES * SIDE_BYTES;
+    static constexpr int STAGE_BYTES = 2 * PLANES * SIDE_BYTES, STAGES = 2;
+    static constexpr int OFF_RAW = STAGES * STAGE_BYTES;           // raw ring behind the planes
+    static constexpr int RAW_BYTES = 2 * RAW_SIDE, RAW_STAGES = 4;
+    static constexpr int RING_BYTES = STAGES * STAGE_BYTES + RAW_STAGES * RAW_BYTES;
     static constexpr int SMEM_BYTES = RING_BYTES + 256 + 1024;
 };
 
@@ -98,7 +92,7 @@ struct Layer {
     int nkb;                       // stages of a tile (GRAD) or of an item (NORM)
     int tile0, tiles;              // GRAD: the launch covers tiles tile0 .. tile0 + tiles - 1 of the layer
     int tile_base, unit_base;      // first tile / first unit of the layer in the launch
-    int do_bias, split;
+    int do_bias;
     const float* clip;             // GRAD: [B] or NULL
     float* gW; float* gb; long ldg; int vec_ok;
     float* sq;                     // NORM: [B]
@@ -121,8 +115,8 @@ struct Params {
 };
 struct Maps { CUtensorMap m[MAX_LAYERS], n[MAX_LAYERS]; };
 
-// Tensor memory is two slots of 256 columns.  A window takes one of them in turn -- F32: the large products in the first N
-// columns, the small ones 128 further -- or, F32 with N > 128, both: the large products in slot 0, the small ones in 1, and
+// Tensor memory is two slots of 256 columns.  A window takes one of them in turn -- the large products in the first N
+// columns, the small ones 128 further -- or, with N > 128, both: the large products in slot 0, the small ones in 1, and
 // the next window waits for its drain.  A segment of at most FLUSH_ONE stages (48 additions in all) keeps everything in one
 // accumulator of one slot: the drain, 1.5 us of the 6 us of such an item at N = 256, then runs beside the next one's MMAs.
 // Every role walks the same sequence.
@@ -173,26 +167,25 @@ __device__ __forceinline__ Seg segment_at(const Params& p, int u, int u_end, int
 }
 }  // namespace zg
 
-template <int MODE, bool NORM>
+template <bool NORM>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(zg::THREADS, 1)
 zta_group_kernel(const __grid_constant__ zg::Maps maps, const __grid_constant__ zg::Params p) {
     using namespace zg;
-    using C = Cfg<MODE>;
+    using C = Cfg;
     constexpr int STAGES = C::STAGES, STAGE_BYTES = C::STAGE_BYTES, BK = C::BK, CHUNK_BYTES = C::CHUNK_BYTES;
     constexpr int RAW_STAGES = C::RAW_STAGES;
     extern __shared__ uint8_t smem_raw[];
     // 1024-byte aligned by an OFFSET from the array (keeps the accesses in the shared state space), the same in both CTAs
     uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + C::RING_BYTES);          // [RAW_STAGES] TMA landed (this CTA)
-    uint64_t* raw_free = full + RAW_STAGES;                                      // [RAW_STAGES] F32: raw stage read (own)
+    uint64_t* raw_free = full + RAW_STAGES;                                      // [RAW_STAGES] raw stage read (own)
     uint64_t* ready = raw_free + RAW_STAGES;                                     // stage prepared (rank 0's is used)
     uint64_t* empty = ready + STAGES;                                            // MMAs done with the stage (each CTA's own)
     uint64_t* acc_full = empty + STAGES;                                         // [2] accumulator complete (each CTA's own)
     uint64_t* acc_empty = acc_full + 2;                                          // [2] accumulator drained (rank 0's is used)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    volatile int* has_lo = abort_flag + 1;                                       // BF16_SPLIT: [STAGES]
-    static_assert((2 * RAW_STAGES + 2 * STAGES + 4) * 8 + 8 + (MODE == BF16_SPLIT ? 4 * STAGES : 0) <= 256, "barrier area");
+    static_assert((2 * RAW_STAGES + 2 * STAGES + 4) * 8 + 8 <= 256, "barrier area");
     static_assert(C::SMEM_BYTES <= 227 * 1024, "shared memory");
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -227,7 +220,7 @@ zta_group_kernel(const __grid_constant__ zg::Maps maps, const __grid_constant__ 
                 const int xm = w.tm * BM + (int)rank * BM_CTA, half = y.N >> 1, xn = w.tn * y.N + (int)rank * half;
                 const int n_boxes = (half + C::BOX - 1) / C::BOX;
                 for (int kb = w.kb0; kb < w.kb1; ++kb) {
-                    ok = mbar_wait(MODE == F32 ? &raw_free[stage] : &empty[stage], phase ^ 1, abort_flag, p.status);
+                    ok = mbar_wait(&raw_free[stage], phase ^ 1, abort_flag, p.status);
                     if (!ok) break;
                     DPCLIP_TRACE_AT(0, tr); ++tr;
                     uint8_t* dst = smem + C::OFF_RAW + stage * C::RAW_BYTES;
@@ -255,11 +248,11 @@ zta_group_kernel(const __grid_constant__ zg::Maps maps, const __grid_constant__ 
                 const Seg w = segment_at<NORM>(p, u, u_end, run);
                 const Layer& y = p.layer[w.layer];
                 const uint32_t idesc = make_idesc_bf16(BM, y.N, 1, 1);
-                const bool two = MODE == F32 && w.kb1 - w.kb0 > FLUSH_ONE;
+                const bool two = w.kb1 - w.kb0 > FLUSH_ONE;
                 uint32_t d_tmem = tmem_base, d_small = tmem_base;
                 for (int kb = w.kb0; kb < w.kb1; ++kb) {
                     const int k = kb - w.kb0;
-                    const bool start = MODE == F32 ? (k % FLUSH) == 0 : k == 0;
+                    const bool start = (k % FLUSH) == 0;
                     if (start) {
                         ring.take(two && y.N > 128);
                         ok = mbar_wait(&acc_empty[ring.slot], (ring.uses(ring.slot) & 1) ^ 1, abort_flag, p.status) &&
@@ -275,33 +268,19 @@ zta_group_kernel(const __grid_constant__ zg::Maps maps, const __grid_constant__ 
                     tc_fence_after_sync();
                     const uint32_t base = smem_u32(smem + stage * STAGE_BYTES);
                     // MN-major, 128-byte swizzle: 64-column chunks CHUNK_BYTES apart, 8-row groups 1024 bytes apart
-                    if (MODE == F32) {
-                        constexpr int PM[6] = {2, 0, 1, 1, 0, 0}, PN[6] = {0, 2, 1, 0, 1, 0};
+                    constexpr int PM[6] = {2, 0, 1, 1, 0, 0}, PN[6] = {0, 2, 1, 0, 1, 0};
 #pragma unroll
-                        for (int k4 = 0; k4 < BK / 16; ++k4) {
+                    for (int k4 = 0; k4 < BK / 16; ++k4) {
 #pragma unroll
-                            for (int x = 0; x < 6; ++x)
-                                mma_bf16_ss_pair(x == 5 ? d_tmem : d_small,
-                                                 make_smem_desc_sw128(base + C::OFF_M + PM[x] * C::SIDE_BYTES + k4 * 2048, CHUNK_BYTES, 1024),
-                                                 make_smem_desc_sw128(base + C::OFF_N + PN[x] * C::SIDE_BYTES + k4 * 2048, CHUNK_BYTES, 1024),
-                                                 idesc, (start && k4 == 0 && (x == 0 || (x == 5 && two))) ? 0u : 1u);
-                        }
-                    } else {
-                        const bool lo = MODE == BF16_SPLIT && has_lo[stage] != 0;
-#pragma unroll
-                        for (int k4 = 0; k4 < BK / 16; ++k4) {
-                            const uint64_t dm = make_smem_desc_sw128(base + C::OFF_M + k4 * 2048, CHUNK_BYTES, 1024);
-                            const uint64_t dn = make_smem_desc_sw128(base + C::OFF_N + k4 * 2048, CHUNK_BYTES, 1024);
-                            mma_bf16_ss_pair(d_tmem, dm, dn, idesc, (start && k4 == 0) ? 0u : 1u);
-                            if (lo) {
-                                const uint64_t dl = make_smem_desc_sw128(base + C::OFF_LO + k4 * 2048, CHUNK_BYTES, 1024);
-                                mma_bf16_ss_pair(d_tmem, y.z_on_m ? dl : dm, y.z_on_m ? dn : dl, idesc, 1u);
-                            }
-                        }
+                        for (int x = 0; x < 6; ++x)
+                            mma_bf16_ss_pair(x == 5 ? d_tmem : d_small,
+                                             make_smem_desc_sw128(base + C::OFF_M + PM[x] * C::SIDE_BYTES + k4 * 2048, CHUNK_BYTES, 1024),
+                                             make_smem_desc_sw128(base + C::OFF_N + PN[x] * C::SIDE_BYTES + k4 * 2048, CHUNK_BYTES, 1024),
+                                             idesc, (start && k4 == 0 && (x == 0 || (x == 5 && two))) ? 0u : 1u);
                     }
                     mma_commit_pair(&empty[stage], 3);          // frees the stage in both CTAs
                     if (++stage == STAGES) { stage = 0; phase ^= 1; }
-                    if (kb == w.kb1 - 1 || (MODE == F32 && (k % FLUSH) == FLUSH - 1)) {
+                    if (kb == w.kb1 - 1 || (k % FLUSH) == FLUSH - 1) {
                         mma_commit_pair(&acc_full[ring.slot], 3);
                         if (ring.wide) mma_commit_pair(&acc_full[1], 3);
                         ring.done();
@@ -312,18 +291,17 @@ zta_group_kernel(const __grid_constant__ zg::Maps maps, const __grid_constant__ 
         }
     } else if (warp < 2 + PREP) {
         // ------------------------------------------------ preparation
-        // A side of a stage is 128 columns; warp wk takes 8 of them over all rows, lane = row (twice for the 64 rows of a bf16
-        // stage): a column's bias sum stays inside a warp, and eight lanes' 16-byte accesses fall on different banks.  The
+        // A side of a stage is 128 columns; warp wk takes 8 of them over all rows, lane = row: a column's bias sum stays inside a warp, and eight lanes' 16-byte accesses fall on different banks.  The
         // 16-byte units of a row sit where the 128-byte swizzle puts them, at the same place for all rows of a thread.
         const int wk = warp - 2;
         constexpr int NR = BK / 32;
         const uint32_t off = (wk >> 3) * CHUNK_BYTES + lane * 128 + (((wk & 7) ^ (lane & 7)) << 4);
-        // F32: the two fp32 units of those columns in a raw stage
+        // the two fp32 units of those columns in a raw stage
         const uint32_t raw0 = (wk >> 2) * C::BOX_BYTES + lane * 128 + (((2 * (wk & 3)) ^ (lane & 7)) << 4);
         const uint32_t raw1 = (wk >> 2) * C::BOX_BYTES + lane * 128 + (((2 * (wk & 3) + 1) ^ (lane & 7)) << 4);
         const uint32_t ready0 = mapa_shared(smem_u32(ready), 0);
         int stage = 0; uint32_t phase = 0;
-        int raw = 0; uint32_t raw_phase = 0;                   // F32: position in the raw ring
+        int raw = 0; uint32_t raw_phase = 0;                   // position in the raw ring
         bool ok = true;
         [[maybe_unused]] int tr = 0;
         for (int u = u_begin; u < u_end && ok;) {
@@ -333,7 +311,6 @@ zta_group_kernel(const __grid_constant__ zg::Maps maps, const __grid_constant__ 
             const int half = y.N >> 1;
             const bool n_live = wk * 8 < half;                 // this warp's columns exist on the N side
             const bool z_live = z_on_m || n_live;
-            const int z_off = z_on_m ? C::OFF_M : C::OFF_N;
             const float* clip = NORM ? nullptr : y.clip;
             // every tile of the other side sees the same Zb rows: GRAD deals the bias sums of stage kb to the tile with kb %
             // tiles == its index there; NORM squares them, so one tile takes them all
@@ -359,86 +336,47 @@ zta_group_kernel(const __grid_constant__ zg::Maps maps, const __grid_constant__ 
                     }
                 }
                 const bool bias_here = y.do_bias && z_live && (NORM ? o_tile == 0 : (kb % o_tiles) == o_tile);
-                ok = mbar_wait(MODE == F32 ? &full[raw] : &full[stage], MODE == F32 ? raw_phase : phase, abort_flag, p.status);
+                ok = mbar_wait(&full[raw], raw_phase, abort_flag, p.status);
                 if (!ok) break;
                 if (threadIdx.x == 64) { DPCLIP_TRACE_AT(1, tr); ++tr; }
                 uint8_t* st = smem + stage * STAGE_BYTES + off;
-                if (MODE == F32) {
-                    const uint8_t* rw = smem + C::OFF_RAW + raw * C::RAW_BYTES;
-                    float4 x[2][2];
+                const uint8_t* rw = smem + C::OFF_RAW + raw * C::RAW_BYTES;
+                float4 x[2][2];
 #pragma unroll
-                    for (int side = 0; side < 2; ++side) {                   // 0: M, 1: N
-                        x[side][0] = *reinterpret_cast<const float4*>(rw + side * C::RAW_SIDE + raw0);
-                        x[side][1] = *reinterpret_cast<const float4*>(rw + side * C::RAW_SIDE + raw1);
-                    }
-                    uint4 b3[2][3];
+                for (int side = 0; side < 2; ++side) {                   // 0: M, 1: N
+                    x[side][0] = *reinterpret_cast<const float4*>(rw + side * C::RAW_SIDE + raw0);
+                    x[side][1] = *reinterpret_cast<const float4*>(rw + side * C::RAW_SIDE + raw1);
+                }
+                uint4 b3[2][3];
 #pragma unroll
-                    for (int side = 0; side < 2; ++side) {
-                        if (side == 1 && !n_live) continue;
-                        float v[8] = {x[side][0].x, x[side][0].y, x[side][0].z, x[side][0].w,
-                                      x[side][1].x, x[side][1].y, x[side][1].z, x[side][1].w};
-                        if ((side == 0) == (z_on_m != 0)) {
+                for (int side = 0; side < 2; ++side) {
+                    if (side == 1 && !n_live) continue;
+                    float v[8] = {x[side][0].x, x[side][0].y, x[side][0].z, x[side][0].w,
+                                  x[side][1].x, x[side][1].y, x[side][1].z, x[side][1].w};
+                    if ((side == 0) == (z_on_m != 0)) {
 #pragma unroll
-                            for (int k = 0; k < 8; ++k) v[k] *= fr[0];
-                            if (bias_here) {
-#pragma unroll
-                                for (int k = 0; k < 8; ++k) cs[k] += v[k];
-                            }
-                        }
-                        split_bf16x3(v, b3[side]);
-                    }
-                    ok = mbar_wait(&empty[stage], phase ^ 1, abort_flag, p.status);
-                    if (!ok) break;
-#pragma unroll
-                    for (int side = 0; side < 2; ++side) {
-                        if (side == 1 && !n_live) continue;
-#pragma unroll
-                        for (int k = 0; k < 3; ++k)
-                            *reinterpret_cast<uint4*>(st + side * C::OFF_N + k * C::SIDE_BYTES) = b3[side][k];
-                    }
-                    // The raw stage is given back only here: the stores above used the values, so the loads are complete.  (Given
-                    // back right after the loads were issued, it was refilled under them now and then.)
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&raw_free[raw]);
-                    if (++raw == RAW_STAGES) { raw = 0; raw_phase ^= 1; }
-                } else {
-                    const bool any = fr[0] != 1.f || fr[NR - 1] != 1.f;
-                    bool split = false;
-                    if (MODE == BF16_SPLIT) {
-                        // every warp of both CTAs sees the same rows, so all agree
-                        split = y.split && __any_sync(0xFFFFFFFFu, any);
-                        if (threadIdx.x == 64) has_lo[stage] = split ? 1 : 0;
-                    }
-                    if (z_live && (any || split || bias_here)) {
-                        uint4 v[NR], lo[NR];
-#pragma unroll
-                        for (int i = 0; i < NR; ++i) { v[i] = *reinterpret_cast<const uint4*>(st + z_off + i * 4096); lo[i] = make_uint4(0u, 0u, 0u, 0u); }
-#pragma unroll
-                        for (int i = 0; i < NR; ++i) {
-                            if (fr[i] != 1.f) {
-                                if (split) scale_bf16x8_split(v[i], lo[i], fr[i]);
-                                else scale_bf16x8(v[i], fr[i]);
-                                *reinterpret_cast<uint4*>(st + z_off + i * 4096) = v[i];
-                            }
-                            if (split) *reinterpret_cast<uint4*>(st + C::OFF_LO + i * 4096) = lo[i];
-                        }
+                        for (int k = 0; k < 8; ++k) v[k] *= fr[0];
                         if (bias_here) {
 #pragma unroll
-                            for (int i = 0; i < NR; ++i) {
-                                const uint32_t a[4] = {v[i].x, v[i].y, v[i].z, v[i].w}, b[4] = {lo[i].x, lo[i].y, lo[i].z, lo[i].w};
-#pragma unroll
-                                for (int k = 0; k < 4; ++k) {
-                                    cs[2 * k] += __uint_as_float(a[k] << 16);
-                                    cs[2 * k + 1] += __uint_as_float(a[k] & 0xFFFF0000u);
-                                    if (split) {
-                                        cs[2 * k] += __uint_as_float(b[k] << 16);
-                                        cs[2 * k + 1] += __uint_as_float(b[k] & 0xFFFF0000u);
-                                    }
-                                }
-                            }
+                            for (int k = 0; k < 8; ++k) cs[k] += v[k];
                         }
                     }
+                    split_bf16x3(v, b3[side]);
                 }
+                ok = mbar_wait(&empty[stage], phase ^ 1, abort_flag, p.status);
+                if (!ok) break;
+#pragma unroll
+                for (int side = 0; side < 2; ++side) {
+                    if (side == 1 && !n_live) continue;
+#pragma unroll
+                    for (int k = 0; k < 3; ++k)
+                        *reinterpret_cast<uint4*>(st + side * C::OFF_N + k * C::SIDE_BYTES) = b3[side][k];
+                }
+                // The raw stage is given back only here: the stores above used the values, so the loads are complete.  (Given
+                // back right after the loads were issued, it was refilled under them now and then.)
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&raw_free[raw]);
+                if (++raw == RAW_STAGES) { raw = 0; raw_phase ^= 1; }
                 fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) mbar_arrive_cluster(ready0 + stage * 8);
@@ -477,8 +415,8 @@ zta_group_kernel(const __grid_constant__ zg::Maps maps, const __grid_constant__ 
             const int nq = y.N >> 1;                           // columns of this warp: 32, 64, 96 or 128
             const bool in_range = DPCLIP_IN_RANGE(w.slot, p.n_slots, p.status);
             float* dst = p.part + (size_t)w.slot * SLOT_ELEMS + (size_t)(g * nq) * PITCH + rank * BM_CTA + quarter * 32 + lane;
-            const int windows = MODE == F32 ? (w.kb1 - w.kb0 + FLUSH - 1) / FLUSH : 1;
-            const bool two = MODE == F32 && w.kb1 - w.kb0 > FLUSH_ONE;
+            const int windows = (w.kb1 - w.kb0 + FLUSH - 1) / FLUSH;
+            const bool two = w.kb1 - w.kb0 > FLUSH_ONE;
             float fro = 0.f;
             for (int win = 0; win < windows; ++win) {
                 ring.take(two && y.N > 128);
@@ -496,13 +434,13 @@ zta_group_kernel(const __grid_constant__ zg::Maps maps, const __grid_constant__ 
                     float x[16];
 #pragma unroll
                     for (int j = 0; j < 16; ++j) x[j] = 0.f;
-                    if (MODE == F32 && win > 0 && in_range) {
+                    if (win > 0 && in_range) {
 #pragma unroll
                         for (int j = 0; j < 16; ++j) x[j] = dst[(size_t)(h + j) * PITCH];
                     }
                     uint32_t v[16];
                     tmem_ld_32x16(t_row + h, v);
-                    if (MODE == F32 && two) {
+                    if (two) {
                         uint32_t v2[16];
                         tmem_ld_32x16(t_row + to_small + h, v2);
                         tmem_ld_wait();
