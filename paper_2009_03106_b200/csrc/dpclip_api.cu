@@ -444,10 +444,11 @@ inline bool gram_two_blocks(int T) {
 // T = 90, 320 + 3296 features, 264 examples: 55 / 47 us; T = 374, 1024, 64: 34 / 21; T = 512, 5120, 256: 608 / 383; T = 2048, 8192,
 // 32: 3813 / 844.  Below 88 rows the empty part of a block costs more (T = 77, six layers of 300 to 1100 features, 50 examples: the
 // step 139 us flattened, 145 this way), and so does a second block of few rows (256 examples of 2048 features, T = 140: 46 / 53;
-// T = 176: 60 / 54).
+// T = 176: 60 / 54) or a third (seven layers of 352 to 1392 features, T = 276, 244 examples: 361 / 398; T = 300, 512 + 2048, 200:
+// 146 / 101).
 inline bool gram_per_ex(int T) {
     namespace g = tc::gram;
-    return T >= 88 && T != g::BM && !(T > g::BM && T < 168) && !gram_two_blocks(T) && !path_switch(SW_NO_GRAM_PER_EX);
+    return T >= 88 && T != g::BM && !(T > g::BM && T < 168) && !(T > 2 * g::BM && T < 288) && !gram_two_blocks(T) && !path_switch(SW_NO_GRAM_PER_EX);
 }
 // every item is on the diagonal when an example spans at most two aligned row blocks
 inline bool gram_diag_only(int T) {
