@@ -670,6 +670,7 @@ int launch_zta_tc_mt(const tc::zta::Maps& maps, tc::zta::Params p, int B, bool n
         if (ksplit > nkb) ksplit = nkb;
         if (ksplit < 1) ksplit = 1;
         p.kb_per_split = ceil_div(nkb, ksplit);
+        p.windows = ceil_div(p.kb_per_split, (long)z::SPLIT_WINDOW);
         ksplit = ceil_div(nkb, p.kb_per_split);
         p.n_items = tiles * ksplit;
         if (grp && grp->n > 0 && ksplit == 1) return 1;        // a group's outputs go through the partial tiles

@@ -667,7 +667,13 @@ constexpr int SMEM_BYTES = 192 * 1024 + 256 + OUT_STAGE_BYTES + 1024;
 // per-stage cost of the transform warps (barrier round trips, proxy fence) weighing twice.
 // SPLIT (GRAD, MT = 1): the scaled operand c * zb is held as two bf16 terms, hi + lo (relative error 2^-18 instead of
 //           2^-9), and every stage whose rows are not all unscaled runs a second set of MMAs on the lo plane.  For layers
-//           that would otherwise run on the fp32 ALUs, where the product is taken in fp32; 3 stages of 64 KB.
+//           that would otherwise run on the fp32 ALUs, where the product is taken in fp32; 3 stages of 64 KB.  The tensor
+//           core's accumulation truncates, a bias toward zero that grows with the number of additions, eight a stage: sums
+//           of two terms are drained every SPLIT_WINDOW stages and the windows are added up in fp32 (red.add of one thread,
+//           in order).  237618 rows, 321 -> 1531: relative error of the sums 3.3e-5 in one window (301 stages), 3.0e-6 with
+//           windows of 24, 2.5e-6 with 16 (two terms alone: 2.2e-6; the fp32 ALUs: 3.6e-6); step 1031, 1129 and 1177 us.
+//           read, add, store in place of red: 1242.
+constexpr int SPLIT_WINDOW = 24;
 template <int MT, bool SPLIT = false> struct Cfg {
     static_assert(!SPLIT || MT == 1, "two planes of a 256-row tile leave room for two stages only");
     static constexpr int BM = 128 * MT;
@@ -688,6 +694,7 @@ struct Params {
     int tiles_m_layer;             // d_out tiles of one layer (= tiles_m for a single layer)
     int n_items;
     int kb_per_split;              // GRAD: stages (blocks of Cfg::BK rows) per item
+    int windows;                   // SPLIT: windows of an item
     int do_bias;                   // GRAD: gb != NULL; NORM: has_bias
     const float* clip;             // GRAD: [B] or NULL
     float* gW; long ldg; float* gb; int vec_ok;
@@ -706,9 +713,20 @@ struct Maps { CUtensorMap a[MAX_LAYERS], z[MAX_LAYERS]; };
 
 struct Item { int m0, n0, tn; int row_begin, row_end; int nkb; int example; int layer; };
 
-template <int MT>
-__device__ __forceinline__ Item decode(const Params& p, int item) {
+// The items of a CTA, with SPLIT window by window.
+template <bool SPLIT>
+struct Walk {
+    int item = blockIdx.x, window = 0;
+    __device__ __forceinline__ void next(const Params& p) {
+        if (SPLIT && ++window < p.windows) return;
+        window = 0; item += gridDim.x;
+    }
+};
+
+template <int MT, bool SPLIT>
+__device__ __forceinline__ Item decode(const Params& p, const Walk<SPLIT>& at) {
     Item w;
+    const int item = at.item;
     const int n_tiles = p.tiles_m * p.tiles_n;
     const int tile = item % n_tiles, outer = item / n_tiles;
     const int tm = tile / p.tiles_n;
@@ -726,6 +744,12 @@ __device__ __forceinline__ Item decode(const Params& p, int item) {
         w.row_end = min(w.row_begin + p.kb_per_split * Cfg<MT>::BK, p.R);
     }
     w.nkb = (w.row_end - w.row_begin + Cfg<MT>::BK - 1) / Cfg<MT>::BK;
+    if (SPLIT) {                                            // 0 stages: the last slice of the rows has fewer windows
+        const int k0 = at.window * SPLIT_WINDOW;
+        w.row_begin += k0 * Cfg<MT>::BK;
+        w.nkb = max(0, min(w.nkb - k0, SPLIT_WINDOW));
+        w.row_end = min(w.row_end, w.row_begin + w.nkb * Cfg<MT>::BK);
+    }
     return w;
 }
 }  // namespace zta
@@ -797,8 +821,9 @@ zta_tc_kernel(const __grid_constant__ zta::Maps maps, const zta::Params p) {
             bool ok = true;
             int tr = 0;
             DPCLIP_TRACE_AT(0, 255);
-            for (int item = blockIdx.x; item < p.n_items && ok; item += gridDim.x) {
-                const Item w = decode<MT>(p, item);
+            for (Walk<SPLIT> at; at.item < p.n_items && ok; at.next(p)) {
+                const Item w = decode<MT, SPLIT>(p, at);
+                if (SPLIT && w.nkb == 0) continue;
                 const CUtensorMap* map_a = &maps.a[w.layer];
                 const CUtensorMap* map_z = &maps.z[w.layer];
                 for (int kb = 0; kb < w.nkb; ++kb) {
@@ -825,8 +850,9 @@ zta_tc_kernel(const __grid_constant__ zta::Maps maps, const zta::Params p) {
             int stage = 0; uint32_t phase = 0; int it = 0;
             bool ok = true;
             int tr = 0;
-            for (int item = blockIdx.x; item < p.n_items && ok; item += gridDim.x) {
-                const Item w = decode<MT>(p, item);
+            for (Walk<SPLIT> at; at.item < p.n_items && ok; at.next(p)) {
+                const Item w = decode<MT, SPLIT>(p, at);
+                if (SPLIT && w.nkb == 0) continue;
                 const int buf = it % NBUF; const uint32_t acc_phase = (it / NBUF) & 1;
                 ok = mbar_wait(&acc_empty[buf], acc_phase ^ 1, abort_flag, p.status);
                 if (!ok) break;
@@ -878,8 +904,9 @@ zta_tc_kernel(const __grid_constant__ zta::Maps maps, const zta::Params p) {
         int stage = 0; uint32_t phase = 0;
         bool ok = true;
         int tr = 0;
-        for (int item = blockIdx.x; item < p.n_items && ok; item += gridDim.x) {
-            const Item w = decode<MT>(p, item);
+        for (Walk<SPLIT> at; at.item < p.n_items && ok; at.next(p)) {
+            const Item w = decode<MT, SPLIT>(p, at);
+            if (SPLIT && w.nkb == 0) continue;
             // bias gradient = column sums of the scaled Zb tile; the values pass through these threads'
             // registers anyway, so the sums cost no extra shared-memory traffic
             float cs[MT][8];
@@ -1024,8 +1051,10 @@ zta_tc_kernel(const __grid_constant__ zta::Maps maps, const zta::Params p) {
                         ssq = fmaf(c, c, ssq);
                         if (!p.norm_mode && rs == 0) {
                             const int ml = h * 128 + q * 8 + j;
-                            if (p.bias_part) p.bias_part[(size_t)item * C::BM + ml] = c;
-                            else if (w.m0 + ml < p.d_out) red_add_f32(p.gb + w.m0 + ml, c);
+                            if (p.bias_part) {
+                                float* dst = p.bias_part + (size_t)at.item * C::BM + ml;
+                                *dst = SPLIT && at.window > 0 ? *dst + c : c;
+                            } else if (w.m0 + ml < p.d_out) red_add_f32(p.gb + w.m0 + ml, c);
                         }
                     }
                 if (p.norm_mode) {
@@ -1046,8 +1075,9 @@ zta_tc_kernel(const __grid_constant__ zta::Maps maps, const zta::Params p) {
         const int col_begin = MT == 2 ? 0 : g * (BN / 2);
         const int col_end = MT == 2 ? BN : col_begin + BN / 2;
         int it = 0;
-        for (int item = blockIdx.x; item < p.n_items; item += gridDim.x) {
-            const Item w = decode<MT>(p, item);
+        for (Walk<SPLIT> at; at.item < p.n_items; at.next(p)) {
+            const Item w = decode<MT, SPLIT>(p, at);
+            if (SPLIT && w.nkb == 0) continue;
             const int buf = it % NBUF; const uint32_t acc_phase = (it / NBUF) & 1;
             if (!mbar_wait(&acc_full[buf], acc_phase, abort_flag, p.status)) break;
             if (threadIdx.x == 64 + 32 * N_TRANSFORM_WARPS) DPCLIP_TRACE_AT(3, 2 * it);
@@ -1055,6 +1085,7 @@ zta_tc_kernel(const __grid_constant__ zta::Maps maps, const zta::Params p) {
             const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + (buf * MT + h) * BN;
             const int m_base = w.m0 + h * 128 + quarter * 32;     // first output row of this warp
             float fro = 0.f;
+            const bool add = SPLIT && at.window > 0;              // this thread's own sums of the windows before
 #pragma unroll 1
             for (int c0 = col_begin; c0 < col_end; c0 += 32) {
                 uint32_t v[32];
@@ -1083,19 +1114,21 @@ zta_tc_kernel(const __grid_constant__ zta::Maps maps, const zta::Params p) {
                         if (p.part) {
                             // rows split over several items: store the partial tile (dense, no bounds);
                             // reduce_partials_kernel adds the items of a tile in a fixed order
-                            float* dst = p.part + ((size_t)item * C::BM + (h * 128 + quarter * 32 + rr)) * BN + c0 + 4 * jj;
-                            *reinterpret_cast<float4*>(dst) = x;
+                            float* dst = p.part + ((size_t)at.item * C::BM + (h * 128 + quarter * 32 + rr)) * BN + c0 + 4 * jj;
+                            if (add) red_add_v4_f32(dst, x.x, x.y, x.z, x.w);
+                            else *reinterpret_cast<float4*>(dst) = x;
                         } else {
                             const int mm = m_base + rr;
                             if (mm < p.d_out) {
                                 float* dst = p.gW + (size_t)mm * p.ldg + n;
                                 if (p.vec_ok && n + 4 <= p.d_in) {
-                                    *reinterpret_cast<float4*>(dst) = x;
+                                    if (add) red_add_v4_f32(dst, x.x, x.y, x.z, x.w);
+                                    else *reinterpret_cast<float4*>(dst) = x;
                                 } else {
                                     const float xs[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
                                     for (int u = 0; u < 4; ++u)
-                                        if (n + u < p.d_in) dst[u] = xs[u];
+                                        if (n + u < p.d_in) dst[u] = add ? dst[u] + xs[u] : xs[u];
                                 }
                             }
                         }

@@ -66,9 +66,11 @@ constexpr int A_BYTES = (BN_CTA / 64) * CHUNK_BYTES;     // 16 KB
 constexpr int LOAD_BYTES = Z_BYTES + A_BYTES;            // 48 KB
 // SPLIT: the scaled A half in two bf16 terms, hi + lo (see zta::Cfg), for layers that would otherwise run on the fp32
 // ALUs: 64 KB per stage, three stages instead of four, and a second set of MMAs where a row of the stage is scaled.
+// Their accumulators are drained every WINDOW stages (see zta::SPLIT_WINDOW), the windows of a segment add up in its partial tile.
 template <bool SPLIT> struct Cfg {
     static constexpr int STAGE_BYTES = LOAD_BYTES + (SPLIT ? A_BYTES : 0);
     static constexpr int STAGES = 192 * 1024 / STAGE_BYTES;
+    static constexpr int WINDOW = SPLIT ? zta::SPLIT_WINDOW : 1 << 30;
 };
 constexpr int N_TRANSFORM_WARPS = 8, N_EPILOGUE_WARPS = 8;
 constexpr int THREADS = 64 + 32 * (N_TRANSFORM_WARPS + N_EPILOGUE_WARPS);
@@ -119,15 +121,23 @@ __device__ __forceinline__ float row_factor(const Params& p, const float* clip, 
 
 __host__ __device__ __forceinline__ long segment_of(long u, int S, int U, long lcm) { return u / S + u / U - u / lcm; }
 
-struct Seg { int layer, m0, n0, tn, kb0, kb1; long slot; };       // layer < 0: this pair has no tile in the segment
+// layer < 0: this pair has no tile in the segment; first: the segment's first window
+struct Seg { int layer, m0, n0, tn, kb0, kb1; bool first; long slot; };
 
-// the segment that starts at unit u of a run that ends before unit u_end, for pair j of the gang
-__device__ __forceinline__ Seg segment_at(const Params& p, long u, long u_end, int j) {
+// the window of a segment that starts at unit u of the run [u_begin, u_end), for pair j of the gang; without SPLIT a segment
+// is one window
+template <bool SPLIT>
+__device__ __forceinline__ Seg segment_at(const Params& p, long u, long u_begin, long u_end, int j) {
     Seg s;
     const int sl = (int)(u / p.S);
     s.kb0 = (int)(u - (long)sl * p.S);
     const long left = u_end - u;
     s.kb1 = (int)min((long)p.S, s.kb0 + left);
+    s.first = true;
+    if (SPLIT) {
+        s.kb1 = min(s.kb1, s.kb0 + Cfg<SPLIT>::WINDOW);
+        s.first = s.kb0 == 0 || u == u_begin;
+    }
     const int g = p.super_tile[sl * p.W + j];
     s.layer = -1; s.m0 = s.n0 = s.tn = 0; s.slot = 0;
     if (g < 0) return s;
@@ -202,7 +212,7 @@ zta_pair_kernel(const __grid_constant__ zta::Maps maps, const __grid_constant__ 
             int tr = 0;
             DPCLIP_TRACE_AT(0, 255);
             for (long u = u_begin; u < u_end && ok;) {
-                const Seg w = segment_at(p, u, u_end, gj);
+                const Seg w = segment_at<SPLIT>(p, u, u_begin, u_end, gj);
                 if (w.layer < 0) { u += w.kb1 - w.kb0; continue; }
                 const CUtensorMap* map_a = &maps.a[w.layer];
                 const CUtensorMap* map_z = &maps.z[w.layer];
@@ -234,7 +244,7 @@ zta_pair_kernel(const __grid_constant__ zta::Maps maps, const __grid_constant__ 
             bool ok = true;
             int tr = 0;
             for (long u = u_begin; u < u_end && ok;) {
-                const Seg w = segment_at(p, u, u_end, gj);
+                const Seg w = segment_at<SPLIT>(p, u, u_begin, u_end, gj);
                 if (w.layer < 0) { u += w.kb1 - w.kb0; continue; }
                 ok = mbar_wait(acc_empty, (it & 1) ^ 1, abort_flag, p.status);
                 if (!ok) break;
@@ -294,7 +304,7 @@ zta_pair_kernel(const __grid_constant__ zta::Maps maps, const __grid_constant__ 
         bool ok = true;
         int tr = 0;
         for (long u = u_begin; u < u_end && ok;) {
-            const Seg w = segment_at(p, u, u_end, gj);
+            const Seg w = segment_at<SPLIT>(p, u, u_begin, u_end, gj);
             if (w.layer < 0) { u += w.kb1 - w.kb0; continue; }
             const float* lclip = p.layer[w.layer].clip;
             for (int kb = w.kb0; kb < w.kb1; ++kb) {
@@ -384,7 +394,7 @@ zta_pair_kernel(const __grid_constant__ zta::Maps maps, const __grid_constant__ 
         int it = 0;
         bool ok = true;
         for (long u = u_begin; u < u_end && ok;) {
-            const Seg w = segment_at(p, u, u_end, gj);
+            const Seg w = segment_at<SPLIT>(p, u, u_begin, u_end, gj);
             if (w.layer < 0) { u += w.kb1 - w.kb0; continue; }
             const Layer& y = p.layer[w.layer];
             const float* lclip = y.clip;
@@ -455,8 +465,10 @@ zta_pair_kernel(const __grid_constant__ zta::Maps maps, const __grid_constant__ 
                         c += __shfl_xor_sync(0xFFFFFFFFu, c, 2);
                         c += __shfl_xor_sync(0xFFFFFFFFu, c, 4);
                         c += __shfl_xor_sync(0xFFFFFFFFu, c, 8);
-                        if (rs == 0 && DPCLIP_IN_RANGE(w.slot, p.n_segments, p.status))
-                            p.bias_part[(size_t)w.slot * BM + (int)rank * BM_CTA + h2 * 128 + q * 8 + j] = c;
+                        if (rs == 0 && DPCLIP_IN_RANGE(w.slot, p.n_segments, p.status)) {
+                            float* dst = p.bias_part + (size_t)w.slot * BM + (int)rank * BM_CTA + h2 * 128 + q * 8 + j;
+                            *dst = SPLIT && !w.first ? *dst + c : c;
+                        }
                     }
             }
             if (!mbar_wait(acc_full, it & 1, abort_flag, p.status)) break;
@@ -486,8 +498,11 @@ zta_pair_kernel(const __grid_constant__ zta::Maps maps, const __grid_constant__ 
                     const float4 x = st[rr * 8 + (jj ^ (rr & 7))];
                     // the segment's partial tile (dense 512 x 256, no bounds: rows and columns past the layer's
                     // extent hold the zeros TMA filled in)
-                    if (DPCLIP_IN_RANGE(w.slot, p.n_segments, p.status) && DPCLIP_IN_RANGE(ml0 + rr, BM, p.status))
-                        *reinterpret_cast<float4*>(seg + (size_t)(ml0 + rr) * BN + c0 + 4 * jj) = x;
+                    if (DPCLIP_IN_RANGE(w.slot, p.n_segments, p.status) && DPCLIP_IN_RANGE(ml0 + rr, BM, p.status)) {
+                        float* dst = seg + (size_t)(ml0 + rr) * BN + c0 + 4 * jj;
+                        if (SPLIT && !w.first) red_add_v4_f32(dst, x.x, x.y, x.z, x.w);
+                        else *reinterpret_cast<float4*>(dst) = x;
+                    }
                 }
                 __syncwarp();
             }

@@ -1178,6 +1178,29 @@ def test_step_staged_operands(dp, B, specs, dtype, path_switch):
         assert rel_fro(g.cpu().numpy(), h.cpu().numpy()) <= 2 * TOL["f32"]["grad"]
 
 
+# Staged bf16 layers of many rows: the sums of two-term operands in windows of 24 stages.  One narrow layer (single-CTA kernel,
+# two tiles), one on CTA pairs, and two of several tiles sharing a launch, where runs begin and end inside a tile
+STAGED_LONG = [(512, 1024, ((65, 130),)), (512, 1024, ((65, 260),)), (256, 200, ((300, 301), (301, 700)))]
+
+
+@pytest.mark.parametrize("B,T,widths", STAGED_LONG)
+def test_step_staged_sums_of_many_rows(dp, B, T, widths):
+    gen = torch.Generator(device="cuda"); gen.manual_seed(3)
+    randn = lambda *s: torch.randn(*s, generator=gen, device="cuda")   # noqa: E731
+    scale = torch.exp(torch.rand(B, 1, 1, generator=gen, device="cuda") * 2.8 - 1.4) / np.sqrt(T * sum(i * o for i, o in widths))
+    plan = dp.StepPlan([dp.Layer(randn(B, T, i).bfloat16(), (randn(B, T, o) * scale).bfloat16(), True) for i, o in widths])
+    plan.run(1.0, 0.0, 1)
+    assert dp.dpclip_read_status(plan.workspace) == 0
+    assert 0 < int((plan.clip < 1).sum()) < B
+    for y, gW, gb in zip(plan.layers, plan.gW, plan.gb):
+        a = y.A.double().view(B * T, -1)
+        cz = (y.Zbar.double() * plan.clip.double()[:, None, None]).view(B * T, -1)
+        # two bf16 terms: 2^-18 a product at most, 2.2e-6 as a root mean square; truncation of a window's 192 additions,
+        # about 1e-8 each.  (In one window the three cases err by 6.1e-6, 1.2e-5 and 7e-6.)
+        assert rel_fro(gW.cpu().numpy(), (cz.T @ a).cpu().numpy()) <= 4.5e-6
+        assert rel_fro(gb.cpu().numpy(), cz.sum(0).cpu().numpy()) <= 4.5e-6
+
+
 STAGED_CONVS = [  # B, C, H, W, k, pad, stride, d_out, channel-major dL/dZ
     (5, 3, 28, 28, 3, 1, 1, 16, True), (6, 33, 15, 14, 3, 1, 2, 160, True), (4, 40, 9, 11, (3, 2), 1, 1, 257, False),
     (3, 9, 14, 14, 5, 2, 2, 30, True), (4, 64, 7, 7, 1, 0, 1, 65, True), (33, 64, 14, 14, 3, 1, 1, 128, True)]
