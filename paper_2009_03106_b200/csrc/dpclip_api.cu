@@ -2803,11 +2803,13 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
         // the factors came from the tail of the Gram launch, the last kernel of this stream: the first clipped-sum
         // launch may start loading while that tail runs
         const OverlapPrevScope overlap(factors_done);
-        // layers of several T would share several launches, one after the other on lane 0, where side by side on the lanes they
-        // are faster (four convolutions of 49 and 16 positions, 78 examples, four lanes: 97 us, 80 apart)
+        // Layers of several T would share several launches, one after the other on lane 0, where side by side on the lanes they
+        // are faster (four convolutions of 49 and 16 positions, 78 examples, four lanes: 68 us, 47 apart; layers of 100 and 50
+        // positions: 70, 45).  On one lane sharing would win (77 us, 117 apart), but the shared kernel rounds c a where the
+        // layers' own round c zb, and a step's results do not depend on the number of lanes.
         bool join = true;
         int T_dense = 0;
-        for (int l = 0; l < L && lanes.n > 1; ++l) {
+        for (int l = 0; l < L; ++l) {
             if (other_kind(l) || layers[l].T <= 1) continue;
             join = join && (T_dense == 0 || layers[l].T == T_dense);
             T_dense = layers[l].T;

@@ -1340,3 +1340,24 @@ def test_step_t1_bf16_stage_groups(dp, B, widths):
         a, z = A.reshape(B, -1).astype(np.float64), Z.reshape(B, -1).astype(np.float64)
         assert rel_fro(plan.gW[l].cpu().numpy(), (z * clip[:, None]).T @ a) <= TOL["bf16"]["grad"]
         assert rel_fro(plan.gb[l].cpu().numpy(), (z * clip[:, None]).sum(0)) <= TOL["bf16"]["grad"]
+
+
+# Narrow bf16 layers of two T: the kernels that share a launch and those that do not round another operand to bf16, so which of
+# them a layer takes must not depend on the number of streams
+@pytest.mark.parametrize("B,specs", [(16, ((49, 136, 72), (49, 72, 136), (40, 136, 200), (40, 200, 72))),
+                                     (33, ((64, 264, 96), (31, 264, 96), (31, 96, 304)))])
+def test_step_rounds_alike_on_one_and_several_streams(dp, B, specs):
+    data = [workloads.random_layer(110 + k, B, T, i, o, "bf16", scale_z=0.05) for k, (T, i, o) in enumerate(specs)]
+    sq = np.stack([oracle.layer_sqnorms(A, Z, True) for A, Z in data])
+    C = float(np.median(np.sqrt(sq.sum(0)))) * 1.001
+    plan = dp.StepPlan([dp.Layer(to_device(A, "bf16"), to_device(Z, "bf16"), True) for A, Z in data])
+    plan.run(C, 0.0, 3)
+    one = [g.cpu().numpy() for g in plan.gW]
+    for branches in (2, 4):
+        plan.run_streams(C, 0.0, 3, branches=branches)
+        torch.cuda.synchronize()
+        assert all(dp.dpclip_read_status(w) == 0 for w in plan.workspaces())
+        for g, h in zip(one, plan.gW):
+            # the same products in another order: fp32 rounding.  c a against c zb is 1e-3; factors that differ in the last
+            # bit move a few roundings of c zb (2^-9 of an element in a hundred thousand)
+            assert rel_fro(h.cpu().numpy(), g) <= 2e-5
