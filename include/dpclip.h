@@ -244,7 +244,9 @@ int dpclip_step(const dpclip_layer* layers /* host */, int L, int B, dpclip_dtyp
 /* dpclip_step with the launches of a stage spread over several streams INSIDE the library (Algorithm 1
  * fixes only the order norms -> factors -> clipped sums; within the norm stage and within the clipped-sum
  * stage the layers are independent, so one layer's kernel can start on the SMs another layer's kernel has
- * already left).  Same arguments and results as dpclip_step, bit for bit, except:
+ * already left).  Same arguments as dpclip_step, and the same results
+ * up to the rounding of fp32 sums: rows may be cut elsewhere, and narrow fp32 layers take the kernel that is faster
+ * beside others.  A bf16 layer takes the same kernel, which rounds the same operand, on any number of streams.  Except:
  *   streams     host array of n_streams (1..8) distinct cudaStream_t.  streams[0] is the caller's stream:
  *               the step waits for nothing but what is already enqueued there, and when the call returns
  *               everything the step enqueued, on any stream, is ordered before whatever the caller enqueues

@@ -1084,11 +1084,28 @@ inline GroupTiling group_tiling(int d_in, int d_out) {
     return cz < ca ? z : a;
 }
 // fp32: layers with a side of at most 128 leave the 256-column tiles mostly prepared for few products, and are as fast in
-// zta_tf32_kernel (128 x 128 tiles), one or two of them; from three on the shared launch wins (convolutions 288 -> 64 and
-// 576 -> 128 of a CNN, two streams: 139 us a step by layer, 147 together; seven layers of 148 to 592 features, B = 61, T = 48:
-// 252 us a step by layer, 83 together).
+// zta_tf32_kernel (128 x 128 tiles), one or two of them; from three on the shared launch wins on one stream (three layers 288 -> 64,
+// T = 256, 128 examples: 215 us a step by layer, 194 together; 576 -> 128, T = 64: 143 / 108; four 100 -> 100, T = 200, 64: 136 / 84).
 inline bool group_wide(int d_in, int d_out) { return d_in > 128 && d_out > 128; }
 constexpr int kGroupFrom = 3;
+// On several streams the launches of zta_tf32_kernel run side by side, so a narrow layer joins only where the shared launch's
+// extra work on it takes less than the launches it saves: microseconds over all SMs, a pair's stage 0.00225 a column, a CTA's
+// 128 x 128 stage 0.7, a tile's drain 1 and 1.5, saved 1.1 per layer of the clipped sum and 2 in the norms.  Steps on four streams,
+// by layer / sums together / norms together / both: three layers 288 -> 64, T = 256, 128 examples: 169 / 178 / 182 / 189;
+// 576 -> 128, T = 64: 111 / 107 / 107 / 103; 512 -> 64, T = 256, 64: 131 / 121 / 124 / 113; four 100 -> 100, T = 200, 64:
+// 70 / 66 / 80 / 78.
+inline double group_stage_us(int d_in, int d_out) {
+    const GroupTiling t = group_tiling(d_in, d_out);
+    return t.tiles_m * t.tiles_n * (256 + t.N) * 0.00225;
+}
+inline bool group_joins(const dpclip_layer& y, int B, int n, bool norm) {
+    if (group_wide(y.d_in, y.d_out)) return true;
+    const GroupTiling t = group_tiling(y.d_in, y.d_out);
+    const double pair = group_stage_us(y.d_in, y.d_out) / (kNumSMs / 2), tiles = ceil_div(y.d_out, 128) * ceil_div(y.d_in, 128);
+    if (!norm) return ceil_div((long)B * y.T, 32L) * (pair - tiles * 0.7 / kNumSMs) <= 1.1 * n;
+    const int stages = ceil_div(y.T, 32L);
+    return B * (stages * pair + t.tiles_m * t.tiles_n / (kNumSMs / 2.0) - tiles * (stages * 0.7 + 1.5) / kNumSMs) <= 2.0;
+}
 inline int group_tiles(int d_in, int d_out) { const GroupTiling t = group_tiling(d_in, d_out); return t.tiles_m * t.tiles_n; }
 
 // Clears the rows of sq that a launch accumulates into, adjacent rows in one memset.
@@ -2582,18 +2599,24 @@ static bool group_candidate(const dpclip_layer& y, int B, dpclip_dtype dtype) {
     return dtype == DPCLIP_F32 && tf32_eligible(y.A, y.lda, y.Zbar, y.ldz, B, y.T, y.d_in, y.d_out, dtype) &&
            !narrow_layer(y.T, y.d_in, y.d_out, y.has_bias, y.lda, y.ldz);
 }
-// of one or two fp32 layers only the wide ones stay
-static int keep_wide(GroupLayer* g, const dpclip_layer* layers, int L, int* taken) {
-    int k = 0, i = 0;
-    for (int l = 0; l < L; ++l) {
-        if (!taken[l]) continue;
-        if (group_wide(layers[l].d_in, layers[l].d_out)) g[k++] = g[i]; else taken[l] = 0;
-        ++i;
-    }
-    return k;
+// The layers that stay of the n taken: on several streams those that pay, of one or two fp32 layers the wide ones
+static int keep_group(GroupLayer* g, int n, const dpclip_layer* layers, int L, int B, bool norm, int streams, int* taken) {
+    auto keep = [&](auto&& stays) {
+        int k = 0, i = 0;
+        for (int l = 0; l < L; ++l) {
+            if (!taken[l]) continue;
+            if (stays(layers[l])) g[k++] = g[i]; else taken[l] = 0;
+            ++i;
+        }
+        return k;
+    };
+    const int all = n;
+    if (streams > 1) n = keep([&](const dpclip_layer& y) { return group_joins(y, B, all, norm); });
+    if (n < kGroupFrom) n = keep([](const dpclip_layer& y) { return group_wide(y.d_in, y.d_out); });
+    return n;
 }
 static int group_norms(const dpclip_layer* layers, int L, int B, dpclip_dtype dtype, float* sq_layers, const int* skip, int* taken,
-                       void* workspace, size_t workspace_bytes, void* stream, const tc::gram::FactorsTail* tail, bool* tail_done) {
+                       void* workspace, size_t workspace_bytes, void* stream, const tc::gram::FactorsTail* tail, bool* tail_done, int streams) {
     GroupLayer g[64];
     int n = 0;
     for (int l = 0; l < L; ++l) {
@@ -2606,7 +2629,7 @@ static int group_norms(const dpclip_layer* layers, int L, int B, dpclip_dtype dt
         g[n++] = {y.A, y.lda, y.Zbar, y.ldz, y.T, y.d_in, y.d_out, y.has_bias != 0, sq_layers + (size_t)l * B};
         taken[l] = 1;
     }
-    if (n < kGroupFrom) n = keep_wide(g, layers, L, taken);
+    n = keep_group(g, n, layers, L, B, true, streams, taken);
     if (n == 0) return DPCLIP_OK;
     if (!workspace || workspace_bytes < (size_t)kHeaderBytes) return DPCLIP_ERR_WORKSPACE;
     const bool with_tail = tail && n == L;
@@ -2616,7 +2639,7 @@ static int group_norms(const dpclip_layer* layers, int L, int B, dpclip_dtype dt
 // clip_ld as in shared_clipped_grad_launches
 static int group_grads(const dpclip_layer* layers, int L, int B, dpclip_dtype dtype, const float* clip, long clip_ld,
                        float C, float sigma, unsigned long long seed, unsigned long long stream_id0, const int* skip, int* taken,
-                       void* workspace, size_t workspace_bytes, void* stream) {
+                       void* workspace, size_t workspace_bytes, void* stream, int streams) {
     GroupLayer g[64];
     int n = 0;
     for (int l = 0; l < L; ++l) {
@@ -2627,7 +2650,7 @@ static int group_grads(const dpclip_layer* layers, int L, int B, dpclip_dtype dt
                   y.gW, y.ldg, y.has_bias ? y.gb : nullptr, stream_id0 + 2ull * l, stream_id0 + 2ull * l + 1};
         taken[l] = 1;
     }
-    if (n < kGroupFrom) n = keep_wide(g, layers, L, taken);
+    n = keep_group(g, n, layers, L, B, false, streams, taken);
     if (n == 0) return DPCLIP_OK;
     const NoiseSpec ns = {sigma * C, seed, 0, 0};
     bool noise_done = false;
@@ -2728,7 +2751,7 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
         const int b = any_gram && lanes.n > 1 ? 1 : 0;
         rc = group_norms(layers, L, B, dtype, sq_layers, skip, taken, lanes.ws[b], workspace_bytes, lanes.st[b],
                          (!t1.active && !any_other && !any_gram && !path_switch(SW_NO_FACTORS_TAIL)) ? &tail : nullptr,
-                         any_gram ? nullptr : &factors_done);
+                         any_gram ? nullptr : &factors_done, lanes.n);
         if (rc) return rc;
         for (int l = 0; l < L; ++l) {
             any_mat = any_mat || taken[l];
@@ -2822,7 +2845,7 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
         for (int l = 0; l < L; ++l) skip[l] = in_grad_group[l] || other_kind(l) || (t1.active && layers[l].T == 1);
         const int b = any_group && lanes.n > 1 ? 1 : 0;
         rc = group_grads(layers, L, B, dtype, clip, 0, C, sigma, seed, stream_id0, skip, taken, lanes.ws[b], workspace_bytes,
-                         lanes.st[b]);
+                         lanes.st[b], lanes.n);
         if (rc) return rc;
         for (int l = 0; l < L; ++l) if (taken[l]) { any_rest = true; in_grad_group[l] = 1; }
     }
@@ -2995,7 +3018,7 @@ int dpclip_step_per_layer(const dpclip_layer* layers, int L, int B, dpclip_dtype
         rc = dpclip_gram_layers_sqnorms(layers, L, B, dtype, sq_layers, in_gram, workspace, workspace_bytes, stream);
         if (rc) return rc;
         int taken[kMaxTracked];
-        rc = group_norms(layers, L, B, dtype, sq_layers, in_gram, taken, workspace, workspace_bytes, stream, nullptr, nullptr);
+        rc = group_norms(layers, L, B, dtype, sq_layers, in_gram, taken, workspace, workspace_bytes, stream, nullptr, nullptr, 1);
         if (rc) return rc;
         for (int l = 0; l < L; ++l) in_gram[l] = in_gram[l] || taken[l];
     }
@@ -3016,7 +3039,7 @@ int dpclip_step_per_layer(const dpclip_layer* layers, int L, int B, dpclip_dtype
         if (rc) return rc;
         int taken[kMaxTracked];
         rc = group_grads(layers, L, B, dtype, clip_layers, (long)B, C_total, sigma, seed, stream_id0, in_pairs, taken, workspace,
-                         workspace_bytes, stream);
+                         workspace_bytes, stream, 1);
         if (rc) return rc;
         for (int l = 0; l < L; ++l) in_pairs[l] = in_pairs[l] || taken[l];
     } else {

@@ -1361,3 +1361,24 @@ def test_step_rounds_alike_on_one_and_several_streams(dp, B, specs):
             # the same products in another order: fp32 rounding.  c a against c zb is 1e-3; factors that differ in the last
             # bit move a few roundings of c zb (2^-9 of an element in a hundred thousand)
             assert rel_fro(h.cpu().numpy(), g) <= 2e-5
+
+
+# Three narrow fp32 layers share the launches on one stream; on four, those whose padding costs more than the launches saved keep
+# launches of their own (288 -> 64: 56 % of two 256 x 64 tiles are used; 512 -> 64: all of them)
+@pytest.mark.parametrize("widths,apart", [((288, 64), True), ((512, 64), False)])
+def test_step_fp32_narrow_layers_on_several_streams(dp, widths, apart):
+    gen = torch.Generator(device="cuda"); gen.manual_seed(5)
+    B, T = 90, 256
+    plan = dp.StepPlan([dp.Layer(torch.randn(B, T, widths[0], generator=gen, device="cuda"),
+                                 torch.randn(B, T, widths[1], generator=gen, device="cuda") * 1e-3, True) for _ in range(3)])
+    counts, results = [], []
+    for step in (lambda: plan.run(0.5, 0.02, 1), lambda: plan.run_streams(0.5, 0.02, 1, branches=4)):
+        n0 = dp.dpclip_launch_count()
+        step()
+        torch.cuda.synchronize()
+        counts.append(dp.dpclip_launch_count() - n0)
+        results.append([t.clone() for t in (plan.norms, plan.clip, *plan.gW, *plan.gb)])
+        assert all(dp.dpclip_read_status(w) == 0 for w in plan.workspaces())
+    assert counts[1] > counts[0] if apart else counts[1] == counts[0]
+    for one, four in zip(*results):
+        assert rel_fro(four.cpu().numpy(), one.cpu().numpy()) <= TOL["f32"]["grad"]
