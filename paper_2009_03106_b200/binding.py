@@ -383,9 +383,11 @@ class StepPlan:
             self._branch_ws = [self.workspace] + [torch.empty_like(self.workspace) for _ in range(branches - 1)]
             for w in self._branch_ws[1:]:
                 dpclip_workspace_init(w)
-            self._streams = [torch.cuda.Stream() for _ in range(branches - 1)]
+            # one to spare: torch hands its streams out in rotation, so the caller's stream may be one of these
+            self._streams = [torch.cuda.Stream() for _ in range(branches)]
             torch.cuda.synchronize()
-        return self._streams[:branches - 1], self._branch_ws[:branches]
+        current = torch.cuda.current_stream()
+        return [s for s in self._streams if s != current][:branches - 1], self._branch_ws[:branches]
 
     def run_streams(self, C: float, sigma: float, seed: int, stream_id0: int = 0, branches: int = 4) -> None:
         """One dpclip_step_streams call: the library spreads the launches of a stage over `branches` streams,

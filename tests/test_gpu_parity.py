@@ -1382,3 +1382,20 @@ def test_step_fp32_narrow_layers_on_several_streams(dp, widths, apart):
     assert counts[1] > counts[0] if apart else counts[1] == counts[0]
     for one, four in zip(*results):
         assert rel_fro(four.cpu().numpy(), one.cpu().numpy()) <= TOL["f32"]["grad"]
+
+
+def test_run_streams_from_one_of_the_plans_own_streams(dp):
+    """torch hands its streams out in rotation: the stream a caller works on (or captures on) may be one the plan was given."""
+    w = workloads.seq("bf16", B=4, T=40, d=64, d_ff=128)
+    layers = workloads.generate(w, 1)
+    plan = dp.StepPlan([dp.Layer(to_device(A, w.dtype), to_device(Z, w.dtype), s.has_bias) for (A, Z), s in zip(layers, w.layers)])
+    plan.run_streams(w.C, w.sigma, 1, branches=4)
+    torch.cuda.synchronize()
+    first = plan.flat.clone()
+    for s in list(plan._streams):
+        plan.flat.zero_()
+        torch.cuda.synchronize()
+        with torch.cuda.stream(s):
+            plan.run_streams(w.C, w.sigma, 1, branches=4)
+        torch.cuda.synchronize()
+        assert rel_fro(plan.flat.cpu().numpy(), first.cpu().numpy()) <= 2e-6
