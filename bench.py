@@ -14,7 +14,7 @@ and, with per-kernel detail, under "workloads".  Rank 0 prints ONE JSON line.
 
 Timing: CUDA events on the launching stream, max over ranks.  Models with T > 1
 layers (hundreds of microseconds per step): one step = one replay of a CUDA
-graph that holds ONE dpclip_step_streams call (the library forks over four
+graph that holds ONE dpclip_step_lanes call (the library forks over four
 streams inside the call); events around every step, the L2 flushed by a 256 MB
 write between steps (outside the events).  All-T=1 models (one launch of about
 ten microseconds per step): the K timed steps are recorded back to back into
@@ -1005,7 +1005,7 @@ def main():
                                     "call each); one event pair around the region, median of 3 regions")
         line["single_step_graph_ms_per_step"] = res["single_graph_ms"]
     else:
-        line["launch"] = ("CUDA graph replay of one step = ONE dpclip_step_streams call (the library forks over 4 "
+        line["launch"] = ("CUDA graph replay of one step = ONE dpclip_step_lanes call (the library forks over 4 "
                                     "streams); events around every step")
     line["breakdown_us"] = res["breakdown"]
     line["e2e"] = dict(value=w.B / (res["e2e_ms"] * 1e-3), unit=UNIT, h2d_bytes_per_step=res["h2d"],

@@ -244,9 +244,9 @@ int dpclip_step(const dpclip_layer* layers /* host */, int L, int B, dpclip_dtyp
 /* dpclip_step with the launches of a stage spread over several streams INSIDE the library (Algorithm 1
  * fixes only the order norms -> factors -> clipped sums; within the norm stage and within the clipped-sum
  * stage the layers are independent, so one layer's kernel can start on the SMs another layer's kernel has
- * already left).  Same arguments as dpclip_step, and the same results
- * up to the rounding of fp32 sums: rows may be cut elsewhere, and narrow fp32 layers take the kernel that is faster
- * beside others.  A bf16 layer takes the same kernel, which rounds the same operand, on any number of streams.  Except:
+ * already left).  Results agree with dpclip_step up to the rounding of fp32 sums: rows may be cut elsewhere, and
+ * narrow fp32 layers take the kernel that is faster beside others; a bf16 layer takes the same kernel, which rounds
+ * the same operand, on any number of streams.  Same arguments as dpclip_step, except:
  *   streams     host array of n_streams (1..8) distinct cudaStream_t.  streams[0] is the caller's stream:
  *               the step waits for nothing but what is already enqueued there, and when the call returns
  *               everything the step enqueued, on any stream, is ordered before whatever the caller enqueues
@@ -266,6 +266,14 @@ int dpclip_step_streams(const dpclip_layer* layers /* host */, int L, int B, dpc
                         float* sq_layers, float* clip, float* norms,
                         int n_streams, void* const* streams /* host */, void* const* workspaces /* host */,
                         size_t workspace_bytes);
+/* dpclip_step_streams with a size per workspace (host array of n_streams): workspaces[0] as for dpclip_step, the others
+ * need only dpclip_step_side_workspace_bytes(), because the copies of layers whose rows TMA cannot address lie in the
+ * first alone.  INVALID_ARG for a null size array. */
+int dpclip_step_lanes(const dpclip_layer* layers /* host */, int L, int B, dpclip_dtype dtype,
+                      float C, float sigma, unsigned long long seed, unsigned long long stream_id0,
+                      float* sq_layers, float* clip, float* norms,
+                      int n_streams, void* const* streams /* host */, void* const* workspaces /* host */,
+                      const size_t* workspace_bytes /* host */);
 
 /* Convolution layers given by their INPUT feature map (implicit im2col).  Algorithm 3 unfolds the input into
  * the patch matrix (kh * kw copies of every pixel) and reshapes dL/dZ to [tau, c_out, T]; here element
@@ -353,6 +361,14 @@ int dpclip_model_step_streams(const dpclip_model_layer* layers /* host */, int L
                               float* sq_layers, float* clip, float* norms,
                               int n_streams, void* const* streams /* host */, void* const* workspaces /* host */,
                               size_t workspace_bytes);
+/* The same with a size per workspace, as dpclip_step_lanes: the first of dpclip_model_workspace_bytes(), the others of
+ * dpclip_model_side_workspace_bytes(). */
+int dpclip_model_step_lanes(const dpclip_model_layer* layers /* host */, int L, int B, dpclip_dtype dtype,
+                            float C, float sigma, unsigned long long seed, unsigned long long stream_id0,
+                            float* sq_layers, float* clip, float* norms,
+                            int n_streams, void* const* streams /* host */, void* const* workspaces /* host */,
+                            const size_t* workspace_bytes /* host */);
+size_t dpclip_model_side_workspace_bytes(const dpclip_model_layer* layers /* host */, int L, int B, dpclip_dtype dtype);
 
 /* Parameter updates with the noise folded in (one pass over the parameters instead of a noise pass and
  * an optimiser pass).  gsum is the PRE-noise clipped sum of one tensor (run the step with sigma = 0);
@@ -460,9 +476,12 @@ size_t dpclip_workspace_bytes(int B, int T, int d_in, int d_out, dpclip_dtype dt
 /* Workspace for dpclip_step / dpclip_step_streams / dpclip_step_per_layer over these layers: the largest
  * per-layer need, and room for the launches several layers share (bf16 layers of one T whose d_out is wide
  * enough for 512-row tiles go into one clipped-sum launch: one fp32 partial tile of 512 x 256 per output tile
- * of all of them and one per pair of SMs).  With less (but at least the per-layer needs) the step still
- * runs, those layers in launches of their own. */
+ * of all of them and one per pair of SMs; fp32 layers likewise), and 16-byte aligned copies of the operands that TMA
+ * cannot address (at most 3 GB).  With less (but at least the per-layer needs) the step still runs, those layers in
+ * launches of their own and the unaligned ones on the fp32 ALUs. */
 size_t dpclip_step_workspace_bytes(const dpclip_layer* layers /* host */, int L, int B, dpclip_dtype dtype);
+/* What the workspaces of the streams after the first need (dpclip_step_lanes): the above without the staged copies. */
+size_t dpclip_step_side_workspace_bytes(const dpclip_layer* layers /* host */, int L, int B, dpclip_dtype dtype);
 
 /* Zero the 256-byte status header.  Call once after allocating a workspace. */
 int dpclip_workspace_init(void* workspace, size_t workspace_bytes, void* stream);

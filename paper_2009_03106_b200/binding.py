@@ -107,6 +107,13 @@ def load_library():
     L.dpclip_model_step_streams.argtypes = [ctypes.POINTER(_CModelLayer), _i, _i, _i, _f, _f, _u64, _u64, _vp, _vp, _vp,
                                             _i, ctypes.POINTER(_vp), ctypes.POINTER(_vp), _sz]
     L.dpclip_model_step_streams.restype = _i
+    for f, desc in ((L.dpclip_step_lanes, _CLayer), (L.dpclip_model_step_lanes, _CModelLayer)):
+        f.argtypes = [ctypes.POINTER(desc), _i, _i, _i, _f, _f, _u64, _u64, _vp, _vp, _vp, _i, ctypes.POINTER(_vp),
+                      ctypes.POINTER(_vp), ctypes.POINTER(_sz)]
+        f.restype = _i
+    for f, desc in ((L.dpclip_step_side_workspace_bytes, _CLayer), (L.dpclip_model_side_workspace_bytes, _CModelLayer)):
+        f.argtypes = [ctypes.POINTER(desc), _i, _i, _i]
+        f.restype = _sz
     L.dpclip_step_host.argtypes = [ctypes.POINTER(_CLayer), _i, _i, _i, _f, _f, _u64, _u64, _vp, _vp, _vp, _sz, _vp]
     L.dpclip_step_host_arena_bytes.argtypes = [ctypes.POINTER(_CLayer), _i, _i, _i]
     L.dpclip_step_host_arena_bytes.restype = _sz
@@ -377,10 +384,15 @@ class StepPlan:
     def run(self, C: float, sigma: float, seed: int, stream_id0: int = 0, stream=None) -> None:
         dpclip_step(self, C, sigma, seed, stream_id0, stream)
 
+    def _side_workspace_bytes(self) -> int:
+        return dpclip_step_side_workspace_bytes(self)
+
     def _branches(self, branches: int):
         """Side streams and their workspaces for the several-streams entry points (allocated once)."""
         if len(getattr(self, "_branch_ws", [])) < branches:
-            self._branch_ws = [self.workspace] + [torch.empty_like(self.workspace) for _ in range(branches - 1)]
+            side = self._side_workspace_bytes()
+            self._branch_ws = [self.workspace] + [torch.empty((side,), dtype=torch.uint8, device=self.workspace.device)
+                                                  for _ in range(branches - 1)]
             for w in self._branch_ws[1:]:
                 dpclip_workspace_init(w)
             # one to spare: torch hands its streams out in rotation, so the caller's stream may be one of these
@@ -390,10 +402,10 @@ class StepPlan:
         return [s for s in self._streams if s != current][:branches - 1], self._branch_ws[:branches]
 
     def run_streams(self, C: float, sigma: float, seed: int, stream_id0: int = 0, branches: int = 4) -> None:
-        """One dpclip_step_streams call: the library spreads the launches of a stage over `branches` streams,
+        """One dpclip_step_lanes call: the library spreads the launches of a stage over `branches` streams,
         starting from and joining back into the current stream."""
         side, ws = self._branches(branches)
-        dpclip_step_streams(self, C, sigma, seed, stream_id0, [torch.cuda.current_stream()] + side, ws)
+        dpclip_step_lanes(self, C, sigma, seed, stream_id0, [torch.cuda.current_stream()] + side, ws)
 
     def workspaces(self) -> List[torch.Tensor]:
         """Every workspace the plan has used (their status words are checked separately)."""
@@ -403,7 +415,7 @@ class StepPlan:
         """Record one step into a CUDA graph (the launch-bound small workloads spend most of a step
         in launch gaps).  Returns the graph; `graph.replay()` re-runs the same kernels on the same
         buffers with the same (C, sigma, seed, stream ids).  The graph holds exactly ONE library call:
-        dpclip_step (branches = 1) or dpclip_step_streams (the fork/join over `branches` streams happens
+        dpclip_step (branches = 1) or dpclip_step_lanes (the fork/join over `branches` streams happens
         inside the library and becomes the graph's parallel branches)."""
         step = self.run if branches <= 1 else (lambda *a: self.run_streams(*a, branches=branches))
         step(C, sigma, seed, stream_id0)               # warm-up outside capture (function attributes, maps)
@@ -526,6 +538,11 @@ def dpclip_step_workspace_bytes(plan) -> int:
     return load_library().dpclip_step_workspace_bytes(plan._c, plan.L, plan.B, plan.dtype_code)
 
 
+def dpclip_step_side_workspace_bytes(plan) -> int:
+    """The same for the workspaces of the streams after the first."""
+    return load_library().dpclip_step_side_workspace_bytes(plan._c, plan.L, plan.B, plan.dtype_code)
+
+
 def dpclip_step(plan: StepPlan, C: float, sigma: float, seed: int, stream_id0: int = 0, stream=None) -> None:
     _check("dpclip_step", load_library().dpclip_step(
         plan._c, plan.L, plan.B, plan.dtype_code, C, sigma, seed, stream_id0, _ptr(plan.sq_layers),
@@ -534,25 +551,43 @@ def dpclip_step(plan: StepPlan, C: float, sigma: float, seed: int, stream_id0: i
 
 def _stream_args(streams, workspaces):
     n = len(streams)
-    assert n == len(workspaces) and all(w.numel() == workspaces[0].numel() for w in workspaces)
+    assert n == len(workspaces)
     st = (_vp * n)(*[s.cuda_stream for s in streams])
     ws = (_vp * n)(*[w.data_ptr() for w in workspaces])
-    return n, st, ws, workspaces[0].numel()
+    return n, st, ws, (_sz * n)(*[w.numel() for w in workspaces])
+
+
+def dpclip_step_lanes(plan: StepPlan, C: float, sigma: float, seed: int, stream_id0: int, streams, workspaces) -> None:
+    """dpclip_step with the library forking over `streams` (torch streams; streams[0] = the caller's), each with a workspace of its
+    own size: the first of dpclip_step_workspace_bytes, the others of dpclip_step_side_workspace_bytes at least."""
+    n, st, ws, nbytes = _stream_args(streams, workspaces)
+    _check("dpclip_step_lanes", load_library().dpclip_step_lanes(
+        plan._c, plan.L, plan.B, plan.dtype_code, C, sigma, seed, stream_id0, _ptr(plan.sq_layers), _ptr(plan.clip),
+        _ptr(plan.norms), n, st, ws, nbytes))
+
+
+def dpclip_model_step_lanes(plan, C: float, sigma: float, seed: int, stream_id0: int, streams, workspaces) -> None:
+    n, st, ws, nbytes = _stream_args(streams, workspaces)
+    _check("dpclip_model_step_lanes", load_library().dpclip_model_step_lanes(
+        plan._c, plan.L, plan.B, plan.dtype_code, C, sigma, seed, stream_id0, _ptr(plan.sq_layers), _ptr(plan.clip),
+        _ptr(plan.norms), n, st, ws, nbytes))
 
 
 def dpclip_step_streams(plan: StepPlan, C: float, sigma: float, seed: int, stream_id0: int, streams, workspaces) -> None:
-    """dpclip_step with the library forking over `streams` (torch streams; streams[0] = the caller's)."""
+    """dpclip_step_lanes with workspaces of one size."""
     n, st, ws, nbytes = _stream_args(streams, workspaces)
+    assert len(set(nbytes)) == 1
     _check("dpclip_step_streams", load_library().dpclip_step_streams(
         plan._c, plan.L, plan.B, plan.dtype_code, C, sigma, seed, stream_id0, _ptr(plan.sq_layers), _ptr(plan.clip),
-        _ptr(plan.norms), n, st, ws, nbytes))
+        _ptr(plan.norms), n, st, ws, nbytes[0]))
 
 
 def dpclip_model_step_streams(plan, C: float, sigma: float, seed: int, stream_id0: int, streams, workspaces) -> None:
     n, st, ws, nbytes = _stream_args(streams, workspaces)
+    assert len(set(nbytes)) == 1
     _check("dpclip_model_step_streams", load_library().dpclip_model_step_streams(
         plan._c, plan.L, plan.B, plan.dtype_code, C, sigma, seed, stream_id0, _ptr(plan.sq_layers), _ptr(plan.clip),
-        _ptr(plan.norms), n, st, ws, nbytes))
+        _ptr(plan.norms), n, st, ws, nbytes[0]))
 
 
 DPCLIP_KIND_DENSE, DPCLIP_KIND_ELEMENTWISE, DPCLIP_KIND_CONV = 0, 1, 2
@@ -576,7 +611,7 @@ class ModelLayer:
 
 class ModelPlan(StepPlan):
     """Buffers and the C descriptor array of a model with dense, element-wise and convolution layers.
-    Holds no arithmetic: `run` is one dpclip_model_step call, `run_streams` one dpclip_model_step_streams call
+    Holds no arithmetic: `run` is one dpclip_model_step call, `run_streams` one dpclip_model_step_lanes call
     (which `capture` with several branches records).  gW[l] is (d_out, d_in)
     for dense and convolution layers (d_in = C*kh*kw) and (d,) for element-wise layers; all live in `flat`."""
 
@@ -635,12 +670,15 @@ class ModelPlan(StepPlan):
         self.workspace = torch.empty((ws,), dtype=torch.uint8, device=dev)
         dpclip_workspace_init(self.workspace)
 
+    def _side_workspace_bytes(self) -> int:
+        return dpclip_model_side_workspace_bytes(self)
+
     def run(self, C: float, sigma: float, seed: int, stream_id0: int = 0, stream=None) -> None:
         dpclip_model_step(self, C, sigma, seed, stream_id0, stream)
 
     def run_streams(self, C: float, sigma: float, seed: int, stream_id0: int = 0, branches: int = 4) -> None:
         side, ws = self._branches(branches)
-        dpclip_model_step_streams(self, C, sigma, seed, stream_id0, [torch.cuda.current_stream()] + side, ws)
+        dpclip_model_step_lanes(self, C, sigma, seed, stream_id0, [torch.cuda.current_stream()] + side, ws)
 
 
 def dpclip_step_per_layer(plan: StepPlan, C_layer: Sequence[float], sigma: float, seed: int, stream_id0: int = 0,
@@ -663,6 +701,10 @@ def dpclip_step_per_layer(plan: StepPlan, C_layer: Sequence[float], sigma: float
 
 def dpclip_model_workspace_bytes(plan: ModelPlan) -> int:
     return load_library().dpclip_model_workspace_bytes(plan._c, plan.L, plan.B, plan.dtype_code)
+
+
+def dpclip_model_side_workspace_bytes(plan: ModelPlan) -> int:
+    return load_library().dpclip_model_side_workspace_bytes(plan._c, plan.L, plan.B, plan.dtype_code)
 
 
 def dpclip_model_step(plan: ModelPlan, C: float, sigma: float, seed: int, stream_id0: int = 0, stream=None) -> None:

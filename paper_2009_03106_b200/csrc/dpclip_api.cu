@@ -1599,12 +1599,17 @@ static size_t step_scratch_bytes(const dpclip_layer* layers, int L, int B, dpcli
     return ws;
 }
 
-struct StagePlan;
-static size_t staged_workspace_bytes(const dpclip_layer* layers, const dpclip_model_layer* other, int L, int B, dpclip_dtype dtype);
+static size_t staged_workspace_bytes(const dpclip_layer* layers, const dpclip_model_layer* other, int L, int B, dpclip_dtype dtype,
+                                     bool with_copies);
 
 size_t dpclip_step_workspace_bytes(const dpclip_layer* layers, int L, int B, dpclip_dtype dtype) {
     const size_t ws = step_scratch_bytes(layers, L, B, dtype);
-    const size_t staged = staged_workspace_bytes(layers, nullptr, L, B, dtype);
+    const size_t staged = staged_workspace_bytes(layers, nullptr, L, B, dtype, true);
+    return staged > ws ? staged : ws;
+}
+size_t dpclip_step_side_workspace_bytes(const dpclip_layer* layers, int L, int B, dpclip_dtype dtype) {
+    const size_t ws = step_scratch_bytes(layers, L, B, dtype);
+    const size_t staged = staged_workspace_bytes(layers, nullptr, L, B, dtype, false);
     return staged > ws ? staged : ws;
 }
 
@@ -2382,8 +2387,7 @@ static int other_kind_clipped_grad_noise(const dpclip_model_layer& m, int B, dpc
 // from the first launch of the step to its last.
 // ---------------------------------------------------------------------------
 constexpr int kStageMaxLayers = 64;
-// Copies of one step; a layer that no longer fits keeps its fp32-ALU form.  (Every lane of a several-streams step owns
-// a workspace of this size.)
+// Copies of one step; a layer that no longer fits keeps its fp32-ALU form.
 constexpr size_t kStageCapBytes = (size_t)3 << 30;
 struct StagePlan {
     bool active = false;
@@ -2566,10 +2570,12 @@ static bool stage_plan(StagePlan& sp, const dpclip_layer* layers, const dpclip_m
     return true;
 }
 
-static size_t staged_workspace_bytes(const dpclip_layer* layers, const dpclip_model_layer* other, int L, int B, dpclip_dtype dtype) {
+static size_t staged_workspace_bytes(const dpclip_layer* layers, const dpclip_model_layer* other, int L, int B, dpclip_dtype dtype,
+                                     bool with_copies) {
     if (!layers || L <= 0 || B <= 0) return 0;
     StagePlan sp;
-    return stage_plan(sp, layers, other, L, B, dtype, reinterpret_cast<char*>(256), true) ? sp.bytes : 0;
+    if (!stage_plan(sp, layers, other, L, B, dtype, reinterpret_cast<char*>(256), true)) return 0;
+    return with_copies ? sp.bytes : sp.scratch;
 }
 
 static int launch_stage(StagePlan& sp, cudaStream_t st) {
@@ -2668,7 +2674,7 @@ struct Lanes {
     int n = 1;
     cudaStream_t st[kMax] = {};
     void* ws[kMax] = {};
-    size_t ws_bytes = 0;
+    size_t ws_bytes[kMax] = {};
     cudaEvent_t ev[2 * kMax + 2] = {};
     int n_ev = 0;
     ~Lanes() { for (int i = 0; i < n_ev; ++i) cudaEventDestroy(ev[i]); }     // pending work keeps what it needs
@@ -2719,11 +2725,10 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
     for (int l = 0; l < L; ++l) any_other = any_other || other_kind(l);
     const int last = lanes.n - 1;
     void* const ws0 = lanes.ws[0];
-    const size_t workspace_bytes = lanes.ws_bytes;
     T1Group t1;
     rc = prepare_t1_group(t1, layers, L, B, t1_dtype, C, sigma, seed, stream_id0, sq_layers, clip);
     if (rc) return rc;
-    if (t1.active && (!lanes.ws[last] || workspace_bytes < (size_t)kHeaderBytes)) t1.active = false;
+    if (t1.active && (!lanes.ws[last] || lanes.ws_bytes[last] < (size_t)kHeaderBytes)) t1.active = false;
     if (!t1.active && sp && t1_dtype != dtype) {                        // not taken together after all: the inputs as given
         for (int l = 0; l < L; ++l) if (layers_in[l].T == 1) sp->eff[l] = layers_in[l];
         t1_dtype = dtype;
@@ -2741,7 +2746,7 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
     if (track) {
         // when one Gram launch takes every layer of the model, its last CTA also computes the factors
         const tc::gram::FactorsTail tail = {sq_layers, L, (long)B, B, C, clip, norms, nullptr};
-        rc = gram_layers_sqnorms(layers, L, B, dtype, sq_layers, in_gram_group, ws0, workspace_bytes, lanes.st[0],
+        rc = gram_layers_sqnorms(layers, L, B, dtype, sq_layers, in_gram_group, ws0, lanes.ws_bytes[0], lanes.st[0],
                                  (!t1.active && !any_other && !path_switch(SW_NO_FACTORS_TAIL)) ? &tail : nullptr, &factors_done);
         if (rc) return rc;
         for (int l = 0; l < L; ++l) any_gram = any_gram || in_gram_group[l];
@@ -2749,7 +2754,7 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
         int skip[64], taken[64];
         for (int l = 0; l < L; ++l) skip[l] = in_gram_group[l] || other_kind(l);
         const int b = any_gram && lanes.n > 1 ? 1 : 0;
-        rc = group_norms(layers, L, B, dtype, sq_layers, skip, taken, lanes.ws[b], workspace_bytes, lanes.st[b],
+        rc = group_norms(layers, L, B, dtype, sq_layers, skip, taken, lanes.ws[b], lanes.ws_bytes[b], lanes.st[b],
                          (!t1.active && !any_other && !any_gram && !path_switch(SW_NO_FACTORS_TAIL)) ? &tail : nullptr,
                          any_gram ? nullptr : &factors_done, lanes.n);
         if (rc) return rc;
@@ -2802,11 +2807,11 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
         const SmBudgetScope share(track ? budget[l] : 0);
         const int b = k++ % lanes.n;
         if (is_other)
-            rc = other_kind_sqnorms(other[l], B, dtype, sq_layers + (size_t)l * B, lanes.ws[b], workspace_bytes, lanes.st[b]);
+            rc = other_kind_sqnorms(other[l], B, dtype, sq_layers + (size_t)l * B, lanes.ws[b], lanes.ws_bytes[b], lanes.st[b]);
         else
             rc = dpclip_layer_sqnorms(y.A, y.lda, y.Zbar, y.ldz, B, y.T, y.d_in, y.d_out, dtype, y.has_bias,
                                       (dpclip_method)y.method, sq_layers + (size_t)l * B, lanes.ws[b],
-                                      workspace_bytes, lanes.st[b]);
+                                      lanes.ws_bytes[b], lanes.st[b]);
         if (rc) return rc;
     }
     if ((rc = lanes.join())) return rc;
@@ -2816,7 +2821,7 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
     }
     if ((rc = lanes.fork())) return rc;
     if (t1.active) {
-        rc = launch_fused_t1_tf32(t1.p, false, t1_dtype, lanes.ws[last], workspace_bytes, lanes.st[last]);
+        rc = launch_fused_t1_tf32(t1.p, false, t1_dtype, lanes.ws[last], lanes.ws_bytes[last], lanes.st[last]);
         if (rc < 0) return rc;
         if (rc > 0) return DPCLIP_ERR_UNSUPPORTED;           // prepare_t1_group checked the same conditions
     }
@@ -2838,13 +2843,13 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
             T_dense = layers[l].T;
         }
         rc = shared_clipped_grad_launches(layers, split, join, L, B, dtype, clip, 0, C, sigma, seed, stream_id0, in_grad_group, ws0,
-                                          workspace_bytes, lanes.st[0]);
+                                          lanes.ws_bytes[0], lanes.st[0]);
         if (rc) return rc;
         for (int l = 0; l < L; ++l) any_group = any_group || in_grad_group[l];
         int skip[64], taken[64];
         for (int l = 0; l < L; ++l) skip[l] = in_grad_group[l] || other_kind(l) || (t1.active && layers[l].T == 1);
         const int b = any_group && lanes.n > 1 ? 1 : 0;
-        rc = group_grads(layers, L, B, dtype, clip, 0, C, sigma, seed, stream_id0, skip, taken, lanes.ws[b], workspace_bytes,
+        rc = group_grads(layers, L, B, dtype, clip, 0, C, sigma, seed, stream_id0, skip, taken, lanes.ws[b], lanes.ws_bytes[b],
                          lanes.st[b], lanes.n);
         if (rc) return rc;
         for (int l = 0; l < L; ++l) if (taken[l]) { any_rest = true; in_grad_group[l] = 1; }
@@ -2859,6 +2864,7 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
         const int b = k++ % lanes.n;
         void* const stream = lanes.st[b];
         void* const workspace = lanes.ws[b];
+        const size_t workspace_bytes = lanes.ws_bytes[b];
         if (is_other) {
             rc = other_kind_clipped_grad_noise(other[l], B, dtype, clip, C, sigma, seed, stream_id0 + 2ull * l,
                                                stream_id0 + 2ull * l + 1, workspace, workspace_bytes, stream);
@@ -2891,13 +2897,16 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
 
 // Lanes of a one-stream call, and of a several-streams call (argument checks included).
 static void one_lane(Lanes& lanes, void* workspace, size_t workspace_bytes, void* stream) {
-    lanes.n = 1; lanes.st[0] = (cudaStream_t)stream; lanes.ws[0] = workspace; lanes.ws_bytes = workspace_bytes;
+    lanes.n = 1; lanes.st[0] = (cudaStream_t)stream; lanes.ws[0] = workspace; lanes.ws_bytes[0] = workspace_bytes;
 }
-static int many_lanes(Lanes& lanes, int n_streams, void* const* streams, void* const* workspaces, size_t workspace_bytes) {
+// sizes: bytes of every lane's workspace, or NULL: workspace_bytes each
+static int many_lanes(Lanes& lanes, int n_streams, void* const* streams, void* const* workspaces, const size_t* sizes,
+                      size_t workspace_bytes) {
     if (n_streams < 1 || n_streams > Lanes::kMax || !streams || !workspaces) return DPCLIP_ERR_INVALID_ARG;
-    lanes.n = n_streams; lanes.ws_bytes = workspace_bytes;
+    lanes.n = n_streams;
     for (int i = 0; i < n_streams; ++i) {
         lanes.st[i] = (cudaStream_t)streams[i]; lanes.ws[i] = workspaces[i];
+        lanes.ws_bytes[i] = sizes ? sizes[i] : workspace_bytes;
         for (int j = 0; j < i; ++j)
             if (streams[i] == streams[j] || (workspaces[i] && workspaces[i] == workspaces[j])) return DPCLIP_ERR_INVALID_ARG;
     }
@@ -2917,8 +2926,8 @@ static int step_args_ok(const void* layers, int L, int B, dpclip_dtype dtype, fl
 static int stage_step(StagePlan& sp, const dpclip_layer* layers, const dpclip_model_layer* other, int L, int B,
                       dpclip_dtype dtype, Lanes& lanes, bool t1_too) {
     if (!lanes.ws[0] || !stage_plan(sp, layers, other, L, B, dtype, static_cast<char*>(lanes.ws[0]), t1_too)) return DPCLIP_OK;
-    if (lanes.ws_bytes < sp.bytes) { sp.active = false; return DPCLIP_OK; }
-    lanes.ws_bytes = sp.scratch;
+    if (lanes.ws_bytes[0] < sp.bytes) { sp.active = false; return DPCLIP_OK; }
+    lanes.ws_bytes[0] = sp.scratch;                            // the copies lie behind lane 0's scratch
     return launch_stage(sp, lanes.st[0]);
 }
 
@@ -2929,7 +2938,7 @@ static int step_dense(const dpclip_layer* layers, int L, int B, dpclip_dtype dty
     int rc = stage_step(sp, layers, nullptr, L, B, dtype, lanes, true);
     if (rc) return rc;
     rc = try_fused_t1_step(sp.active ? sp.eff : layers, L, B, sp.active ? sp.t1_dtype : dtype, C, sigma, seed, stream_id0,
-                           sq_layers, clip, norms, lanes.ws[0], lanes.ws_bytes, lanes.st[0]);
+                           sq_layers, clip, norms, lanes.ws[0], lanes.ws_bytes[0], lanes.st[0]);
     if (rc <= 0) return rc;                  // done (0) or argument error (< 0); 1 = take the general path
     return step_general(layers, nullptr, L, B, dtype, C, sigma, seed, stream_id0, sq_layers, clip, norms, lanes,
                         sp.active ? &sp : nullptr);
@@ -2973,7 +2982,19 @@ int dpclip_step_streams(const dpclip_layer* layers, int L, int B, dpclip_dtype d
     int rc = step_args_ok(layers, L, B, dtype, C, sigma, sq_layers, clip);
     if (rc) return rc;
     Lanes lanes;
-    if ((rc = many_lanes(lanes, n_streams, streams, workspaces, workspace_bytes))) return rc;
+    if ((rc = many_lanes(lanes, n_streams, streams, workspaces, nullptr, workspace_bytes))) return rc;
+    return step_dense(layers, L, B, dtype, C, sigma, seed, stream_id0, sq_layers, clip, norms, lanes);
+}
+
+int dpclip_step_lanes(const dpclip_layer* layers, int L, int B, dpclip_dtype dtype, float C, float sigma,
+                        unsigned long long seed, unsigned long long stream_id0, float* sq_layers, float* clip,
+                        float* norms, int n_streams, void* const* streams, void* const* workspaces,
+                        const size_t* workspace_bytes) {
+    if (!workspace_bytes) return DPCLIP_ERR_INVALID_ARG;
+    int rc = step_args_ok(layers, L, B, dtype, C, sigma, sq_layers, clip);
+    if (rc) return rc;
+    Lanes lanes;
+    if ((rc = many_lanes(lanes, n_streams, streams, workspaces, workspace_bytes, 0))) return rc;
     return step_dense(layers, L, B, dtype, C, sigma, seed, stream_id0, sq_layers, clip, norms, lanes);
 }
 
@@ -3010,7 +3031,7 @@ int dpclip_step_per_layer(const dpclip_layer* layers, int L, int B, dpclip_dtype
         Lanes lanes;
         one_lane(lanes, workspace, workspace_bytes, stream);
         if ((rc = stage_step(sp, layers, nullptr, L, B, dtype, lanes, false))) return rc;
-        workspace_bytes = lanes.ws_bytes;
+        workspace_bytes = lanes.ws_bytes[0];
     }
     const bool* split = sp.active ? sp.split : nullptr;
     if (sp.active) layers = sp.eff;
@@ -3070,7 +3091,7 @@ int dpclip_step_per_layer(const dpclip_layer* layers, int L, int B, dpclip_dtype
     return DPCLIP_OK;
 }
 
-size_t dpclip_model_workspace_bytes(const dpclip_model_layer* layers, int L, int B, dpclip_dtype dtype) {
+static size_t model_workspace_bytes(const dpclip_model_layer* layers, int L, int B, dpclip_dtype dtype, bool with_copies) {
     size_t ws = kHeaderBytes;
     if (!layers || L <= 0 || L > 256 || B <= 0) return ws;
     {
@@ -3080,7 +3101,7 @@ size_t dpclip_model_workspace_bytes(const dpclip_model_layer* layers, int L, int
             else memset(&dense[l], 0, sizeof(dense[l]));
         }
         ws = step_scratch_bytes(dense, L, B, dtype);
-        const size_t staged = staged_workspace_bytes(dense, layers, L, B, dtype);
+        const size_t staged = staged_workspace_bytes(dense, layers, L, B, dtype, with_copies);
         if (staged > ws) ws = staged;
     }
     for (int l = 0; l < L; ++l) {
@@ -3093,6 +3114,13 @@ size_t dpclip_model_workspace_bytes(const dpclip_model_layer* layers, int L, int
         if (w > ws) ws = w;
     }
     return ws;
+}
+
+size_t dpclip_model_workspace_bytes(const dpclip_model_layer* layers, int L, int B, dpclip_dtype dtype) {
+    return model_workspace_bytes(layers, L, B, dtype, true);
+}
+size_t dpclip_model_side_workspace_bytes(const dpclip_model_layer* layers, int L, int B, dpclip_dtype dtype) {
+    return model_workspace_bytes(layers, L, B, dtype, false);
 }
 
 int dpclip_model_step(const dpclip_model_layer* layers, int L, int B, dpclip_dtype dtype, float C, float sigma,
@@ -3112,7 +3140,19 @@ int dpclip_model_step_streams(const dpclip_model_layer* layers, int L, int B, dp
     int rc = step_args_ok(layers, L, B, dtype, C, sigma, sq_layers, clip);
     if (rc) return rc;
     Lanes lanes;
-    if ((rc = many_lanes(lanes, n_streams, streams, workspaces, workspace_bytes))) return rc;
+    if ((rc = many_lanes(lanes, n_streams, streams, workspaces, nullptr, workspace_bytes))) return rc;
+    return step_model(layers, L, B, dtype, C, sigma, seed, stream_id0, sq_layers, clip, norms, lanes);
+}
+
+int dpclip_model_step_lanes(const dpclip_model_layer* layers, int L, int B, dpclip_dtype dtype, float C, float sigma,
+                              unsigned long long seed, unsigned long long stream_id0, float* sq_layers, float* clip,
+                              float* norms, int n_streams, void* const* streams, void* const* workspaces,
+                              const size_t* workspace_bytes) {
+    if (!workspace_bytes) return DPCLIP_ERR_INVALID_ARG;
+    int rc = step_args_ok(layers, L, B, dtype, C, sigma, sq_layers, clip);
+    if (rc) return rc;
+    Lanes lanes;
+    if ((rc = many_lanes(lanes, n_streams, streams, workspaces, workspace_bytes, 0))) return rc;
     return step_model(layers, L, B, dtype, C, sigma, seed, stream_id0, sq_layers, clip, norms, lanes);
 }
 

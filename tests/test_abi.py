@@ -113,6 +113,30 @@ def test_streams_step_argument_errors(lib):
     assert f(layers, 1, 2, 0, 0.0, 0.0, 0, 0, fake, fake, None, 2, st2, ws2, 1 << 20) == INVALID     # C must be > 0
 
 
+def test_side_workspaces_hold_no_staged_copies(lib):
+    """A step over several streams keeps the 16-byte aligned copies of its operands in the first workspace alone."""
+    from paper_2009_03106_b200 import binding as b
+    B, T, d, f = 50, 77, 300, 1100
+
+    def layers(bf16):
+        es = 2 if bf16 else 4
+        return (b._CLayer * 2)(b._CLayer(256, d, 512, f, T, d, f, 0, 0, 768, d, None),
+                               b._CLayer(256, f, 512 + (0 if bf16 else es), d, T, f, d, 0, 0, 768, f, None))
+    up = lambda n, m: -(-n // m) * m                                                 # noqa: E731
+    rows = B * T
+    # bf16: all four operands, rows of 304 and 1104 elements; fp32: one misaligned base, 300 elements are 16-byte rows
+    for dtype, copies in ((1, 2 * (up(rows * 304 * 2, 256) + up(rows * 1104 * 2, 256))), (0, up(rows * 300 * 4, 256))):
+        whole = lib.dpclip_step_workspace_bytes(layers(dtype), 2, B, dtype)
+        side = lib.dpclip_step_side_workspace_bytes(layers(dtype), 2, B, dtype)
+        assert side >= lib.dpclip_workspace_bytes(B, T, d, f, dtype, 0) and 0 <= whole - copies - side < 256
+    conv = (b._CModelLayer * 1)()
+    conv[0].kind, conv[0].conv, conv[0].z_channel_major = 2, b._CConv(64, 32, 32, 3, 3, 2, 1), 1
+    conv[0].layer = b._CLayer(256, 0, 512, 0, 0, 0, 128, 0, 0, 768, 576, None)
+    whole = lib.dpclip_model_workspace_bytes(conv, 1, 64, 1)
+    side = lib.dpclip_model_side_workspace_bytes(conv, 1, 64, 1)
+    assert whole - side >= 64 * 256 * (576 + 128) * 2
+
+
 def test_workspace_queries_without_a_gpu(lib):
     """The workspace queries are host arithmetic: the fixed scratch for ordinary layers, room for one partial
     tile per row slice for long bf16 layers whose 64 tiles leave SMs idle in one wave, and the copies of the

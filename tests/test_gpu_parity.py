@@ -1399,3 +1399,28 @@ def test_run_streams_from_one_of_the_plans_own_streams(dp):
             plan.run_streams(w.C, w.sigma, 1, branches=4)
         torch.cuda.synchronize()
         assert rel_fro(plan.flat.cpu().numpy(), first.cpu().numpy()) <= 2e-6
+
+
+def test_step_streams_stay_inside_side_workspaces(dp):
+    """The workspaces of the streams after the first are only as large as dpclip_step_side_workspace_bytes says: bytes behind them
+    keep their pattern, and the results are those of one stream."""
+    B, specs = 64, ((100, 250, 130), (100, 130, 250), (60, 250, 250), (60, 250, 330))
+    data = [workloads.random_layer(130 + k, B, T, i, o, "bf16", scale_z=0.05) for k, (T, i, o) in enumerate(specs)]
+    plan = dp.StepPlan([dp.Layer(to_device(A, "bf16"), to_device(Z, "bf16"), True) for A, Z in data])
+    plan.run(1.0, 0.0, 3)
+    one = [g.cpu().numpy() for g in (plan.norms, *plan.gW, *plan.gb)]
+    plan.run_streams(1.0, 0.0, 3, branches=4)
+    side = plan.workspaces()[1].numel()
+    copies = sum(B * T * (-(-i // 8) + -(-o // 8)) * 16 for T, i, o in specs)
+    assert all(w.numel() == side for w in plan.workspaces()[1:]) and plan.workspace.numel() - side >= copies
+    raw = [torch.full((side + 4096,), 0xA5, dtype=torch.uint8, device="cuda") for _ in range(3)]
+    ws = [plan.workspace] + [r[:side] for r in raw]
+    for w in ws[1:]:
+        dp.dpclip_workspace_init(w)
+    plan.flat.fill_(float("nan"))
+    dp.dpclip_step_lanes(plan, 1.0, 0.0, 3, 0, [torch.cuda.current_stream()] + plan._branches(4)[0], ws)
+    torch.cuda.synchronize()
+    assert all(dp.dpclip_read_status(w) == 0 for w in ws)
+    assert all(bool((r[side:] == 0xA5).all()) for r in raw)
+    for g, h in zip(one, (plan.norms, *plan.gW, *plan.gb)):
+        assert rel_fro(h.cpu().numpy(), g) <= TOL["f32"]["grad"]
