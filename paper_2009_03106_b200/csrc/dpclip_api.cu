@@ -2591,7 +2591,8 @@ static int launch_stage(StagePlan& sp, cudaStream_t st) {
             else q.blocks += ceil_div((long)j.rows * (j.dst_ld / ((j.es == 4 || j.kind == stage::ROWS_TO_F32) ? 4 : 8)),
                                       (long)stage::ROWS_UNROLL * stage::THREADS);
         }
-        if (sp.smem > 48 * 1024 && !enable_smem(stage_operands_kernel, sp.smem)) return DPCLIP_ERR_CUDA;
+        // the limit is the kernel's, not the launch's: a smaller one would fail the launch another thread is about to make
+        if (sp.smem > 48 * 1024 && !enable_smem(stage_operands_kernel, stage::SMEM_MAX)) return DPCLIP_ERR_CUDA;
         stage_operands_kernel<<<q.blocks, stage::THREADS, sp.smem, st>>>(q);
         if (launch_status()) return DPCLIP_ERR_CUDA;
     }

@@ -1229,6 +1229,35 @@ def test_model_step_staged_convolutions(dp, case, dtype):
     assert rel_fro(plan.gb[0].cpu().numpy(), refb) <= TOL["f32"]["grad"]
 
 
+def test_staged_convolutions_of_two_kernel_sizes_from_four_threads(dp):
+    """Their patch windows need 64 and 53 KB of shared memory: a thread's launch must not depend on what another sets meanwhile."""
+    import threading
+    plans = []
+    for k in (11, 10, 11, 10):
+        X = torch.randn(8, 16, 32, 32, device="cuda").bfloat16()
+        Z = (torch.randn(8, 48, 33 - k, 33 - k, device="cuda") * 1e-2).bfloat16()
+        plans.append(dp.ModelPlan([dp.ModelLayer(dp.DPCLIP_KIND_CONV, X, Z.flatten(2), True, conv=(k, k, 1, 0), z_channel_major=True)]))
+    errors = []
+
+    def work(plan):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for k in range(4000):
+                    plan.run(1.0, 0.0, 1)
+                    if k % 200 == 199:
+                        torch.cuda.current_stream().synchronize()
+        except Exception as e:                                               # noqa: BLE001
+            errors.append(e)
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=work, args=(p,)) for p in plans]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+    assert all(dp.dpclip_read_status(p.workspace) == 0 for p in plans)
+
+
 # fp32 layers that share the CTA-pair launch: a run boundary inside a tile, items of one stage to several drains (T = 30,
 # 128, 800: one accumulator, two, several windows), N = 64 .. 256 tiles, either operand on the M side, ragged widths
 GROUP_MODELS = [
