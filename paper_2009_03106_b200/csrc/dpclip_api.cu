@@ -1137,7 +1137,7 @@ int launch_group_kernel(const tc::zg::Maps& maps, const tc::zg::Params& p, cudaS
 }
 
 // Norms (norm = true) or clipped sums with noise of n fp32 layers.  Returns DPCLIP_OK, a negative status, or 1 when the
-// workspace cannot hold a few partial tiles (clipped sums only; nothing has been launched then).
+// workspace cannot hold a few partial tiles (clipped sums, norms of more than FLUSH stages; nothing has been launched then).
 int launch_group(const GroupLayer* ls, int n, int B, bool norm, const NoiseSpec* noise, bool* noise_done,
                  void* workspace, size_t workspace_bytes, cudaStream_t st, const tc::gram::FactorsTail* tail = nullptr) {
     namespace g = tc::zg;
@@ -1148,7 +1148,7 @@ int launch_group(const GroupLayer* ls, int n, int B, bool norm, const NoiseSpec*
     // norms of long examples keep the sums between two drains in a slot per run
     bool long_norms = false;
     for (int l = 0; norm && l < n; ++l) long_norms = long_norms || ls[l].T > g::FLUSH * bk;
-    if ((!norm || long_norms) && cap < 8) return norm ? DPCLIP_ERR_WORKSPACE : 1;
+    if ((!norm || long_norms) && cap < 8) return 1;
     bool fuse_noise = !norm && noise && noise->scale > 0.f;
     for (int l = 0; l < n && fuse_noise; ++l) fuse_noise = ls[l].ldg == ls[l].d_in;
     if (norm) {
@@ -1264,13 +1264,14 @@ int clipped_grad_impl(const void* A, long lda, const void* Zbar, long ldz, int B
         return launch_zta_tc(A, lda, Zbar, ldz, B, T, d_in, d_out, false, 0, clip, gW, ldg, gb, nullptr, workspace,
                              workspace_bytes, noise, noise_done, st, false, split);
     if (tf32_eligible(A, lda, Zbar, ldz, B, T, d_in, d_out, dtype) && !narrow_layer(T, d_in, d_out, gb != nullptr, lda, ldz)) {
-        if (!group_wide(d_in, d_out))
-            return launch_zta_tf32(A, lda, Zbar, ldz, B, T, d_in, d_out, false, 0, clip, gW, ldg, gb, nullptr, workspace,
-                                   workspace_bytes, noise, noise_done, st);
-        GroupLayer y = {A, lda, Zbar, ldz, T, d_in, d_out, false, nullptr, clip, gW, ldg, gb,
-                        noise ? noise->sid_w : 0ull, noise ? noise->sid_b : 0ull};
-        const int rc = launch_group(&y, 1, B, false, noise, noise_done, workspace, workspace_bytes, st);
-        return rc > 0 ? DPCLIP_ERR_WORKSPACE : rc;
+        if (group_wide(d_in, d_out)) {
+            GroupLayer y = {A, lda, Zbar, ldz, T, d_in, d_out, false, nullptr, clip, gW, ldg, gb,
+                            noise ? noise->sid_w : 0ull, noise ? noise->sid_b : 0ull};
+            const int rc = launch_group(&y, 1, B, false, noise, noise_done, workspace, workspace_bytes, st);
+            if (rc <= 0) return rc;
+        }
+        return launch_zta_tf32(A, lda, Zbar, ldz, B, T, d_in, d_out, false, 0, clip, gW, ldg, gb, nullptr, workspace,
+                               workspace_bytes, noise, noise_done, st);
     }
     return launch_simt_grad(A, lda, Zbar, ldz, B, T, d_in, d_out, dtype, clip, gW, ldg, gb, st, workspace,
                             workspace_bytes, noise, noise_done);
@@ -1660,11 +1661,13 @@ int dpclip_layer_sqnorms(const void* A, long lda, const void* Zbar, long ldz, in
             if (dtype == DPCLIP_F32) {                    // fp32: materialised tiles via error-compensated tf32
                 if (method != DPCLIP_MATERIALIZE || !aligned_to(A, 16) || !aligned_to(Zbar, 16) || lda % 4 || ldz % 4)
                     return DPCLIP_ERR_UNSUPPORTED;
-                if (!group_wide(d_in, d_out))
-                    return launch_zta_tf32(A, lda, Zbar, ldz, B, T, d_in, d_out, true, has_bias, nullptr, nullptr, 0,
-                                           nullptr, sq_layer, workspace, workspace_bytes, nullptr, nullptr, st);
-                GroupLayer y = {A, lda, Zbar, ldz, T, d_in, d_out, has_bias != 0, sq_layer};
-                return launch_group(&y, 1, B, true, nullptr, nullptr, workspace, workspace_bytes, st);
+                if (group_wide(d_in, d_out)) {
+                    GroupLayer y = {A, lda, Zbar, ldz, T, d_in, d_out, has_bias != 0, sq_layer};
+                    rc = launch_group(&y, 1, B, true, nullptr, nullptr, workspace, workspace_bytes, st);
+                    if (rc <= 0) return rc;              // 1: small layers come with the header alone
+                }
+                return launch_zta_tf32(A, lda, Zbar, ldz, B, T, d_in, d_out, true, has_bias, nullptr, nullptr, 0,
+                                       nullptr, sq_layer, workspace, workspace_bytes, nullptr, nullptr, st);
             }
             if (!aligned_to(A, 16) || !aligned_to(Zbar, 16) || lda % 8 || ldz % 8)
                 return DPCLIP_ERR_UNSUPPORTED;
@@ -2640,8 +2643,10 @@ static int group_norms(const dpclip_layer* layers, int L, int B, dpclip_dtype dt
     if (n == 0) return DPCLIP_OK;
     if (!workspace || workspace_bytes < (size_t)kHeaderBytes) return DPCLIP_ERR_WORKSPACE;
     const bool with_tail = tail && n == L;
+    const int rc = launch_group(g, n, B, true, nullptr, nullptr, workspace, workspace_bytes, (cudaStream_t)stream, with_tail ? tail : nullptr);
+    if (rc > 0) { for (int l = 0; l < L; ++l) taken[l] = 0; return DPCLIP_OK; }         // no room: layer by layer
     if (tail_done) *tail_done = with_tail;
-    return launch_group(g, n, B, true, nullptr, nullptr, workspace, workspace_bytes, (cudaStream_t)stream, with_tail ? tail : nullptr);
+    return rc;
 }
 // clip_ld as in shared_clipped_grad_launches
 static int group_grads(const dpclip_layer* layers, int L, int B, dpclip_dtype dtype, const float* clip, long clip_ld,

@@ -1453,3 +1453,20 @@ def test_step_streams_stay_inside_side_workspaces(dp):
     assert all(bool((r[side:] == 0xA5).all()) for r in raw)
     for g, h in zip(one, (plan.norms, *plan.gW, *plan.gb)):
         assert rel_fro(h.cpu().numpy(), g) <= TOL["f32"]["grad"]
+
+
+@pytest.mark.parametrize("T,d_in,d_out", [(769, 132, 140), (1000, 132, 132), (768, 136, 260)])
+def test_fp32_norms_of_small_long_layers_with_the_header_alone(dp, T, d_in, d_out):
+    """Layers below the size where fp32 takes the tensor cores by itself need no scratch (dpclip_workspace_bytes), also when the
+    caller asks for the materialised product."""
+    B = 1
+    nbytes = dp.dpclip_workspace_bytes(B, T, d_in, d_out, dp.DPCLIP_F32, dp.DPCLIP_MATERIALIZE)
+    assert nbytes == 256
+    A, Z = workloads.random_layer(3, B, T, d_in, d_out, "f32", scale_z=0.05)
+    guard = Guarded(B, fill=-1.0)
+    ws = _ws(dp, nbytes)
+    dp.dpclip_layer_sqnorms(to_device(A, "f32"), to_device(Z, "f32"), True, guard.t, ws, dp.DPCLIP_MATERIALIZE)
+    torch.cuda.synchronize()
+    assert dp.dpclip_read_status(ws) == 0
+    guard.check()
+    assert max_rel(np.sqrt(guard.t.cpu().numpy()), np.sqrt(oracle.layer_sqnorms(A, Z, True))) <= TOL["f32"]["norm"]
