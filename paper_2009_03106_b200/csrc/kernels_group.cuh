@@ -322,10 +322,7 @@ zta_group_kernel(const __grid_constant__ zg::Maps maps, const __grid_constant__ 
                 // factors of this stage's rows, fetched before waiting for the tile
                 const int blk0 = w.row0 + kb * BK;
                 float fr[NR];
-                if (NORM) {
-#pragma unroll
-                    for (int i = 0; i < NR; ++i) fr[i] = blk0 + lane + 32 * i < w.row_end ? 1.f : 0.f;
-                } else {
+                if (!NORM) {
                     const int e_first = blk0 / T, rem0 = blk0 - e_first * T;
                     const bool uniform = rem0 + BK <= T && blk0 + BK <= w.row_end;
 #pragma unroll
@@ -347,6 +344,12 @@ zta_group_kernel(const __grid_constant__ zg::Maps maps, const __grid_constant__ 
                     x[side][0] = *reinterpret_cast<const float4*>(rw + side * C::RAW_SIDE + raw0);
                     x[side][1] = *reinterpret_cast<const float4*>(rw + side * C::RAW_SIDE + raw1);
                 }
+                if (NORM && blk0 + lane >= w.row_end) {
+                    // rows of the next example are cleared on both sides: an infinity or NaN there times a factor of 0 would
+                    // be this one's norm
+#pragma unroll
+                    for (int side = 0; side < 2; ++side) x[side][0] = x[side][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+                }
                 uint4 b3[2][3];
 #pragma unroll
                 for (int side = 0; side < 2; ++side) {
@@ -354,8 +357,10 @@ zta_group_kernel(const __grid_constant__ zg::Maps maps, const __grid_constant__ 
                     float v[8] = {x[side][0].x, x[side][0].y, x[side][0].z, x[side][0].w,
                                   x[side][1].x, x[side][1].y, x[side][1].z, x[side][1].w};
                     if ((side == 0) == (z_on_m != 0)) {
+                        if (!NORM) {
 #pragma unroll
-                        for (int k = 0; k < 8; ++k) v[k] *= fr[0];
+                            for (int k = 0; k < 8; ++k) v[k] *= fr[0];
+                        }
                         if (bias_here) {
 #pragma unroll
                             for (int k = 0; k < 8; ++k) cs[k] += v[k];

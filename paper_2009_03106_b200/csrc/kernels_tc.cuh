@@ -940,6 +940,19 @@ zta_tc_kernel(const __grid_constant__ zta::Maps maps, const zta::Params p) {
                 if (!ok) break;
                 if (t == 0) { DPCLIP_TRACE_AT(1, tr); ++tr; }
                 uint8_t* zt = smem + stage * STAGE_BYTES;
+                if (!SPLIT && p.norm_mode && blk0 + BK > w.row_end) {
+                    // rows of the next example: cleared on both sides, because an infinity or NaN of that example
+                    // times a factor of 0 would be this one's norm (the A tile is BN columns, two units a thread)
+#pragma unroll
+                    for (int i = 0; i < NR; ++i) {
+                        if (blk0 + rs + 16 * i < w.row_end) continue;
+                        const uint4 none = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+                        for (int h = 0; h < MT; ++h) *reinterpret_cast<uint4*>(zt + h * 2 * CHUNK_BYTES + off + i * 2048) = none;
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) *reinterpret_cast<uint4*>(zt + A_BYTES + h * 2 * CHUNK_BYTES + off + i * 2048) = none;
+                    }
+                }
                 auto add8 = [](float* c, const uint4& v) {
                     const uint32_t wds[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll

@@ -1470,3 +1470,31 @@ def test_fp32_norms_of_small_long_layers_with_the_header_alone(dp, T, d_in, d_ou
     assert dp.dpclip_read_status(ws) == 0
     guard.check()
     assert max_rel(np.sqrt(guard.t.cpu().numpy()), np.sqrt(oracle.layer_sqnorms(A, Z, True))) <= TOL["f32"]["norm"]
+
+
+# An example's infinities and NaNs are its own: norms of the others are what they are without it.  The materialised product's last
+# stage of an example holds rows of the next: fp32 in 128 x 128 tiles and on pairs (one and several accumulators), bf16, rows
+# that TMA can address and staged ones; and the Gram form
+NEIGHBOURS = [("f32", 77, 256, 100), ("f32", 77, 250, 101), ("f32", 77, 260, 132), ("f32", 145, 261, 132), ("f32", 1000, 260, 133),
+              ("bf16", 200, 136, 72), ("bf16", 200, 131, 70), ("bf16", 200, 136, 264), ("bf16", 77, 300, 302), ("bf16", 300, 520, 512)]
+
+
+@pytest.mark.parametrize("dtype,T,d_in,d_out", NEIGHBOURS)
+def test_norms_do_not_see_the_next_example(dp, dtype, T, d_in, d_out):
+    B = max(6, 40 * 2 ** 20 // (T * d_in * d_out) + 1)
+    A, Z = workloads.random_layer(17, B, T, d_in, d_out, dtype, scale_z=0.05)
+    dA, dZ = to_device(A, dtype), to_device(Z, dtype)
+    plan = dp.StepPlan([dp.Layer(dA, dZ, True)])
+    plan.run(1.0, 0.0, 1)
+    clean = plan.norms.cpu().numpy()
+    for bad in (float("nan"), float("inf")):
+        for t in (dA, dZ):
+            keep = t[2, 0, 3].clone()
+            t[2, 0, 3] = bad
+            plan.run(1.0, 0.0, 1)
+            got = plan.norms.cpu().numpy()
+            t[2, 0, 3] = keep
+            assert not np.isfinite(got[2])
+            others = np.arange(B) != 2
+            assert max_rel(got[others], clean[others]) <= 2e-6, (bad, np.nonzero(others & ~np.isfinite(got)))
+    assert dp.dpclip_read_status(plan.workspace) == 0
