@@ -291,7 +291,8 @@ int launch_simt_norms(const void* A, long lda, const void* Z, long ldz, int B, i
     return launch_status();
 }
 
-struct NoiseSpec { float scale; unsigned long long seed, sid_w, sid_b; };
+// after_sum: the result has to be that of the sum followed by the noise, bit for bit
+struct NoiseSpec { float scale; unsigned long long seed, sid_w, sid_b; bool after_sum = false; };
 
 // noise in the epilogue of the fp32-ALU kernel; it indexes the dense tensor
 void simt_noise(SimtParams& p, const NoiseSpec* noise, bool* noise_done) {
@@ -373,7 +374,8 @@ int launch_simt_grad(const void* A, long lda, const void* Z, long ldz, int B, in
         if (gb && cudaMemsetAsync(gb, 0, sizeof(float) * (size_t)d_out, st) != cudaSuccess)
             return DPCLIP_ERR_CUDA;
     }
-    simt_noise(p, noise, noise_done);
+    // slices add up in any order, the noise among them
+    if (ksplit == 1 || !noise || !noise->after_sum) simt_noise(p, noise, noise_done);
     dim3 grid(n_tiles, (unsigned)ksplit);
     if (dtype == DPCLIP_F32) zta_simt_kernel<float, true><<<grid, SIMT_THREADS, 0, st>>>(p);
     else zta_simt_kernel<__nv_bfloat16, true><<<grid, SIMT_THREADS, 0, st>>>(p);
@@ -1875,7 +1877,7 @@ int dpclip_clipped_grad_noise(const void* A, long lda, const void* Zbar, long ld
     if (!aligned_to(gW, 4) || (gb && !aligned_to(gb, 4))) return DPCLIP_ERR_MISALIGNED;
     if (!workspace || workspace_bytes < workspace_floor(B, T, d_in, d_out, dtype))
         return DPCLIP_ERR_WORKSPACE;
-    NoiseSpec ns = {sigma * C, seed, stream_id_w, stream_id_b};
+    NoiseSpec ns = {sigma * C, seed, stream_id_w, stream_id_b, true};
     bool noise_done = false;
     rc = clipped_grad_impl(A, lda, Zbar, ldz, B, T, d_in, d_out, dtype, clip, gW, d_in, gb, workspace,
                            workspace_bytes, &ns, &noise_done, (cudaStream_t)stream);

@@ -1498,3 +1498,17 @@ def test_norms_do_not_see_the_next_example(dp, dtype, T, d_in, d_out):
             others = np.arange(B) != 2
             assert max_rel(got[others], clean[others]) <= 2e-6, (bad, np.nonzero(others & ~np.isfinite(got)))
     assert dp.dpclip_read_status(plan.workspace) == 0
+
+
+@pytest.mark.parametrize("B,d_in,d_out", [(64, 37, 53), (128, 37, 53), (128, 130, 70)])
+def test_clipped_grad_noise_is_the_sum_then_the_noise(dp, B, d_in, d_out):
+    """On the fp32 ALUs, one slice of rows and two (more add up in any order): the bits of the two separate calls."""
+    A, Z = workloads.random_layer(19, B, 1, d_in, d_out, "f32", scale_z=0.1)
+    dA, dZ, clip = to_device(A, "f32"), to_device(Z, "f32"), torch.rand(B, device="cuda")
+    ws = _ws(dp)
+    out = [(torch.empty(d_out, d_in, device="cuda"), torch.empty(d_out, device="cuda")) for _ in range(2)]
+    dp.dpclip_clipped_grad(dA, dZ, clip, out[0][0], out[0][1], ws)
+    for g, sid in zip(out[0], (4, 5)):
+        dp.dpclip_add_noise(g, 0.3, 1.0, 7, sid)
+    dp.dpclip_clipped_grad_noise(dA, dZ, clip, out[1][0], out[1][1], 0.3, 1.0, 7, 4, 5, ws)
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
