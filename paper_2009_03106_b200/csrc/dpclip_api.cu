@@ -435,36 +435,85 @@ struct GramLayer {
     const void* A; long lda; const void* Z; long ldz;
     int B, T, d_in, d_out, has_bias;
     float* sq;
+    bool per_ex;                   // row blocks begin with their example (gram_per_ex)
 };
 
 // Examples of two row blocks: their own kernel, one HBM pass per example.
 inline bool gram_two_blocks(int T) {
     return T == 2 * tc::gram::BM && !path_switch(SW_NO_GRAM_Q2);
 }
-// Row blocks that begin with their example, not with a multiple of 128 rows.  Flattened, a row block of T = 90 meets two column
-// blocks (1.4 blocks of products an example, 1 this way), and long examples were re-read from HBM.  Kernel, flattened / this way:
-// T = 90, 320 + 3296 features, 264 examples: 55 / 47 us; T = 374, 1024, 64: 34 / 21; T = 512, 5120, 256: 608 / 383; T = 2048, 8192,
-// 32: 3813 / 844.  Below 88 rows the empty part of a block costs more (T = 77, six layers of 300 to 1100 features, 50 examples: the
-// step 139 us flattened, 145 this way), and so does a second block of few rows (256 examples of 2048 features, T = 140: 46 / 53;
-// T = 176: 60 / 54) or a third (seven layers of 352 to 1392 features, T = 276, 244 examples: 361 / 398; T = 300, 512 + 2048, 200:
-// 146 / 101).
-inline bool gram_per_ex(int T) {
+// Row blocks that begin with their example, not with a multiple of 128 rows; width[0 .. n) are the d_in + d_out of the launch's
+// layers, widest first.  Flattened over the examples, a block that crosses into the next example meets a column block more, and
+// a long example was re-read from HBM; beginning with the example, its last block is partly empty and there are more work
+// items.  Which takes less follows from T, B and the layers: the items are dealt to the CTAs as the launch deals them, an item
+// costing one unit a feature, half a unit more for every column block and for a row block of its own, and 300 for its drain; the
+// order whose busiest CTA has less to do wins, by 5 % for the re-reads of examples of several blocks, else by 2 %.
+// Kernel, flattened / by example: T = 96, three layers of 1536 features, 64 examples: 17 / 24 us; T = 192, 260 examples of 1024 +
+// 2560: 77 / 88; T = 200, 250: 129 / 87; T = 156, 16 of 4096: 47 / 28; T = 512, 256 of 5120: 608 / 383; T = 2048, 32 of 8192:
+// 3813 / 844.  551 launches (T = 66 to 383, 16 to 320 examples, one to seven layers of 768 to 2560 features): 0.3 % over the
+// faster order of each, where ranges of T alone (by example from 88 rows, but for 129 to 167 and 257 to 287) were 4.5 % over.
+inline bool gram_per_ex(int T, int B, const int* width, int n) {
     namespace g = tc::gram;
-    return T >= 88 && T != g::BM && !(T > g::BM && T < 168) && !(T > 2 * g::BM && T < 288) && !gram_two_blocks(T) && !path_switch(SW_NO_GRAM_PER_EX);
+    if (T <= g::BM / 2 || T == g::BM || gram_two_blocks(T) || path_switch(SW_NO_GRAM_PER_EX)) return false;
+    const int q = ceil_div(T, (long)g::BM), subs = g::subs_of(q), sms = sm_budget();
+    if (T >= 3 * g::BM) return (long)B * subs < 1L << 27;               // items of a launch are counted in an int
+    struct Item { double features; int subs; };
+    auto row_block = [](int rb, int cb_max) {                           // rb against column blocks rb .. cb_max, two at a time
+        Item c = {0.0, 0};
+        for (int cb = rb; cb <= cb_max; cb += 2, ++c.subs) c.features += 1.0 + (cb < cb_max ? 1.0 : 0.5) + (cb > rb ? 0.5 : 0.0);
+        return c;
+    };
+    // steady: the period divides the number of CTAs, so a CTA always gets the same item of it
+    auto busiest = [&](const Item* item, int period, long items, bool steady) {
+        if (n * items <= 2400) {
+            double load[kNumSMs] = {0.0}, most = 0.0;
+            int cta = 0;
+            for (int l = 0; l < n; ++l)
+                for (long i = 0, k = 0; i < items; ++i) {
+                    load[cta] += item[k].features * width[l] + 300.0 * item[k].subs;
+                    if (++k == period) k = 0;
+                    if (++cta == sms) cta = 0;
+                }
+            for (int c = 0; c < sms; ++c) most = load[c] > most ? load[c] : most;
+            return most;
+        }
+        double mean = 0.0, most = 0.0, drains = 0.0, sum = 0.0;
+        for (int k = 0; k < period; ++k) {
+            mean += item[k].features / period; drains += 300.0 * item[k].subs / period;
+            most = item[k].features > most ? item[k].features : most;
+        }
+        const double one = steady ? most : mean;
+        for (int l = 0; l < n; ++l) sum += (one * width[l] + drains) * items / sms;
+        const double part = (double)ceil_div(n * items, (long)sms) - (double)n * items / sms;       // of a last wave
+        return sum + part * (one * width[n - 1] + drains);
+    };
+    Item own[4], flat[3 * g::BM];
+    int k = 0;
+    for (int rb = 0; rb < q; ++rb)
+        for (int cb = rb; cb < q; cb += 2) own[k++] = {1.0 + (cb + 1 < q ? 1.0 : 0.5) + (cb > rb ? 0.5 : 0.0), 1};
+    const long blocks = ceil_div((long)B * T, (long)g::BM);
+    int period = T;                                                     // blocks after which the examples lie alike: T / gcd(T, 128)
+    for (int two = 1; two < g::BM && period % 2 == 0; two *= 2) period /= 2;
+    if (period > blocks) period = (int)blocks;
+    for (int rb = 0, end = T - 1; rb < period; ++rb) {                  // end: last row of the block's last example
+        while (end < rb * g::BM + g::BM - 1) end += T;
+        flat[rb] = row_block(rb, end / g::BM);
+    }
+    return busiest(own, subs, (long)B * subs, true) <= busiest(flat, period, blocks, false) * (q > 1 ? 1.05 : 0.98);
 }
 // every item is on the diagonal when an example spans at most two aligned row blocks
-inline bool gram_diag_only(int T) {
+inline bool gram_diag_only(int T, bool per_ex) {
     namespace g = tc::gram;
-    return (gram_per_ex(T) && T <= 2 * g::BM) || (T % g::BM == 0 && T <= 2 * g::BM) || (g::BM % T == 0);
+    return (per_ex && T <= 2 * g::BM) || (T % g::BM == 0 && T <= 2 * g::BM) || (g::BM % T == 0);
 }
 
 // Which Gram kernel a layer takes; layers of one class can share a launch, and the kernel of class 2 takes layers of class 1 too.
 //   0: examples of exactly two row blocks (their own kernel: one HBM pass per example)
 //   1: other layers whose items all sit on the diagonal (stages of two tiles, six of them)
 //   2: the rest
-inline int gram_class(int T) {
+inline int gram_class(int T, bool per_ex) {
     if (gram_two_blocks(T)) return 0;
-    return gram_diag_only(T) ? 1 : 2;
+    return gram_diag_only(T, per_ex) ? 1 : 2;
 }
 
 // Norms of up to gram::MAX_LAYERS layers by the Gram identity in ONE launch of kernel class `cls`.  Layers go in descending order of bytes per group, so that the round-robin deal
@@ -475,10 +524,7 @@ int launch_gram_group(const GramLayer* ls, int n, int cls, int* status, cudaStre
     if (n <= 0 || n > g::MAX_LAYERS) return DPCLIP_ERR_INVALID_ARG;
     int order[g::MAX_LAYERS];
     for (int i = 0; i < n; ++i) order[i] = i;
-    auto cost = [&](int i) {
-        const long rows = ls[i].T % g::BM == 0 ? ls[i].T : g::BM;
-        return rows * (long)(ls[i].d_in + ls[i].d_out);
-    };
+    auto cost = [&](int i) { return (long)ls[i].d_in + ls[i].d_out; };
     for (int i = 1; i < n; ++i)                       // insertion sort, stable
         for (int j = i; j > 0 && cost(order[j]) > cost(order[j - 1]); --j) { const int t = order[j]; order[j] = order[j - 1]; order[j - 1] = t; }
     static_assert(sizeof(g::Launch) <= 4096, "kernel parameter space");
@@ -488,7 +534,8 @@ int launch_gram_group(const GramLayer* ls, int n, int cls, int* status, cudaStre
     int groups = 0;
     for (int k = 0; k < n; ++k) {
         const GramLayer& y = ls[order[k]];
-        if (gram_class(y.T) != cls && !(cls == 2 && gram_class(y.T) == 1)) return DPCLIP_ERR_INVALID_ARG;
+        const int own = gram_class(y.T, y.per_ex);
+        if (own != cls && !(cls == 2 && own == 1)) return DPCLIP_ERR_INVALID_ARG;
         const long R = (long)y.B * y.T;
         if (!make_map_bf16(&q.map_a[k], y.A, R, y.d_in, y.lda, g::BK, g::BM) ||
             !make_map_bf16(&q.map_z[k], y.Z, R, y.d_out, y.ldz, g::BK, g::BM))
@@ -497,17 +544,11 @@ int launch_gram_group(const GramLayer* ls, int n, int cls, int* status, cudaStre
         p.R = (int)R; p.T = y.T; p.d_in = y.d_in; p.d_out = y.d_out; p.has_bias = y.has_bias ? 1 : 0;
         p.sq = y.sq;
         if (cls == 0) {
-            p.dense = 1; p.q = 2;
-            p.n_groups = y.B;
-        } else if (gram_per_ex(y.T)) {
-            p.per_ex = 1; p.q = ceil_div(y.T, g::BM); p.subs = g::subs_of(p.q);
-            if ((long)y.B * p.subs > 0x3FFFFFFFL) return DPCLIP_ERR_UNSUPPORTED;
-            p.n_groups = y.B * p.subs;
-        } else if (y.T % g::BM == 0) {
-            p.dense = 1; p.q = y.T / g::BM;
             p.n_groups = y.B;                     // one example per group
+        } else if (y.per_ex) {
+            p.per_ex = 1; p.q = ceil_div(y.T, g::BM); p.subs = g::subs_of(p.q);
+            p.n_groups = y.B * p.subs;
         } else {
-            p.dense = 0;
             p.n_groups = ceil_div(R, g::BM);      // one 128-row block per group
         }
         q.group_begin[k] = groups;
@@ -552,8 +593,10 @@ int launch_gram_group(const GramLayer* ls, int n, int cls, int* status, cudaStre
 
 int launch_gram_norms(const void* A, long lda, const void* Z, long ldz, int B, int T, int d_in, int d_out,
                       int has_bias, float* sq, int* status, cudaStream_t st) {
-    const GramLayer y = {A, lda, Z, ldz, B, T, d_in, d_out, has_bias, sq};
-    return launch_gram_group(&y, 1, gram_class(T), status, st);
+    const int width = d_in + d_out;
+    const bool per_ex = gram_per_ex(T, B, &width, 1);
+    const GramLayer y = {A, lda, Z, ldz, B, T, d_in, d_out, has_bias, sq, per_ex};
+    return launch_gram_group(&y, 1, gram_class(T, per_ex), status, st);
 }
 
 // Largest scratch the split-row clipped sum can ask for: one partial tile per item, at most one
@@ -1712,9 +1755,31 @@ static int gram_layers_sqnorms(const dpclip_layer* layers, int L, int B, dpclip_
         const int method = y.method == DPCLIP_AUTO ? dpclip_pick_method(B, y.T, y.d_in, y.d_out, y.lda, y.ldz, dtype) : y.method;
         return method == DPCLIP_GRAM;
     };
-    bool any_long = false;
-    for (int l = 0; l < L; ++l) any_long = any_long || (takes(layers[l]) && gram_class(layers[l].T) == 2);
-    auto class_of = [&](int T) { const int c = gram_class(T); return c == 1 && any_long ? 2 : c; };
+    // the numbers of positions that occur, the widest layers of each and the order of their row blocks; a thirteenth is flattened
+    struct { int T, n, width[g::MAX_LAYERS]; bool per_ex; } seen[12] = {};
+    int n_seen = 0;
+    bool more = false;
+    auto of = [&](int T) { int k = 0; while (k < n_seen && seen[k].T != T) ++k; return k; };
+    for (int l = 0; l < L; ++l) {
+        if (!takes(layers[l])) continue;
+        const int k = of(layers[l].T), w = layers[l].d_in + layers[l].d_out;
+        if (k == n_seen) {
+            if (n_seen == 12) { more = true; continue; }
+            seen[n_seen++].T = layers[l].T;
+        }
+        auto& y = seen[k];
+        int i = y.n < g::MAX_LAYERS ? y.n++ : w > y.width[g::MAX_LAYERS - 1] ? g::MAX_LAYERS - 1 : g::MAX_LAYERS;
+        if (i == g::MAX_LAYERS) continue;
+        for (; i > 0 && y.width[i - 1] < w; --i) y.width[i] = y.width[i - 1];
+        y.width[i] = w;
+    }
+    bool any_long = more;
+    for (int k = 0; k < n_seen; ++k) {
+        seen[k].per_ex = gram_per_ex(seen[k].T, B, seen[k].width, seen[k].n);
+        any_long = any_long || gram_class(seen[k].T, seen[k].per_ex) == 2;
+    }
+    auto per_ex_of = [&](int T) { const int k = of(T); return k < n_seen && seen[k].per_ex; };
+    auto class_of = [&](int T) { const int c = gram_class(T, per_ex_of(T)); return c == 1 && any_long ? 2 : c; };
     for (int cls = 0; cls < 3; ++cls) {
         GramLayer batch[g::MAX_LAYERS];
         int idx[g::MAX_LAYERS];
@@ -1734,7 +1799,8 @@ static int gram_layers_sqnorms(const dpclip_layer* layers, int L, int B, dpclip_
         for (int l = 0; l < L; ++l) {
             const dpclip_layer& y = layers[l];
             if (!takes(y) || class_of(y.T) != cls) continue;
-            batch[n] = {y.A, y.lda, y.Zbar, y.ldz, B, y.T, y.d_in, y.d_out, y.has_bias ? 1 : 0, sq_layers + (size_t)l * B};
+            batch[n] = {y.A, y.lda, y.Zbar, y.ldz, B, y.T, y.d_in, y.d_out, y.has_bias ? 1 : 0, sq_layers + (size_t)l * B,
+                        per_ex_of(y.T)};
             idx[n] = l;
             if (++n == g::MAX_LAYERS) { const int rc = flush(); if (rc) return rc; }
         }

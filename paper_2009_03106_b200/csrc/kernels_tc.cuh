@@ -68,9 +68,8 @@ constexpr int MAX_LAYERS = 8;                 // layers one launch can take
 
 struct Params {            // one layer
     int R, T, d_in, d_out, has_bias;
-    int n_groups;          // dense (T % 128 == 0): examples; otherwise: 128-row blocks
-    int dense, q;          // q = T / 128 blocks per example in the dense case
-    int per_ex, subs;      // row blocks begin with their example: q = ceil(T / 128), a group is one of the example's `subs` sub-items
+    int n_groups;          // 128-row blocks; per_ex: sub-items; in the kernel of two row blocks: examples
+    int per_ex, q, subs;   // row blocks begin with their example: q = ceil(T / 128), a group is one of the example's `subs` sub-items
     float* sq;
 };
 
@@ -141,14 +140,8 @@ __host__ __device__ __forceinline__ int subs_of(int q) { int n = 0; for (int rb 
 // With per_ex the row blocks begin with their example and every sub-item is a group of its own, so that neighbouring CTAs
 // stream the same example at the same time and all but the first read of a block hit L2.  One CTA walking an example of
 // 512 rows and 5120 features read it three times from HBM, 148 examples (770 MB) being in flight: 617 us for 256 of them.
-// In the dense case the row blocks of an example are walked from the LAST to the first: row block rb needs
-// the column blocks rb .. q-1, so every pass then fetches exactly one block that has not been read before
-// (its own) and re-reads the others from L2.  Walking upwards, the first pass streams the whole example
-// from HBM and the later ones run out of L2; CTAs that start together then alternate in lockstep between
-// a phase that saturates HBM and one that leaves it idle (measured: 23 us per 512 KB example instead of the
-// 12.5 us its bytes take).
 struct SubIter {
-    int rb, rb_first, rb_last, cb, cb_max;
+    int rb, cb, cb_max;
     int base;                                   // first row of block 0
     __device__ __forceinline__ static int cbmax(const Params& p, int rb) {
         const long last_row = min((long)rb * BM + BM - 1, (long)p.R - 1);
@@ -156,27 +149,23 @@ struct SubIter {
         return (int)(min((e_last + 1) * p.T - 1, (long)p.R - 1) / BM);
     }
     __device__ __forceinline__ SubIter(const Params& p, int g) {
-        base = 0;
         if (p.per_ex) {
             const int ex = g / p.subs;
             int i = g - ex * p.subs;
             rb = 0;
             while (i >= (p.q - rb + 1) >> 1) { i -= (p.q - rb + 1) >> 1; ++rb; }
-            rb_first = rb_last = rb;
             cb = rb + 2 * i; cb_max = min(cb + 1, p.q - 1);
             base = ex * p.T;
-            return;
+        } else {
+            rb = cb = g; cb_max = cbmax(p, g);
+            base = 0;
         }
-        if (p.dense) { rb_first = g * p.q; rb_last = rb_first + p.q - 1; } else { rb_first = g; rb_last = g; }
-        rb = rb_last;
-        cb = rb; cb_max = cbmax(p, rb);
     }
     __device__ __forceinline__ bool next(const Params& p, Sub& s) {
-        if (rb < rb_first) return false;
+        if (cb > cb_max) return false;
         s.rb = rb; s.cb = cb; s.ncb = cb + 1 <= cb_max ? 2 : 1;
         s.row0 = base + rb * BM; s.col0 = base + cb * BM;
         cb += 2;
-        if (cb > cb_max) { --rb; if (rb >= rb_first) { cb = rb; cb_max = cbmax(p, rb); } }
         return true;
     }
 };

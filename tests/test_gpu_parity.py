@@ -1290,13 +1290,18 @@ def test_step_fp32_layers_in_one_launch(dp, B, specs):
             assert np.linalg.norm(got.cpu().numpy() - sigma * C * xi - ref) <= bound, (l, sid)
 
 
-# Gram norms with row blocks that begin with their example (65 rows on, more than two blocks) and the two-block kernel with
-# masked rows and columns: one row behind a block's edge, one short of it, several layers with and without a bias in one launch
-GRAM_ROWS = [(5, (65, 127)), (3, (129, 159, 255)), (2, (257, 300, 383)), (2, (513, 640)), (4, (192, 256))]
+# Gram norms in row blocks that begin with their example and in blocks flattened over the examples (the switch): one row behind a
+# block's edge, one short of it, several layers with and without a bias in one launch, and lengths at which batches of 2 to 5
+# or of 300 go over from one order to the other
+GRAM_ROWS = [(5, (65, 127)), (3, (129, 159, 255)), (2, (257, 300, 383)), (2, (513, 640)), (4, (192, 256)),
+             (5, (88, 96)), (3, (168, 288)), (300, (66,)), (300, (96, 100)), (300, (160, 192)), (2, (384, 128, 64, 30))]
 
 
+@pytest.mark.parametrize("flattened", [False, True])
 @pytest.mark.parametrize("B,Ts", GRAM_ROWS)
-def test_gram_norms_row_blocks_of_an_example(dp, B, Ts):
+def test_gram_norms_row_blocks_of_an_example(dp, B, Ts, flattened, path_switch):
+    if flattened:
+        path_switch("DPCLIP_NO_GRAM_PER_EX", "1")
     specs = [(T, i, o, k % 2 == 0) for k, T in enumerate(Ts) for i, o in ((136, 72), (64, 200))]
     data = [workloads.random_layer(90 + k, B, T, i, o, "bf16", scale_z=0.05) for k, (T, i, o, _) in enumerate(specs)]
     plan = dp.StepPlan([dp.Layer(to_device(A, "bf16"), to_device(Z, "bf16"), s[3], dp.DPCLIP_GRAM) for (A, Z), s in zip(data, specs)])
