@@ -9,8 +9,10 @@ paper's workloads.  The headline workload is the largest single-GPU
 configuration: the sequence-model layers at B = 128, T = 256 in bf16 (cfg4).
 The other configurations (the two MLPs, the CNN in both precisions, the
 Gram-vs-materialise sweep) are timed in the same run; their step times and
-roofline fractions are in the JSON line under "configs" (compact, printed last)
-and, with per-kernel detail, under "workloads".  Rank 0 prints ONE JSON line.
+roofline fractions are in the JSON line under "configs".  Rank 0 prints ONE JSON
+line on stdout, short enough to be kept whole where only the end of the output
+is (`headline`); the full record, with per-kernel detail and the sweep, goes to
+stderr as a JSON line of its own.
 
 Timing: CUDA events on the launching stream, max over ranks.  Models with T > 1
 layers (hundreds of microseconds per step): one step = one replay of a CUDA
@@ -892,6 +894,33 @@ def config_summary(name, w, r, ms):
                 frac_sustained=round(sr["roof_sustained_us"] / (ms * 1e3), 4))
 
 
+# Of the record the printed line keeps what the benchmark's contract names and one pair of numbers per configuration.
+HEADLINE_KEYS = ("impl", "metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+                 "vs_baseline", "dtype", "data", "config", "e2e", "gpu_launches", "clocks", "launch", "cpu_baseline",
+                 "step_roofline_frac", "eager_ms_per_step", "warm_l2_ms_per_step", "single_step_graph_ms_per_step")
+ROOFLINE_KEYS = ("kernel", "bound", "achieved", "peak", "unit", "frac", "traffic", "kernel_ms", "share_of_step", "peak_source")
+HEADLINE_MAX = 2600
+
+
+def headline(record):
+    line = {k: record[k] for k in HEADLINE_KEYS if k in record}
+    if record.get("e2e"):
+        line["e2e"] = {k: v for k, v in record["e2e"].items() if k != "note"}
+    if record.get("roofline"):
+        line["roofline"] = {k: record["roofline"][k] for k in ROOFLINE_KEYS if k in record["roofline"]}
+    # workload: [microseconds, fraction of its step roofline]
+    line["configs"] = {k: [v["us"], v["frac"]] for k, v in record.get("configs", {}).items() if "us" in v}
+    for k in ("single_step_graph_ms_per_step", "warm_l2_ms_per_step", "eager_ms_per_step", "launch"):
+        if len(json.dumps(line)) > HEADLINE_MAX:
+            line.pop(k, None)
+    return line
+
+
+def emit(record):
+    print(json.dumps(record), file=sys.stderr)
+    print(json.dumps(headline(record)), flush=True)
+
+
 # ---------------------------------------------------------------------------
 def main():
     ap = argparse.ArgumentParser()
@@ -977,7 +1006,7 @@ def main():
         line["launch"] = res["how"]
         line["e2e"] = None
         dist.destroy_process_group()
-        print(json.dumps(line))
+        emit(line)
         return
 
     if res.get("clip_cases"):
@@ -1054,11 +1083,8 @@ def main():
     line["workloads"] = others
     if not args.no_cpu_baseline:
         line["cpu_baseline"], _, _ = oracle_sample(w)
-    # per-configuration step times and roofline fractions: inside `roofline` (kept with the headline) and,
-    # compact, as the LAST key of the line
-    roof["per_config"] = {k: (v if k == "cfg5" else dict(us=v["us"], frac=v["frac"], bound=v["bound"])) for k, v in configs.items()}
     line["configs"] = configs
-    print(json.dumps(line))
+    emit(line)
 
 
 if __name__ == "__main__":
