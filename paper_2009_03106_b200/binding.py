@@ -161,10 +161,17 @@ def _dtype_code(t: torch.Tensor) -> int:
     raise TypeError(f"unsupported dtype {t.dtype}")
 
 
+# The raw handle of the current stream (0.1 us): torch.cuda.current_stream() builds a Stream object, 3 us of a 10 us step.  Both
+# functions are torch's own and may be renamed.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream) -> int:
     if stream is None:
-        # the raw handle (0.1 us): torch.cuda.current_stream() builds a Stream object, 3 us of a 10 us step
-        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        if _raw_stream is None or _raw_device is None:
+            return torch.cuda.current_stream().cuda_stream
+        return _raw_stream(_raw_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 

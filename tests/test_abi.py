@@ -168,3 +168,23 @@ def test_workspace_queries_without_a_gpu(lib):
     g1 = Conv(3, 32, 32, 3, 3, 1, 1)
     first = lib.dpclip_conv_workspace_bytes(128, ctypes.byref(g1), 32, 0, 0)
     assert first == rows + 128 * 1024 * 32 * 4 + 128 * 1024 * 27 * 4                # dL/dZ rows + the patch matrix
+
+
+@pytest.mark.parametrize("missing", ["_cuda_getCurrentRawStream", "_cuda_getDevice"])
+def test_current_stream_without_torchs_private_functions(monkeypatch, missing):
+    """The binding's short way to the current stream's handle goes through private names of torch; without one of them it asks the
+    public call."""
+    import importlib.util
+    import sys
+    import types
+
+    import torch
+    from paper_2009_03106_b200 import binding
+    monkeypatch.setattr(torch, "_C", types.SimpleNamespace(**{k: getattr(torch._C, k) for k in dir(torch._C) if k != missing}))
+    spec = importlib.util.spec_from_file_location("binding_without", binding.__file__)
+    other = importlib.util.module_from_spec(spec)
+    monkeypatch.setitem(sys.modules, "binding_without", other)
+    spec.loader.exec_module(other)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=1234))
+    assert other._stream(None) == 1234
+    assert other._stream(7) == 7
