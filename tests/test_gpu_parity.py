@@ -1146,6 +1146,41 @@ STAGED_MODELS = [
 ]
 
 
+# Sizes from which on every unaligned layer of the model IS copied (below, the fp32 ALUs keep it: the models above mix both)
+STAGED_LARGE = [
+    # all T = 1: copied from 2e8 multiply-adds on, bf16 as fp32 (64 examples), fp32 as it is (256); a thin head beside
+    (130, ("bf16",), ((1, 783, 1101, True), (1, 1101, 1003, False), (1, 1003, 10, True))),
+    (256, ("f32", "bf16"), ((1, 783, 1001, True), (1, 1001, 301, True))),
+    # T > 1, and a T = 1 group beside it whose type differs after staging
+    (64, ("f32", "bf16"), ((33, 515, 301, True), (20, 301, 130, False))),
+    (70, ("bf16",), ((20, 301, 514, True), (1, 2101, 1403, True), (1, 1403, 11, True))),
+    # one operand copied, the other addressed as it is
+    (16, ("f32", "bf16"), ((80, 304, 301, True), (80, 301, 304, True))),
+]
+
+
+def test_step_staged_models_are_staged(dp):
+    for B, dtypes, specs in STAGED_LARGE:
+        for dtype in dtypes:
+            t = torch.float32 if dtype == "f32" else torch.bfloat16
+            plan = dp.StepPlan([dp.Layer(torch.empty(B, T, i, dtype=t, device="cuda"), torch.empty(B, T, o, dtype=t, device="cuda"), b)
+                                for T, i, o, b in specs])
+            staged = dp.dpclip_step_workspace_bytes(plan) - dp.dpclip_step_side_workspace_bytes(plan)
+            unit = 4 if dtype == "f32" else 8
+            copies = 0
+            for T, i, o, _ in specs:
+                if T == 1 and dtype == "bf16":               # the whole group becomes fp32
+                    copies += B * (-(-i // 4) + -(-o // 4)) * 16
+                else:
+                    copies += sum(B * T * -(-d // unit) * 16 for d in (i, o) if d % unit)
+            assert copies <= staged <= copies + 512 * len(specs), (B, dtype, specs)
+
+
+@pytest.mark.parametrize("B,dtype,specs", [(B, d, specs) for B, dtypes, specs in STAGED_LARGE for d in dtypes])
+def test_step_staged_operands_at_size(dp, B, dtype, specs, path_switch):
+    test_step_staged_operands(dp, B, specs, dtype, path_switch)
+
+
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("B,specs", STAGED_MODELS)
 def test_step_staged_operands(dp, B, specs, dtype, path_switch):
@@ -1204,11 +1239,16 @@ def test_step_staged_sums_of_many_rows(dp, B, T, widths):
 STAGED_CONVS = [  # B, C, H, W, k, pad, stride, d_out, channel-major dL/dZ
     (5, 3, 28, 28, 3, 1, 1, 16, True), (6, 33, 15, 14, 3, 1, 2, 160, True), (4, 40, 9, 11, (3, 2), 1, 1, 257, False),
     (3, 9, 14, 14, 5, 2, 2, 30, True), (4, 64, 7, 7, 1, 0, 1, 65, True), (33, 64, 14, 14, 3, 1, 1, 128, True)]
+# large enough to be copied in both types: 5 x 5, 1 x 1 with both layouts, 3 channels of 7 x 7, and a narrow first layer, whose fp32
+# copies are dense rows of 27 and 30 elements
+STAGED_CONVS_LARGE = [
+    (16, 16, 20, 20, 5, 2, 1, 40, True), (16, 128, 14, 14, 1, 0, 1, 130, True), (16, 130, 14, 14, 1, 0, 1, 129, False),
+    (16, 3, 33, 33, 7, 3, 2, 65, True), (54, 3, 28, 28, 3, 1, 1, 30, True), (40, 64, 13, 15, (3, 2), 1, 2, 136, True)]
 
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
-@pytest.mark.parametrize("case", STAGED_CONVS)
-def test_model_step_staged_convolutions(dp, case, dtype):
+@pytest.mark.parametrize("case", STAGED_CONVS + STAGED_CONVS_LARGE)
+def test_model_step_staged_convolutions(dp, case, dtype, path_switch):
     """Convolutions from their feature maps in a model step: maps and gradients the implicit kernels do not take
     (strides, odd widths, many channels) are staged as patch matrix and rows; bounds as above."""
     B, cin, H, W, k, pad, stride, cout, cm = case
@@ -1221,7 +1261,13 @@ def test_model_step_staged_convolutions(dp, case, dtype):
     dZ = to_device(Z, dtype)
     plan = dp.ModelPlan([dp.ModelLayer(dp.DPCLIP_KIND_CONV, to_device(X, dtype), dZ.transpose(1, 2).contiguous() if cm else dZ,
                                        True, conv=(kh, kw, stride, pad), z_channel_major=cm)])
-    plan.run(C, 0.0, 1)
+    counts = []
+    for off in ("1", "0"):
+        path_switch("DPCLIP_NO_STAGE", off)
+        n0 = dp.dpclip_launch_count()
+        plan.run(C, 0.0, 1)
+        counts.append(dp.dpclip_launch_count() - n0)
+    assert case not in STAGED_CONVS_LARGE or counts[0] != counts[1]          # the copies' launch and others than without them
     assert dp.dpclip_read_status(plan.workspace) == 0
     assert max_rel(plan.norms.cpu().numpy(), norms_ref) <= TOL["f32"]["norm"]
     refW, refb = oracle.clipped_grad(A, Z, clip_ref)
@@ -1259,12 +1305,17 @@ def test_staged_convolutions_of_two_kernel_sizes_from_four_threads(dp):
 
 
 # fp32 layers that share the CTA-pair launch: a run boundary inside a tile, items of one stage to several drains (T = 30,
-# 128, 800: one accumulator, two, several windows), N = 64 .. 256 tiles, either operand on the M side, ragged widths
+# 128, 800: one accumulator, two, several windows), either operand on the M side, ragged widths; layers below 2^25 multiply-adds
+# beside them keep the fp32 ALUs.  The last two models share with all their layers: N = 64 and 128, where the two accumulators of
+# a tile lie in one slot, T of at most a stage, and N = 192 and 256
 GROUP_MODELS = [
     (3, ((30, 516, 64, True), (128, 260, 520, True), (800, 140, 196, False))),
     (9, ((128, 512, 256, False), (128, 196, 640, True), (33, 100, 300, True), (65, 320, 68, True))),
     (1, ((1700, 132, 516, True),)),
+    (40, ((30, 516, 64, True), (33, 300, 100, True), (65, 320, 68, False), (20, 128, 512, True))),
+    (24, ((200, 100, 128, True), (128, 64, 260, True), (100, 132, 196, True), (31, 516, 260, False))),
 ]
+GROUP_ALL = GROUP_MODELS[3:]
 
 
 @pytest.mark.parametrize("B,specs", GROUP_MODELS)
@@ -1276,7 +1327,11 @@ def test_step_fp32_layers_in_one_launch(dp, B, specs):
     norms_ref, clip_ref = oracle.factors(sq, C)
     plan = dp.StepPlan([dp.Layer(to_device(A, "f32"), to_device(Z, "f32"), b) for (A, Z), b in zip(data, hb)])
     for _ in range(2):                                       # the second step reuses every counter and slot
+        n0 = dp.dpclip_launch_count()
         plan.run(C, sigma, seed)
+        launches = dp.dpclip_launch_count() - n0
+    if (B, specs) in GROUP_ALL:                              # norms with the factors, sums, reduce
+        assert launches == 3
     assert dp.dpclip_read_status(plan.workspace) == 0
     assert max_rel(np.sqrt(plan.sq_layers.cpu().numpy()), np.sqrt(sq)) <= TOL["f32"]["norm"]
     check_saturation(plan.clip.cpu().numpy(), norms_ref, clip_ref, C)
@@ -1288,6 +1343,39 @@ def test_step_fp32_layers_in_one_launch(dp, B, specs):
             xi = oracle.normals(ref.size, seed, sid).reshape(ref.shape)
             bound = TOL["f32"]["grad"] * np.linalg.norm(ref) + 1e-5 * sigma * C * np.sqrt(ref.size)
             assert np.linalg.norm(got.cpu().numpy() - sigma * C * xi - ref) <= bound, (l, sid)
+
+
+def test_fp32_sums_of_more_tiles_than_the_workspace_holds(dp):
+    """147 partial tiles fit the workspace of one layer: 80 tiles and as many runs go in two launches, whose bias sums add up."""
+    A, Z = workloads.random_layer(84, 8, 5, 4096, 1280, "f32", scale_z=0.05)
+    clip = np.linspace(0.2, 1.0, 8).astype(np.float32)
+    W, gb = oracle.clipped_grad(A, Z, clip)
+    ws = _ws(dp, dp.dpclip_workspace_bytes(8, 5, 4096, 1280, dp.DPCLIP_F32, 0))
+    gW, gB = Guarded(1280, 4096), Guarded(1280)
+    n0 = dp.dpclip_launch_count()
+    dp.dpclip_clipped_grad(to_device(A, "f32"), to_device(Z, "f32"), torch.from_numpy(clip).cuda(), gW.t, gB.t, ws)
+    assert dp.dpclip_launch_count() - n0 == 4                # two launches and their reduces
+    torch.cuda.synchronize()
+    assert dp.dpclip_read_status(ws) == 0
+    gW.check(); gB.check()
+    assert rel_fro(gW.t.cpu().numpy(), W) <= TOL["f32"]["grad"] and rel_fro(gB.t.cpu().numpy(), gb) <= TOL["f32"]["grad"]
+
+
+def test_step_fp32_layers_in_the_workspace_of_one(dp):
+    """The smallest workspace a step accepts, with noise: layers and tiles in several launches, every output's noise once."""
+    B, specs = 8, ((5, 4096, 1280, True), (6, 1032, 1300, True), (20, 516, 516, False))
+    data = [workloads.random_layer(85 + k, B, T, i, o, "f32", scale_z=0.05) for k, (T, i, o, _) in enumerate(specs)]
+    plan = dp.StepPlan([dp.Layer(to_device(A, "f32"), to_device(Z, "f32"), s[3]) for (A, Z), s in zip(data, specs)])
+    plan.run(1.0, 0.3, 9)
+    whole = [g.cpu().numpy() for g in (*plan.gW, *plan.gb) if g is not None]
+    full = plan.workspace
+    plan.workspace = full[:max(dp.dpclip_workspace_bytes(B, T, i, o, dp.DPCLIP_F32, 0) for T, i, o, _ in specs)]
+    assert plan.workspace.numel() < full.numel()
+    plan.flat.fill_(float("nan"))
+    plan.run(1.0, 0.3, 9)
+    assert dp.dpclip_read_status(plan.workspace) == 0
+    for g, h in zip(whole, [g for g in (*plan.gW, *plan.gb) if g is not None]):
+        assert rel_fro(h.cpu().numpy(), g) <= 2e-6
 
 
 # Gram norms in row blocks that begin with their example and in blocks flattened over the examples (the switch): one row behind a
