@@ -235,7 +235,10 @@ typedef struct {
  * input rows are 16-byte multiples (4 fp32 / 8 bf16 elements; the zb rows of
  * a layer with at most 16 outputs excepted): norms, a grid-wide barrier with a
  * bounded wait, factors, clipped sums on the tensor cores, noise; else as two
- * launches; other models run layer by layer, their T = 1 layers together. */
+ * launches; other models run layer by layer, their T = 1 layers together.
+ * With a workspace of dpclip_step_workspace_bytes() several layers share
+ * launches, and operands whose rows are no 16-byte multiples are copied to such
+ * rows once per step where that pays (models of at most 64 layers). */
 int dpclip_step(const dpclip_layer* layers /* host */, int L, int B, dpclip_dtype dtype,
                 float C, float sigma, unsigned long long seed, unsigned long long stream_id0,
                 float* sq_layers, float* clip, float* norms,
@@ -339,7 +342,8 @@ int dpclip_step_per_layer(const dpclip_layer* layers /* host */, int L, int B, d
  * Row l of sq_layers [L][B] and the noise streams stream_id0 + 2l (gW) and + 2l + 1 (gb) belong to layer l
  * whatever its kind; factors and norms are over all L layers.  Dense layers take the same launches as in
  * dpclip_step (a model of dense layers only IS dpclip_step); the other kinds run through their per-layer
- * entry points followed by dpclip_add_noise.  workspace >= dpclip_model_workspace_bytes().  L <= 256.
+ * entry points with the noise added, but for convolutions outside the implicit kernels, which are copied as
+ * patch matrices where that pays and the workspace has room, and then are dense layers too.  workspace >= dpclip_model_workspace_bytes().  L <= 256.
  * Errors as for the per-layer entry points; INVALID_ARG for an unknown kind or d_in != d_out in an
  * element-wise layer; UNSUPPORTED for padded output rows. */
 typedef enum { DPCLIP_KIND_DENSE = 0, DPCLIP_KIND_ELEMENTWISE = 1, DPCLIP_KIND_CONV = 2 } dpclip_layer_kind;
@@ -427,7 +431,7 @@ int dpclip_gram_layers_sqnorms(const dpclip_layer* layers /* host */, int L, int
 
 /* Clipped sums with noise (Eq. 1 applied to the sum over examples of c_i Zbar_i^T A_i, Algorithm 1's
  * last two steps) of layers taken together: bf16 layers with T > 1, rows TMA can address, dense output
- * rows and d_in a multiple of 4.  Layers with ONE T and d_out wide enough for 512-row tiles (d_out >
+ * rows.  Layers with ONE T and d_out wide enough for 512-row tiles (d_out >
  * 256 and little padding) share a launch whatever their shapes, up to eight at a time: their tiles'
  * work is cut into equal runs over all pairs of SMs (needs the workspace dpclip_step_workspace_bytes
  * reports).  Other layers share a launch when they have ONE shape (T, d_in, d_out) and would be short

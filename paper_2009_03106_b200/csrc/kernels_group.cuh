@@ -3,7 +3,7 @@
 //
 // Why one launch.  A small model's layers are each a chain of latencies (set-up, first loads, drain) that fills few
 // SMs, and launched one after the other they add up: seven fp32 layers of 148 to 592 features (B = 61, T = 48) were 7
-// norm launches of 10 to 20 us and 14 clipped-sum launches, 261 us for 1.1 GFLOP.  Here the layers' work is one sequence
+// norm launches of 10 to 20 us and 14 clipped-sum launches, 252 us a step for 1.1 GFLOP.  Here the layers' work is one sequence
 // of units cut into equal shares, one per CTA pair.
 //
 // Why pairs.  What bounds the fp32 product is the shared-memory port: an fp32 operand tile is written by TMA, read and
@@ -21,8 +21,8 @@
 //       NORM: unit = one (example, tile); runs end between units; squares are summed into sq with atomics.
 //
 // Numbers.      fp32 inputs: x = b0 + b1 + b2, three bf16 terms cut off the top of the fp32 word: 3 x 8 bits, exact.  Six products,
-//                         b0 b0, b0 b1, b1 b0, b1 b1, b0 b2, b2 b0; what is dropped is below 2^-22 of a product, 2^-24 on
-//                         average.  The tensor core needs as long for them as for three tf32 products (which drop as much),
+//                         b0 b0, b0 b1, b1 b0, b1 b1, b0 b2, b2 b0; what is dropped (b1 b2, b2 b1) is below 2^-21 of a
+//                         product, 2^-24 on average, always toward zero.  The tensor core needs as long for them as for three tf32 products (which drop as much),
 //                         but 16-bit operands come out of the MN-major layout at full rate: the twelve tf32 MMAs of a 256 x
 //                         256 stage took 1.2 us where 0.8 is nominal.
 //                         The tensor core's accumulation truncates, a bias toward zero that grows with the number of additions:
@@ -31,9 +31,11 @@
 //                         one accumulator every four stages into registers of the warps that also prepare the stages took 2 us
 //                         each time, a quarter of the kernel.)
 //
-// Measured (fp32): the clipped-sum loop of 256 x 256 tiles takes 1.15 us a stage, 1.6 PFLOP/s of bf16 products, the tensor
-// core's rate (two plane stages and four raw ones, or three and two: the same).  Seven layers of 512 and 2048 features, B = 32,
-// T = 128: norms 172 us, clipped sums 164 us, reduce 28 us, where one launch per layer took 305, 310 and 38.
+// Measured (fp32): the loop of 256 x 256 tiles takes 1.15 us a stage, 1.6 PFLOP/s of bf16 products, the tensor core's rate
+// (two plane stages and four raw ones, or three and two: the same).  Seven layers of 512 and 2048 features, B = 32, T = 128:
+// norms 172 us, clipped sums 164 us, reduce 28 us, where one launch per layer took 305, 310 and 38.  Of those the loop is 127
+// us each (8192 stages on 74 pairs; tensor pipe active 56 and 54 % of a launch under ncu); the norms lose the rest to the
+// drain of 1.5 us behind the four stages of an example, the sums to fill, drains and partial tiles.
 //
 // Roles: warp 0 TMA (each CTA its own operands, plain loads), warp 1 MMA issuer (rank 0), 16 warps that prepare every
 // stage (factor, planes, bias column sums), 8 epilogue warps that take the finished accumulators.

@@ -1,9 +1,9 @@
 // fp32-ALU tile kernel for the product Zbar^T A over a range of rows.
 //
-// Used (1) for every fp32 layer with T > 1 -- the 1e-5 tolerance of fp32
-// inputs rules out plain bf16/tf32 tensor-core math -- and (2) as the path for
-// bf16 layers whose rows are not 16-byte multiples (e.g. d_in = 27) and so
-// cannot be fetched by TMA.
+// Used for layers below the sizes from which the tensor-core kernels pay, for
+// layers whose rows TMA cannot fetch where a call does not copy them to 16-byte
+// rows (the per-layer entry points), and for convolutions outside the implicit
+// kernels there.
 //
 // One CTA computes 64 x 64 output tiles (d_out x d_in) with 4 x 4 register
 // micro-tiles, marching over rows in slabs of 16 staged through shared memory
