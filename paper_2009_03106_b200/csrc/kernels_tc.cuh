@@ -940,6 +940,7 @@ zta_tc_kernel(const __grid_constant__ zta::Maps maps, const zta::Params p) {
                         for (int h = 0; h < MT; ++h) *reinterpret_cast<uint4*>(zt + h * 2 * CHUNK_BYTES + off + i * 2048) = none;
 #pragma unroll
                         for (int h = 0; h < 2; ++h) *reinterpret_cast<uint4*>(zt + A_BYTES + h * 2 * CHUNK_BYTES + off + i * 2048) = none;
+                        fr[i] = 1.f;                                 // nothing left to scale
                     }
                 }
                 auto add8 = [](float* c, const uint4& v) {
