@@ -163,14 +163,14 @@ def _dtype_code(t: torch.Tensor) -> int:
 
 # The raw handle of the current stream (0.1 us): torch.cuda.current_stream() builds a Stream object, 3 us of a 10 us step.  Both
 # functions are torch's own and may be renamed.
-_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
-_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+try:
+    _raw_stream, _raw_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+except AttributeError:
+    _raw_stream, _raw_device = (lambda _: torch.cuda.current_stream().cuda_stream), (lambda: 0)
 
 
 def _stream(stream) -> int:
     if stream is None:
-        if _raw_stream is None or _raw_device is None:
-            return torch.cuda.current_stream().cuda_stream
         return _raw_stream(_raw_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
