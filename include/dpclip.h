@@ -342,7 +342,9 @@ int dpclip_step_per_layer(const dpclip_layer* layers /* host */, int L, int B, d
  * Row l of sq_layers [L][B] and the noise streams stream_id0 + 2l (gW) and + 2l + 1 (gb) belong to layer l
  * whatever its kind; factors and norms are over all L layers.  Dense layers take the same launches as in
  * dpclip_step (a model of dense layers only IS dpclip_step); the other kinds run through their per-layer
- * entry points with the noise added, but for convolutions outside the implicit kernels, which are copied as
+ * entry points with the noise added, but for element-wise layers of at least 8 positions, whose per-example
+ * gradients (2 d floats an example) stay in the workspace between the stages when it has room, and for
+ * convolutions outside the implicit kernels, which are copied as
  * patch matrices where that pays and the workspace has room, and then are dense layers too.  workspace >= dpclip_model_workspace_bytes().  L <= 256.
  * Errors as for the per-layer entry points; INVALID_ARG for an unknown kind or d_in != d_out in an
  * element-wise layer; UNSUPPORTED for padded output rows. */

@@ -429,6 +429,14 @@ template <typename K>
 bool enable_smem(K kernel, int bytes) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
 }
+// The same for a kernel whose SMs small launches on other streams may share: the smallest division of L1 and shared memory that
+// holds the kernel (196 KB for a Gram kernel) would leave those none.  One transformer block (B = 128, T = 256, d = 512): the norms
+// of its LayerNorms ran behind the Gram launch, 100 to 135 us; beside it they end at 111 us, the Gram launch at 129 instead of 114.
+template <typename K>
+bool enable_smem_shared(K kernel, int bytes) {
+    return enable_smem(kernel, bytes) &&
+           cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess;
+}
 
 // One layer of a Gram-norm launch.
 struct GramLayer {
@@ -579,13 +587,13 @@ int launch_gram_group(const GramLayer* ls, int n, int cls, int* status, cudaStre
     const int grid = groups < sm_budget() ? groups : sm_budget();
     if (cls == 0) {
         q.work_counter = reinterpret_cast<unsigned int*>(reinterpret_cast<char*>(status) + kWorkCounterOffset);
-        if (!enable_smem(tc::gram_norm_q2_kernel, g::SMEM_BYTES)) return DPCLIP_ERR_CUDA;
+        if (!enable_smem_shared(tc::gram_norm_q2_kernel, g::SMEM_BYTES)) return DPCLIP_ERR_CUDA;
         tc::gram_norm_q2_kernel<<<grid, g::THREADS, g::SMEM_BYTES, st>>>(q);
     } else if (cls == 1) {
-        if (!enable_smem(tc::gram_norm_kernel<true>, g::SMEM_BYTES)) return DPCLIP_ERR_CUDA;
+        if (!enable_smem_shared(tc::gram_norm_kernel<true>, g::SMEM_BYTES)) return DPCLIP_ERR_CUDA;
         tc::gram_norm_kernel<true><<<grid, g::THREADS, g::SMEM_BYTES, st>>>(q);
     } else {
-        if (!enable_smem(tc::gram_norm_kernel<false>, g::SMEM_BYTES)) return DPCLIP_ERR_CUDA;
+        if (!enable_smem_shared(tc::gram_norm_kernel<false>, g::SMEM_BYTES)) return DPCLIP_ERR_CUDA;
         tc::gram_norm_kernel<false><<<grid, g::THREADS, g::SMEM_BYTES, st>>>(q);
     }
     return launch_status();
@@ -2341,8 +2349,9 @@ int dpclip_t1_layers_clipped_grad_noise(const dpclip_layer* layers, int L, int B
     return rc > 0 ? DPCLIP_ERR_UNSUPPORTED : rc;
 }
 
-int dpclip_elementwise_sqnorms(const void* Hbar, long ldh, const void* Zbar, long ldz, int B, int T, int d,
-                               dpclip_dtype dtype, int has_shift, float* sq_layer, void* stream) {
+// per_example: [B][2][d] for the examples' gradients (scale, shift), or NULL
+static int elementwise_sqnorms(const void* Hbar, long ldh, const void* Zbar, long ldz, int B, int T, int d, dpclip_dtype dtype,
+                               int has_shift, float* sq_layer, float* per_example, void* stream) {
     int rc = check_layer_args(Hbar, ldh, Zbar, ldz, B, T, d, d, dtype);
     if (rc) return rc;
     if (!sq_layer) return DPCLIP_ERR_INVALID_ARG;
@@ -2354,9 +2363,13 @@ int dpclip_elementwise_sqnorms(const void* Hbar, long ldh, const void* Zbar, lon
     const dim3 grid(ceil_div(d, cg * v), B);
     const int use_atomic = grid.x > 1;
     if (use_atomic && cudaMemsetAsync(sq_layer, 0, sizeof(float) * (size_t)B, st) != cudaSuccess) return DPCLIP_ERR_CUDA;
-    if (dtype == DPCLIP_F32) launch_ew_norm<float>(vec, cg, grid, st, Hbar, ldh, Zbar, ldz, T, d, has_shift, sq_layer, use_atomic);
-    else launch_ew_norm<__nv_bfloat16>(vec, cg, grid, st, Hbar, ldh, Zbar, ldz, T, d, has_shift, sq_layer, use_atomic);
+    if (dtype == DPCLIP_F32) launch_ew_norm<float>(vec, cg, grid, st, Hbar, ldh, Zbar, ldz, T, d, has_shift, sq_layer, use_atomic, per_example);
+    else launch_ew_norm<__nv_bfloat16>(vec, cg, grid, st, Hbar, ldh, Zbar, ldz, T, d, has_shift, sq_layer, use_atomic, per_example);
     return launch_status();
+}
+int dpclip_elementwise_sqnorms(const void* Hbar, long ldh, const void* Zbar, long ldz, int B, int T, int d,
+                               dpclip_dtype dtype, int has_shift, float* sq_layer, void* stream) {
+    return elementwise_sqnorms(Hbar, ldh, Zbar, ldz, B, T, d, dtype, has_shift, sq_layer, nullptr, stream);
 }
 
 int dpclip_elementwise_clipped_grad(const void* Hbar, long ldh, const void* Zbar, long ldz, int B, int T, int d,
@@ -2406,12 +2419,12 @@ int dpclip_add_noise(float* g, size_t n, float sigma, float C, unsigned long lon
 
 // Norms / clipped sum + noise of a layer that is not a dense product (element-wise parameters, convolution
 // given by its feature map): the per-layer entry points, with the layer's row of sq and its noise streams.
-static int other_kind_sqnorms(const dpclip_model_layer& m, int B, dpclip_dtype dtype, float* sq_row, void* workspace,
-                              size_t workspace_bytes, void* stream) {
+static int other_kind_sqnorms(const dpclip_model_layer& m, int B, dpclip_dtype dtype, float* sq_row, float* per_example,
+                              void* workspace, size_t workspace_bytes, void* stream) {
     const dpclip_layer& y = m.layer;
     if (m.kind == DPCLIP_KIND_ELEMENTWISE) {
         if (y.d_in != y.d_out) return DPCLIP_ERR_INVALID_ARG;
-        return dpclip_elementwise_sqnorms(y.A, y.lda, y.Zbar, y.ldz, B, y.T, y.d_in, dtype, y.has_bias, sq_row, stream);
+        return elementwise_sqnorms(y.A, y.lda, y.Zbar, y.ldz, B, y.T, y.d_in, dtype, y.has_bias, sq_row, per_example, stream);
     }
     if (m.kind == DPCLIP_KIND_CONV)
         return dpclip_conv_sqnorms(y.A, y.Zbar, m.z_channel_major, B, &m.conv, y.d_out, dtype, y.has_bias, sq_row,
@@ -2450,6 +2463,42 @@ static int other_kind_clipped_grad_noise(const dpclip_model_layer& m, int B, dpc
     if (gb) rc = dpclip_add_noise(gb, m.kind == DPCLIP_KIND_ELEMENTWISE ? (size_t)y.d_in : (size_t)y.d_out, sigma, C,
                                   seed, sid_b, stream);
     return rc;
+}
+
+// Per-example gradients of element-wise layers between the two stages of a step ([B][2][d] per layer).  Layers of fewer than 8
+// positions keep their second pass: their inputs are about as many bytes.
+static size_t ew_rows_bytes(const dpclip_model_layer& m, int B) {
+    const dpclip_layer& y = m.layer;
+    if (m.kind != DPCLIP_KIND_ELEMENTWISE || y.T < 8 || y.d_in <= 0 || y.d_in != y.d_out || B <= 0) return 0;
+    return round_up((size_t)B * 2 * y.d_in * sizeof(float), 256);
+}
+static size_t ew_rows_total(const dpclip_model_layer* layers, int L, int B) {
+    size_t total = 0;
+    for (int l = 0; l < L; ++l) total += ew_rows_bytes(layers[l], B);
+    return total;
+}
+// Clipped sums with noise of the element-wise layers whose per-example gradients are there.
+static int ew_rows_grads(const dpclip_model_layer* other, float* const* rows, int L, int B, const float* clip, float C, float sigma,
+                         unsigned long long seed, unsigned long long stream_id0, cudaStream_t st) {
+    EwRowsParams p;
+    int blocks = 0;
+    p.n = 0; p.B = B; p.clip = clip; p.noise_scale = sigma * C; p.k0 = (uint32_t)seed; p.k1 = (uint32_t)(seed >> 32);
+    for (int l = 0; l < L; ++l) {
+        if (rows[l]) {
+            const dpclip_layer& y = other[l].layer;
+            const unsigned long long sw = stream_id0 + 2ull * l, sb = sw + 1;
+            EwRowsLayer& q = p.layer[p.n++];
+            q.rows = rows[l]; q.g_scale = y.gW; q.g_shift = y.has_bias ? y.gb : nullptr; q.d = y.d_in; q.blk_begin = blocks;
+            q.sw0 = (uint32_t)sw; q.sw1 = (uint32_t)(sw >> 32); q.sb0 = (uint32_t)sb; q.sb1 = (uint32_t)(sb >> 32);
+            blocks += ceil_div(y.d_in, 32L) * (q.g_shift ? 2 : 1);
+        }
+        if (p.n == EW_ROWS_MAX_LAYERS || (l == L - 1 && p.n > 0)) {
+            elementwise_rows_grad_kernel<<<blocks, EW_THREADS, 0, st>>>(p);
+            if (launch_status()) return DPCLIP_ERR_CUDA;
+            p.n = 0; blocks = 0;
+        }
+    }
+    return DPCLIP_OK;
 }
 
 // ---------------------------------------------------------------------------
@@ -2789,7 +2838,7 @@ struct Lanes {
 // functions above.
 static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer* other, int L, int B, dpclip_dtype dtype,
                         float C, float sigma, unsigned long long seed, unsigned long long stream_id0,
-                        float* sq_layers, float* clip, float* norms, Lanes& lanes, StagePlan* sp) {
+                        float* sq_layers, float* clip, float* norms, Lanes& lanes, StagePlan* sp, float* const* ew_rows = nullptr) {
     int rc;
     const dpclip_layer* layers = sp ? sp->eff : layers_in;              // the layers with their staged operands
     dpclip_dtype t1_dtype = sp ? sp->t1_dtype : dtype;
@@ -2881,7 +2930,8 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
         const SmBudgetScope share(track ? budget[l] : 0);
         const int b = k++ % lanes.n;
         if (is_other)
-            rc = other_kind_sqnorms(other[l], B, dtype, sq_layers + (size_t)l * B, lanes.ws[b], lanes.ws_bytes[b], lanes.st[b]);
+            rc = other_kind_sqnorms(other[l], B, dtype, sq_layers + (size_t)l * B, ew_rows ? ew_rows[l] : nullptr, lanes.ws[b],
+                                    lanes.ws_bytes[b], lanes.st[b]);
         else
             rc = dpclip_layer_sqnorms(y.A, y.lda, y.Zbar, y.ldz, B, y.T, y.d_in, y.d_out, dtype, y.has_bias,
                                       (dpclip_method)y.method, sq_layers + (size_t)l * B, lanes.ws[b],
@@ -2930,10 +2980,16 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
     }
     if (track) stage_budgets(in_grad_group, any_group || any_rest, budget);
     k = (any_group ? 1 : 0) + (any_rest ? 1 : 0);
+    if (ew_rows) {
+        rc = ew_rows_grads(other, ew_rows, L, B, clip, C, sigma, seed, stream_id0, lanes.st[k % lanes.n]);
+        if (rc) return rc;
+        ++k;
+    }
     for (int l = 0; l < L; ++l) {
         const dpclip_layer& y = layers[l];
         const bool is_other = other_kind(l);
         if (!is_other && ((t1.active && y.T == 1) || (track && in_grad_group[l]))) continue;
+        if (ew_rows && ew_rows[l]) continue;
         const SmBudgetScope share(track ? budget[l] : 0);
         const int b = k++ % lanes.n;
         void* const stream = lanes.st[b];
@@ -3018,6 +3074,21 @@ static int step_dense(const dpclip_layer* layers, int L, int B, dpclip_dtype dty
                         sp.active ? &sp : nullptr);
 }
 
+// Scratch of a step over these layers, copies and per-example gradients aside; dense: the layers with T = 0 for other kinds.
+static size_t model_scratch_bytes(const dpclip_model_layer* layers, const dpclip_layer* dense, int L, int B, dpclip_dtype dtype) {
+    size_t ws = step_scratch_bytes(dense, L, B, dtype);
+    for (int l = 0; l < L; ++l) {
+        const dpclip_layer& y = layers[l].layer;
+        size_t w = kHeaderBytes;
+        if (layers[l].kind == DPCLIP_KIND_DENSE)
+            w = dpclip_workspace_bytes(B, y.T, y.d_in, y.d_out, dtype, (dpclip_method)y.method);
+        else if (layers[l].kind == DPCLIP_KIND_CONV)
+            w = dpclip_conv_workspace_bytes(B, &layers[l].conv, y.d_out, dtype, layers[l].z_channel_major);
+        if (w > ws) ws = w;
+    }
+    return ws;
+}
+
 static int step_model(const dpclip_model_layer* layers, int L, int B, dpclip_dtype dtype, float C, float sigma,
                       unsigned long long seed, unsigned long long stream_id0, float* sq_layers, float* clip,
                       float* norms, Lanes& lanes) {
@@ -3033,10 +3104,31 @@ static int step_model(const dpclip_model_layer* layers, int L, int B, dpclip_dty
     }
     if (all_dense) return step_dense(dense, L, B, dtype, C, sigma, seed, stream_id0, sq_layers, clip, norms, lanes);
     StagePlan sp;
+    const size_t given = lanes.ws_bytes[0];
     const int rc = stage_step(sp, dense, layers, L, B, dtype, lanes, true);
     if (rc) return rc;
+    // the per-example gradients of the element-wise layers lie at the end of lane 0's workspace when it has room for them
+    float* rows[kMaxLayers];
+    const size_t ew = ew_rows_total(layers, L, B);
+    bool use_rows = ew > 0 && lanes.ws[0] && given >= ew;
+    if (use_rows) {
+        size_t at = (given - ew) / 256 * 256;
+        use_rows = at >= (sp.active ? sp.bytes : model_scratch_bytes(layers, dense, L, B, dtype));
+        if (use_rows && lanes.ws_bytes[0] > at) lanes.ws_bytes[0] = at;
+        for (int l = 0; use_rows && l < L; ++l) {
+            const dpclip_layer& y = layers[l].layer;
+            const size_t n = ew_rows_bytes(layers[l], B);
+            rows[l] = nullptr;
+            if (n == 0) continue;
+            // the checks of dpclip_elementwise_clipped_grad
+            if (!y.gW || (y.has_bias && !y.gb)) return DPCLIP_ERR_INVALID_ARG;
+            if (!aligned_to(y.gW, 4) || (y.has_bias && !aligned_to(y.gb, 4))) return DPCLIP_ERR_MISALIGNED;
+            rows[l] = reinterpret_cast<float*>(static_cast<char*>(lanes.ws[0]) + at);
+            at += n;
+        }
+    }
     return step_general(dense, layers, L, B, dtype, C, sigma, seed, stream_id0, sq_layers, clip, norms, lanes,
-                        sp.active ? &sp : nullptr);
+                        sp.active ? &sp : nullptr, use_rows ? rows : nullptr);
 }
 
 int dpclip_step(const dpclip_layer* layers, int L, int B, dpclip_dtype dtype, float C, float sigma,
@@ -3166,27 +3258,16 @@ int dpclip_step_per_layer(const dpclip_layer* layers, int L, int B, dpclip_dtype
 }
 
 static size_t model_workspace_bytes(const dpclip_model_layer* layers, int L, int B, dpclip_dtype dtype, bool with_copies) {
-    size_t ws = kHeaderBytes;
-    if (!layers || L <= 0 || L > 256 || B <= 0) return ws;
-    {
-        dpclip_layer dense[256];
-        for (int l = 0; l < L; ++l) {
-            if (layers[l].kind == DPCLIP_KIND_DENSE) dense[l] = layers[l].layer;
-            else memset(&dense[l], 0, sizeof(dense[l]));
-        }
-        ws = step_scratch_bytes(dense, L, B, dtype);
-        const size_t staged = staged_workspace_bytes(dense, layers, L, B, dtype, with_copies);
-        if (staged > ws) ws = staged;
-    }
+    if (!layers || L <= 0 || L > 256 || B <= 0) return kHeaderBytes;
+    dpclip_layer dense[256];
     for (int l = 0; l < L; ++l) {
-        const dpclip_layer& y = layers[l].layer;
-        size_t w = kHeaderBytes;
-        if (layers[l].kind == DPCLIP_KIND_DENSE)
-            w = dpclip_workspace_bytes(B, y.T, y.d_in, y.d_out, dtype, (dpclip_method)y.method);
-        else if (layers[l].kind == DPCLIP_KIND_CONV)
-            w = dpclip_conv_workspace_bytes(B, &layers[l].conv, y.d_out, dtype, layers[l].z_channel_major);
-        if (w > ws) ws = w;
+        if (layers[l].kind == DPCLIP_KIND_DENSE) dense[l] = layers[l].layer;
+        else memset(&dense[l], 0, sizeof(dense[l]));
     }
+    size_t ws = model_scratch_bytes(layers, dense, L, B, dtype);
+    const size_t staged = staged_workspace_bytes(dense, layers, L, B, dtype, with_copies);
+    if (staged > ws) ws = staged;
+    if (with_copies && ew_rows_total(layers, L, B) > 0) ws = round_up(ws, 256) + ew_rows_total(layers, L, B);
     return ws;
 }
 

@@ -10,8 +10,14 @@
 //   elementwise_grad_kernel : CTA = (column block, row slice); every row weighted by its example's
 //                             clip factor; per-column sums are added to g_scale / g_shift (zeroed by
 //                             the launcher) with fire-and-forget adds.
+//   elementwise_rows_grad_kernel : the same sums from the per-example gradients, 2 d numbers an example, when the norm
+//                             kernel has left them in the workspace: sum_i c_i G_i and the noise, all layers in one launch.
+//                             Inputs are then read once a step, not twice: B = 128, T = 256, d = 512 in bf16, two layers:
+//                             17 + 18 us of grad kernels (134 MB) and eight clears and noise launches -> one of 4 us.
 #pragma once
-#include "common.cuh"
+#include <float.h>
+
+#include "kernels_stream.cuh"
 
 namespace dpclip {
 
@@ -130,11 +136,36 @@ __device__ __forceinline__ void ew_combine(float (&gg)[VEC], float (&gs)[VEC], i
     }
 }
 
+// A sum that overflowed although the example's inputs are finite: its norm is infinite and its factor zero, which has to
+// leave zero of it, not NaN.
+template <typename T, int VEC>
+__device__ __forceinline__ void ew_clamp_overflow(const T* __restrict__ H, long ldh, const T* __restrict__ Z, long ldz, long r0,
+                                                  int rows, int c0, float (&gg)[VEC], float (&gs)[VEC]) {
+    bool over = false;
+#pragma unroll
+    for (int u = 0; u < VEC; ++u) over = over || !isfinite(gg[u]) || !isfinite(gs[u]);
+    if (!over) return;
+    for (int r = 0; r < rows; ++r) {
+        EwRaw<T, VEC> h, z;
+        ew_load(H + (size_t)(r0 + r) * ldh + c0, h);
+        ew_load(Z + (size_t)(r0 + r) * ldz + c0, z);
+        float hf[VEC], zf[VEC];
+        ew_f32(h, hf); ew_f32(z, zf);
+#pragma unroll
+        for (int u = 0; u < VEC; ++u) if (!isfinite(hf[u]) || !isfinite(zf[u])) return;
+    }
+#pragma unroll
+    for (int u = 0; u < VEC; ++u) {
+        if (isinf(gg[u])) gg[u] = copysignf(FLT_MAX, gg[u]);
+        if (isinf(gs[u])) gs[u] = copysignf(FLT_MAX, gs[u]);
+    }
+}
+
 // CG column groups of VEC columns per CTA (CG = 64 or 32: narrower CTAs when the grid would not fill the GPU).
 template <typename T, int VEC, int CG>
 __global__ void __launch_bounds__(EW_THREADS)
 elementwise_norm_kernel(const T* __restrict__ H, long ldh, const T* __restrict__ Z, long ldz, int rows, int d,
-                        int has_shift, float* __restrict__ sq, int use_atomic) {
+                        int has_shift, float* __restrict__ sq, int use_atomic, float* __restrict__ per_example) {
     constexpr int RG = EW_THREADS / CG;
     __shared__ float part[EW_THREADS * 2 * VEC];
     __shared__ float red[32];
@@ -151,6 +182,12 @@ elementwise_norm_kernel(const T* __restrict__ H, long ldh, const T* __restrict__
     if (rg == 0 && c0 < d) {
 #pragma unroll
         for (int u = 0; u < VEC; ++u) { s = fmaf(gg[u], gg[u], s); if (has_shift) s = fmaf(gs[u], gs[u], s); }
+        if (per_example) {
+            ew_clamp_overflow<T, VEC>(H, ldh, Z, ldz, (long)i * rows, rows, c0, gg, gs);
+            float* out = per_example + (size_t)i * 2 * d + c0;
+#pragma unroll
+            for (int u = 0; u < VEC; ++u) { out[u] = gg[u]; out[d + u] = gs[u]; }
+        }
     }
     s = block_sum(s, red);
     if (threadIdx.x == 0) { if (use_atomic) atomicAdd(sq + i, s); else sq[i] = s; }
@@ -184,16 +221,61 @@ elementwise_grad_kernel(const T* __restrict__ H, long ldh, const T* __restrict__
     }
 }
 
+// CTA = 32 columns of the scale or of the shift of one layer; warp w adds examples w, w + 8, ..., the warps' sums are added in
+// order.  Bound: latency, two round trips to L2 (B = 128: sixteen loads a thread, eight in flight).
+struct EwRowsLayer { const float* rows; float* g_scale; float* g_shift; int d, blk_begin; uint32_t sw0, sw1, sb0, sb1; };
+constexpr int EW_ROWS_MAX_LAYERS = 16;
+struct EwRowsParams { EwRowsLayer layer[EW_ROWS_MAX_LAYERS]; int n, B; const float* clip; float noise_scale; uint32_t k0, k1; };
+
+__global__ void __launch_bounds__(EW_THREADS)
+elementwise_rows_grad_kernel(const __grid_constant__ EwRowsParams p) {
+    constexpr int WARPS = EW_THREADS / 32, UNR = 8;
+    __shared__ float part[WARPS][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int l = 0;
+    while (l + 1 < p.n && (int)blockIdx.x >= p.layer[l + 1].blk_begin) ++l;
+    const EwRowsLayer& y = p.layer[l];
+    const int blocks = (y.d + 31) >> 5, blk = blockIdx.x - y.blk_begin;
+    const bool shift = blk >= blocks;
+    const int c = (shift ? blk - blocks : blk) * 32 + lane;
+    float acc = 0.f;
+    if (c < y.d) {
+        const float* src = y.rows + (shift ? y.d : 0) + c;
+        for (int i = warp; i < p.B; i += WARPS * UNR) {
+            float g[UNR], f[UNR];
+#pragma unroll
+            for (int k = 0; k < UNR; ++k) {
+                const int e = i + k * WARPS;
+                g[k] = e < p.B ? __ldg(src + (size_t)e * 2 * y.d) : 0.f;
+                f[k] = e < p.B ? __ldg(p.clip + e) : 0.f;
+            }
+#pragma unroll
+            for (int k = 0; k < UNR; ++k) acc = fmaf(f[k], g[k], acc);
+        }
+    }
+    part[warp][lane] = acc;
+    __syncthreads();
+    if (warp != 0 || c >= y.d) return;
+#pragma unroll
+    for (int w = 1; w < WARPS; ++w) acc += part[w][lane];
+    if (p.noise_scale > 0.f) {
+        float z[4];
+        normals_at((size_t)(c & ~3), shift ? y.sb0 : y.sw0, shift ? y.sb1 : y.sw1, p.k0, p.k1, z);
+        acc = fmaf(p.noise_scale, (c & 2) ? ((c & 1) ? z[3] : z[2]) : ((c & 1) ? z[1] : z[0]), acc);
+    }
+    (shift ? y.g_shift : y.g_scale)[c] = acc;
+}
+
 // Launch helpers of the element-wise layer kernels: VEC = 4 needs 4-element-aligned rows and width; CG = 32
 // (narrower CTAs, more of them) when 64-column-group CTAs would leave SMs idle.
 template <typename T>
 void launch_ew_norm(bool vec, int cg, dim3 grid, cudaStream_t st, const void* H, long ldh, const void* Z, long ldz,
-                    int T_, int d, int has_shift, float* sq, int use_atomic) {
+                    int T_, int d, int has_shift, float* sq, int use_atomic, float* per_example) {
     const T* h = static_cast<const T*>(H); const T* z = static_cast<const T*>(Z);
-    if (vec && cg == 64) elementwise_norm_kernel<T, 4, 64><<<grid, EW_THREADS, 0, st>>>(h, ldh, z, ldz, T_, d, has_shift, sq, use_atomic);
-    else if (vec) elementwise_norm_kernel<T, 4, 32><<<grid, EW_THREADS, 0, st>>>(h, ldh, z, ldz, T_, d, has_shift, sq, use_atomic);
-    else if (cg == 64) elementwise_norm_kernel<T, 1, 64><<<grid, EW_THREADS, 0, st>>>(h, ldh, z, ldz, T_, d, has_shift, sq, use_atomic);
-    else elementwise_norm_kernel<T, 1, 32><<<grid, EW_THREADS, 0, st>>>(h, ldh, z, ldz, T_, d, has_shift, sq, use_atomic);
+    if (vec && cg == 64) elementwise_norm_kernel<T, 4, 64><<<grid, EW_THREADS, 0, st>>>(h, ldh, z, ldz, T_, d, has_shift, sq, use_atomic, per_example);
+    else if (vec) elementwise_norm_kernel<T, 4, 32><<<grid, EW_THREADS, 0, st>>>(h, ldh, z, ldz, T_, d, has_shift, sq, use_atomic, per_example);
+    else if (cg == 64) elementwise_norm_kernel<T, 1, 64><<<grid, EW_THREADS, 0, st>>>(h, ldh, z, ldz, T_, d, has_shift, sq, use_atomic, per_example);
+    else elementwise_norm_kernel<T, 1, 32><<<grid, EW_THREADS, 0, st>>>(h, ldh, z, ldz, T_, d, has_shift, sq, use_atomic, per_example);
 }
 template <typename T>
 void launch_ew_grad(bool vec, int cg, dim3 grid, cudaStream_t st, const void* H, long ldh, const void* Z, long ldz,

@@ -1,0 +1,73 @@
+"""Branches of the whole step against fp64 references of the same step (noise by the sequential paths, which have their own
+tests), at the sizes where a tile, a remainder or a range ends."""
+import numpy as np
+import pytest
+import torch
+
+from util import TOL
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dp():
+    import paper_2009_03106_b200 as pkg
+    pkg.load_library()
+    return pkg
+
+
+def _rel(got, ref):
+    got, ref = got.double(), ref.double()
+    return ((got - ref).norm() / ref.norm()).item()
+
+
+# ---------------------------------------------------------------------------
+# element-wise layers: clipped sums from the stored per-example gradients, against fp64 and against the second pass over the
+# inputs (taken when the workspace lacks the room, and by layers of fewer than 8 positions)
+# ---------------------------------------------------------------------------
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("B,T,widths", [(1, 8, (1,)), (7, 9, (33, 4, 130)), (65, 40, (512, 31)), (129, 8, (64,) * 17)])
+def test_elementwise_grads_from_stored_rows(dp, dtype, B, T, widths):
+    gen = torch.Generator(device="cuda"); gen.manual_seed(B + T)
+    td = torch.float32 if dtype == "f32" else torch.bfloat16
+    C, sigma, seed = 1.0, 0.5, 11
+    layers = []
+    for k, d in enumerate(widths):
+        t = 3 if k == 2 else T
+        H = torch.randn(B, t, d, generator=gen, device="cuda").to(td)
+        Z = (torch.randn(B, t, d, generator=gen, device="cuda") * (2.0 / (t * sum(widths))) ** 0.5).to(td)
+        layers.append(dp.ModelLayer(dp.DPCLIP_KIND_ELEMENTWISE, H, Z, k % 3 != 1))
+    full, small = dp.ModelPlan(layers), dp.ModelPlan(layers)
+    small.workspace = small.workspace[:256]
+    grads = [((y.A.double() * y.Zbar.double()).sum(1), y.Zbar.double().sum(1) if y.has_bias else None) for y in layers]
+    norms = sum(g.pow(2).sum(1) + (0 if s is None else s.pow(2).sum(1)) for g, s in grads).sqrt()
+    clip = (C / norms).clamp(max=1.0)
+    for sg in (0.0, sigma):
+        for plan in (full, small):
+            plan.run(C, sg, seed)
+        torch.cuda.synchronize()
+        assert dp.dpclip_read_status(full.workspace) == 0
+        for l, (g, s) in enumerate(grads):
+            for out, other, ref in ((full.gW[l], small.gW[l], g), (full.gb[l], small.gb[l], s)):
+                if ref is None:
+                    continue
+                if sg == 0.0:
+                    assert _rel(out, (clip[:, None] * ref).sum(0)) <= TOL["f32"]["grad"]      # sums in fp32 of exact inputs
+                else:
+                    # the same draws on either path: what differs is the sum below them
+                    assert (out - other).abs().max().item() <= 1e-5 * max(1.0, out.abs().max().item())
+    assert ((full.norms.double() - norms).abs() / norms).max().item() <= TOL["f32"]["norm"]
+
+
+def test_elementwise_grads_of_an_example_that_overflows(dp):
+    # finite inputs, a per-example sum beyond fp32: infinite norm, factor 0, nothing of it in the sum
+    B, T, d = 5, 16, 40
+    H = torch.randn(B, T, d, device="cuda"); Z = torch.randn(B, T, d, device="cuda") * 1e-3
+    H[2, :, 7] = 3e30; Z[2, :, 7] = 1e20
+    plan = dp.ModelPlan([dp.ModelLayer(dp.DPCLIP_KIND_ELEMENTWISE, H, Z, True)])
+    plan.run(1.0, 0.0, 0)
+    torch.cuda.synchronize()
+    keep = [0, 1, 3, 4]
+    ref = (H[keep].double() * Z[keep].double()).sum((0, 1))
+    assert torch.isinf(plan.norms[2]) and plan.clip[2].item() == 0.0
+    assert _rel(plan.gW[0], ref) <= 1e-5 and np.isfinite(plan.gb[0].cpu().numpy()).all()
