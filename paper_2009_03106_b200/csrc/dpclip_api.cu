@@ -103,6 +103,18 @@ struct SmBudgetScope {
     ~SmBudgetScope() { t_sm_budget = prev; }
 };
 
+// Set while a step runs its norm stage with all rows of sq already at zero: launches that add their norms up with atomics then
+// leave out their own clear.
+thread_local bool t_sq_cleared = false;
+struct SqClearedScope {
+    bool prev;
+    explicit SqClearedScope(bool on) : prev(t_sq_cleared) { t_sq_cleared = on; }
+    ~SqClearedScope() { t_sq_cleared = prev; }
+};
+inline bool clear_sq(float* sq, size_t n, cudaStream_t st) {
+    return t_sq_cleared || cudaMemsetAsync(sq, 0, sizeof(float) * n, st) == cudaSuccess;
+}
+
 // DPCLIP_LOG=1: one line on stderr per dispatch decision (which form of a kernel a layer takes and how its
 // work is cut) -- host side only, nothing changes on the device.
 #define DPCLIP_LOGF(...) do { if (path_switch(SW_LOG)) { fprintf(stderr, "[dpclip] " __VA_ARGS__); fputc('\n', stderr); } } while (0)
@@ -202,7 +214,7 @@ int launch_narrow_tc(const NarrowParams& p, int grid, int n_items, int* status, 
     q.n_items = n_items; q.rows_total = p.rows_total; q.rows_per_cta = p.rows_per_cta;
     q.clip = p.clip; q.sq = p.sq; q.part = p.part; q.part_m = p.d_out <= 32 ? 32 : 64;
     q.status = status;
-    if (!GRAD && p.d_out > 32 && cudaMemsetAsync(p.sq, 0, sizeof(float) * (size_t)n_items, st) != cudaSuccess)
+    if (!GRAD && p.d_out > 32 && !clear_sq(p.sq, (size_t)n_items, st))
         return DPCLIP_ERR_CUDA;
     if (cudaFuncSetAttribute(tc::narrow_tc_kernel<GRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, n::SMEM_BYTES) !=
         cudaSuccess) return DPCLIP_ERR_CUDA;
@@ -243,7 +255,7 @@ int launch_narrow_pack(const NarrowParams& p, int grid, int n_items, dpclip_dtyp
     q.A = p.A; q.Z = p.Z; q.T = p.T; q.d_in = p.d_in; q.d_out = p.d_out; q.has_bias = p.has_bias;
     q.n_items = n_items; q.rows_total = p.rows_total; q.rows_per_cta = p.rows_per_cta;
     q.clip = p.clip; q.sq = p.sq; q.part = p.part; q.status = status;
-    if (!GRAD && cudaMemsetAsync(p.sq, 0, sizeof(float) * (size_t)n_items, st) != cudaSuccess) return DPCLIP_ERR_CUDA;
+    if (!GRAD && !clear_sq(p.sq, (size_t)n_items, st)) return DPCLIP_ERR_CUDA;
     return dtype == DPCLIP_F32 ? launch_narrow_pack_inst<float, GRAD>(q, grid, st)
                                : launch_narrow_pack_inst<__nv_bfloat16, GRAD>(q, grid, st);
 }
@@ -283,7 +295,7 @@ int launch_simt_norms(const void* A, long lda, const void* Z, long ldz, int B, i
     if (split < 1) split = 1;
     p.sq = sq;
     p.use_atomic = split > 1;
-    if (p.use_atomic && cudaMemsetAsync(sq, 0, sizeof(float) * (size_t)B, st) != cudaSuccess)
+    if (p.use_atomic && !clear_sq(sq, (size_t)B, st))
         return DPCLIP_ERR_CUDA;
     dim3 grid(split, B);
     if (dtype == DPCLIP_F32) zta_simt_kernel<float, false><<<grid, SIMT_THREADS, 0, st>>>(p);
@@ -574,7 +586,7 @@ int launch_gram_group(const GramLayer* ls, int n, int cls, int* status, cudaStre
             float* end = begin + ls[by_ptr[i]].B;
             int j = i + 1;
             while (j < n && ls[by_ptr[j]].sq == end) { end += ls[by_ptr[j]].B; ++j; }
-            if (cudaMemsetAsync(begin, 0, sizeof(float) * (size_t)(end - begin), st) != cudaSuccess) return DPCLIP_ERR_CUDA;
+            if (!clear_sq(begin, (size_t)(end - begin), st)) return DPCLIP_ERR_CUDA;
             i = j;
         }
     }
@@ -700,7 +712,7 @@ int launch_zta_tc_mt(const tc::zta::Maps& maps, tc::zta::Params p, int B, bool n
     int ksplit = 1;
     if (norm_mode) {
         p.n_items = B * tiles;
-        if (cudaMemsetAsync(sq, 0, sizeof(float) * (size_t)B, st) != cudaSuccess) return DPCLIP_ERR_CUDA;
+        if (!clear_sq(sq, (size_t)B, st)) return DPCLIP_ERR_CUDA;
     } else {
         const int nkb = ceil_div(R, z::Cfg<MT>::BK);
         // One wave of equally long items: the kernel is bound by L2->SM traffic, so what matters is that
@@ -1064,7 +1076,7 @@ int launch_zta_tf32(const void* A, long lda, const void* Z, long ldz, int B, int
         p.do_bias = has_bias ? 1 : 0;
         p.sq = sq;
         p.n_items = B * tiles;
-        if (cudaMemsetAsync(sq, 0, sizeof(float) * (size_t)B, st) != cudaSuccess) return DPCLIP_ERR_CUDA;
+        if (!clear_sq(sq, (size_t)B, st)) return DPCLIP_ERR_CUDA;
     } else {
         p.clip = clip; p.gW = gW; p.ldg = ldg; p.gb = gb;
         p.do_bias = gb ? 1 : 0;
@@ -1175,7 +1187,7 @@ inline int clear_rows(float* const* rows, int n, int B, cudaStream_t st) {
         float* end = begin + B;
         int j = i + 1;
         while (j < n && rows[order[j]] == end) { end += B; ++j; }
-        if (cudaMemsetAsync(begin, 0, sizeof(float) * (size_t)(end - begin), st) != cudaSuccess) return DPCLIP_ERR_CUDA;
+        if (!clear_sq(begin, (size_t)(end - begin), st)) return DPCLIP_ERR_CUDA;
         i = j;
     }
     return DPCLIP_OK;
@@ -2086,7 +2098,7 @@ static int launch_conv_tc(const SimtParams& sp, const void* X, const void* Zbar,
         p.ex_per_item = 1;
         p.n_items = B * p.tiles_n;
         p.sq = sq;
-        if (cudaMemsetAsync(sq, 0, sizeof(float) * (size_t)B, st) != cudaSuccess) return DPCLIP_ERR_CUDA;
+        if (!clear_sq(sq, (size_t)B, st)) return DPCLIP_ERR_CUDA;
     }
     if (!enable_smem(tc::conv_tc_kernel<GRAD>, c::SMEM_BYTES)) return DPCLIP_ERR_CUDA;
     const int grid = p.n_items < sm_budget() ? p.n_items : sm_budget();
@@ -2213,7 +2225,7 @@ int dpclip_conv_sqnorms(const void* X, const void* Zbar, int z_channel_major, in
     if (split < 1) split = 1;
     p.sq = sq_layer;
     p.use_atomic = split > 1;
-    if (p.use_atomic && cudaMemsetAsync(sq_layer, 0, sizeof(float) * (size_t)B, st) != cudaSuccess) return DPCLIP_ERR_CUDA;
+    if (p.use_atomic && !clear_sq(sq_layer, (size_t)B, st)) return DPCLIP_ERR_CUDA;
     dim3 grid(split, B);
     if (dtype == DPCLIP_F32) zta_simt_kernel<float, false, true><<<grid, SIMT_THREADS, 0, st>>>(p);
     else zta_simt_kernel<__nv_bfloat16, false, true><<<grid, SIMT_THREADS, 0, st>>>(p);
@@ -2362,7 +2374,7 @@ static int elementwise_sqnorms(const void* Hbar, long ldh, const void* Zbar, lon
     const int cg = (long)ceil_div(d, 64 * v) * B >= 4L * kNumSMs ? 64 : 32;
     const dim3 grid(ceil_div(d, cg * v), B);
     const int use_atomic = grid.x > 1;
-    if (use_atomic && cudaMemsetAsync(sq_layer, 0, sizeof(float) * (size_t)B, st) != cudaSuccess) return DPCLIP_ERR_CUDA;
+    if (use_atomic && !clear_sq(sq_layer, (size_t)B, st)) return DPCLIP_ERR_CUDA;
     if (dtype == DPCLIP_F32) launch_ew_norm<float>(vec, cg, grid, st, Hbar, ldh, Zbar, ldz, T, d, has_shift, sq_layer, use_atomic, per_example);
     else launch_ew_norm<__nv_bfloat16>(vec, cg, grid, st, Hbar, ldh, Zbar, ldz, T, d, has_shift, sq_layer, use_atomic, per_example);
     return launch_status();
@@ -2698,11 +2710,13 @@ static size_t staged_workspace_bytes(const dpclip_layer* layers, const dpclip_mo
     return with_copies ? sp.bytes : sp.scratch;
 }
 
-static int launch_stage(StagePlan& sp, cudaStream_t st) {
+// sq [n_sq]: cleared by the way
+static int launch_stage(StagePlan& sp, float* sq, size_t n_sq, cudaStream_t st) {
     for (int i0 = 0; i0 < sp.n_jobs; i0 += stage::MAX_JOBS) {
         stage::Launch q;
         memset(&q, 0, sizeof(q));
         q.n = sp.n_jobs - i0 < stage::MAX_JOBS ? sp.n_jobs - i0 : stage::MAX_JOBS;
+        if (i0 == 0) { q.clear = sq; q.n_clear = n_sq; }
         for (int i = 0; i < q.n; ++i) {
             stage::Job& j = q.job[i] = sp.job[i0 + i];
             j.blk_begin = q.blocks;
@@ -2856,6 +2870,15 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
         for (int l = 0; l < L; ++l) if (layers_in[l].T == 1) sp->eff[l] = layers_in[l];
         t1_dtype = dtype;
     }
+    // The rows of sq that launches add up with atomics: cleared by the staging launch, else on several streams all at once in
+    // front of the fork.
+    bool cleared = sp != nullptr;
+    if (!cleared && lanes.n > 1) {
+        const size_t n = (size_t)L * B;
+        clear_kernel<<<(unsigned)(n < 256 * 64 ? (n + 255) / 256 : 64), 256, 0, lanes.st[0]>>>(sq_layers, n);
+        if (launch_status()) return DPCLIP_ERR_CUDA;
+        cleared = true;
+    }
     if ((rc = lanes.fork())) return rc;
     if (t1.active) {
         if (t1_dtype == DPCLIP_F32) t1_all_norms_kernel<float><<<t1.p.L * B, 128, 0, lanes.st[last]>>>(t1.p);
@@ -2866,6 +2889,7 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
     const bool track = L <= 64;
     bool any_gram = false, any_mat = false;
     bool factors_done = false;
+    SqClearedScope cleared_scope(cleared);
     if (track) {
         // when one Gram launch takes every layer of the model, its last CTA also computes the factors
         const tc::gram::FactorsTail tail = {sq_layers, L, (long)B, B, C, clip, norms, nullptr};
@@ -3054,18 +3078,18 @@ static int step_args_ok(const void* layers, int L, int B, dpclip_dtype dtype, fl
 // Plans and launches the staging of a step when the workspace has room for the copies (sp.active says so); the
 // lanes' scratch then ends where the copies begin.
 static int stage_step(StagePlan& sp, const dpclip_layer* layers, const dpclip_model_layer* other, int L, int B,
-                      dpclip_dtype dtype, Lanes& lanes, bool t1_too) {
+                      dpclip_dtype dtype, float* sq_layers, Lanes& lanes, bool t1_too) {
     if (!lanes.ws[0] || !stage_plan(sp, layers, other, L, B, dtype, static_cast<char*>(lanes.ws[0]), t1_too)) return DPCLIP_OK;
     if (lanes.ws_bytes[0] < sp.bytes) { sp.active = false; return DPCLIP_OK; }
     lanes.ws_bytes[0] = sp.scratch;                            // the copies lie behind lane 0's scratch
-    return launch_stage(sp, lanes.st[0]);
+    return launch_stage(sp, sq_layers, (size_t)L * B, lanes.st[0]);
 }
 
 static int step_dense(const dpclip_layer* layers, int L, int B, dpclip_dtype dtype, float C, float sigma,
                       unsigned long long seed, unsigned long long stream_id0, float* sq_layers, float* clip,
                       float* norms, Lanes& lanes) {
     StagePlan sp;
-    int rc = stage_step(sp, layers, nullptr, L, B, dtype, lanes, true);
+    int rc = stage_step(sp, layers, nullptr, L, B, dtype, sq_layers, lanes, true);
     if (rc) return rc;
     rc = try_fused_t1_step(sp.active ? sp.eff : layers, L, B, sp.active ? sp.t1_dtype : dtype, C, sigma, seed, stream_id0,
                            sq_layers, clip, norms, lanes.ws[0], lanes.ws_bytes[0], lanes.st[0]);
@@ -3105,7 +3129,7 @@ static int step_model(const dpclip_model_layer* layers, int L, int B, dpclip_dty
     if (all_dense) return step_dense(dense, L, B, dtype, C, sigma, seed, stream_id0, sq_layers, clip, norms, lanes);
     StagePlan sp;
     const size_t given = lanes.ws_bytes[0];
-    const int rc = stage_step(sp, dense, layers, L, B, dtype, lanes, true);
+    const int rc = stage_step(sp, dense, layers, L, B, dtype, sq_layers, lanes, true);
     if (rc) return rc;
     // the per-example gradients of the element-wise layers lie at the end of lane 0's workspace when it has room for them
     float* rows[kMaxLayers];
@@ -3196,11 +3220,13 @@ int dpclip_step_per_layer(const dpclip_layer* layers, int L, int B, dpclip_dtype
     {
         Lanes lanes;
         one_lane(lanes, workspace, workspace_bytes, stream);
-        if ((rc = stage_step(sp, layers, nullptr, L, B, dtype, lanes, false))) return rc;
+        if ((rc = stage_step(sp, layers, nullptr, L, B, dtype, sq_layers, lanes, false))) return rc;
         workspace_bytes = lanes.ws_bytes[0];
     }
     const bool* split = sp.active ? sp.split : nullptr;
     if (sp.active) layers = sp.eff;
+    {
+    const SqClearedScope cleared(sp.active);                            // by the staging launch
     if (track) {
         rc = dpclip_gram_layers_sqnorms(layers, L, B, dtype, sq_layers, in_gram, workspace, workspace_bytes, stream);
         if (rc) return rc;
@@ -3215,6 +3241,7 @@ int dpclip_step_per_layer(const dpclip_layer* layers, int L, int B, dpclip_dtype
         rc = dpclip_layer_sqnorms(y.A, y.lda, y.Zbar, y.ldz, B, y.T, y.d_in, y.d_out, dtype, y.has_bias,
                                   (dpclip_method)y.method, sq_layers + (size_t)l * B, workspace, workspace_bytes, stream);
         if (rc) return rc;
+    }
     }
     if (track) {
         LayerThresholds th;

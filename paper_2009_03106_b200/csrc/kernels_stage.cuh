@@ -36,7 +36,7 @@ struct Job {
     int C, H, W, kh, kw, stride, pad, Wo, ct, pitch;     // IM2COL: ct channels per CTA, pitch = shared-memory bytes of a patch row
     int cta_rows;                  // IM2COL: patch rows per CTA
 };
-struct Launch { Job job[MAX_JOBS]; int n, blocks; };
+struct Launch { Job job[MAX_JOBS]; int n, blocks; float* clear; size_t n_clear; };     // clear: fp32 words set to zero by the way
 
 // eight bf16 elements that start at any 2-byte boundary; reads exactly those sixteen bytes
 __device__ __forceinline__ uint4 load_bf16x8(const uint16_t* p) {
@@ -232,6 +232,7 @@ __global__ void __launch_bounds__(stage::THREADS, 6)
 stage_operands_kernel(const __grid_constant__ stage::Launch q) {
     using namespace stage;
     extern __shared__ __align__(16) uint8_t stage_smem[];
+    for (size_t i = (size_t)blockIdx.x * THREADS + threadIdx.x; i < q.n_clear; i += (size_t)gridDim.x * THREADS) q.clear[i] = 0.f;
     int k = 0;
     while (k + 1 < q.n && (int)blockIdx.x >= q.job[k + 1].blk_begin) ++k;
     const Job& j = q.job[k];

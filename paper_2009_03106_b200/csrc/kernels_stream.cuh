@@ -188,6 +188,10 @@ noise_kernel(float* __restrict__ g, size_t n, float scale, uint32_t k0, uint32_t
     }
 }
 
+__global__ void __launch_bounds__(256) clear_kernel(float* __restrict__ p, size_t n) {
+    for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (size_t)gridDim.x * 256) p[i] = 0.f;
+}
+
 // ---------------------------------------------------------------------------
 // Parameter updates with the noise folded in (one pass over the parameters instead of a noise pass
 // followed by an optimiser pass).  g = (gsum + scale * xi) * inv_tau is the noisy mean gradient of
