@@ -19,6 +19,7 @@
 #include "kernels_narrow_pack.cuh"
 #include "kernels_elementwise.cuh"
 #include "kernels_stage.cuh"
+#include "kernels_t1_thin.cuh"
 
 #include <stdio.h>
 #include <stdlib.h>
@@ -316,6 +317,29 @@ void simt_noise(SimtParams& p, const NoiseSpec* noise, bool* noise_done) {
     if (noise_done) *noise_done = true;
 }
 
+// T = 1 layers of at most 16 outputs (kernels_t1_thin.cuh).  Up to 1024 examples, 128 rows a warp: beyond, rows in slices over more
+// CTAs (the tile kernel) take less.
+inline bool t1_thin_ok(int B, int T, int d_out) { return T == 1 && d_out <= THIN_OUT && B <= 1024 && !path_switch(SW_FORCE_SIMT); }
+int launch_t1_thin_grad(const void* A, long lda, const void* Z, long ldz, int B, int d_in, int d_out, dpclip_dtype dtype,
+                        const float* clip, float* gW, long ldg, float* gb, cudaStream_t st, const NoiseSpec* noise, bool* noise_done) {
+    ThinParams p;
+    memset(&p, 0, sizeof(p));
+    p.A = A; p.lda = lda; p.Z = Z; p.ldz = ldz; p.B = B; p.d_in = d_in; p.d_out = d_out;
+    p.pairs_ok = aligned_to(A, 2 * elt_size(dtype)) && lda % 2 == 0;
+    p.clip = clip; p.gW = gW; p.ldg = ldg; p.gb = gb;
+    if (noise && noise->scale > 0.f && ldg == d_in) {
+        p.noise_scale = noise->scale;
+        p.k0 = (uint32_t)noise->seed; p.k1 = (uint32_t)(noise->seed >> 32);
+        p.sw0 = (uint32_t)noise->sid_w; p.sw1 = (uint32_t)(noise->sid_w >> 32);
+        p.sb0 = (uint32_t)noise->sid_b; p.sb1 = (uint32_t)(noise->sid_b >> 32);
+        if (noise_done) *noise_done = true;
+    }
+    const int grid = ceil_div(d_in, (long)THIN_COLS);
+    if (dtype == DPCLIP_F32) t1_thin_grad_kernel<float><<<grid, THIN_THREADS, 0, st>>>(p);
+    else t1_thin_grad_kernel<__nv_bfloat16><<<grid, THIN_THREADS, 0, st>>>(p);
+    return launch_status();
+}
+
 int launch_simt_grad(const void* A, long lda, const void* Z, long ldz, int B, int T, int d_in, int d_out,
                      dpclip_dtype dtype, const float* clip, float* gW, long ldg, float* gb, cudaStream_t st,
                      void* workspace = nullptr, size_t workspace_bytes = 0, const NoiseSpec* noise = nullptr,
@@ -365,6 +389,8 @@ int launch_simt_grad(const void* A, long lda, const void* Z, long ldz, int B, in
         if (gb && cudaMemsetAsync(gb, 0, sizeof(float) * (size_t)d_out, st) != cudaSuccess) return DPCLIP_ERR_CUDA;
         return launch_narrow<true>(q, grid, d_out, dtype, st);
     }
+    if (t1_thin_ok(B, T, d_out))
+        return launch_t1_thin_grad(A, lda, Z, ldz, B, d_in, d_out, dtype, clip, gW, ldg, gb, st, noise, noise_done);
     SimtParams p;
     fill_simt_params(p, A, lda, Z, ldz, T, d_in, d_out, gb != nullptr, dtype);
     const int n_tiles = p.tiles_m * p.tiles_n;
@@ -3004,18 +3030,23 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
     }
     if (track) stage_budgets(in_grad_group, any_group || any_rest, budget);
     k = (any_group ? 1 : 0) + (any_rest ? 1 : 0);
+    // On several streams the small layers of one position go first, on the last one: a few microseconds in front of that stream's
+    // larger layer, where at their place in the order they ended the stage.
+    auto first = [&](int l) { return lanes.n > 1 && !other_kind(l) && t1_thin_ok(B, layers[l].T, layers[l].d_out); };
     if (ew_rows) {
         rc = ew_rows_grads(other, ew_rows, L, B, clip, C, sigma, seed, stream_id0, lanes.st[k % lanes.n]);
         if (rc) return rc;
         ++k;
     }
+    for (int pass = lanes.n > 1 ? 0 : 1; pass < 2; ++pass)
     for (int l = 0; l < L; ++l) {
         const dpclip_layer& y = layers[l];
         const bool is_other = other_kind(l);
         if (!is_other && ((t1.active && y.T == 1) || (track && in_grad_group[l]))) continue;
         if (ew_rows && ew_rows[l]) continue;
+        if (first(l) != (pass == 0)) continue;
         const SmBudgetScope share(track ? budget[l] : 0);
-        const int b = k++ % lanes.n;
+        const int b = pass == 0 ? last : k++ % lanes.n;
         void* const stream = lanes.st[b];
         void* const workspace = lanes.ws[b];
         const size_t workspace_bytes = lanes.ws_bytes[b];

@@ -71,3 +71,32 @@ def test_elementwise_grads_of_an_example_that_overflows(dp):
     ref = (H[keep].double() * Z[keep].double()).sum((0, 1))
     assert torch.isinf(plan.norms[2]) and plan.clip[2].item() == 0.0
     assert _rel(plan.gW[0], ref) <= 1e-5 and np.isfinite(plan.gb[0].cpu().numpy()).all()
+
+
+# ---------------------------------------------------------------------------
+# classifier heads of one position on their own: rows and columns around the kernel's 64, odd rows, noise, 1025 examples (the
+# tile kernel again)
+# ---------------------------------------------------------------------------
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("B,d_in,d_out,lda", [(1, 1, 1, 1), (64, 256, 10, 256), (65, 63, 16, 63), (130, 130, 7, 131), (1024, 65, 2, 66), (1025, 64, 3, 64)])
+def test_heads_of_few_outputs(dp, dtype, B, d_in, d_out, lda):
+    gen = torch.Generator(device="cuda"); gen.manual_seed(B)
+    td = torch.float32 if dtype == "f32" else torch.bfloat16
+    A = torch.randn(B, 1, lda, generator=gen, device="cuda").to(td)[:, :, :d_in]
+    Z = torch.randn(B, 1, d_out, generator=gen, device="cuda").to(td)
+    clip = torch.rand(B, generator=gen, device="cuda")
+    ws = torch.zeros(max(dp.dpclip_workspace_bytes(B, 1, d_in, d_out, 0 if dtype == "f32" else 1), 256), dtype=torch.uint8, device="cuda")
+    gW, gb = torch.full((d_out, d_in), 9.0, device="cuda"), torch.full((d_out,), 9.0, device="cuda")
+    for c in (clip, None):
+        dp.dpclip_clipped_grad(A, Z, c, gW, gb, ws)
+        w = torch.ones(B, device="cuda") if c is None else c
+        zc = w.double()[:, None] * Z[:, 0].double()
+        # bf16 operands that TMA can address take the tensor cores, which round c zb to bf16
+        tol = 1e-2 if dtype == "bf16" and d_in % 8 == 0 and d_out % 8 == 0 else 1e-5
+        assert _rel(gW, zc.T @ A[:, 0].double()) <= tol and _rel(gb, zc.sum(0)) <= tol
+    # with noise: the same sum followed by the same draws
+    dp.dpclip_add_noise(gW, 0.5, 1.0, 3, 4); dp.dpclip_add_noise(gb, 0.5, 1.0, 3, 5)
+    nW, nb = torch.empty_like(gW), torch.empty_like(gb)
+    dp.dpclip_clipped_grad_noise(A, Z, None, nW, nb, 0.5, 1.0, 3, 4, 5, ws)
+    torch.cuda.synchronize()
+    assert (nW - gW).abs().max().item() <= 1e-5 * gW.abs().max().item() and (nb - gb).abs().max().item() <= 1e-5 * gb.abs().max().item()
