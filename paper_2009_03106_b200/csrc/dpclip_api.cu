@@ -2609,21 +2609,38 @@ static bool stage_plan(StagePlan& sp, const dpclip_layer* layers, const dpclip_m
             const bool narrow = dtype == DPCLIP_F32 && narrow_layer(T, p.d_in, p.d_out, 1, p.d_in, p.d_out);
             const long ldp = narrow ? p.d_in : (long)round_up(p.d_in, unit), ldz = narrow ? p.d_out : (long)round_up(p.d_out, unit);
             const int kk = g.kh * g.kw;
-            int ct = (int)(1152 / (kk * es)) / unit * unit;         // about 36 KB of lines per CTA
-            if (ct < unit) ct = unit;
-            if (ct > (int)round_up(g.C, unit)) ct = (int)round_up(g.C, unit);
-            const int pitch = (int)round_up((size_t)ct * kk * es, 16) + 4;
-            int cta_rows = 32;
-            while (cta_rows * 2 <= stage::IM_MAX_ROWS && cta_rows * 2 * pitch <= 40 * 1024) cta_rows *= 2;
-            const int im_bytes = cta_rows * pitch + stage::IM_MAX_ROWS * (int)sizeof(int2);
-            if (im_bytes > stage::SMEM_MAX || (double)B * T * ldp / unit > 4.0e9 || g.kh > 16 || g.kw > 16) continue;
-            if ((double)(cta_rows / T + 2) * g.C * g.H * g.W > 2.0e9) continue;
+            // A CTA: about 144 columns in whole channels whose columns are a multiple of 16 bytes, and 32 to 256 positions, about 18432
+            // elements in all: rows of positions of one example, or whole examples (9216 and 36864 elements, 288 and 576 columns:
+            // up to 15 % slower on the layers of two CNNs).  Odd rows of a narrow layer take one block of all channels.
+            stage::Job im;
+            memset(&im, 0, sizeof(im));
+            const int Ho = T / p.Wo;
+            im.T = T; im.C = g.C; im.H = g.H; im.W = g.W; im.kh = g.kh; im.kw = g.kw; im.stride = g.stride; im.pad = g.pad; im.Wo = p.Wo;
+            im.es = (int)es; im.dst_ld = (int)ldp; im.cols = p.d_in; im.rows = B * T;
+            im.vec = g.W % unit == 0 && aligned_to(y.A, 16);
+            auto cut = [&](int ct, int positions) {
+                im.ct = ct;
+                im.n_ex = positions / T > 1 ? positions / T : 1;
+                if (im.n_ex > B) im.n_ex = B;
+                im.r_out = positions / p.Wo < 1 ? 1 : positions / p.Wo > Ho ? Ho : positions / p.Wo;
+                im.tiles_a = ceil_div(Ho, (long)im.r_out); im.tiles_b = ceil_div(g.C, (long)ct);
+                return stage::im_smem(im);
+            };
+            int ct = ldp % unit ? g.C : 144 / kk / unit * unit;
+            if (ct < unit && ldp % unit == 0) ct = unit;
+            if (ct > g.C) ct = g.C;
+            int positions = 18432 / (ct * kk);
+            positions = positions < 32 ? 32 : positions > 256 ? 256 : positions;
+            size_t im_bytes = cut(ct, positions);
+            while (im_bytes > 48 * 1024 && positions > 32) im_bytes = cut(ct, positions /= 2);
+            while (im_bytes > (size_t)stage::SMEM_MAX && ct > unit && ldp % unit == 0) im_bytes = cut(ct = (int)round_up((size_t)ct / 2, unit), positions);
+            if (im_bytes > (size_t)stage::SMEM_MAX || (double)B * T * ldp / unit > 4.0e9 || g.kh > 16 || g.kw > 16) continue;
+            if ((double)im.n_ex * g.C * g.H * g.W > 2.0e9) continue;
             {
                 stage::Job& j = add_job(l, false, stage::IM2COL, y.A, 0, (int)ldp, B * T, p.d_in, es);
-                j.T = T; j.C = g.C; j.H = g.H; j.W = g.W; j.kh = g.kh; j.kw = g.kw; j.stride = g.stride; j.pad = g.pad;
-                j.Wo = p.Wo; j.ct = ct; j.pitch = pitch; j.tiles_b = ceil_div(g.C, ct);
-                j.cta_rows = cta_rows;
-                if (im_bytes > sp.smem) sp.smem = im_bytes;
+                im.kind = j.kind; im.src = j.src; im.src_ld = 0;
+                j = im;
+                if ((int)im_bytes > sp.smem) sp.smem = (int)im_bytes;
             }
             dpclip_layer& e = sp.eff[l];
             e = y;
@@ -2746,7 +2763,7 @@ static int launch_stage(StagePlan& sp, float* sq, size_t n_sq, cudaStream_t st) 
         for (int i = 0; i < q.n; ++i) {
             stage::Job& j = q.job[i] = sp.job[i0 + i];
             j.blk_begin = q.blocks;
-            if (j.kind == stage::IM2COL) q.blocks += ceil_div(j.rows, j.cta_rows) * j.tiles_b;
+            if (j.kind == stage::IM2COL) q.blocks += ceil_div((long)j.rows / j.T, (long)j.n_ex) * j.tiles_a * j.tiles_b;
             else if (j.kind == stage::TRANSPOSE) q.blocks += j.rows / j.T * j.tiles_a * j.tiles_b;
             else q.blocks += ceil_div((long)j.rows * (j.dst_ld / ((j.es == 4 || j.kind == stage::ROWS_TO_F32) ? 4 : 8)),
                                       (long)stage::ROWS_UNROLL * stage::THREADS);

@@ -8,9 +8,8 @@
 //   im2col     [B][C][H][W] -> [B*T][ld'], columns (c, ky, kx), zeros for the padding: the patch matrix of Sec.
 //              "Convolutional Layers"
 //
-// Bound: latency of the loads and stores (strided CNN from feature maps, 31 us: load/store pipe and shared memory 30 %, DRAM
-// 11 %).  The copies of one step are a few to a few dozen MB and mostly stay in the 126 MB L2 until the two stages have read
-// them.  Columns between the width and ld' need no value: the tensor maps end at the width.
+// The copies of one step are a few to a few dozen MB and mostly stay in the 126 MB L2 until the two stages have read them.
+// Columns between the width and ld' need no value: the tensor maps end at the width.
 #pragma once
 #include "common.cuh"
 
@@ -22,7 +21,6 @@ constexpr int MAX_JOBS = 32;
 constexpr int THREADS = 256;
 constexpr int ROWS_UNROLL = 4;                 // 16-byte output chunks per thread
 constexpr int TILE = 4096;                     // elements of a transpose tile: 64 x 64, or 128 positions x 32 channels
-constexpr int IM_MAX_ROWS = 256;               // im2col: patch rows per CTA, 32 to 256
 constexpr int SMEM_MAX = 160 * 1024;
 
 struct Job {
@@ -33,9 +31,14 @@ struct Job {
     int blk_begin;
     // TRANSPOSE / IM2COL
     int T, tiles_a, tiles_b;       // TRANSPOSE: tiles along T and along M, ct = channels of a tile; IM2COL: channel blocks in tiles_b
-    int C, H, W, kh, kw, stride, pad, Wo, ct, pitch;     // IM2COL: ct channels per CTA, pitch = shared-memory bytes of a patch row
-    int cta_rows;                  // IM2COL: patch rows per CTA
+    int C, H, W, kh, kw, stride, pad, Wo, ct;
+    int n_ex, r_out, vec;          // IM2COL: examples and rows of output positions per CTA (tiles_a of them), ct channels; 16-byte loads
 };
+// Shared memory of an im2col CTA: places of the columns in the window, the window.
+__host__ __device__ inline int im_plane(const Job& j) { return ((j.r_out - 1) * j.stride + j.kh) * (j.W + 2 * j.pad); }
+__host__ __device__ inline int im_table(const Job& j) { return (j.ct * j.kh * j.kw + 15) / 16 * 16; }
+__host__ __device__ inline int im_tile_elems(const Job& j) { return (j.n_ex * j.ct * im_plane(j) + 7) / 8 * 8; }
+inline size_t im_smem(const Job& j) { return (size_t)im_table(j) * 4 + (size_t)im_tile_elems(j) * j.es + 16; }
 struct Launch { Job job[MAX_JOBS]; int n, blocks; float* clear; size_t n_clear; };     // clear: fp32 words set to zero by the way
 
 // eight bf16 elements that start at any 2-byte boundary; reads exactly those sixteen bytes
@@ -138,93 +141,100 @@ __device__ __forceinline__ void transpose_job(const Job& j, int blk, uint8_t* sm
     }
 }
 
-// cta_rows patch rows x ct channels.  Where a row's window lies and which of its rows and columns are inside the map is
-// worked out once per row; then a warp takes (32 rows, channel) at a time -- lane = row, so that neighbouring lanes read
-// neighbouring pixels -- and writes the window to kh*kw consecutive elements of the row's line in shared memory; the lines
-// leave in 16-byte chunks.  Rows are added until a CTA holds about 36 KB: CTAs of 32 rows of a 3-channel image were all
-// latency.
+// A CTA takes ct channels of r_out rows of output positions (of n_ex whole examples when the maps are small).  The input window
+// comes into shared memory once, in 16-byte loads and with zeros around it, so the gather needs no bounds.  A thread then keeps
+// the places of N consecutive columns and walks along a row of positions: a patch element costs one load from shared memory at a
+// constant distance from the one before and an Nth of a store, and neighbouring threads write neighbouring 16 bytes.
+// Bound: issue slots, then latency.  Window elements taken one by one from the map, with masks, through lines of patch rows in
+// shared memory were 16 instructions an element, and so was a window in shared memory with a table look-up an element: 288
+// columns of 32768 positions in fp32 16 us either way, here 13 (2.9 TB/s written).  All copies of a CNN of three layers 41 -> 29
+// us (fp32, 100 MB), of a strided one in bf16 30 -> 24.
+template <typename E, int N, int STRIDE>
+__device__ __forceinline__ void im2col_rows(const Job& j, const E* tile, const int* off, E* dst, int n_rows, int nyo, int width) {
+    const int chunks = (width + N - 1) / N, PW = j.W + 2 * j.pad, plane = im_plane(j);
+    const int stride = STRIDE ? STRIDE : j.stride;
+    for (int i = threadIdx.x; i < n_rows * chunks; i += THREADS) {
+        const int r = i / chunks, k0 = (i - r * chunks) * N;
+        const int e = r / nyo;
+        const E* x = tile + e * j.ct * plane + (r - e * nyo) * j.stride * PW;
+        const E* src[N];
+#pragma unroll
+        for (int k = 0; k < N; ++k) src[k] = x + off[k0 + k];
+        E* out = dst + (size_t)r * j.Wo * j.dst_ld + k0;
+#pragma unroll 4
+        for (int xo = 0; xo < j.Wo; ++xo) {
+            union { E e[N]; uint4 q; } v;
+#pragma unroll
+            for (int k = 0; k < N; ++k) v.e[k] = src[k][xo * stride];
+            if (N == 1) *out = v.e[0];
+            else *reinterpret_cast<uint4*>(out) = v.q;
+            out += j.dst_ld;
+        }
+    }
+}
+
 template <typename E>
 __device__ __forceinline__ void im2col_job(const Job& j, int blk, uint8_t* smem) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int rb = blk / j.tiles_b, cb = blk - rb * j.tiles_b;
-    const int row0 = rb * j.cta_rows, c0 = cb * j.ct;
-    const int kk = j.kh * j.kw, map = j.H * j.W;
-    const int nc = min(j.ct, j.C - c0);
-    int2* info = reinterpret_cast<int2*>(smem);                   // [cta_rows]: offset of the window, row and column masks
-    uint8_t* lines = smem + IM_MAX_ROWS * sizeof(int2);
-    const int b0 = row0 / j.T;
-    for (int r = threadIdx.x; r < j.cta_rows; r += THREADS) {
-        const int row = row0 + r;
-        int2 v = make_int2(0, 0);
-        if (row < j.rows) {
-            const int b = row / j.T, t = row - b * j.T;
-            const int yo = t / j.Wo, xo = t - yo * j.Wo;
-            const int y0 = yo * j.stride - j.pad, x0 = xo * j.stride - j.pad;
-            uint32_t ym = 0, xm = 0;
-            for (int k = 0; k < j.kh; ++k) ym |= (y0 + k >= 0 && y0 + k < j.H) ? 1u << k : 0u;
-            for (int k = 0; k < j.kw; ++k) xm |= (x0 + k >= 0 && x0 + k < j.W) ? 1u << k : 0u;
-            v = make_int2((b - b0) * j.C * map + y0 * j.W + x0, (int)(ym | xm << 16));
-        }
-        info[r] = v;
+    constexpr int VEC = 16 / sizeof(E);
+    const int cb = blk % j.tiles_b, at = blk / j.tiles_b;
+    const int rg = at % j.tiles_a, b0 = at / j.tiles_a * j.n_ex;
+    const int Ho = j.T / j.Wo, B = j.rows / j.T, kk = j.kh * j.kw;
+    const int nb = min(j.n_ex, B - b0), yo0 = rg * j.r_out, nyo = min(j.r_out, Ho - yo0);
+    const int c0 = cb * j.ct, nc = min(j.ct, j.C - c0), width = nc * kk;
+    const int PW = j.W + 2 * j.pad, plane = im_plane(j);
+    int* off = reinterpret_cast<int*>(smem);                               // [ct * kk, rounded up]
+    E* tile = reinterpret_cast<E*>(off + im_table(j));
+    // valid input rows: one contiguous run of a channel
+    const int y_lo = yo0 * j.stride - j.pad, y0 = max(y_lo, 0), y1 = min(y_lo + (nyo - 1) * j.stride + j.kh, j.H);
+    const int ny = max(y1 - y0, 0);
+    const int vec = j.vec ? VEC : 1, wv = j.W / vec, units = nb * nc * ny * wv;
+    {
+        uint4* z = reinterpret_cast<uint4*>(tile);
+        for (int i = threadIdx.x; i < im_tile_elems(j) / VEC; i += THREADS) z[i] = make_uint4(0, 0, 0, 0);
+    }
+    for (int i = threadIdx.x; i < im_table(j); i += THREADS) {
+        const int c = i / kk, k = i - c * kk, ky = k / j.kw;
+        off[i] = i < width ? c * plane + ky * PW + (k - ky * j.kw) : 0;   // columns behind the width need no value
     }
     __syncthreads();
-    const E* src = static_cast<const E*>(j.src) + ((size_t)b0 * j.C + c0) * map;
-    // a window element is a load and a store of its own size, a chain the kernel waits for: of two channels of bf16 windows of
-    // nine the 18 elements leave as nine words (the line of an even channel starts on a word): step of the strided
-    // CNN from feature maps 115.1 -> 113.8 us
-    constexpr int CH = sizeof(E) == 2 ? 2 : 1;
-    const bool nine = j.kh * j.kw == 9 && j.kw == 3;
-    const int groups = nine ? (nc + CH - 1) / CH : nc;
-    const int pairs = (j.cta_rows >> 5) * groups;
-    for (int p = warp; p < pairs; p += THREADS / 32) {
-        const int rg = p / groups, ci = (p - rg * groups) * (nine ? CH : 1);
-        const int r = rg * 32 + lane;
-        const int2 v = info[r];
-        const E* x = src + (ptrdiff_t)ci * map + v.x;
-        E* line = reinterpret_cast<E*>(lines + r * j.pitch) + ci * kk;
-        const uint32_t ym = (uint32_t)v.y & 0xFFFFu, xm = (uint32_t)v.y >> 16;
-        if (nine) {
-            E e[9 * CH];
-            const bool both = ci + CH <= nc;
+    const E* src = static_cast<const E*>(j.src) + ((size_t)b0 * j.C + c0) * j.H * j.W + (size_t)y0 * j.W;
+    constexpr int UNR = 2;
+    for (int u0 = threadIdx.x; u0 < units; u0 += UNR * THREADS) {
+        uint4 v[UNR];
+        int dst[UNR];
 #pragma unroll
-            for (int k = 0; k < 9 * CH; ++k) {
-                const int w = k % 9;
-                e[k] = ((k < 9 || both) && (ym >> (w / 3) & xm >> (w % 3) & 1u)) ? __ldg(x + (k / 9) * map + (w / 3) * j.W + w % 3) : E(0);
-            }
-            if (CH == 2 && both) {
+        for (int k = 0; k < UNR; ++k) {
+            const int u = u0 + k * THREADS;
+            dst[k] = -1;
+            if (u >= units) continue;
+            const int row = u / wv, x = (u - row * wv) * vec;
+            const int ec = row / ny, y = row - ec * ny;
+            const int e = ec / nc, c = ec - e * nc;
+            const E* p = src + ((size_t)(e * j.C + c) * j.H + y) * j.W + x;
+            dst[k] = (e * j.ct + c) * plane + (y0 - y_lo + y) * PW + j.pad + x;
+            if (vec > 1) v[k] = __ldg(reinterpret_cast<const uint4*>(p));
+            else v[k].x = *p;
+        }
 #pragma unroll
-                for (int k = 0; k < 9; ++k) reinterpret_cast<uint32_t*>(line)[k] = (uint32_t)e[2 * k % (9 * CH)] | (uint32_t)e[(2 * k + 1) % (9 * CH)] << 16;
+        for (int k = 0; k < UNR; ++k) {
+            if (dst[k] < 0) continue;
+            if (vec > 1) {
+                union { uint4 q; E e[VEC]; } w;
+                w.q = v[k];
+#pragma unroll
+                for (int i = 0; i < VEC; ++i) tile[dst[k] + i] = w.e[i];
             } else {
-#pragma unroll
-                for (int k = 0; k < 9; ++k) line[k] = e[k];
+                tile[dst[k]] = (E)v[k].x;
             }
-        } else {
-            for (int ky = 0, k = 0; ky < j.kh; ++ky)
-                for (int kx = 0; kx < j.kw; ++kx, ++k) line[k] = (ym >> ky & xm >> kx & 1u) ? __ldg(x + ky * j.W + kx) : E(0);
         }
     }
     __syncthreads();
-    constexpr int PER = 16 / sizeof(E);
-    const int width = nc * kk, rows = min(j.cta_rows, j.rows - row0);
-    E* dst = static_cast<E*>(j.dst) + (size_t)row0 * j.dst_ld + c0 * kk;
-    auto chunk = [&](int r, int c) {
-        const uint32_t* s = reinterpret_cast<const uint32_t*>(lines + r * j.pitch + c * 16);
-        *reinterpret_cast<uint4*>(dst + (size_t)r * j.dst_ld + c * PER) = make_uint4(s[0], s[1], s[2], s[3]);
-    };
-    if ((j.dst_ld % PER) == 0) {
-        const int cpr = (width + PER - 1) / PER;                  // the last chunk may run into the row's padding
-        if (cpr >= 16) {
-            for (int r = warp; r < rows; r += THREADS / 32)
-                for (int c = lane; c < cpr; c += 32) chunk(r, c);
-        } else {
-            for (int k = threadIdx.x; k < rows * cpr; k += THREADS) { const int r = k / cpr; chunk(r, k - r * cpr); }
-        }
-    } else {
-        for (int k = threadIdx.x; k < rows * width; k += THREADS) {
-            const int r = k / width, c = k - r * width;
-            dst[(size_t)r * j.dst_ld + c] = reinterpret_cast<const E*>(lines + r * j.pitch)[c];
-        }
-    }
+    // the CTA's patch rows are consecutive
+    E* dst = static_cast<E*>(j.dst) + ((size_t)b0 * j.T + yo0 * j.Wo) * j.dst_ld + c0 * kk;
+    if (j.dst_ld % VEC != 0) im2col_rows<E, 1, 0>(j, tile, off, dst, nb * nyo, nyo, width);
+    else if (j.stride == 1) im2col_rows<E, VEC, 1>(j, tile, off, dst, nb * nyo, nyo, width);
+    else if (j.stride == 2) im2col_rows<E, VEC, 2>(j, tile, off, dst, nb * nyo, nyo, width);
+    else im2col_rows<E, VEC, 0>(j, tile, off, dst, nb * nyo, nyo, width);
 }
 }  // namespace stage
 

@@ -74,6 +74,38 @@ def test_elementwise_grads_of_an_example_that_overflows(dp):
 
 
 # ---------------------------------------------------------------------------
+# convolutions from feature maps, copied as patch matrices: widths that are no multiple of 16 bytes, several examples per CTA,
+# channel blocks with a remainder, strides, paddings beyond the map, odd rows of narrow layers
+# ---------------------------------------------------------------------------
+@pytest.mark.parametrize("dtype,B,C,size,d_out,k,stride,pad,cm", [
+    ("f32", 9, 40, (8, 8), 160, 3, 1, 1, True), ("f32", 33, 33, (13, 10), 48, 3, 1, 1, True), ("f32", 16, 3, (32, 32), 32, 3, 1, 1, True),
+    ("f32", 24, 3, (33, 31), 30, 3, 1, 1, True), ("f32", 8, 72, (12, 20), 64, 5, 2, 2, False), ("f32", 40, 64, (4, 4), 130, 3, 1, 1, True),
+    ("f32", 4, 48, (56, 56), 16, 1, 2, 0, True), ("bf16", 9, 40, (8, 8), 160, 3, 1, 1, True), ("bf16", 33, 33, (13, 10), 48, 3, 1, 1, True),
+    ("bf16", 16, 64, (16, 16), 128, 3, 2, 1, True), ("bf16", 50, 100, (4, 6), 40, 3, 1, 1, False), ("bf16", 5, 24, (28, 28), 72, 5, 1, 4, True),
+    ("bf16", 3, 20, (56, 40), 200, 3, 3, 0, True), ("bf16", 64, 80, (7, 7), 33, 2, 1, 3, True)])
+def test_convolutions_from_feature_maps(dp, dtype, B, C, size, d_out, k, stride, pad, cm):
+    gen = torch.Generator(device="cuda"); gen.manual_seed(7)
+    td = torch.float32 if dtype == "f32" else torch.bfloat16
+    X = torch.randn(B, C, *size, generator=gen, device="cuda").to(td)
+    T = ((size[0] + 2 * pad - k) // stride + 1) * ((size[1] + 2 * pad - k) // stride + 1)
+    Z = (torch.randn(B, T, d_out, generator=gen, device="cuda") / (T * d_out * C * k * k) ** 0.5).to(td)
+    plan = dp.ModelPlan([dp.ModelLayer(dp.DPCLIP_KIND_CONV, X, Z.transpose(1, 2).contiguous() if cm else Z, True,
+                                       conv=(k, k, stride, pad), z_channel_major=cm)])
+    plan.run(1.0, 0.0, 0)
+    torch.cuda.synchronize()
+    assert dp.dpclip_read_status(plan.workspace) == 0
+    A = torch.nn.functional.unfold(X.double(), k, padding=pad, stride=stride).transpose(1, 2)
+    G = torch.einsum("bto,bti->boi", Z.double(), A)
+    gb = Z.double().sum(1)
+    norms = (G.pow(2).sum((1, 2)) + gb.pow(2).sum(1)).sqrt()
+    clip = (1.0 / norms).clamp(max=1.0)
+    tol = TOL[dtype]
+    assert ((plan.norms.double() - norms).abs() / norms).max().item() <= tol["norm"]
+    assert _rel(plan.gW[0], (clip[:, None, None] * G).sum(0)) <= tol["grad"]
+    assert _rel(plan.gb[0], (clip[:, None] * gb).sum(0)) <= tol["grad"]
+
+
+# ---------------------------------------------------------------------------
 # classifier heads of one position on their own: rows and columns around the kernel's 64, odd rows, noise, 1025 examples (the
 # tile kernel again)
 # ---------------------------------------------------------------------------
