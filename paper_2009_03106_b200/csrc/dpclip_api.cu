@@ -2617,13 +2617,13 @@ static bool stage_plan(StagePlan& sp, const dpclip_layer* layers, const dpclip_m
             const int Ho = T / p.Wo;
             im.T = T; im.C = g.C; im.H = g.H; im.W = g.W; im.kh = g.kh; im.kw = g.kw; im.stride = g.stride; im.pad = g.pad; im.Wo = p.Wo;
             im.es = (int)es; im.dst_ld = (int)ldp; im.cols = p.d_in; im.rows = B * T;
-            im.vec = g.W % unit == 0 && aligned_to(y.A, 16);
             auto cut = [&](int ct, int positions) {
                 im.ct = ct;
                 im.n_ex = positions / T > 1 ? positions / T : 1;
                 if (im.n_ex > B) im.n_ex = B;
                 im.r_out = positions / p.Wo < 1 ? 1 : positions / p.Wo > Ho ? Ho : positions / p.Wo;
                 im.tiles_a = ceil_div(Ho, (long)im.r_out); im.tiles_b = ceil_div(g.C, (long)ct);
+                stage::im_pitches(im);
                 return stage::im_smem(im);
             };
             int ct = ldp % unit ? g.C : 144 / kk / unit * unit;
@@ -2632,10 +2632,14 @@ static bool stage_plan(StagePlan& sp, const dpclip_layer* layers, const dpclip_m
             int positions = 18432 / (ct * kk);
             positions = positions < 32 ? 32 : positions > 256 ? 256 : positions;
             size_t im_bytes = cut(ct, positions);
-            while (im_bytes > 48 * 1024 && positions > 32) im_bytes = cut(ct, positions /= 2);
+            while ((im_bytes > 48 * 1024 || (long)ceil_div(B, (long)im.n_ex) * im.tiles_a * im.tiles_b < kNumSMs) && positions > 32)
+                im_bytes = cut(ct, positions /= 2);
             while (im_bytes > (size_t)stage::SMEM_MAX && ct > unit && ldp % unit == 0) im_bytes = cut(ct = (int)round_up((size_t)ct / 2, unit), positions);
             if (im_bytes > (size_t)stage::SMEM_MAX || (double)B * T * ldp / unit > 4.0e9 || g.kh > 16 || g.kw > 16) continue;
             if ((double)im.n_ex * g.C * g.H * g.W > 2.0e9) continue;
+            // loads start at a channel's first valid row: a multiple of W elements, or the channel's start when a CTA takes it whole
+            for (im.vec = unit; im.vec > 1; im.vec /= 2)
+                if (aligned_to(y.A, im.vec * es) && (g.H * g.W) % im.vec == 0 && (im.tiles_a == 1 || g.W % im.vec == 0)) break;
             {
                 stage::Job& j = add_job(l, false, stage::IM2COL, y.A, 0, (int)ldp, B * T, p.d_in, es);
                 im.kind = j.kind; im.src = j.src; im.src_ld = 0;

@@ -32,12 +32,37 @@ struct Job {
     // TRANSPOSE / IM2COL
     int T, tiles_a, tiles_b;       // TRANSPOSE: tiles along T and along M, ct = channels of a tile; IM2COL: channel blocks in tiles_b
     int C, H, W, kh, kw, stride, pad, Wo, ct;
-    int n_ex, r_out, vec;          // IM2COL: examples and rows of output positions per CTA (tiles_a of them), ct channels; 16-byte loads
+    int n_ex, r_out, vec;          // IM2COL: examples and rows of output positions per CTA (tiles_a of them), ct channels; elements per load
+    int pitch, plane;              // IM2COL: elements of a row and of a channel of the window
 };
 // Shared memory of an im2col CTA: places of the columns in the window, the window.
-__host__ __device__ inline int im_plane(const Job& j) { return ((j.r_out - 1) * j.stride + j.kh) * (j.W + 2 * j.pad); }
 __host__ __device__ inline int im_table(const Job& j) { return (j.ct * j.kh * j.kw + 15) / 16 * 16; }
-__host__ __device__ inline int im_tile_elems(const Job& j) { return (j.n_ex * j.ct * im_plane(j) + 7) / 8 * 8; }
+__host__ __device__ inline int im_tile_elems(const Job& j) { return (j.n_ex * j.ct * j.plane + 7) / 8 * 8; }
+// Row and channel pitch of the window.  A warp reads one element of each of 32 chunks of columns at a time: the channels lie so
+// far apart that these meet as few times as possible on a bank (windows of 16 x 14 pixels in bf16, unpadded: six times; 132 examples
+// of 14 x 14 maps, 32 to 256 channels: 91 us of staging, padded 60).
+inline void im_pitches(Job& j) {
+    const int kk = j.kh * j.kw, width = (j.ct < j.C ? j.ct : j.C) * kk, n = 16 / j.es;
+    j.pitch = j.W + 2 * j.pad;
+    const int plane = ((j.r_out - 1) * j.stride + j.kh) * j.pitch;
+    int best = 1 << 30, pad = 0;
+    for (int b = 0; b < 16 && best > n * (j.es == 4 ? 2 : 1); ++b) {
+        int sum = 0;
+        for (int e = 0; e < n; ++e) {
+            int hits[32] = {0}, word[32], most = 0;
+            for (int l = 0; l < 32 && l * n + e < width; ++l) {
+                const int col = l * n + e, c = col / kk, k = col - c * kk, ky = k / j.kw;
+                const int w = (c * (plane + b) + ky * j.pitch + k - ky * j.kw) * j.es / 4, bank = w & 31;
+                if (hits[bank] > 0 && word[bank] == w) continue;
+                word[bank] = w;
+                if (++hits[bank] > most) most = hits[bank];
+            }
+            sum += most;
+        }
+        if (sum < best) { best = sum; pad = b; }
+    }
+    j.plane = plane + pad;
+}
 inline size_t im_smem(const Job& j) { return (size_t)im_table(j) * 4 + (size_t)im_tile_elems(j) * j.es + 16; }
 struct Launch { Job job[MAX_JOBS]; int n, blocks; float* clear; size_t n_clear; };     // clear: fp32 words set to zero by the way
 
@@ -142,7 +167,7 @@ __device__ __forceinline__ void transpose_job(const Job& j, int blk, uint8_t* sm
 }
 
 // A CTA takes ct channels of r_out rows of output positions (of n_ex whole examples when the maps are small).  The input window
-// comes into shared memory once, in 16-byte loads and with zeros around it, so the gather needs no bounds.  A thread then keeps
+// comes into shared memory once, in loads of up to 16 bytes and with zeros around it, so the gather needs no bounds.  A thread then keeps
 // the places of N consecutive columns and walks along a row of positions: a patch element costs one load from shared memory at a
 // constant distance from the one before and an Nth of a store, and neighbouring threads write neighbouring 16 bytes.
 // Bound: issue slots, then latency.  Window elements taken one by one from the map, with masks, through lines of patch rows in
@@ -150,25 +175,30 @@ __device__ __forceinline__ void transpose_job(const Job& j, int blk, uint8_t* sm
 // columns of 32768 positions in fp32 16 us either way, here 13 (2.9 TB/s written).  All copies of a CNN of three layers 41 -> 29
 // us (fp32, 100 MB), of a strided one in bf16 30 -> 24.
 template <typename E, int N, int STRIDE>
-__device__ __forceinline__ void im2col_rows(const Job& j, const E* tile, const int* off, E* dst, int n_rows, int nyo, int width) {
-    const int chunks = (width + N - 1) / N, PW = j.W + 2 * j.pad, plane = im_plane(j);
-    const int stride = STRIDE ? STRIDE : j.stride;
-    for (int i = threadIdx.x; i < n_rows * chunks; i += THREADS) {
+__device__ __forceinline__ void im2col_rows(const Job& j, const E* tile, const int* off, E* dst, int nb, int nyo, int width) {
+    const int chunks = (width + N - 1) / N, stride = STRIDE ? STRIDE : j.stride;
+    // a thread walks along a whole row of positions, along several of narrow maps
+    const int per = j.Wo >= 16 ? 1 : (16 + j.Wo - 1) / j.Wo, runs = (nyo + per - 1) / per;
+    for (int i = threadIdx.x; i < nb * runs * chunks; i += THREADS) {
         const int r = i / chunks, k0 = (i - r * chunks) * N;
-        const int e = r / nyo;
-        const E* x = tile + e * j.ct * plane + (r - e * nyo) * j.stride * PW;
+        const int e = r / runs, y0 = (r - e * runs) * per, y1 = min(y0 + per, nyo);
+        const E* x = tile + e * j.ct * j.plane + y0 * j.stride * j.pitch;
         const E* src[N];
 #pragma unroll
         for (int k = 0; k < N; ++k) src[k] = x + off[k0 + k];
-        E* out = dst + (size_t)r * j.Wo * j.dst_ld + k0;
+        E* out = dst + (size_t)((e * nyo + y0) * j.Wo) * j.dst_ld + k0;
+        for (int y = y0; y < y1; ++y) {
 #pragma unroll 4
-        for (int xo = 0; xo < j.Wo; ++xo) {
-            union { E e[N]; uint4 q; } v;
+            for (int xo = 0; xo < j.Wo; ++xo) {
+                union { E e[N]; uint4 q; } v;
 #pragma unroll
-            for (int k = 0; k < N; ++k) v.e[k] = src[k][xo * stride];
-            if (N == 1) *out = v.e[0];
-            else *reinterpret_cast<uint4*>(out) = v.q;
-            out += j.dst_ld;
+                for (int k = 0; k < N; ++k) v.e[k] = src[k][xo * stride];
+                if (N == 1) *out = v.e[0];
+                else *reinterpret_cast<uint4*>(out) = v.q;
+                out += j.dst_ld;
+            }
+#pragma unroll
+            for (int k = 0; k < N; ++k) src[k] += j.stride * j.pitch;
         }
     }
 }
@@ -181,13 +211,37 @@ __device__ __forceinline__ void im2col_job(const Job& j, int blk, uint8_t* smem)
     const int Ho = j.T / j.Wo, B = j.rows / j.T, kk = j.kh * j.kw;
     const int nb = min(j.n_ex, B - b0), yo0 = rg * j.r_out, nyo = min(j.r_out, Ho - yo0);
     const int c0 = cb * j.ct, nc = min(j.ct, j.C - c0), width = nc * kk;
-    const int PW = j.W + 2 * j.pad, plane = im_plane(j);
+    const int PW = j.pitch, plane = j.plane;
     int* off = reinterpret_cast<int*>(smem);                               // [ct * kk, rounded up]
     E* tile = reinterpret_cast<E*>(off + im_table(j));
     // valid input rows: one contiguous run of a channel
     const int y_lo = yo0 * j.stride - j.pad, y0 = max(y_lo, 0), y1 = min(y_lo + (nyo - 1) * j.stride + j.kh, j.H);
     const int ny = max(y1 - y0, 0);
-    const int vec = j.vec ? VEC : 1, wv = j.W / vec, units = nb * nc * ny * wv;
+    // loads of a channel's run: they may cross its rows, the last may go beyond them inside the channel
+    const int vec = j.vec, run = (ny * j.W + vec - 1) / vec, units = nb * nc * run;
+    const E* src = static_cast<const E*>(j.src) + ((size_t)b0 * j.C + c0) * j.H * j.W + (size_t)y0 * j.W;
+    constexpr int UNR = 2;
+    union { uint4 q; uint2 d; uint32_t w; E e[VEC]; } v[UNR];
+    int to[UNR], x0[UNR], n[UNR];
+    auto load = [&](int u0) {
+#pragma unroll
+        for (int k = 0; k < UNR; ++k) {
+            const int u = u0 + k * THREADS;
+            to[k] = -1;
+            if (u >= units) continue;
+            const int ec = u / run, at = (u - ec * run) * vec;
+            const int e = ec / nc, c = ec - e * nc, y = at / j.W;
+            const E* p = src + (size_t)(e * j.C + c) * j.H * j.W + at;
+            x0[k] = at - y * j.W;
+            n[k] = min(vec, ny * j.W - at);
+            to[k] = (e * j.ct + c) * plane + (y0 - y_lo + y) * PW + j.pad + x0[k];
+            if (vec == VEC) v[k].q = __ldg(reinterpret_cast<const uint4*>(p));
+            else if (vec * (int)sizeof(E) == 8) v[k].d = __ldg(reinterpret_cast<const uint2*>(p));
+            else if (vec * (int)sizeof(E) == 4) v[k].w = __ldg(reinterpret_cast<const uint32_t*>(p));
+            else v[k].e[0] = *p;
+        }
+    };
+    load(threadIdx.x);                                                     // on their way while the zeros and the table are written
     {
         uint4* z = reinterpret_cast<uint4*>(tile);
         for (int i = threadIdx.x; i < im_tile_elems(j) / VEC; i += THREADS) z[i] = make_uint4(0, 0, 0, 0);
@@ -197,44 +251,28 @@ __device__ __forceinline__ void im2col_job(const Job& j, int blk, uint8_t* smem)
         off[i] = i < width ? c * plane + ky * PW + (k - ky * j.kw) : 0;   // columns behind the width need no value
     }
     __syncthreads();
-    const E* src = static_cast<const E*>(j.src) + ((size_t)b0 * j.C + c0) * j.H * j.W + (size_t)y0 * j.W;
-    constexpr int UNR = 2;
     for (int u0 = threadIdx.x; u0 < units; u0 += UNR * THREADS) {
-        uint4 v[UNR];
-        int dst[UNR];
+        if (u0 != (int)threadIdx.x) load(u0);
 #pragma unroll
         for (int k = 0; k < UNR; ++k) {
-            const int u = u0 + k * THREADS;
-            dst[k] = -1;
-            if (u >= units) continue;
-            const int row = u / wv, x = (u - row * wv) * vec;
-            const int ec = row / ny, y = row - ec * ny;
-            const int e = ec / nc, c = ec - e * nc;
-            const E* p = src + ((size_t)(e * j.C + c) * j.H + y) * j.W + x;
-            dst[k] = (e * j.ct + c) * plane + (y0 - y_lo + y) * PW + j.pad + x;
-            if (vec > 1) v[k] = __ldg(reinterpret_cast<const uint4*>(p));
-            else v[k].x = *p;
-        }
+            if (to[k] < 0) continue;
+            int d = to[k], x = x0[k];
 #pragma unroll
-        for (int k = 0; k < UNR; ++k) {
-            if (dst[k] < 0) continue;
-            if (vec > 1) {
-                union { uint4 q; E e[VEC]; } w;
-                w.q = v[k];
-#pragma unroll
-                for (int i = 0; i < VEC; ++i) tile[dst[k] + i] = w.e[i];
-            } else {
-                tile[dst[k]] = (E)v[k].x;
+            for (int i = 0; i < VEC; ++i) {
+                if (i >= n[k]) break;
+                tile[d] = v[k].e[i];
+                ++d;
+                if (++x == j.W) { x = 0; d += PW - j.W; }
             }
         }
     }
     __syncthreads();
     // the CTA's patch rows are consecutive
     E* dst = static_cast<E*>(j.dst) + ((size_t)b0 * j.T + yo0 * j.Wo) * j.dst_ld + c0 * kk;
-    if (j.dst_ld % VEC != 0) im2col_rows<E, 1, 0>(j, tile, off, dst, nb * nyo, nyo, width);
-    else if (j.stride == 1) im2col_rows<E, VEC, 1>(j, tile, off, dst, nb * nyo, nyo, width);
-    else if (j.stride == 2) im2col_rows<E, VEC, 2>(j, tile, off, dst, nb * nyo, nyo, width);
-    else im2col_rows<E, VEC, 0>(j, tile, off, dst, nb * nyo, nyo, width);
+    if (j.dst_ld % VEC != 0) im2col_rows<E, 1, 0>(j, tile, off, dst, nb, nyo, width);
+    else if (j.stride == 1) im2col_rows<E, VEC, 1>(j, tile, off, dst, nb, nyo, width);
+    else if (j.stride == 2) im2col_rows<E, VEC, 2>(j, tile, off, dst, nb, nyo, width);
+    else im2col_rows<E, VEC, 0>(j, tile, off, dst, nb, nyo, width);
 }
 }  // namespace stage
 

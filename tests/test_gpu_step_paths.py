@@ -82,7 +82,9 @@ def test_elementwise_grads_of_an_example_that_overflows(dp):
     ("f32", 24, 3, (33, 31), 30, 3, 1, 1, True), ("f32", 8, 72, (12, 20), 64, 5, 2, 2, False), ("f32", 40, 64, (4, 4), 130, 3, 1, 1, True),
     ("f32", 4, 48, (56, 56), 16, 1, 2, 0, True), ("bf16", 9, 40, (8, 8), 160, 3, 1, 1, True), ("bf16", 33, 33, (13, 10), 48, 3, 1, 1, True),
     ("bf16", 16, 64, (16, 16), 128, 3, 2, 1, True), ("bf16", 50, 100, (4, 6), 40, 3, 1, 1, False), ("bf16", 5, 24, (28, 28), 72, 5, 1, 4, True),
-    ("bf16", 3, 20, (56, 40), 200, 3, 3, 0, True), ("bf16", 64, 80, (7, 7), 33, 2, 1, 3, True)])
+    ("bf16", 3, 20, (56, 40), 200, 3, 3, 0, True), ("bf16", 64, 80, (7, 7), 33, 2, 1, 3, True),
+    ("bf16", 40, 32, (14, 14), 64, 3, 2, 0, True), ("bf16", 40, 32, (14, 14), 64, 3, 1, 1, True), ("f32", 80, 24, (6, 7), 64, 3, 2, 0, True),
+    ("f32", 70, 36, (10, 5), 48, 2, 2, 0, True)])
 def test_convolutions_from_feature_maps(dp, dtype, B, C, size, d_out, k, stride, pad, cm):
     gen = torch.Generator(device="cuda"); gen.manual_seed(7)
     td = torch.float32 if dtype == "f32" else torch.bfloat16
