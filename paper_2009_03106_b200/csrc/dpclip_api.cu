@@ -835,7 +835,7 @@ int launch_zta_stream(const StreamLayer* ls, int n, int B, int T, const NoiseSpe
     memset(&p, 0, sizeof(p));
     p.R = (int)R; p.T = T; p.S = (int)ceil_div(R, (long)zp::BK); p.n_layers = n;
     p.status = static_cast<int*>(workspace);
-    bool fuse_noise = noise && noise->scale > 0.f, any_split = false;
+    bool fuse_noise = noise && noise->scale > 0.f, any_split = false, cut = false;
     int G = 0;
     for (int l = 0; l < n; ++l) {
         const StreamLayer& y = ls[l];
@@ -845,12 +845,14 @@ int launch_zta_stream(const StreamLayer* ls, int n, int B, int T, const NoiseSpe
         zp::Layer& q = p.layer[l];
         q.d_in = y.d_in; q.d_out = y.d_out;
         q.tiles_n = ceil_div(y.d_in, zp::BN);
+        q.N = (int)round_up(ceil_div(y.d_in, (long)q.tiles_n), 32);
         q.tile_base = G; q.tiles = pair_tiles(y.d_in, y.d_out);
         G += q.tiles;
         q.do_bias = y.gb ? 1 : 0;
         q.clip = y.clip;
         q.split = y.split ? 1 : 0;
         any_split = any_split || y.split;
+        cut = cut || q.N != zp::BN || (y.d_out - 1) % zp::BM < zp::BM_CTA;
         q.gW = y.gW; q.gb = y.gb; q.ldg = y.ldg;
         q.vec_ok = aligned_to(y.gW, 16) && y.ldg % 4 == 0;
         q.sw0 = (uint32_t)y.sid_w; q.sw1 = (uint32_t)(y.sid_w >> 32);
@@ -935,7 +937,7 @@ int launch_zta_stream(const StreamLayer* ls, int n, int B, int T, const NoiseSpe
         p.k0 = (uint32_t)noise->seed; p.k1 = (uint32_t)(noise->seed >> 32);
         if (noise_done) *noise_done = true;
     }
-    const auto kernel = any_split ? tc::zta_pair_kernel<true> : tc::zta_pair_kernel<false>;
+    const auto kernel = any_split ? tc::zta_pair_kernel<true, true> : cut ? tc::zta_pair_kernel<false, true> : tc::zta_pair_kernel<false, false>;
     if (!enable_smem(kernel, zp::SMEM_BYTES)) return DPCLIP_ERR_CUDA;
     const int pairs = (int)ceil_div(p.total, U) * W;
     DPCLIP_LOGF("clipped sum, CTA pairs: %d layer(s), B*T=%ld, %d tiles of 512x256 in %d super-layer(s) of %d, %d stages per tile, "
