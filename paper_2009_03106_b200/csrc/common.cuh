@@ -11,6 +11,16 @@ namespace dpclip {
 constexpr int kHeaderBytes = 256;   // status header at the start of every workspace
 constexpr int kNumSMs = 148;        // B200: 2 dies x 74 SMs
 
+// Programmatic dependent launch.  A kernel that calls griddep_launch_dependents lets the next kernel of its stream,
+// if that one was launched with the programmatic-serialization attribute, start its CTAs as soon as every CTA of
+// this grid has made the call (or exited) and there is room for them; that kernel's threads call griddep_wait
+// before they touch anything this grid (or an earlier one) writes or reads for writing: the wait returns once
+// this grid has completed and its writes are visible.  Without the attribute both are no-ops.  A kernel that was itself
+// launched so makes the call only behind its own wait: whoever follows may then read, without waiting, what lies two
+// launches back.
+__device__ __forceinline__ void griddep_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ float to_f32(float x) { return x; }
 __device__ __forceinline__ float to_f32(__nv_bfloat16 x) { return __bfloat162float(x); }
 

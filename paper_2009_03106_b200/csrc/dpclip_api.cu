@@ -116,6 +116,22 @@ inline bool clear_sq(float* sq, size_t n, cudaStream_t st) {
     return t_sq_cleared || cudaMemsetAsync(sq, 0, sizeof(float) * n, st) == cudaSuccess;
 }
 
+// Launch with programmatic serialization: for kernels that call griddep_wait, right behind another kernel of their stream.
+template <typename... P, typename... A>
+inline int launch_behind(void (*kernel)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, const A&... args) {
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = grid; cfg.blockDim = dim3(block); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = path_switch(SW_NO_OVERLAP) ? 0 : 1;
+    if (cudaLaunchKernelEx(&cfg, kernel, args...) != cudaSuccess) { cudaGetLastError(); return DPCLIP_ERR_CUDA; }
+    return launch_status();
+}
+// The kernel that this thread is about to launch directly follows one of the same step in its stream (takes the flag).
+inline bool take_overlap() { const bool on = t_overlap_prev; t_overlap_prev = false; return on; }
+
 // DPCLIP_LOG=1: one line on stderr per dispatch decision (which form of a kernel a layer takes and how its
 // work is cut) -- host side only, nothing changes on the device.
 #define DPCLIP_LOGF(...) do { if (path_switch(SW_LOG)) { fprintf(stderr, "[dpclip] " __VA_ARGS__); fputc('\n', stderr); } } while (0)
@@ -381,8 +397,7 @@ int launch_simt_grad(const void* A, long lda, const void* Z, long ldz, int B, in
                 r.sid_w = noise->sid_w; r.sid_b = noise->sid_b;
                 if (noise_done) *noise_done = true;
             }
-            narrow_reduce_kernel<<<d_out, 256, 0, st>>>(r);
-            return launch_status();
+            return launch_behind(narrow_reduce_kernel, dim3(d_out), 256, 0, st, r);
         }
         if (cudaMemset2DAsync(gW, sizeof(float) * (size_t)ldg, 0, sizeof(float) * (size_t)d_in, d_out, st) !=
             cudaSuccess) return DPCLIP_ERR_CUDA;
@@ -623,17 +638,11 @@ int launch_gram_group(const GramLayer* ls, int n, int cls, int* status, cudaStre
         q.tail.done = reinterpret_cast<unsigned int*>(reinterpret_cast<char*>(status) + kTailCounterOffset);
     }
     const int grid = groups < sm_budget() ? groups : sm_budget();
-    if (cls == 0) {
-        q.work_counter = reinterpret_cast<unsigned int*>(reinterpret_cast<char*>(status) + kWorkCounterOffset);
-        if (!enable_smem_shared(tc::gram_norm_q2_kernel, g::SMEM_BYTES)) return DPCLIP_ERR_CUDA;
-        tc::gram_norm_q2_kernel<<<grid, g::THREADS, g::SMEM_BYTES, st>>>(q);
-    } else if (cls == 1) {
-        if (!enable_smem_shared(tc::gram_norm_kernel<true>, g::SMEM_BYTES)) return DPCLIP_ERR_CUDA;
-        tc::gram_norm_kernel<true><<<grid, g::THREADS, g::SMEM_BYTES, st>>>(q);
-    } else {
-        if (!enable_smem_shared(tc::gram_norm_kernel<false>, g::SMEM_BYTES)) return DPCLIP_ERR_CUDA;
-        tc::gram_norm_kernel<false><<<grid, g::THREADS, g::SMEM_BYTES, st>>>(q);
-    }
+    if (cls == 0) q.work_counter = reinterpret_cast<unsigned int*>(reinterpret_cast<char*>(status) + kWorkCounterOffset);
+    const auto kernel = cls == 0 ? tc::gram_norm_q2_kernel : cls == 1 ? tc::gram_norm_kernel<true> : tc::gram_norm_kernel<false>;
+    if (!enable_smem_shared(kernel, g::SMEM_BYTES)) return DPCLIP_ERR_CUDA;
+    if (take_overlap()) return launch_behind(kernel, dim3(grid), g::THREADS, g::SMEM_BYTES, st, q);
+    kernel<<<grid, g::THREADS, g::SMEM_BYTES, st>>>(q);
     return launch_status();
 }
 
@@ -717,8 +726,7 @@ int launch_reduce_partials(const tc::zta::Params& p, int tiles, int ksplit, int 
     r.lanes = lanes;
     long blocks = (n_vec + (256 / lanes) - 1) / (256 / lanes);
     if (blocks > 8L * kNumSMs) blocks = 8L * kNumSMs;
-    tc::reduce_partials_kernel<<<dim3((unsigned)blocks, r.n_layers > 0 ? r.n_layers : 1), 256, 0, st>>>(r);
-    return launch_status();
+    return launch_behind(tc::reduce_partials_kernel, dim3((unsigned)blocks, r.n_layers > 0 ? r.n_layers : 1), 256, 0, st, r);
 }
 
 // Tile shape: 256 x 256 (MT = 2) cuts the L2->SM traffic per flop by a third but has a single
@@ -943,27 +951,18 @@ int launch_zta_stream(const StreamLayer* ls, int n, int B, int T, const NoiseSpe
     DPCLIP_LOGF("clipped sum, CTA pairs: %d layer(s), B*T=%ld, %d tiles of 512x256 in %d super-layer(s) of %d, %d stages per tile, "
                 "%d pairs in gangs of %d, runs of %ld stages, %ld segments, noise %s", n, R, G, n_super, W, p.S, pairs, W, U,
                 n_segments, fuse_noise ? "in the reduce" : "separate");
-    if (t_overlap_prev && !path_switch(SW_NO_OVERLAP)) {
-        t_overlap_prev = false;                    // only the launch that directly follows
-        cudaLaunchConfig_t cfg;
-        memset(&cfg, 0, sizeof(cfg));
-        cfg.gridDim = dim3(2 * pairs); cfg.blockDim = dim3(zp::THREADS);
-        cfg.dynamicSmemBytes = zp::SMEM_BYTES; cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr; cfg.numAttrs = 1;
-        if (cudaLaunchKernelEx(&cfg, kernel, maps, p) != cudaSuccess) { cudaGetLastError(); return DPCLIP_ERR_CUDA; }
+    int rc;
+    if (take_overlap()) {
+        rc = launch_behind(kernel, dim3(2 * pairs), zp::THREADS, zp::SMEM_BYTES, st, maps, p);
     } else {
         kernel<<<2 * pairs, zp::THREADS, zp::SMEM_BYTES, st>>>(maps, p);
+        rc = launch_status();
     }
-    int rc = launch_status();
     if (rc) return rc;
     // one wave of CTAs (six of 256 threads and 40 registers per SM) over the 4-row blocks of all tiles
     long blocks = (long)G * (zp::BM / 4);
     if (blocks > 6L * kNumSMs) blocks = 6L * kNumSMs;
-    tc::reduce_segments_kernel<<<(unsigned)blocks, 256, 0, st>>>(p);
-    return launch_status();
+    return launch_behind(tc::reduce_segments_kernel, dim3((unsigned)blocks), 256, 0, st, p);
 }
 
 int launch_zta_tc(const void* A, long lda, const void* Z, long ldz, int B, int T, int d_in, int d_out,
@@ -1225,6 +1224,7 @@ template <bool NORM>
 int launch_group_kernel(const tc::zg::Maps& maps, const tc::zg::Params& p, cudaStream_t st) {
     constexpr int smem = tc::zg::Cfg::SMEM_BYTES;
     if (!enable_smem(tc::zta_group_kernel<NORM>, smem)) return DPCLIP_ERR_CUDA;
+    if (take_overlap()) return launch_behind(tc::zta_group_kernel<NORM>, dim3(2 * p.n_runs), tc::zg::THREADS, smem, st, maps, p);
     tc::zta_group_kernel<NORM><<<2 * p.n_runs, tc::zg::THREADS, smem, st>>>(maps, p);
     return launch_status();
 }
@@ -1337,8 +1337,7 @@ int launch_group(const GroupLayer* ls, int n, int B, bool norm, const NoiseSpec*
         if (rc) return rc;
         if (norm) continue;
         const int blocks = p.n_blocks < 8 * kNumSMs ? p.n_blocks : 8 * kNumSMs;
-        tc::reduce_group_kernel<<<blocks, 256, 0, st>>>(p);
-        if ((rc = launch_status())) return rc;
+        if ((rc = launch_behind(tc::reduce_group_kernel, dim3(blocks), 256, 0, st, p))) return rc;
     }
     if (fuse_noise && noise_done) *noise_done = true;
     return DPCLIP_OK;
@@ -2024,9 +2023,7 @@ static int launch_dp_update(bool adam, float* theta, float* m, float* v, const f
     size_t blocks = (nq + 255) / 256;
     const size_t cap = (size_t)kNumSMs * 16;
     if (blocks > cap) blocks = cap;
-    if (adam) dp_update_kernel<true><<<(unsigned)blocks, 256, 0, (cudaStream_t)stream>>>(p);
-    else dp_update_kernel<false><<<(unsigned)blocks, 256, 0, (cudaStream_t)stream>>>(p);
-    return launch_status();
+    return launch_behind(adam ? dp_update_kernel<true> : dp_update_kernel<false>, dim3((unsigned)blocks), 256, 0, (cudaStream_t)stream, p);
 }
 
 int dpclip_dp_sgd_step(float* theta, const float* gsum, size_t n, float inv_tau, float C, float sigma,
@@ -2155,8 +2152,7 @@ static int launch_conv_tc(const SimtParams& sp, const void* X, const void* Zbar,
     r.lanes = lanes;
     long blocks = (n_vec + (256 / lanes) - 1) / (256 / lanes);
     if (blocks > 8L * kNumSMs) blocks = 8L * kNumSMs;
-    tc::reduce_partials_kernel<<<(unsigned)blocks, 256, 0, st>>>(r);
-    return launch_status();
+    return launch_behind(tc::reduce_partials_kernel, dim3((unsigned)blocks), 256, 0, st, r);
 }
 }  // extern "C++"
 
@@ -2925,7 +2921,7 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
     if (!cleared && lanes.n > 1) {
         const size_t n = (size_t)L * B;
         clear_kernel<<<(unsigned)(n < 256 * 64 ? (n + 255) / 256 : 64), 256, 0, lanes.st[0]>>>(sq_layers, n);
-        if (launch_status()) return DPCLIP_ERR_CUDA;
+        if (cudaGetLastError() != cudaSuccess) return DPCLIP_ERR_CUDA;     // not in the count of launches, like the memsets it stands for
         cleared = true;
     }
     if ((rc = lanes.fork())) return rc;
@@ -2941,7 +2937,8 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
     SqClearedScope cleared_scope(cleared);
     if (track) {
         // when one Gram launch takes every layer of the model, its last CTA also computes the factors
-        const tc::gram::FactorsTail tail = {sq_layers, L, (long)B, B, C, clip, norms, nullptr};
+        const tc::gram::FactorsTail tail = {sq_layers, L, (long)B, B, C, clip, norms, nullptr, 0, {}};
+        const OverlapPrevScope behind_copies(sp != nullptr && lanes.n == 1);
         rc = gram_layers_sqnorms(layers, L, B, dtype, sq_layers, in_gram_group, ws0, lanes.ws_bytes[0], lanes.st[0],
                                  (!t1.active && !any_other && !path_switch(SW_NO_FACTORS_TAIL)) ? &tail : nullptr, &factors_done);
         if (rc) return rc;
@@ -3013,7 +3010,11 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
     }
     if ((rc = lanes.join())) return rc;
     if (!factors_done) {
-        rc = dpclip_factors(sq_layers, L, B, B, C, clip, norms, nullptr, lanes.st[0]);
+        // on one stream right behind the last of the norms
+        if (lanes.n == 1)
+            rc = launch_behind(factors_kernel, dim3(1), 256, 0, lanes.st[0], (const float*)sq_layers, L, (long)B, B, C, clip, norms, (int*)nullptr);
+        else
+            rc = dpclip_factors(sq_layers, L, B, B, C, clip, norms, nullptr, lanes.st[0]);
         if (rc) return rc;
     }
     if ((rc = lanes.fork())) return rc;
@@ -3025,9 +3026,9 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
     int in_grad_group[64];
     bool any_group = false, any_rest = false;
     if (track) {
-        // the factors came from the tail of the Gram launch, the last kernel of this stream: the first clipped-sum
-        // launch may start loading while that tail runs
-        const OverlapPrevScope overlap(factors_done);
+        // the factors came from the tail of the Gram launch or from factors_kernel, the last kernel of this stream: the first
+        // clipped-sum launch may start loading while that runs
+        const OverlapPrevScope overlap(factors_done || lanes.n == 1);
         // Layers of several T would share several launches, one after the other on lane 0, where side by side on the lanes they
         // are faster (four convolutions of 49 and 16 positions, 78 examples, four lanes: 68 us, 47 apart; layers of 100 and 50
         // positions: 70, 45).  On one lane sharing would win (77 us, 117 apart), but the shared kernel rounds c a where the
@@ -3279,13 +3280,22 @@ int dpclip_step_per_layer(const dpclip_layer* layers, int L, int B, dpclip_dtype
     }
     const bool* split = sp.active ? sp.split : nullptr;
     if (sp.active) layers = sp.eff;
+    bool factors_done = false;
     {
     const SqClearedScope cleared(sp.active);                            // by the staging launch
     if (track) {
-        rc = dpclip_gram_layers_sqnorms(layers, L, B, dtype, sq_layers, in_gram, workspace, workspace_bytes, stream);
+        // when one launch takes every layer, its last CTA computes the factors too
+        tc::gram::FactorsTail tail = {sq_layers, L, (long)B, B, 0.f, clip_layers, norms_layers, nullptr, 1, {}};
+        const bool with_tail = L <= (int)(sizeof(tail.C_row) / sizeof(float)) && !path_switch(SW_NO_FACTORS_TAIL);
+        for (int l = 0; with_tail && l < L; ++l) tail.C_row[l] = C_layer[l];
+        const OverlapPrevScope behind_copies(sp.active);
+        rc = gram_layers_sqnorms(layers, L, B, dtype, sq_layers, in_gram, workspace, workspace_bytes, stream, with_tail ? &tail : nullptr, &factors_done);
         if (rc) return rc;
         int taken[kMaxTracked];
-        rc = group_norms(layers, L, B, dtype, sq_layers, in_gram, taken, workspace, workspace_bytes, stream, nullptr, nullptr, 1);
+        bool any_gram = false;
+        for (int l = 0; l < L; ++l) any_gram = any_gram || in_gram[l];
+        rc = group_norms(layers, L, B, dtype, sq_layers, in_gram, taken, workspace, workspace_bytes, stream,
+                         with_tail && !any_gram ? &tail : nullptr, any_gram ? nullptr : &factors_done, 1);
         if (rc) return rc;
         for (int l = 0; l < L; ++l) in_gram[l] = in_gram[l] || taken[l];
     }
@@ -3298,10 +3308,13 @@ int dpclip_step_per_layer(const dpclip_layer* layers, int L, int B, dpclip_dtype
     }
     }
     if (track) {
-        LayerThresholds th;
-        for (int l = 0; l < L; ++l) th.C[l] = C_layer[l];
-        factors_rows_kernel<<<L, 256, 0, (cudaStream_t)stream>>>(sq_layers, (long)B, B, th, clip_layers, norms_layers);
-        if (launch_status()) return DPCLIP_ERR_CUDA;
+        if (!factors_done) {
+            LayerThresholds th;
+            for (int l = 0; l < L; ++l) th.C[l] = C_layer[l];
+            if (launch_behind(factors_rows_kernel, dim3(L), 256, 0, (cudaStream_t)stream, (const float*)sq_layers, (long)B, B, th, clip_layers,
+                              norms_layers)) return DPCLIP_ERR_CUDA;
+        }
+        const OverlapPrevScope overlap(true);
         rc = shared_clipped_grad_launches(layers, split, true, L, B, dtype, clip_layers, (long)B, C_total, sigma, seed, stream_id0,
                                           in_pairs, workspace, workspace_bytes, stream);
         if (rc) return rc;

@@ -207,6 +207,9 @@ zta_group_kernel(const __grid_constant__ zg::Maps maps, const __grid_constant__ 
     cluster_sync_all();
     tc_fence_after_sync();
     const uint32_t tmem_base = *tmem_slot;
+    // Norms may follow the launch that copies their operands, clipped sums the one that computes the factors: of the latter the loads
+    // run ahead, and whoever passes the launch on (warp 1) waits in either.
+    if (NORM || warp >= 1) griddep_wait();
 
     if (warp == 0) {
         // ------------------------------------------------ TMA producer
@@ -241,6 +244,7 @@ zta_group_kernel(const __grid_constant__ zg::Maps maps, const __grid_constant__ 
         }
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer (rank 0 only)
+        if (lane == 0 && rank != 0) griddep_launch_dependents();
         if (lane == 0 && rank == 0) {
             int stage = 0; uint32_t phase = 0;
             AccRing ring;
@@ -290,6 +294,7 @@ zta_group_kernel(const __grid_constant__ zg::Maps maps, const __grid_constant__ 
                 }
                 u += w.units;
             }
+            griddep_launch_dependents();                        // the reduce may place CTAs beside the last drains
         }
     } else if (warp < 2 + PREP) {
         // ------------------------------------------------ preparation
@@ -504,6 +509,7 @@ __global__ void __launch_bounds__(256)
 reduce_group_kernel(const __grid_constant__ zg::Params p) {
     using namespace zg;
     __shared__ float turn[32][33];
+    griddep_wait();
     auto run_of = [&](int u) {                                 // last run that begins at or before unit u
         int lo = 0, hi = p.n_runs;
         while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (p.run_begin[mid] <= u) lo = mid; else hi = mid; }

@@ -375,6 +375,7 @@ struct NarrowReduceParams {
 __global__ void __launch_bounds__(256)
 narrow_reduce_kernel(const NarrowReduceParams p) {
     __shared__ float comb[8][32];
+    griddep_wait();
     const int m = blockIdx.x, n = threadIdx.x & 31, g = threadIdx.x >> 5;
     const size_t stride = (size_t)p.maxm * 32;
     const float* src = p.part + (size_t)m * 32 + n;

@@ -281,6 +281,7 @@ stage_operands_kernel(const __grid_constant__ stage::Launch q) {
     using namespace stage;
     extern __shared__ __align__(16) uint8_t stage_smem[];
     for (size_t i = (size_t)blockIdx.x * THREADS + threadIdx.x; i < q.n_clear; i += (size_t)gridDim.x * THREADS) q.clear[i] = 0.f;
+    griddep_launch_dependents();
     int k = 0;
     while (k + 1 < q.n && (int)blockIdx.x >= q.job[k + 1].blk_begin) ++k;
     const Job& j = q.job[k];

@@ -53,6 +53,8 @@ factors_kernel(const float* __restrict__ sq_layers, int L, long ld_sq, int B, fl
                float* __restrict__ clip, float* __restrict__ norms, int* __restrict__ n_clipped) {
     __shared__ float red[32];
     float cnt = 0.f;
+    griddep_wait();
+    griddep_launch_dependents();
     for (int i = threadIdx.x; i < B; i += blockDim.x) {
         float s = 0.f;
         for (int l = 0; l < L; ++l) s += sq_layers[(size_t)l * ld_sq + i];
@@ -76,6 +78,8 @@ factors_rows_kernel(const float* __restrict__ sq_layers, long ld_sq, int B, cons
                     float* __restrict__ clip_layers, float* __restrict__ norms_layers) {
     const int l = blockIdx.x;
     const float C = th.C[l];
+    griddep_wait();
+    griddep_launch_dependents();
     for (int i = threadIdx.x; i < B; i += blockDim.x) {
         const float n = sqrtf(sq_layers[(size_t)l * ld_sq + i]);
         float c = 1.0f;
@@ -208,6 +212,8 @@ struct UpdateParams {
 template <bool ADAM>
 __global__ void __launch_bounds__(256)
 dp_update_kernel(const UpdateParams p) {
+    griddep_wait();
+    griddep_launch_dependents();
     const size_t nq = (p.n + 3) >> 2;
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     for (size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q < nq; q += stride) {

@@ -85,6 +85,9 @@ struct FactorsTail {
     const float* sq; int L; long ld; int B; float C;
     float* clip; float* norms;           // clip == NULL: no tail
     unsigned int* done;                  // CTAs finished so far (workspace header; back at zero after the launch)
+    // per-layer clipping: row l of sq against C_row[l] alone, its factors and norms in row l of clip[L][B], norms[L][B]
+    int per_row;
+    float C_row[16];
 };
 
 struct Launch {
@@ -107,6 +110,14 @@ __device__ __forceinline__ void factors_tail(const FactorsTail& t) {
     __syncthreads();
     if (s_prev != gridDim.x - 1) return;               // not the last CTA
     __threadfence();
+    if (t.per_row) {
+        for (int k = threadIdx.x; k < t.L * t.B; k += blockDim.x) {
+            const int l = k / t.B, i = k - l * t.B;
+            const float n = sqrtf(__ldcg(t.sq + (size_t)l * t.ld + i)), C = t.C_row[l];
+            t.clip[k] = n > C ? C / n : 1.0f;
+            if (t.norms) t.norms[k] = n;
+        }
+    } else
     for (int i = threadIdx.x; i < t.B; i += blockDim.x) {
         float s = 0.f;
         for (int l = 0; l < t.L; ++l) s += __ldcg(t.sq + (size_t)l * t.ld + i);      // L2: where the atomics landed
@@ -201,6 +212,8 @@ gram_norm_kernel(const __grid_constant__ gram::Launch q) {
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem_base = *tmem_slot;      // A A^T in columns 0..255, Zb Zb^T in 256..511
+    griddep_wait();                             // the launch may follow the one that copies the operands
+    griddep_launch_dependents();                // the next may place its CTAs as SMs fall idle
 
     if (warp == 0) {
         // ------------------------------------------------ TMA producer
@@ -432,6 +445,7 @@ gram_norm_q2_kernel(const __grid_constant__ gram::Launch q) {
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem_base = *tmem_slot;
+    griddep_wait();                 // the launch may follow the one that copies the operands
     griddep_launch_dependents();    // the clipped-sum launch that follows may place its CTAs as SMs fall idle
 
     if (warp == 0) {
@@ -1193,6 +1207,7 @@ namespace tc {
 __global__ void __launch_bounds__(256)
 reduce_partials_kernel(const ReduceParams q) {
     __shared__ float4 part_s[256];
+    griddep_wait();
     ReduceParams p = q;
     if (q.n_layers > 0) {
         const int y = blockIdx.y;

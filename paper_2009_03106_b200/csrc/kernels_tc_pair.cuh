@@ -211,8 +211,8 @@ zta_pair_kernel(const __grid_constant__ zta::Maps maps, const __grid_constant__ 
     const uint32_t tmem_base = *tmem_slot;
     // When the launch overlaps the tail of the kernel that computes the factors, only the loads of the layers'
     // inputs (which no kernel of a step writes) may run ahead: the warps that read the factors or write the
-    // workspace wait for that kernel here.
-    if (warp >= 2) griddep_wait();
+    // workspace wait for that kernel here, and so does the warp that passes the launch on.
+    if (warp >= 1) griddep_wait();
 
     if (warp == 0) {
         // ------------------------------------------------ TMA producer (each CTA loads its own operands)
@@ -251,6 +251,7 @@ zta_pair_kernel(const __grid_constant__ zta::Maps maps, const __grid_constant__ 
         }
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer (rank 0 only)
+        if (lane == 0 && rank != 0) griddep_launch_dependents();
         if (lane == 0 && rank == 0) {
             int stage = 0; uint32_t phase = 0; int it = 0;
             bool ok = true;
@@ -304,6 +305,7 @@ zta_pair_kernel(const __grid_constant__ zta::Maps maps, const __grid_constant__ 
                 ++it;
                 u += w.kb1 - w.kb0;
             }
+            griddep_launch_dependents();                        // the reduce may place CTAs beside the last drains
         }
     } else if (warp < 2 + N_TRANSFORM_WARPS) {
         // ------------------------------------------------ transform (256 threads)
@@ -554,6 +556,7 @@ reduce_segments_kernel(const __grid_constant__ ztp::Params p) {
     // 64-bit divisions per block).  A thread issues the loads of up to four segments before the first add and draws
     // its noise while they are in flight: with one load in flight per thread the kernel was bound by the latency of
     // its serial loads; what binds it now is instruction issue (the Philox rounds and Box-Muller of every float4).
+    griddep_wait();
     constexpr int ROWS = 4, SG = 4;
     constexpr int ROW_BLOCKS = BM / ROWS;
     const int n_blocks = p.G * ROW_BLOCKS;

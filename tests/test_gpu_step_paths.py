@@ -164,3 +164,51 @@ def test_clipped_sums_on_pairs_of_cut_tiles(dp, d_in, d_out, odd):
             tol = 4e-3                                     # not copied: whatever form it takes
         assert _rel(plan.gW[l], torch.einsum("b,bto,bti->oi", clip, Z, A)) <= tol, (l, tol)
         assert _rel(plan.gb[l], torch.einsum("b,bto->o", clip, Z)) <= 1e-5
+
+
+# ---------------------------------------------------------------------------
+# launches that start behind their predecessor's tail: a step recorded after a memset, a copy, a kernel and a join, and per-layer
+# factors from the tail of the norm launch, equal the step on its own
+# ---------------------------------------------------------------------------
+@pytest.mark.parametrize("before", ["nothing", "memset", "copy", "join"])
+@pytest.mark.parametrize("dtype,T,d", [("bf16", 50, 300), ("bf16", 256, 128), ("f32", 64, 192), ("f32", 48, 146)])
+def test_recorded_steps_behind_other_work(dp, dtype, T, d, before):
+    gen = torch.Generator(device="cuda"); gen.manual_seed(T)
+    td = torch.float32 if dtype == "f32" else torch.bfloat16
+    B, n = 40, 3
+    layers = [dp.Layer(torch.randn(B, T, d, generator=gen, device="cuda").to(td),
+                       (torch.randn(B, T, 2 * d, generator=gen, device="cuda") * 1e-2).to(td), True) for _ in range(n)]
+    plan, C = dp.StepPlan(layers), [0.5, 1.0, 2.0]
+    theta = torch.randn(plan.flat.numel(), generator=gen, device="cuda")
+
+    def step():
+        clip = dp.dpclip_step_per_layer(plan, C, 0.1, 5)
+        dp.dpclip_dp_sgd_step(theta, plan.flat, 0.5, 1.0, 0.1, 7, 9, 1e-2)
+        return clip
+
+    theta0 = theta.clone()
+    want = [step().clone(), plan.flat.clone(), theta.clone()]
+    theta.copy_(theta0)
+    x, y, side = torch.zeros(1 << 20, device="cuda"), torch.ones(1 << 20, device="cuda"), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        if before == "memset":
+            x.zero_()
+        elif before == "copy":
+            x.copy_(y)
+        elif before == "join":
+            side.wait_stream(torch.cuda.current_stream())
+            with torch.cuda.stream(side):
+                x.add_(y)
+            torch.cuda.current_stream().wait_stream(side)
+        clip = step()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert dp.dpclip_read_status(plan.workspace) == 0
+    for l, (y, c) in enumerate(zip(layers, C)):
+        G = torch.einsum("bto,bti->boi", y.Zbar.double(), y.A.double())
+        norm = (G.pow(2).sum((1, 2)) + y.Zbar.double().sum(1).pow(2).sum(1)).sqrt()
+        assert ((clip[l].double() - (c / norm).clamp(max=1.0)).abs()).max().item() <= TOL[dtype]["norm"]
+    # sums of norms and of windows may add up in another order from run to run
+    assert _rel(clip, want[0]) <= 1e-5 and _rel(plan.flat, want[1]) <= 1e-4 and _rel(theta, want[2]) <= 1e-4
