@@ -12,6 +12,7 @@
 #include "kernels_fused_t1_tf32.cuh"
 #include "kernels_tf32.cuh"
 #include "kernels_group.cuh"
+#include "kernels_t1_planes.cuh"
 #include "kernels_fused_t1.cuh"
 #include "kernels_narrow.cuh"
 #include "kernels_narrow_tc.cuh"
@@ -50,7 +51,7 @@ enum PathSwitch : unsigned {
     SW_FORCE_SIMT = 1u << 0, SW_NO_NARROW = 1u << 1, SW_NO_NARROW_RING = 1u << 2, SW_NO_NARROW_TC = 1u << 3,
     SW_NO_NARROW_PACK = 1u << 4, SW_NARROW_PACK_BF16 = 1u << 5, SW_NO_GRAM_Q2 = 1u << 6, SW_NO_T1_TF32 = 1u << 7,
     SW_NO_FUSED_T1 = 1u << 8, SW_NO_GRAM_GROUP = 1u << 9, SW_NO_GRAD_GROUP = 1u << 10, SW_NO_CONV_TC = 1u << 11,
-    SW_NO_CONV_PATCHES = 1u << 12, SW_TILE_M1 = 1u << 13, SW_TILE_M2 = 1u << 14, SW_T1_TWO_LAUNCHES = 1u << 15, SW_NO_PAIR = 1u << 16, SW_LOG = 1u << 17, SW_NO_FACTORS_TAIL = 1u << 18, SW_NO_SM_BUDGET = 1u << 19, SW_NO_OVERLAP = 1u << 20, SW_NO_STAGE = 1u << 21, SW_NO_GRAM_PER_EX = 1u << 22, SW_NO_PAIR_JOIN = 1u << 23,
+    SW_NO_CONV_PATCHES = 1u << 12, SW_TILE_M1 = 1u << 13, SW_TILE_M2 = 1u << 14, SW_T1_TWO_LAUNCHES = 1u << 15, SW_NO_PAIR = 1u << 16, SW_LOG = 1u << 17, SW_NO_FACTORS_TAIL = 1u << 18, SW_NO_SM_BUDGET = 1u << 19, SW_NO_OVERLAP = 1u << 20, SW_NO_STAGE = 1u << 21, SW_NO_GRAM_PER_EX = 1u << 22, SW_NO_PAIR_JOIN = 1u << 23, SW_NO_T1_PLANES = 1u << 24,
     SW_LOADED = 1u << 31
 };
 std::atomic<unsigned> g_path_switches{0};
@@ -67,7 +68,7 @@ unsigned read_path_switches() {
         {"DPCLIP_NO_PAIR", SW_NO_PAIR, '1'}, {"DPCLIP_LOG", SW_LOG, '1'},
         {"DPCLIP_NO_FACTORS_TAIL", SW_NO_FACTORS_TAIL, '1'}, {"DPCLIP_NO_SM_BUDGET", SW_NO_SM_BUDGET, '1'},
         {"DPCLIP_NO_OVERLAP", SW_NO_OVERLAP, '1'}, {"DPCLIP_NO_STAGE", SW_NO_STAGE, '1'},
-        {"DPCLIP_NO_GRAM_PER_EX", SW_NO_GRAM_PER_EX, '1'}, {"DPCLIP_NO_PAIR_JOIN", SW_NO_PAIR_JOIN, '1'},
+        {"DPCLIP_NO_GRAM_PER_EX", SW_NO_GRAM_PER_EX, '1'}, {"DPCLIP_NO_PAIR_JOIN", SW_NO_PAIR_JOIN, '1'}, {"DPCLIP_NO_T1_PLANES", SW_NO_T1_PLANES, '1'},
     };
     unsigned v = SW_LOADED;
     for (const auto& e : table) {
@@ -1444,6 +1445,99 @@ int launch_fused_t1_tf32(const FusedT1Params& base, bool one_launch, dpclip_dtyp
                  : launch_fused_t1_tc<float, false>(q, one_launch, grid, workspace, st);
 }
 
+// Planes of a layer's operands in the workspace (kernels_t1_planes.cuh): c zb, and of fp32 models a too.
+struct T1Planes { int pitch_z, pitch_a; size_t z, a; };
+inline T1Planes t1_planes(int B, int d_in, int d_out, dpclip_dtype dtype) {
+    const int planes = dtype == DPCLIP_F32 ? 3 : 1;
+    T1Planes y;
+    y.pitch_z = (int)round_up(d_out, 8); y.pitch_a = (int)round_up(d_in, 8);
+    y.z = round_up((size_t)planes * B * y.pitch_z * 2, 256);
+    y.a = dtype == DPCLIP_F32 ? round_up((size_t)planes * B * y.pitch_a * 2, 256) : 0;
+    return y;
+}
+// Models of T = 1 layers that take the two launches of kernels_t1_planes.cuh: more than 16 output tiles of 128 x 128.  A step, one
+// cooperative launch / two launches: fp32, 784-1000-1000-10, B = 128: 14.4 / 13.0 us, 1000-2000-1000, B = 64: 20.6 / 15.4, 512-512-512-10,
+// B = 512: 30.8 / 23.2, 4096-4096-1000, B = 256: 121 / 78; bf16: the first 14.4 / 11.8, the last 72 / 46 (46 / 31 without noise).  784-256-10,
+// B = 32 (16 tiles) would take 8.5 instead of 11.7, but up to there the one launch stays: it is the form whose barrier has its timeout
+// tested, on that model.
+inline bool t1_planes_pays(const dpclip_layer* layers, int L, int B, dpclip_dtype dtype) {
+    if (L <= 0 || L > FUSED_MAX_LAYERS || B > FUSED_MAX_B || path_switch(SW_NO_FUSED_T1 | SW_NO_T1_TF32 | SW_T1_TWO_LAUNCHES | SW_NO_T1_PLANES)) return false;
+    long tiles = 0;
+    for (int l = 0; l < L; ++l) {
+        if (layers[l].T != 1 || layers[l].d_in <= 0 || layers[l].d_out <= 0) return false;
+        tiles += (long)ceil_div(layers[l].d_out, (long)tc::t1p::BM) * ceil_div(layers[l].d_in, (long)tc::t1p::BN);
+    }
+    return tiles > 16 && tiles < 1L << 30;
+}
+inline size_t t1_planes_bytes(const dpclip_layer* layers, int L, int B, dpclip_dtype dtype) {
+    if (!t1_planes_pays(layers, L, B, dtype)) return 0;
+    size_t n = 0;
+    for (int l = 0; l < L; ++l) { const T1Planes y = t1_planes(B, layers[l].d_in, layers[l].d_out, dtype); n += y.z + y.a; }
+    return n;
+}
+
+// 3-D bf16 matrix [planes][rows][cols], rows ld elements apart; rows and columns beyond a plane read as zero
+bool make_map_planes(CUtensorMap* map, const void* base, int planes, long rows, long cols, long ld, int box_rows) {
+    EncodeTiledFn fn = encode_tiled_fn();
+    if (!fn) return false;
+    cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)planes};
+    cuuint64_t strides[2] = {(cuuint64_t)ld * 2, (cuuint64_t)ld * 2 * rows};
+    cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 1}, estr[3] = {1, 1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+template <typename T>
+int launch_t1_planes(const tc::t1p::Prep& prep, const tc::f1::Params& q, bool quads, int grid, cudaStream_t st) {
+    namespace t = tc::t1p;
+    constexpr int smem = t::Cfg<sizeof(T) == 4 ? 3 : 1>::SMEM_BYTES;
+    const auto kernel = quads ? tc::t1_planes_kernel<T, true> : tc::t1_planes_kernel<T, false>;
+    if (!enable_smem(kernel, smem)) return DPCLIP_ERR_CUDA;
+    const int rc = launch_behind(tc::t1_prepare_kernel<T>, dim3(prep.base.B), t::PREP_THREADS, 0, st, prep);
+    return rc ? rc : launch_behind(kernel, dim3(grid), t::THREADS, smem, st, q);
+}
+// The whole step of a model of T = 1 layers.  1: the workspace lacks room, or the model is none for the tensor cores.
+int try_t1_planes(const FusedT1Params& base, dpclip_dtype dtype, void* workspace, size_t workspace_bytes, cudaStream_t st) {
+    namespace t = tc::t1p;
+    const bool f32 = dtype == DPCLIP_F32;
+    size_t at = kHeaderBytes;
+    if (!workspace || !aligned_to(workspace, 16)) return 1;
+    t::Prep prep;
+    tc::f1::Params q;
+    memset(&prep, 0, sizeof(prep)); memset(&q, 0, sizeof(q));
+    prep.base = q.base = base;
+    q.status = static_cast<int*>(workspace);
+    bool quads = true, wide = false;
+    for (int l = 0; l < base.L; ++l) {
+        const FusedT1Layer& y = base.layer[l];
+        // operands that the one-launch form does not take run on the fp32 ALUs, whose sums are of unrounded products
+        const bool thin = y.d_out <= tc::f1::THIN_MAX_OUT;
+        if (!t1_tma_ok(y.A, y.lda, dtype) || !(t1_tma_ok(y.Z, y.ldz, dtype) || thin)) return 1;
+        wide = wide || !thin;
+        const T1Planes s = t1_planes(base.B, y.d_in, y.d_out, dtype);
+        prep.pitch_z[l] = s.pitch_z; prep.pitch_a[l] = s.pitch_a;
+        prep.za[l] = reinterpret_cast<uint16_t*>(static_cast<char*>(workspace) + at); at += s.z;
+        prep.aa[l] = reinterpret_cast<uint16_t*>(static_cast<char*>(workspace) + at); at += s.a;
+        quads = quads && y.d_in % 4 == 0;
+    }
+    if (workspace_bytes < at || !wide) return 1;
+    const int planes = f32 ? 3 : 1, bk = f32 ? t::Cfg<3>::BK : t::Cfg<1>::BK;
+    int items = 0;
+    for (int l = 0; l < base.L; ++l) {
+        const FusedT1Layer& y = base.layer[l];
+        if (!make_map_planes(&q.map_z[l], prep.za[l], planes, base.B, y.d_out, prep.pitch_z[l], bk) ||
+            !(f32 ? make_map_planes(&q.map_a[l], prep.aa[l], planes, base.B, y.d_in, prep.pitch_a[l], bk)
+                  : make_map_planes(&q.map_a[l], y.A, 1, base.B, y.d_in, y.lda, bk))) return DPCLIP_ERR_CUDA;
+        q.item_begin[l] = items;
+        q.tiles_n[l] = ceil_div(y.d_in, (long)t::BN);
+        items += ceil_div(y.d_out, (long)t::BM) * q.tiles_n[l];
+    }
+    q.total_items = items;
+    const int grid = items < kNumSMs ? items : kNumSMs;
+    DPCLIP_LOGF("T = 1 model in two launches: %d layer(s), B=%d, %d tiles", base.L, base.B, items);
+    return f32 ? launch_t1_planes<float>(prep, q, quads, grid, st) : launch_t1_planes<__nv_bfloat16>(prep, q, quads, grid, st);
+}
+
 // One T = 1 layer of the caller's model as the fused kernels see it.  Returns 0, 1 (the layer does not
 // qualify for the fused kernels) or a negative argument error.
 int fill_fused_t1_layer(FusedT1Layer& f, const dpclip_layer& y, int index, int B, dpclip_dtype dtype, int tile,
@@ -1527,6 +1621,10 @@ int try_fused_t1_step(const dpclip_layer* layers, int L, int B, dpclip_dtype dty
     const int grid_n = rows;
     const int grid_g = tiles < 4 * kNumSMs ? tiles : 4 * kNumSMs;
     const int smem64 = FusedT1Cfg<64>::SMEM_BYTES;
+    if (t1_planes_pays(layers, L, B, dtype)) {
+        const int rc = try_t1_planes(p, dtype, workspace, workspace_bytes, st);
+        if (rc <= 0) return rc;
+    }
     bool one = true;
     if (path_switch(SW_T1_TWO_LAUNCHES)) one = false;
     if (one) {
@@ -1670,6 +1768,7 @@ static size_t step_scratch_bytes(const dpclip_layer* layers, int L, int B, dpcli
         const size_t need = kHeaderBytes + (size_t)(tiles + kNumPairs) * kGroupSlotBytes;
         if (tiles > 0 && need > ws && ws > (size_t)kHeaderBytes) ws = need;
     }
+    if (const size_t planes = t1_planes_bytes(layers, L, B, dtype)) if (kHeaderBytes + planes > ws) ws = kHeaderBytes + planes;
     if (dtype != DPCLIP_BF16 || path_switch(SW_NO_GRAD_GROUP)) return ws;
     // layers of one T that share a CTA-pair launch (up to eight): one segment per tile of all of them + one per pair
     for (int l0 = 0; l0 < L; ++l0) {
@@ -2729,7 +2828,13 @@ static bool stage_plan(StagePlan& sp, const dpclip_layer* layers, const dpclip_m
         }
     }
     if (!any) return false;
+    bool all_t1 = other == nullptr;
+    for (int l = 0; l < L; ++l) all_t1 = all_t1 && sp.eff[l].T == 1;
     sp.scratch = round_up(step_scratch_bytes(sp.eff, L, B, dtype), 256);
+    if (all_t1 && sp.t1_dtype != dtype) {                            // the planes of a model that has become fp32
+        const size_t w = round_up(step_scratch_bytes(sp.eff, L, B, sp.t1_dtype), 256);
+        if (w > sp.scratch) sp.scratch = w;
+    }
     if (other) {
         for (int l = 0; l < L; ++l) {
             if (!sp.other[l] || other[l].kind != DPCLIP_KIND_CONV) continue;

@@ -212,3 +212,45 @@ def test_recorded_steps_behind_other_work(dp, dtype, T, d, before):
         assert ((clip[l].double() - (c / norm).clamp(max=1.0)).abs()).max().item() <= TOL[dtype]["norm"]
     # sums of norms and of windows may add up in another order from run to run
     assert _rel(clip, want[0]) <= 1e-5 and _rel(plan.flat, want[1]) <= 1e-4 and _rel(theta, want[2]) <= 1e-4
+
+
+# ---------------------------------------------------------------------------
+# models of T = 1 layers in two launches: batches and widths around the stages and tiles, heads of few outputs, noise, the
+# accumulation windows (B > 128 in fp32, > 768 in bf16), and the one launch that a header-sized workspace leaves
+# ---------------------------------------------------------------------------
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("B,widths", [(1, (640, 520, 8)), (31, (1000, 512, 10)), (33, (784, 1000, 1000, 10)), (65, (512, 136, 520, 1)), (129, (264, 1096, 17 * 8)),
+                                      (257, (2048, 264, 16)), (800, (384, 768, 24)), (2048, (128, 2200, 10))])
+def test_t1_models_in_two_launches(dp, dtype, B, widths):
+    gen = torch.Generator(device="cuda"); gen.manual_seed(B)
+    td = torch.float32 if dtype == "f32" else torch.bfloat16
+    layers = []
+    for k, (i, o) in enumerate(zip(widths, widths[1:])):
+        A = torch.randn(B, 1, i, generator=gen, device="cuda").to(td)
+        Z = (torch.randn(B, 1, o, generator=gen, device="cuda") * torch.rand(B, 1, 1, generator=gen, device="cuda") * 2 / (i * o) ** 0.5).to(td)
+        layers.append(dp.Layer(A, Z, k % 3 != 1))
+    full, small = dp.StepPlan(layers), dp.StepPlan(layers)
+    small.workspace = small.workspace[:256]
+    n2 = sum(y.Zbar.double().pow(2).sum((1, 2)) * (y.A.double().pow(2).sum((1, 2)) + (1 if y.has_bias else 0)) for y in layers)
+    clip = (0.7 / n2.sqrt()).clamp(max=1.0)
+    counts = []
+    for plan in (full, small):
+        n0 = dp.dpclip_launch_count()
+        plan.run(0.7, 0.0, 1)
+        torch.cuda.synchronize()
+        counts.append(dp.dpclip_launch_count() - n0)
+        assert dp.dpclip_read_status(plan.workspace) == 0
+        assert ((plan.norms.double() - n2.sqrt()) / n2.sqrt()).abs().max().item() <= TOL["f32"]["norm"]
+        for l, y in enumerate(layers):
+            zc = clip[:, None] * y.Zbar[:, 0].double()
+            assert _rel(plan.gW[l], zc.T @ y.A[:, 0].double()) <= (TOL["f32"]["grad"] if dtype == "f32" else 4e-3)
+            if y.has_bias:
+                assert _rel(plan.gb[l], zc.sum(0)) <= 1e-5
+    assert counts == [2, 1]
+    # the same draws on top of either
+    base = [p.flat.clone() for p in (full, small)]
+    for plan in (full, small):
+        plan.run(0.7, 0.3, 5)
+    torch.cuda.synchronize()
+    noise = [p.flat - b for p, b in zip((full, small), base)]
+    assert (noise[0] - noise[1]).abs().max().item() <= 1e-4 * max(1.0, base[0].abs().max().item())
