@@ -441,6 +441,21 @@ zta_group_kernel(const __grid_constant__ zg::Maps maps, const __grid_constant__ 
                 const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + ring.slot * 256 + g * nq;
                 const uint32_t to_small = ring.wide ? 256 : 128;
                 const bool last = win == windows - 1;
+                if (NORM && !two) {
+                    // short examples: one window of one accumulator, only its squares are wanted.  The drain is what such an item waits
+                    // for: 32 columns are under way at a time, in four chains of additions (16 in one chain: norms of 160 examples of
+                    // 32 positions, 512 to 2048 features, 388 us, here 248; 59 positions 250, 209; 128 positions 163, 160)
+                    float f4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+                    for (int h = 0; h < nq; h += 32) {
+                        uint32_t v[32];
+                        tmem_ld_32x32(t_row + h, v);
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) f4[j & 3] = fmaf(__uint_as_float(v[j]), __uint_as_float(v[j]), f4[j & 3]);
+                    }
+                    fro = (f4[0] + f4[1]) + (f4[2] + f4[3]);
+                } else
 #pragma unroll 1
                 for (int h = 0; h < nq; h += 16) {
                     float x[16];

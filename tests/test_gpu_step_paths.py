@@ -254,3 +254,22 @@ def test_t1_models_in_two_launches(dp, dtype, B, widths):
     torch.cuda.synchronize()
     noise = [p.flat - b for p, b in zip((full, small), base)]
     assert (noise[0] - noise[1]).abs().max().item() <= 1e-4 * max(1.0, base[0].abs().max().item())
+
+
+# ---------------------------------------------------------------------------
+# fp32 norms on CTA pairs of examples of one window (up to 128 positions) and of more, every width of the N side
+# ---------------------------------------------------------------------------
+@pytest.mark.parametrize("T", [2, 31, 33, 128, 129])
+@pytest.mark.parametrize("d_in,d_out", [(520, 136), (264, 196), (500, 260), (256, 256)])
+def test_fp32_norms_of_short_examples(dp, T, d_in, d_out):
+    gen = torch.Generator(device="cuda"); gen.manual_seed(T)
+    B = -(-(1 << 25) // (T * d_in * d_out)) + 1                   # just above the size that takes the tensor cores
+    A = torch.randn(B, T, d_in, generator=gen, device="cuda")
+    Z = torch.randn(B, T, d_out, generator=gen, device="cuda") * 1e-2
+    ws = torch.zeros(dp.dpclip_workspace_bytes(B, T, d_in, d_out), dtype=torch.uint8, device="cuda")
+    sq = torch.empty(B, device="cuda")
+    dp.dpclip_layer_sqnorms(A, Z, True, sq, ws)
+    torch.cuda.synchronize()
+    assert dp.dpclip_read_status(ws) == 0
+    ref = torch.stack([(Z[b].double().T @ A[b].double()).pow(2).sum() + Z[b].double().sum(0).pow(2).sum() for b in range(B)])
+    assert ((sq.double().sqrt() - ref.sqrt()) / ref.sqrt()).abs().max().item() <= TOL["f32"]["norm"]
