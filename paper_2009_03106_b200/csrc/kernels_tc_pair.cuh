@@ -556,12 +556,21 @@ reduce_segments_kernel(const __grid_constant__ ztp::Params p) {
     // 64-bit divisions per block).  A thread issues the loads of up to four segments before the first add and draws
     // its noise while they are in flight: with one load in flight per thread the kernel was bound by the latency of
     // its serial loads; what binds it now is instruction issue (the Philox rounds and Box-Muller of every float4).
-    griddep_wait();
     constexpr int ROWS = 4, SG = 4;
     constexpr int ROW_BLOCKS = BM / ROWS;
     const int n_blocks = p.G * ROW_BLOCKS;
     const size_t seg_stride = (size_t)p.W * SEG_ELEMS;
     const int c4 = (threadIdx.x & 63) << 2, r = threadIdx.x >> 6;
+    // the noise of the first block does not wait for the segments
+    float z[4] = {0.f, 0.f, 0.f, 0.f};
+    auto draw = [&](const Layer& y, int m, int n) { normals_at((size_t)m * y.d_in + n, y.sw0, y.sw1, p.k0, p.k1, z); };
+    if (p.noise_scale > 0.f && (int)blockIdx.x < n_blocks) {
+        const int t = blockIdx.x / ROW_BLOCKS, rb = blockIdx.x - t * ROW_BLOCKS;
+        const Layer& y = p.layer[p.tile_layer[t]];
+        const int tile = t - y.tile_base, tm = tile / y.tiles_n;
+        draw(y, tm * BM + rb * ROWS + r, (tile - tm * y.tiles_n) * y.N + c4);
+    }
+    griddep_wait();
     for (int blk = blockIdx.x; blk < n_blocks; blk += gridDim.x) {
         const int t = blk / ROW_BLOCKS, rb = blk - t * ROW_BLOCKS;
         const Layer& y = p.layer[p.tile_layer[t]];
@@ -577,12 +586,7 @@ reduce_segments_kernel(const __grid_constant__ ztp::Params p) {
         for (int k = 0; k < SG; ++k)
             v[k] = k < n_seg ? __ldcs(reinterpret_cast<const float4*>(src + (size_t)k * seg_stride))
                              : make_float4(0.f, 0.f, 0.f, 0.f);
-        float z0 = 0.f, z1 = 0.f, z2 = 0.f, z3 = 0.f;
-        if (p.noise_scale > 0.f) {
-            float z[4];
-            normals_at((size_t)m * y.d_in + n, y.sw0, y.sw1, p.k0, p.k1, z);
-            z0 = z[0]; z1 = z[1]; z2 = z[2]; z3 = z[3];
-        }
+        if (p.noise_scale > 0.f && blk != (int)blockIdx.x) draw(y, m, n);
         float4 acc = v[0];                                                  // segment order
 #pragma unroll
         for (int k = 1; k < SG; ++k) { acc.x += v[k].x; acc.y += v[k].y; acc.z += v[k].z; acc.w += v[k].w; }
@@ -595,8 +599,8 @@ reduce_segments_kernel(const __grid_constant__ ztp::Params p) {
             for (int k = 0; k < SG; ++k) { acc.x += v[k].x; acc.y += v[k].y; acc.z += v[k].z; acc.w += v[k].w; }
         }
         if (p.noise_scale > 0.f) {
-            acc.x = fmaf(p.noise_scale, z0, acc.x); acc.y = fmaf(p.noise_scale, z1, acc.y);
-            acc.z = fmaf(p.noise_scale, z2, acc.z); acc.w = fmaf(p.noise_scale, z3, acc.w);
+            acc.x = fmaf(p.noise_scale, z[0], acc.x); acc.y = fmaf(p.noise_scale, z[1], acc.y);
+            acc.z = fmaf(p.noise_scale, z[2], acc.z); acc.w = fmaf(p.noise_scale, z[3], acc.w);
         }
         float* dst = y.gW + (size_t)m * y.ldg + n;
         if (y.vec_ok && n + 4 <= y.d_in) {
