@@ -3123,11 +3123,12 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
         if (rc) return rc;
     }
     if ((rc = lanes.fork())) return rc;
-    if (t1.active) {
-        rc = launch_fused_t1_tf32(t1.p, false, t1_dtype, lanes.ws[last], lanes.ws_bytes[last], lanes.st[last]);
-        if (rc < 0) return rc;
-        if (rc > 0) return DPCLIP_ERR_UNSUPPORTED;           // prepare_t1_group checked the same conditions
-    }
+    auto t1_grads = [&]() -> int {
+        const int r = t1.active ? launch_fused_t1_tf32(t1.p, false, t1_dtype, lanes.ws[last], lanes.ws_bytes[last], lanes.st[last]) : 0;
+        return r > 0 ? DPCLIP_ERR_UNSUPPORTED : r;           // prepare_t1_group checked the same conditions
+    };
+    const bool t1_last = dtype == DPCLIP_F32 && lanes.n > 1;
+    if (!t1_last && (rc = t1_grads())) return rc;
     int in_grad_group[64];
     bool any_group = false, any_rest = false;
     if (track) {
@@ -3206,6 +3207,7 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
             }
         }
     }
+    if (t1_last && (rc = t1_grads())) return rc;
     return lanes.join();
 }
 
