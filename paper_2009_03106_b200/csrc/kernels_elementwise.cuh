@@ -136,14 +136,14 @@ __device__ __forceinline__ void ew_combine(float (&gg)[VEC], float (&gs)[VEC], i
     }
 }
 
-// A sum that overflowed although the example's inputs are finite: its norm is infinite and its factor zero, which has to
-// leave zero of it, not NaN.
+// A sum that overflowed although the example's inputs in its column are finite: its norm is infinite and its factor zero, which has
+// to leave zero of it, not NaN.
 template <typename T, int VEC>
 __device__ __forceinline__ void ew_clamp_overflow(const T* __restrict__ H, long ldh, const T* __restrict__ Z, long ldz, long r0,
                                                   int rows, int c0, float (&gg)[VEC], float (&gs)[VEC]) {
-    bool over = false;
+    bool over = false, finite[VEC];
 #pragma unroll
-    for (int u = 0; u < VEC; ++u) over = over || !isfinite(gg[u]) || !isfinite(gs[u]);
+    for (int u = 0; u < VEC; ++u) { over = over || isinf(gg[u]) || isinf(gs[u]); finite[u] = true; }
     if (!over) return;
     for (int r = 0; r < rows; ++r) {
         EwRaw<T, VEC> h, z;
@@ -152,12 +152,12 @@ __device__ __forceinline__ void ew_clamp_overflow(const T* __restrict__ H, long 
         float hf[VEC], zf[VEC];
         ew_f32(h, hf); ew_f32(z, zf);
 #pragma unroll
-        for (int u = 0; u < VEC; ++u) if (!isfinite(hf[u]) || !isfinite(zf[u])) return;
+        for (int u = 0; u < VEC; ++u) finite[u] = finite[u] && isfinite(hf[u]) && isfinite(zf[u]);
     }
 #pragma unroll
     for (int u = 0; u < VEC; ++u) {
-        if (isinf(gg[u])) gg[u] = copysignf(FLT_MAX, gg[u]);
-        if (isinf(gs[u])) gs[u] = copysignf(FLT_MAX, gs[u]);
+        if (finite[u] && isinf(gg[u])) gg[u] = copysignf(FLT_MAX, gg[u]);
+        if (finite[u] && isinf(gs[u])) gs[u] = copysignf(FLT_MAX, gs[u]);
     }
 }
 

@@ -1,5 +1,7 @@
 """Branches of the whole step against fp64 references of the same step (noise by the sequential paths, which have their own
 tests), at the sizes where a tile, a remainder or a range ends."""
+import math
+
 import numpy as np
 import pytest
 import torch
@@ -71,6 +73,22 @@ def test_elementwise_grads_of_an_example_that_overflows(dp):
     ref = (H[keep].double() * Z[keep].double()).sum((0, 1))
     assert torch.isinf(plan.norms[2]) and plan.clip[2].item() == 0.0
     assert _rel(plan.gW[0], ref) <= 1e-5 and np.isfinite(plan.gb[0].cpu().numpy()).all()
+
+
+def test_elementwise_overflow_beside_an_infinite_input(dp):
+    # columns 4 to 7 belong to one thread: an infinite input in column 5 makes that column's sum NaN (0 times infinity) and no other
+    B, T, d = 5, 16, 40
+    H = torch.randn(B, T, d, device="cuda"); Z = torch.randn(B, T, d, device="cuda") * 1e-3
+    H[2, :, 7] = 3e30; Z[2, :, 7] = 1e20
+    H[2, 0, 5] = math.inf
+    plan = dp.ModelPlan([dp.ModelLayer(dp.DPCLIP_KIND_ELEMENTWISE, H, Z, True)])
+    plan.run(1.0, 0.0, 0)
+    torch.cuda.synchronize()
+    assert plan.clip[2].item() == 0.0
+    ref = (H[[0, 1, 3, 4]].double() * Z[[0, 1, 3, 4]].double()).sum((0, 1))
+    others = [c for c in range(d) if c != 5]
+    assert torch.isnan(plan.gW[0][5]) and _rel(plan.gW[0][others], ref[others]) <= 1e-5
+    assert torch.isfinite(plan.gb[0]).all()
 
 
 # ---------------------------------------------------------------------------
