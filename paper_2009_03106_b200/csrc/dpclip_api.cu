@@ -2618,6 +2618,8 @@ static int ew_rows_grads(const dpclip_model_layer* other, float* const* rows, in
     EwRowsParams p;
     int blocks = 0;
     p.n = 0; p.B = B; p.clip = clip; p.noise_scale = sigma * C; p.k0 = (uint32_t)seed; p.k1 = (uint32_t)(seed >> 32);
+    p.cluster = 1;
+    while (p.cluster < EW_ROWS_MAX_CLUSTER && (long)p.cluster * EW_ROWS_PER_CTA < B) p.cluster *= 2;
     for (int l = 0; l < L; ++l) {
         if (rows[l]) {
             const dpclip_layer& y = other[l].layer;
@@ -2628,7 +2630,18 @@ static int ew_rows_grads(const dpclip_model_layer* other, float* const* rows, in
             blocks += ceil_div(y.d_in, 32L) * (q.g_shift ? 2 : 1);
         }
         if (p.n == EW_ROWS_MAX_LAYERS || (l == L - 1 && p.n > 0)) {
-            elementwise_rows_grad_kernel<<<blocks, EW_THREADS, 0, st>>>(p);
+            if (B <= EW_ROWS_FEW) elementwise_rows_grad_kernel<EW_THREADS / 32, false><<<blocks, EW_THREADS, 0, st>>>(p);
+            else if (p.cluster == 1) elementwise_rows_grad_kernel<EW_ROWS_WARPS, false><<<blocks, 32 * EW_ROWS_WARPS, 0, st>>>(p);
+            else {
+                cudaLaunchConfig_t cfg;
+                memset(&cfg, 0, sizeof(cfg));
+                cfg.gridDim = dim3(blocks * p.cluster); cfg.blockDim = dim3(32 * EW_ROWS_WARPS); cfg.stream = st;
+                cudaLaunchAttribute attr;
+                attr.id = cudaLaunchAttributeClusterDimension;
+                attr.val.clusterDim.x = p.cluster; attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+                cfg.attrs = &attr; cfg.numAttrs = 1;
+                if (cudaLaunchKernelEx(&cfg, elementwise_rows_grad_kernel<EW_ROWS_WARPS, true>, p) != cudaSuccess) { cudaGetLastError(); return DPCLIP_ERR_CUDA; }
+            }
             if (launch_status()) return DPCLIP_ERR_CUDA;
             p.n = 0; blocks = 0;
         }

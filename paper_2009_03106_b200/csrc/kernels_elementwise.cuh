@@ -15,6 +15,7 @@
 //                             Inputs are then read once a step, not twice: B = 128, T = 256, d = 512 in bf16, two layers:
 //                             17 + 18 us of grad kernels (134 MB) and eight clears and noise launches -> one of 4 us.
 #pragma once
+#include <cooperative_groups.h>
 #include <float.h>
 
 #include "kernels_stream.cuh"
@@ -221,31 +222,37 @@ elementwise_grad_kernel(const T* __restrict__ H, long ldh, const T* __restrict__
     }
 }
 
-// CTA = 32 columns of the scale or of the shift of one layer; warp w adds examples w, w + 8, ..., the warps' sums are added in
-// order.  Bound: latency, two round trips to L2 (B = 128: sixteen loads a thread, eight in flight).
+// CTA = 32 columns of the scale or of the shift of one layer; its warps deal the examples among them, the warps' sums are added in
+// order.  Bound: latency, two round trips to L2 (B = 128: sixteen loads a thread, eight in flight).  Eight warps up to 256 examples, 32
+// beyond, and beyond 1024 the CTAs of a cluster share the examples: with eight warps 4096 examples were 64 round trips one after the other
+// (step of one layer, T = 8, d = 64: 78 us, 38 by a second pass over the inputs; 32 warps 41, four CTAs of them 30).
 struct EwRowsLayer { const float* rows; float* g_scale; float* g_shift; int d, blk_begin; uint32_t sw0, sw1, sb0, sb1; };
-constexpr int EW_ROWS_MAX_LAYERS = 16;
-struct EwRowsParams { EwRowsLayer layer[EW_ROWS_MAX_LAYERS]; int n, B; const float* clip; float noise_scale; uint32_t k0, k1; };
+constexpr int EW_ROWS_MAX_LAYERS = 16, EW_ROWS_WARPS = 32, EW_ROWS_FEW = 256, EW_ROWS_PER_CTA = 1024, EW_ROWS_MAX_CLUSTER = 8;
+struct EwRowsParams { EwRowsLayer layer[EW_ROWS_MAX_LAYERS]; int n, B, cluster; const float* clip; float noise_scale; uint32_t k0, k1; };
 
-__global__ void __launch_bounds__(EW_THREADS)
+// CLUSTER: p.cluster CTAs share the examples.  A kernel of its own: the other one's 6 to 9 us of norms and sums grew by half a microsecond.
+template <int WARPS, bool CLUSTER>
+__global__ void __launch_bounds__(32 * WARPS)
 elementwise_rows_grad_kernel(const __grid_constant__ EwRowsParams p) {
-    constexpr int WARPS = EW_THREADS / 32, UNR = 8;
+    constexpr int UNR = 8;
     __shared__ float part[WARPS][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int block = CLUSTER ? (int)blockIdx.x / p.cluster : (int)blockIdx.x, rank = CLUSTER ? (int)blockIdx.x - block * p.cluster : 0;
     int l = 0;
-    while (l + 1 < p.n && (int)blockIdx.x >= p.layer[l + 1].blk_begin) ++l;
+    while (l + 1 < p.n && block >= p.layer[l + 1].blk_begin) ++l;
     const EwRowsLayer& y = p.layer[l];
-    const int blocks = (y.d + 31) >> 5, blk = blockIdx.x - y.blk_begin;
+    const int blocks = (y.d + 31) >> 5, blk = block - y.blk_begin;
     const bool shift = blk >= blocks;
     const int c = (shift ? blk - blocks : blk) * 32 + lane;
     float acc = 0.f;
     if (c < y.d) {
         const float* src = y.rows + (shift ? y.d : 0) + c;
-        for (int i = warp; i < p.B; i += WARPS * UNR) {
+        const int step = CLUSTER ? p.cluster * WARPS : WARPS;
+        for (int i = rank * WARPS + warp; i < p.B; i += step * UNR) {
             float g[UNR], f[UNR];
 #pragma unroll
             for (int k = 0; k < UNR; ++k) {
-                const int e = i + k * WARPS;
+                const int e = i + k * step;
                 g[k] = e < p.B ? __ldg(src + (size_t)e * 2 * y.d) : 0.f;
                 f[k] = e < p.B ? __ldg(p.clip + e) : 0.f;
             }
@@ -255,9 +262,21 @@ elementwise_rows_grad_kernel(const __grid_constant__ EwRowsParams p) {
     }
     part[warp][lane] = acc;
     __syncthreads();
-    if (warp != 0 || c >= y.d) return;
+    if (!CLUSTER && (warp != 0 || c >= y.d)) return;
+    if (warp == 0) {
 #pragma unroll
-    for (int w = 1; w < WARPS; ++w) acc += part[w][lane];
+        for (int w = 1; w < WARPS; ++w) acc += part[w][lane];
+        if (CLUSTER) part[0][lane] = acc;
+    }
+    if (CLUSTER) {
+        // the CTAs' sums in order, read from their shared memory, which stays until the first CTA has them
+        const cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+        cluster.sync();
+        if (rank == 0 && warp == 0)
+            for (int r = 1; r < p.cluster; ++r) acc += *cluster.map_shared_rank(&part[0][lane], r);
+        cluster.sync();
+    }
+    if (rank != 0 || warp != 0 || c >= y.d) return;
     if (p.noise_scale > 0.f) {
         float z[4];
         normals_at((size_t)(c & ~3), shift ? y.sb0 : y.sw0, shift ? y.sb1 : y.sw1, p.k0, p.k1, z);

@@ -18,6 +18,13 @@ def dp():
     return pkg
 
 
+def _spread(B, scale=4.0):
+    """Factors of the examples' gradients, from 1 / scale to scale, in mixed order: norms on both sides of the threshold."""
+    f = torch.exp(torch.linspace(-1.0, 1.0, B, device="cuda") * math.log(scale))
+    gen = torch.Generator(device="cuda"); gen.manual_seed(B)
+    return f[torch.randperm(B, generator=gen, device="cuda")]
+
+
 def _rel(got, ref):
     got, ref = got.double(), ref.double()
     return ((got - ref).norm() / ref.norm()).item()
@@ -89,6 +96,23 @@ def test_elementwise_overflow_beside_an_infinite_input(dp):
     others = [c for c in range(d) if c != 5]
     assert torch.isnan(plan.gW[0][5]) and _rel(plan.gW[0][others], ref[others]) <= 1e-5
     assert torch.isfinite(plan.gb[0]).all()
+
+
+# sums from stored rows by eight warps (up to 256 examples), 32 and clusters of CTAs, around the ends of each
+@pytest.mark.parametrize("B", [256, 257, 1024, 1025, 2049, 5000, 9000])
+@pytest.mark.parametrize("d", [31, 64])
+def test_elementwise_grads_of_many_examples(dp, B, d):
+    gen = torch.Generator(device="cuda"); gen.manual_seed(B)
+    H = torch.randn(B, 8, d, generator=gen, device="cuda")
+    Z = torch.randn(B, 8, d, generator=gen, device="cuda") * _spread(B)[:, None, None] / (16 * d) ** 0.5
+    plan = dp.ModelPlan([dp.ModelLayer(dp.DPCLIP_KIND_ELEMENTWISE, H, Z, True), dp.ModelLayer(dp.DPCLIP_KIND_ELEMENTWISE, H, Z, False)])
+    plan.run(1.0, 0.0, 0)
+    torch.cuda.synchronize()
+    g, s = (H.double() * Z.double()).sum(1), Z.double().sum(1)
+    clip = (1.0 / (2 * g.pow(2).sum(1) + s.pow(2).sum(1)).sqrt()).clamp(max=1.0)
+    assert clip.max().item() == 1.0 and clip.min().item() < 0.5
+    for got, ref in ((plan.gW[0], g), (plan.gb[0], s), (plan.gW[1], g)):
+        assert _rel(got, (clip[:, None] * ref).sum(0)) <= TOL["f32"]["grad"]
 
 
 # ---------------------------------------------------------------------------

@@ -1,0 +1,57 @@
+"""Steps that once lost time: each against another form of the same work on the same GPU, with a margin well above what two runs
+differ by."""
+import math
+
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dp():
+    import paper_2009_03106_b200 as pkg
+    pkg.load_library()
+    return pkg
+
+
+def _times(*steps, reps=10, rounds=9):
+    """Least time of each step in microseconds: ten to a graph, the graphs in turn (the rate of a training loop)."""
+    graphs = []
+    for step in steps:
+        step()
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=torch.cuda.Stream(priority=-1)):
+            for _ in range(reps):
+                step()
+        graphs.append(g)
+    best = [float("inf")] * len(steps)
+    for _ in range(rounds):
+        for k, g in enumerate(graphs):
+            g.replay()
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(10):
+                g.replay()
+            b.record()
+            torch.cuda.synchronize()
+            best[k] = min(best[k], a.elapsed_time(b) * 1e3 / (10 * reps))
+    return best
+
+
+def _dense(B, T, d_in, d_out, dtype):
+    A = torch.randn(B, T, d_in, device="cuda").to(dtype)
+    Z = torch.randn(B, T, d_out, device="cuda") * (torch.exp((torch.rand(B, 1, 1, device="cuda") * 2 - 1) * math.log(4.0)) / math.sqrt(T * d_in * d_out))
+    return A, Z.to(dtype)
+
+
+# element-wise layers of many examples: the sums from stored per-example gradients beside the second pass over the inputs, which a
+# workspace without room for them leaves
+@pytest.mark.parametrize("B,T,d", [(4096, 8, 64), (16384, 8, 64), (2048, 32, 256)])
+def test_elementwise_sums_of_many_examples(dp, B, T, d):
+    H, Z = _dense(B, T, d, d, torch.bfloat16)
+    stored, second = (dp.ModelPlan([dp.ModelLayer(dp.DPCLIP_KIND_ELEMENTWISE, H, Z, True)]) for _ in range(2))
+    second.workspace = second.workspace[:256]
+    a, b = _times(lambda: stored.run(1.0, 0.05, 1), lambda: second.run(1.0, 0.05, 1))
+    assert a <= 1.05 * b, (a, b)
