@@ -334,9 +334,15 @@ void simt_noise(SimtParams& p, const NoiseSpec* noise, bool* noise_done) {
     if (noise_done) *noise_done = true;
 }
 
-// T = 1 layers of at most 16 outputs (kernels_t1_thin.cuh).  Up to 1024 examples, 128 rows a warp: beyond, rows in slices over more
-// CTAs (the tile kernel) take less.
-inline bool t1_thin_ok(int B, int T, int d_out) { return T == 1 && d_out <= THIN_OUT && B <= 1024 && !path_switch(SW_FORCE_SIMT); }
+// T = 1 layers of at most 16 outputs (kernels_t1_thin.cuh) while a warp's rows are few, or where the tile kernel has as many tiles
+// as there are SMs and gains nothing from its slices of rows.  Call with noise, thin / tile kernel, 10 outputs: bf16, 1024 inputs, B =
+// 192: 12.3 / 16.3 us, 256: 15.4 / 16.3 (301 inputs, odd rows: 17.8 / 16.8), 320: 19.0 / 16.6, 1024: 56 / 18; 4096 inputs, 1024: 56 / 31,
+// 16384: 59 / 97.  fp32, 1024 inputs, 320: 12.7 / 15.4, 384: 14.7 / 15.4 (odd rows: 16.4 / 15.7), 512: 18.9 / 15.4; 4096 inputs, 512: 18.8 / 27.7,
+// 1024: 35.7 / 37.6.
+inline bool t1_thin_ok(int B, int T, int d_in, int d_out, dpclip_dtype dtype) {
+    if (T != 1 || d_out > THIN_OUT || B > 1024 || path_switch(SW_FORCE_SIMT)) return false;
+    return dtype == DPCLIP_F32 ? B <= 360 || d_in >= 4096 : B <= 240 || d_in >= 9216;
+}
 int launch_t1_thin_grad(const void* A, long lda, const void* Z, long ldz, int B, int d_in, int d_out, dpclip_dtype dtype,
                         const float* clip, float* gW, long ldg, float* gb, cudaStream_t st, const NoiseSpec* noise, bool* noise_done) {
     ThinParams p;
@@ -405,7 +411,7 @@ int launch_simt_grad(const void* A, long lda, const void* Z, long ldz, int B, in
         if (gb && cudaMemsetAsync(gb, 0, sizeof(float) * (size_t)d_out, st) != cudaSuccess) return DPCLIP_ERR_CUDA;
         return launch_narrow<true>(q, grid, d_out, dtype, st);
     }
-    if (t1_thin_ok(B, T, d_out))
+    if (t1_thin_ok(B, T, d_in, d_out, dtype))
         return launch_t1_thin_grad(A, lda, Z, ldz, B, d_in, d_out, dtype, clip, gW, ldg, gb, st, noise, noise_done);
     SimtParams p;
     fill_simt_params(p, A, lda, Z, ldz, T, d_in, d_out, gb != nullptr, dtype);
@@ -3175,7 +3181,7 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
     k = (any_group ? 1 : 0) + (any_rest ? 1 : 0);
     // On several streams the small layers of one position go first, on the last one: a few microseconds in front of that stream's
     // larger layer, where at their place in the order they ended the stage.
-    auto first = [&](int l) { return lanes.n > 1 && !other_kind(l) && t1_thin_ok(B, layers[l].T, layers[l].d_out); };
+    auto first = [&](int l) { return lanes.n > 1 && !other_kind(l) && t1_thin_ok(B, layers[l].T, layers[l].d_in, layers[l].d_out, dtype); };
     if (ew_rows) {
         rc = ew_rows_grads(other, ew_rows, L, B, clip, C, sigma, seed, stream_id0, lanes.st[k % lanes.n]);
         if (rc) return rc;

@@ -55,3 +55,17 @@ def test_elementwise_sums_of_many_examples(dp, B, T, d):
     second.workspace = second.workspace[:256]
     a, b = _times(lambda: stored.run(1.0, 0.05, 1), lambda: second.run(1.0, 0.05, 1))
     assert a <= 1.05 * b, (a, b)
+
+
+# heads of few outputs and many examples beside the tile kernel, which a head of 17 outputs takes: as many tiles
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("B,d_in", [(512, 300), (1024, 1000)])
+def test_heads_of_few_outputs_and_many_examples(dp, dtype, B, d_in):
+    steps = []
+    for o in (10, 17):
+        A, Z = _dense(B, 1, d_in, o, dtype)
+        gW, gb, clip = torch.empty(o, d_in, device="cuda"), torch.empty(o, device="cuda"), torch.rand(B, device="cuda")
+        ws = torch.zeros(max(256, dp.dpclip_workspace_bytes(B, 1, d_in, o, dp.DPCLIP_F32 if dtype == torch.float32 else dp.DPCLIP_BF16)), dtype=torch.uint8, device="cuda")
+        steps.append(lambda A=A, Z=Z, gW=gW, gb=gb, ws=ws: dp.dpclip_clipped_grad_noise(A, Z, clip, gW, gb, 0.05, 1.0, 3, 4, 5, ws))
+    few, wide = _times(*steps)
+    assert few <= 1.25 * wide, (few, wide)
