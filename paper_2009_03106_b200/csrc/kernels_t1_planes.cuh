@@ -336,6 +336,44 @@ t1_planes_kernel(const __grid_constant__ f1::Params q) {
                         cs[4] = fmaf(f[k], z.x, cs[4]); cs[5] = fmaf(f[k], z.y, cs[5]); cs[6] = fmaf(f[k], z.z, cs[6]); cs[7] = fmaf(f[k], z.w, cs[7]);
                     }
                 }
+            } else if (y.d_out - m0 <= 16) {
+                // a head of few outputs whose rows take no vector loads: thread = one column on every (128 / columns)-th row, sixteen
+                // rows in flight.  (Eight columns a thread as below: two of four threads had any, and each 64 rows of eight loads at B =
+                // 2048, one round trip after the other: 784-1000-1000-10 in bf16, 49 us of the second launch instead of 21.)
+                const int w = y.d_out - m0, rows = 32 * N_BIAS_WARPS / w, r1 = t / w, c1 = t - r1 * w;
+                float c = 0.f;
+                constexpr int UNR1 = 16;
+                if (r1 < rows)
+                    for (int r0 = r1; r0 < p.B; r0 += rows * UNR1) {
+                        T x[UNR1];
+                        float f[UNR1];
+#pragma unroll
+                        for (int k = 0; k < UNR1; ++k) {
+                            const int r = r0 + rows * k;
+                            x[k] = T(0.f); f[k] = 0.f;
+                            if (r < p.B) { f[k] = __ldcg(p.clip + r); x[k] = Z[(size_t)r * y.ldz + m0 + c1]; }
+                        }
+#pragma unroll
+                        for (int k = 0; k < UNR1; ++k) c = fmaf(f[k], to_f32(x[k]), c);
+                    }
+                // the rows' sums in order: eight groups, then one
+                bias_s[t] = c;
+                f1::named_barrier_sync(1, 32 * N_BIAS_WARPS);
+                c = 0.f;
+                if (t < 8 * w) for (int r = r1; r < rows; r += 8) c += bias_s[r * w + c1];
+                f1::named_barrier_sync(1, 32 * N_BIAS_WARPS);
+                bias_s[t] = c;
+                f1::named_barrier_sync(1, 32 * N_BIAS_WARPS);
+                if (t < w) {
+                    c = 0.f;
+#pragma unroll
+                    for (int g = 0; g < 8; ++g) c += bias_s[g * w + t];
+                    const int m = m0 + t;
+                    if (p.noise_scale > 0.f) c = fmaf(p.noise_scale, philox_normal((size_t)m, p.stream_id0 + 2ull * y.index + 1, p.k0, p.k1), c);
+                    y.gb[m] = c;
+                }
+                f1::named_barrier_sync(1, 32 * N_BIAS_WARPS);
+                continue;
             } else if (c0 < y.d_out) {
                 constexpr int ROWS = 4;
                 for (int r0 = rg; r0 < p.B; r0 += 32 * ROWS) {

@@ -298,6 +298,30 @@ def test_t1_models_in_two_launches(dp, dtype, B, widths):
     assert (noise[0] - noise[1]).abs().max().item() <= 1e-4 * max(1.0, base[0].abs().max().item())
 
 
+# bias sums of heads whose rows take no vector loads: every number of columns up to 16, batches around the rows in flight
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("B,d_out", [(1, 1), (297, 2), (300, 3), (64, 5), (2048, 7), (129, 9), (1025, 10), (333, 13), (700, 15), (96, 16)])
+def test_t1_bias_sums_of_heads(dp, dtype, B, d_out):
+    gen = torch.Generator(device="cuda"); gen.manual_seed(B)
+    td = torch.float32 if dtype == "f32" else torch.bfloat16
+    layers = []
+    for i, o in ((640, 520), (520, 136), (136, d_out)):
+        A = torch.randn(B, 1, i, generator=gen, device="cuda").to(td)
+        Z = (torch.randn(B, 1, o, generator=gen, device="cuda") * _spread(B)[:, None, None] / (3 * i * o) ** 0.5).to(td)
+        layers.append(dp.Layer(A, Z, True))
+    plan = dp.StepPlan(layers)
+    n2 = sum(y.Zbar.double().pow(2).sum((1, 2)) * (y.A.double().pow(2).sum((1, 2)) + 1) for y in layers)
+    clip = (1.0 / n2.sqrt()).clamp(max=1.0)
+    n0 = dp.dpclip_launch_count()
+    plan.run(1.0, 0.0, 1)
+    torch.cuda.synchronize()
+    assert dp.dpclip_launch_count() - n0 == 2 and dp.dpclip_read_status(plan.workspace) == 0
+    for l, y in enumerate(layers):
+        zc = clip[:, None] * y.Zbar[:, 0].double()
+        assert _rel(plan.gb[l], zc.sum(0)) <= 1e-5 * max(1.0, (zc.abs().sum(0).norm() / zc.sum(0).norm()).item() ** 0.5)
+        assert _rel(plan.gW[l], zc.T @ y.A[:, 0].double()) <= (TOL["f32"]["grad"] if dtype == "f32" else 4e-3)
+
+
 # ---------------------------------------------------------------------------
 # fp32 norms on CTA pairs of examples of one window (up to 128 positions) and of more, every width of the N side
 # ---------------------------------------------------------------------------

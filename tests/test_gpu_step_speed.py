@@ -69,3 +69,13 @@ def test_heads_of_few_outputs_and_many_examples(dp, dtype, B, d_in):
         steps.append(lambda A=A, Z=Z, gW=gW, gb=gb, ws=ws: dp.dpclip_clipped_grad_noise(A, Z, clip, gW, gb, 0.05, 1.0, 3, 4, 5, ws))
     few, wide = _times(*steps)
     assert few <= 1.25 * wide, (few, wide)
+
+
+# models of T = 1 layers: the bias sums of a head whose rows take no vector loads beside the same model without them, and the two launches
+# beside the one cooperative launch, many examples and few tiles
+@pytest.mark.parametrize("dtype,widths", [(torch.bfloat16, (784, 1000, 1000, 10)), (torch.float32, (256, 640, 640, 10))])
+def test_bias_sums_of_a_head_of_few_outputs(dp, dtype, widths):
+    data = [_dense(2048, 1, i, o, dtype) for i, o in zip(widths, widths[1:])]
+    plans = [dp.StepPlan([dp.Layer(A, Z, k < len(data) - 1 or bias) for k, (A, Z) in enumerate(data)]) for bias in (True, False)]
+    a, b = _times(*[lambda p=p: p.run(1.0, 0.05, 1) for p in plans])
+    assert a <= 1.1 * b, (a, b)
