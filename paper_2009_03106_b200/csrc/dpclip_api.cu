@@ -1499,7 +1499,9 @@ int launch_t1_planes(const tc::t1p::Prep& prep, const tc::f1::Params& q, bool qu
     constexpr int smem = t::Cfg<sizeof(T) == 4 ? 3 : 1>::SMEM_BYTES;
     const auto kernel = quads ? tc::t1_planes_kernel<T, true> : tc::t1_planes_kernel<T, false>;
     if (!enable_smem(kernel, smem)) return DPCLIP_ERR_CUDA;
-    const int rc = launch_behind(tc::t1_prepare_kernel<T>, dim3(prep.base.B), t::PREP_THREADS, 0, st, prep);
+    const bool few = prep.base.B <= t::PREP_FEW_EXAMPLES;
+    const int rc = few ? launch_behind(tc::t1_prepare_kernel<T, 16>, dim3(prep.base.B), 512, 0, st, prep)
+                       : launch_behind(tc::t1_prepare_kernel<T, 8>, dim3(prep.base.B), 256, 0, st, prep);
     return rc ? rc : launch_behind(kernel, dim3(grid), t::THREADS, smem, st, q);
 }
 // The whole step of a model of T = 1 layers.  1: the workspace lacks room, or the model is none for the tensor cores.

@@ -30,7 +30,10 @@ using f1::BN;
 using f1::decode;
 using f1::Item;
 constexpr int NBUF = 2;
-constexpr int PREP_THREADS = 512, PREP_WARPS = PREP_THREADS / 32, CHUNK = 512;      // elements a warp takes at a time
+// Warps of an example's CTA: sixteen while the CTAs are few, eight beyond (more examples on an SM, fewer idle warps at the barriers).  Step, sixteen
+// / eight: 1024-1024-1024 in bf16, B = 256: 11.1 / 10.9 us, 512: 15.2 / 12.5, 2048: 38 / 28; 784-1000-1000-10 in fp32, 256: 16.3 / 16.6, 512:
+// 25.5 / 22.8, 2048: 82.6 / 75.4 (one cooperative launch 78.2).
+constexpr int PREP_FEW_EXAMPLES = 296, CHUNK = 512;               // CHUNK: elements a warp takes at a time
 constexpr int N_EPILOGUE_WARPS = 16, N_BIAS_WARPS = 4;
 constexpr int THREADS = 64 + 32 * (N_EPILOGUE_WARPS + N_BIAS_WARPS);
 constexpr int OUT_STAGE_BYTES = N_EPILOGUE_WARPS * 4096, BIAS_BYTES = 32 * 32 * 4;     // 32 x 32 outputs per warp; 32 row groups x 32 columns
@@ -103,8 +106,8 @@ __device__ __forceinline__ void store_planes(uint16_t* dst, size_t plane, float4
 }
 }  // namespace t1p
 
-template <typename T>
-__global__ void __launch_bounds__(t1p::PREP_THREADS)
+template <typename T, int PREP_WARPS>
+__global__ void __launch_bounds__(32 * PREP_WARPS)
 t1_prepare_kernel(const __grid_constant__ t1p::Prep q) {
     using namespace t1p;
     constexpr int PLANES = sizeof(T) == 4 ? 3 : 1, U = CHUNK / 128;
@@ -114,6 +117,7 @@ t1_prepare_kernel(const __grid_constant__ t1p::Prep q) {
     griddep_launch_dependents();
     const FusedT1Params& p = q.base;
     const int i = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    static_assert(2 * FUSED_MAX_LAYERS <= 32, "one store a thread");
     if (threadIdx.x < 2 * FUSED_MAX_LAYERS * PREP_WARPS) (&part[0][0])[threadIdx.x] = 0.f;
     __syncthreads();
     // rows in chunks, dealt to the warps; a warp adds up what it has of each row, in order.  all: also the rows of A, whose planes need

@@ -79,3 +79,12 @@ def test_bias_sums_of_a_head_of_few_outputs(dp, dtype, widths):
     plans = [dp.StepPlan([dp.Layer(A, Z, k < len(data) - 1 or bias) for k, (A, Z) in enumerate(data)]) for bias in (True, False)]
     a, b = _times(*[lambda p=p: p.run(1.0, 0.05, 1) for p in plans])
     assert a <= 1.1 * b, (a, b)
+
+
+@pytest.mark.parametrize("widths", [(2000, 300, 300, 300, 300, 300, 300, 2), (784, 1000, 1000, 10)])
+def test_two_launches_of_many_examples(dp, path_switch, widths):
+    plan = dp.StepPlan([dp.Layer(*_dense(2048, 1, i, o, torch.float32), True) for i, o in zip(widths, widths[1:])])
+    two, = _times(lambda: plan.run(1.0, 0.05, 1))
+    path_switch("DPCLIP_NO_T1_PLANES", "1")
+    one, = _times(lambda: plan.run(1.0, 0.05, 1))
+    assert two <= 1.02 * one, (two, one)
