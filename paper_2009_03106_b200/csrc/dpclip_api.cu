@@ -130,6 +130,12 @@ inline int launch_behind(void (*kernel)(P...), dim3 grid, int block, size_t smem
     if (cudaLaunchKernelEx(&cfg, kernel, args...) != cudaSuccess) { cudaGetLastError(); return DPCLIP_ERR_CUDA; }
     return launch_status();
 }
+// Dynamic shared memory that lets no more CTAs of a launch stand on one SM than its share of them.  Placed while the kernel in front
+// leaves the SMs one after the other, a launch of few CTAs would be packed on the first.
+inline int spread_smem(long blocks, int static_bytes) {
+    const long k = ceil_div(blocks, (long)kNumSMs);
+    return (int)((228 * 1024 / k - 1024 - static_bytes) / 1024 * 1024);
+}
 // The kernel that this thread is about to launch directly follows one of the same step in its stream (takes the flag).
 inline bool take_overlap() { const bool on = t_overlap_prev; t_overlap_prev = false; return on; }
 
@@ -969,7 +975,14 @@ int launch_zta_stream(const StreamLayer* ls, int n, int B, int T, const NoiseSpe
     // one wave of CTAs (six of 256 threads and 40 registers per SM) over the 4-row blocks of all tiles
     long blocks = (long)G * (zp::BM / 4);
     if (blocks > 6L * kNumSMs) blocks = 6L * kNumSMs;
-    return launch_behind(tc::reduce_segments_kernel, dim3((unsigned)blocks), 256, 0, st, p);
+    // Behind the sums the reduce draws its first noise on SMs that have no pair, or beside the short drains of cut tiles; beside the full
+    // drains of pairs on all SMs it holds these up.  Steps, behind / in order: one layer of 512 -> 512, 1024 rows 30.7 / 32.3 us, 8192 (32 pairs)
+    // 37.7 / 38.9, 16384 (64 pairs) 41.1 / 38.9, 32768 (74 pairs) 59.3 / 53.5; 1024 -> 1024, 2048 rows (32 pairs) 38.9 / 40.6, 4096 (64) 45.0 /
+    // 42.4, 8192 (72) 55.1 / 51.7; cut tiles, 128 -> 300, 32768 rows 46.0 / 47.2, a text model of 300 and 1100 features 90.3 / 91.2.
+    constexpr int kPairsBeside = 56;                       // nothing measured between 48 and 64
+    if (cut || pairs <= kPairsBeside) return launch_behind(tc::reduce_segments_kernel, dim3((unsigned)blocks), 256, 0, st, p);
+    tc::reduce_segments_kernel<<<(unsigned)blocks, 256, 0, st>>>(p);
+    return launch_status();
 }
 
 int launch_zta_tc(const void* A, long lda, const void* Z, long ldz, int B, int T, int d_in, int d_out,
@@ -1344,7 +1357,13 @@ int launch_group(const GroupLayer* ls, int n, int B, bool norm, const NoiseSpec*
         if (rc) return rc;
         if (norm) continue;
         const int blocks = p.n_blocks < 8 * kNumSMs ? p.n_blocks : 8 * kNumSMs;
-        if ((rc = launch_behind(tc::reduce_group_kernel, dim3(blocks), 256, 0, st, p))) return rc;
+        // 48 CTAs of one 192 -> 256 layer stood on six SMs.  Steps, packed / spread (in order): 192 -> 256, 64 examples of 200 positions 60.0 /
+        // 46.7 us (47.1); 256 -> 512, 32 of 300: 58.1 / 50.1 (51.0); 148 -> 412 with two of 148 -> 148, 61 of 48: 46.6 / 42.7 (42.8); seven
+        // layers of 512 and 2048 features, 32 of 128: the same.
+        const int spread = spread_smem(blocks, sizeof(float) * 32 * 33);
+        // one limit for all launches: a smaller one would fail the launch another thread is about to make
+        if (!enable_smem(tc::reduce_group_kernel, spread_smem(1, sizeof(float) * 32 * 33))) return DPCLIP_ERR_CUDA;
+        if ((rc = launch_behind(tc::reduce_group_kernel, dim3(blocks), 256, spread, st, p))) return rc;
     }
     if (fuse_noise && noise_done) *noise_done = true;
     return DPCLIP_OK;

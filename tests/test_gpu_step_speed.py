@@ -88,3 +88,14 @@ def test_two_launches_of_many_examples(dp, path_switch, widths):
     path_switch("DPCLIP_NO_T1_PLANES", "1")
     one, = _times(lambda: plan.run(1.0, 0.05, 1))
     assert two <= 1.02 * one, (two, one)
+
+
+# reduces of few CTAs, and of full tiles on all SMs, beside the same step with every launch in order
+@pytest.mark.parametrize("dtype,B,T,d_in,d_out", [(torch.float32, 64, 200, 192, 256), (torch.float32, 32, 300, 256, 512),
+                                                  (torch.bfloat16, 512, 64, 256, 512), (torch.bfloat16, 16, 512, 1024, 1024)])
+def test_reduces_beside_the_sums(dp, path_switch, dtype, B, T, d_in, d_out):
+    plan = dp.StepPlan([dp.Layer(*_dense(B, T, d_in, d_out, dtype), True)])
+    behind, = _times(lambda: plan.run(1.0, 0.05, 1))
+    path_switch("DPCLIP_NO_OVERLAP", "1")
+    ordered, = _times(lambda: plan.run(1.0, 0.05, 1))
+    assert behind <= 1.03 * ordered, (behind, ordered)
