@@ -1249,6 +1249,15 @@ int launch_group_kernel(const tc::zg::Maps& maps, const tc::zg::Params& p, cudaS
     return launch_status();
 }
 
+// norms of long examples keep the sums between two drains in a slot per run
+constexpr long kGroupMinSlots = 8;
+bool group_long_norms(const GroupLayer* ls, int n) {
+    for (int l = 0; l < n; ++l) if (ls[l].T > tc::zg::FLUSH * tc::zg::Cfg::BK) return true;
+    return false;
+}
+bool group_norm_room(const GroupLayer* ls, int n, size_t workspace_bytes) {
+    return !group_long_norms(ls, n) || workspace_bytes >= kHeaderBytes + kGroupMinSlots * kGroupSlotBytes;
+}
 // Norms (norm = true) or clipped sums with noise of n fp32 layers.  Returns DPCLIP_OK, a negative status, or 1 when the
 // workspace cannot hold a few partial tiles (clipped sums, norms of more than FLUSH stages; nothing has been launched then).
 int launch_group(const GroupLayer* ls, int n, int B, bool norm, const NoiseSpec* noise, bool* noise_done,
@@ -1258,10 +1267,8 @@ int launch_group(const GroupLayer* ls, int n, int B, bool norm, const NoiseSpec*
     const int max_runs = sm_budget() / 2;
     const size_t room = workspace && workspace_bytes > (size_t)kHeaderBytes ? workspace_bytes - kHeaderBytes : 0;
     const long cap = (long)(room / kGroupSlotBytes);
-    // norms of long examples keep the sums between two drains in a slot per run
-    bool long_norms = false;
-    for (int l = 0; norm && l < n; ++l) long_norms = long_norms || ls[l].T > g::FLUSH * bk;
-    if ((!norm || long_norms) && cap < 8) return 1;
+    const bool long_norms = norm && group_long_norms(ls, n);
+    if ((!norm || long_norms) && cap < kGroupMinSlots) return 1;
     bool fuse_noise = !norm && noise && noise->scale > 0.f;
     for (int l = 0; l < n && fuse_noise; ++l) fuse_noise = ls[l].ldg == ls[l].d_in;
     if (norm) {
@@ -2946,10 +2953,13 @@ static int keep_group(GroupLayer* g, int n, const dpclip_layer* layers, int L, i
     if (n < kGroupFrom) n = keep([](const dpclip_layer& y) { return group_wide(y.d_in, y.d_out); });
     return n;
 }
-static int group_norms(const dpclip_layer* layers, int L, int B, dpclip_dtype dtype, float* sq_layers, const int* skip, int* taken,
-                       void* workspace, size_t workspace_bytes, void* stream, const tc::gram::FactorsTail* tail, bool* tail_done, int streams) {
+struct NormGroup {
     GroupLayer g[64];
     int n = 0;
+};
+static int norm_group_layers(NormGroup& q, const dpclip_layer* layers, int L, int B, dpclip_dtype dtype, float* sq_layers, const int* skip,
+                             int* taken, const void* workspace, size_t workspace_bytes, int streams) {
+    q.n = 0;
     for (int l = 0; l < L; ++l) {
         taken[l] = 0;
         const dpclip_layer& y = layers[l];
@@ -2957,17 +2967,24 @@ static int group_norms(const dpclip_layer* layers, int L, int B, dpclip_dtype dt
         int method = y.method;
         if (method == DPCLIP_AUTO) method = dpclip_pick_method(B, y.T, y.d_in, y.d_out, y.lda, y.ldz, dtype);
         if (method != DPCLIP_MATERIALIZE) continue;
-        g[n++] = {y.A, y.lda, y.Zbar, y.ldz, y.T, y.d_in, y.d_out, y.has_bias != 0, sq_layers + (size_t)l * B};
+        q.g[q.n++] = {y.A, y.lda, y.Zbar, y.ldz, y.T, y.d_in, y.d_out, y.has_bias != 0, sq_layers + (size_t)l * B};
         taken[l] = 1;
     }
-    n = keep_group(g, n, layers, L, B, true, streams, taken);
-    if (n == 0) return DPCLIP_OK;
+    q.n = keep_group(q.g, q.n, layers, L, B, true, streams, taken);
+    if (q.n == 0) return DPCLIP_OK;
     if (!workspace || workspace_bytes < (size_t)kHeaderBytes) return DPCLIP_ERR_WORKSPACE;
-    const bool with_tail = tail && n == L;
-    const int rc = launch_group(g, n, B, true, nullptr, nullptr, workspace, workspace_bytes, (cudaStream_t)stream, with_tail ? tail : nullptr);
-    if (rc > 0) { for (int l = 0; l < L; ++l) taken[l] = 0; return DPCLIP_OK; }         // no room: layer by layer
+    if (!group_norm_room(q.g, q.n, workspace_bytes)) {                                   // layer by layer
+        q.n = 0;
+        for (int l = 0; l < L; ++l) taken[l] = 0;
+    }
+    return DPCLIP_OK;
+}
+static int launch_norm_group(const NormGroup& q, int L, int B, void* workspace, size_t workspace_bytes, void* stream,
+                             const tc::gram::FactorsTail* tail, bool* tail_done) {
+    if (q.n == 0) return DPCLIP_OK;
+    const bool with_tail = tail && q.n == L;
     if (tail_done) *tail_done = with_tail;
-    return rc;
+    return launch_group(q.g, q.n, B, true, nullptr, nullptr, workspace, workspace_bytes, (cudaStream_t)stream, with_tail ? tail : nullptr);
 }
 // clip_ld as in shared_clipped_grad_launches
 static int group_grads(const dpclip_layer* layers, int L, int B, dpclip_dtype dtype, const float* clip, long clip_ld,
@@ -3080,9 +3097,16 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
     bool any_gram = false, any_mat = false;
     bool factors_done = false;
     SqClearedScope cleared_scope(cleared);
+    // when one launch takes every layer of the model, its last CTA also computes the factors
+    const tc::gram::FactorsTail tail = {sq_layers, L, (long)B, B, C, clip, norms, nullptr, 0, {}};
+    NormGroup norm_group;
+    int mat_lane = 0;
+    auto launch_mat_norms = [&]() {
+        return launch_norm_group(norm_group, L, B, lanes.ws[mat_lane], lanes.ws_bytes[mat_lane], lanes.st[mat_lane],
+                                 (!t1.active && !any_other && !any_gram && !path_switch(SW_NO_FACTORS_TAIL)) ? &tail : nullptr,
+                                 any_gram ? nullptr : &factors_done);
+    };
     if (track) {
-        // when one Gram launch takes every layer of the model, its last CTA also computes the factors
-        const tc::gram::FactorsTail tail = {sq_layers, L, (long)B, B, C, clip, norms, nullptr, 0, {}};
         const OverlapPrevScope behind_copies(sp != nullptr && lanes.n == 1);
         rc = gram_layers_sqnorms(layers, L, B, dtype, sq_layers, in_gram_group, ws0, lanes.ws_bytes[0], lanes.st[0],
                                  (!t1.active && !any_other && !path_switch(SW_NO_FACTORS_TAIL)) ? &tail : nullptr, &factors_done);
@@ -3091,15 +3115,14 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
         // the layers whose norms go by the materialised product, also in one launch
         int skip[64], taken[64];
         for (int l = 0; l < L; ++l) skip[l] = in_gram_group[l] || other_kind(l);
-        const int b = any_gram && lanes.n > 1 ? 1 : 0;
-        rc = group_norms(layers, L, B, dtype, sq_layers, skip, taken, lanes.ws[b], lanes.ws_bytes[b], lanes.st[b],
-                         (!t1.active && !any_other && !any_gram && !path_switch(SW_NO_FACTORS_TAIL)) ? &tail : nullptr,
-                         any_gram ? nullptr : &factors_done, lanes.n);
+        mat_lane = any_gram && lanes.n > 1 ? 1 : 0;
+        rc = norm_group_layers(norm_group, layers, L, B, dtype, sq_layers, skip, taken, lanes.ws[mat_lane], lanes.ws_bytes[mat_lane], lanes.n);
         if (rc) return rc;
         for (int l = 0; l < L; ++l) {
             any_mat = any_mat || taken[l];
             if (taken[l]) in_gram_group[l] = 1;                          // nothing left to do for it in this stage
         }
+        if (lanes.n == 1 && (rc = launch_mat_norms())) return rc;
     }
     // SM shares for the per-layer launches of a stage (see t_sm_budget): only when several of them run side by
     // side on different lanes, no launch shared by several layers is in the stage, and the stage is small
@@ -3137,13 +3160,20 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
     };
     int budget[64] = {0};
     if (track) stage_budgets(in_gram_group, any_gram || any_mat, budget);
-    int k = (any_gram ? 1 : 0) + (any_mat ? 1 : 0);        // the first lanes already carry the shared launches
+    auto alone = [&](int l) { return other_kind(l) || !((t1.active && layers[l].T == 1) || (track && in_gram_group[l])); };
+    // The shared fp32 kernel fills every SM, so what stands beside it starts first, from this stream: behind it a layer of 18 CTAs on the
+    // fp32 ALUs (18 examples of 28 x 28 maps, 3 -> 64 channels, beside 64 -> 256 -> 256 -> 256) began when it was over, 342 us a step instead of 268.
+    bool beside = false;
+    for (int l = 0; l < L; ++l) beside = beside || alone(l);
+    if (any_mat && !any_gram && beside && lanes.n > 1 && lanes.ws[1] && group_norm_room(norm_group.g, norm_group.n, lanes.ws_bytes[1])) mat_lane = 1;
+    const bool moved = mat_lane == 1 && !any_gram;
+    int k = moved ? 0 : (any_gram ? 1 : 0) + (any_mat ? 1 : 0);        // the first lanes already carry the shared launches
     for (int l = 0; l < L; ++l) {
         const dpclip_layer& y = layers[l];
+        if (!alone(l)) continue;
         const bool is_other = other_kind(l);
-        if (!is_other && ((t1.active && y.T == 1) || (track && in_gram_group[l]))) continue;
         const SmBudgetScope share(track ? budget[l] : 0);
-        const int b = k++ % lanes.n;
+        const int i = k++ % lanes.n, b = !moved || i == 0 ? i : i == lanes.n - 1 ? 1 : i + 1;      // moved: 0, 2, 3, ..., 1
         if (is_other)
             rc = other_kind_sqnorms(other[l], B, dtype, sq_layers + (size_t)l * B, ew_rows ? ew_rows[l] : nullptr, lanes.ws[b],
                                     lanes.ws_bytes[b], lanes.st[b]);
@@ -3153,6 +3183,7 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
                                       lanes.ws_bytes[b], lanes.st[b]);
         if (rc) return rc;
     }
+    if (lanes.n > 1 && (rc = launch_mat_norms())) return rc;
     if ((rc = lanes.join())) return rc;
     if (!factors_done) {
         // on one stream right behind the last of the norms
@@ -3441,8 +3472,10 @@ int dpclip_step_per_layer(const dpclip_layer* layers, int L, int B, dpclip_dtype
         int taken[kMaxTracked];
         bool any_gram = false;
         for (int l = 0; l < L; ++l) any_gram = any_gram || in_gram[l];
-        rc = group_norms(layers, L, B, dtype, sq_layers, in_gram, taken, workspace, workspace_bytes, stream,
-                         with_tail && !any_gram ? &tail : nullptr, any_gram ? nullptr : &factors_done, 1);
+        NormGroup norm_group;
+        rc = norm_group_layers(norm_group, layers, L, B, dtype, sq_layers, in_gram, taken, workspace, workspace_bytes, 1);
+        if (!rc) rc = launch_norm_group(norm_group, L, B, workspace, workspace_bytes, stream, with_tail && !any_gram ? &tail : nullptr,
+                                        any_gram ? nullptr : &factors_done);
         if (rc) return rc;
         for (int l = 0; l < L; ++l) in_gram[l] = in_gram[l] || taken[l];
     }

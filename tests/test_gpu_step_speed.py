@@ -46,6 +46,13 @@ def _dense(B, T, d_in, d_out, dtype):
     return A, Z.to(dtype)
 
 
+def _conv(dp, B, C, size, d_out, k, stride, pad, dtype):
+    X = torch.relu(torch.randn(B, C, *size, device="cuda")).to(dtype)
+    T = ((size[0] + 2 * pad - k[0]) // stride + 1) * ((size[1] + 2 * pad - k[1]) // stride + 1)
+    Z = (torch.randn(B, d_out, T, device="cuda") / math.sqrt(T * d_out * C * k[0] * k[1])).to(dtype)
+    return dp.ModelLayer(dp.DPCLIP_KIND_CONV, X, Z, True, conv=(*k, stride, pad), z_channel_major=True)
+
+
 # element-wise layers of many examples: the sums from stored per-example gradients beside the second pass over the inputs, which a
 # workspace without room for them leaves
 @pytest.mark.parametrize("B,T,d", [(4096, 8, 64), (16384, 8, 64), (2048, 32, 256)])
@@ -99,3 +106,13 @@ def test_reduces_beside_the_sums(dp, path_switch, dtype, B, T, d_in, d_out):
     path_switch("DPCLIP_NO_OVERLAP", "1")
     ordered, = _times(lambda: plan.run(1.0, 0.05, 1))
     assert behind <= 1.03 * ordered, (behind, ordered)
+
+
+# a long chain of few CTAs beside the shared fp32 norms, which fill every SM: on four streams the two run side by side
+def test_small_layers_beside_the_shared_fp32_norms(dp):
+    f = torch.float32
+    layers = [_conv(dp, 18, 3, (28, 28), 64, (3, 3), 1, 1, f), _conv(dp, 18, 64, (28, 28), 256, (3, 3), 1, 1, f),
+              _conv(dp, 18, 256, (28, 28), 256, (3, 3), 2, 1, f), _conv(dp, 18, 256, (14, 14), 256, (3, 3), 1, 1, f)]
+    plan = dp.ModelPlan(layers)
+    four, one = _times(lambda: plan.run_streams(1.0, 0.05, 1, branches=4), lambda: plan.run(1.0, 0.05, 1), reps=1)
+    assert four <= 0.95 * one, (four, one)
