@@ -53,6 +53,14 @@ def _conv(dp, B, C, size, d_out, k, stride, pad, dtype):
     return dp.ModelLayer(dp.DPCLIP_KIND_CONV, X, Z, True, conv=(*k, stride, pad), z_channel_major=True)
 
 
+# patch matrices of maps with an odd number of elements, loaded element by element, beside maps of one element more a channel
+def test_patch_matrices_of_odd_maps(dp):
+    odd = dp.ModelPlan([_conv(dp, 16, 96, (33, 31), 24, (3, 3), 1, 1, torch.bfloat16)])
+    even = dp.ModelPlan([_conv(dp, 16, 96, (32, 32), 24, (3, 3), 1, 1, torch.bfloat16)])
+    t_odd, t_even = _times(lambda: odd.run(1.0, 0.0, 1), lambda: even.run(1.0, 0.0, 1))
+    assert t_odd <= 1.15 * t_even, (t_odd, t_even)
+
+
 # element-wise layers of many examples: the sums from stored per-example gradients beside the second pass over the inputs, which a
 # workspace without room for them leaves
 @pytest.mark.parametrize("B,T,d", [(4096, 8, 64), (16384, 8, 64), (2048, 32, 256)])
