@@ -2767,20 +2767,30 @@ static bool stage_plan(StagePlan& sp, const dpclip_layer* layers, const dpclip_m
                 if (im.n_ex > B) im.n_ex = B;
                 im.r_out = positions / p.Wo < 1 ? 1 : positions / p.Wo > Ho ? Ho : positions / p.Wo;
                 im.tiles_a = ceil_div(Ho, (long)im.r_out); im.tiles_b = ceil_div(g.C, (long)ct);
-                stage::im_pitches(im);
-                return stage::im_smem(im);
+                im.pitch = g.W + 2 * g.pad;
+                im.plane = ((im.r_out - 1) * g.stride + g.kh) * im.pitch;
+            };
+            // whether the window, its channels apart on the banks, takes more than so many bytes
+            auto above = [&](size_t limit) {
+                if (stage::im_smem(im) > limit) return true;
+                stage::Job widest = im;
+                widest.plane += stage::IM_MAX_PAD;
+                if (stage::im_smem(widest) <= limit) return false;
+                widest.plane = im.plane + stage::im_bank_pad(im);
+                return stage::im_smem(widest) > limit;
             };
             int ct = ldp % unit ? g.C : 144 / kk / unit * unit;
             if (ct < unit && ldp % unit == 0) ct = unit;
             if (ct > g.C) ct = g.C;
             int positions = 18432 / (ct * kk);
             positions = positions < 32 ? 32 : positions > 256 ? 256 : positions;
-            size_t im_bytes = cut(ct, positions);
-            while ((im_bytes > 48 * 1024 || (long)ceil_div(B, (long)im.n_ex) * im.tiles_a * im.tiles_b < kNumSMs) && positions > 32)
-                im_bytes = cut(ct, positions /= 2);
-            while (im_bytes > (size_t)stage::SMEM_MAX && ct > unit && ldp % unit == 0) im_bytes = cut(ct = (int)round_up((size_t)ct / 2, unit), positions);
-            if (im_bytes > (size_t)stage::SMEM_MAX || (double)B * T * ldp / unit > 4.0e9 || g.kh > 16 || g.kw > 16) continue;
+            cut(ct, positions);
+            while (positions > 32 && (above(48 * 1024) || (long)ceil_div(B, (long)im.n_ex) * im.tiles_a * im.tiles_b < kNumSMs)) cut(ct, positions /= 2);
+            while (above(stage::SMEM_MAX) && ct > unit && ldp % unit == 0) cut(ct = (int)round_up((size_t)ct / 2, unit), positions);
+            if (above(stage::SMEM_MAX) || (double)B * T * ldp / unit > 4.0e9 || g.kh > 16 || g.kw > 16) continue;
             if ((double)im.n_ex * g.C * g.H * g.W > 2.0e9) continue;
+            im.plane += stage::im_bank_pad(im);
+            const size_t im_bytes = stage::im_smem(im);
             // loads start at a channel's first valid row: a multiple of W elements, or the channel's start when a CTA takes it whole
             for (im.vec = unit; im.vec > 1; im.vec /= 2)
                 if (aligned_to(y.A, im.vec * es) && (g.H * g.W) % im.vec == 0 && (im.tiles_a == 1 || g.W % im.vec == 0)) break;

@@ -1,0 +1,41 @@
+"""Plans of whole steps, worked out on the host (no GPU): which convolutions are copied as patch matrices, and what planning costs."""
+import time
+
+import pytest
+
+FAKE = 1 << 20                    # an aligned address that nothing reads
+
+
+@pytest.fixture(scope="module")
+def binding():
+    from paper_2009_03106_b200 import binding as b
+    b.load_library()
+    return b
+
+
+def _conv(b, C, H, W, d_out, k, stride, pad):
+    kh, kw = k
+    m = b._CModelLayer()
+    m.kind, m.z_channel_major = b.DPCLIP_KIND_CONV, 1
+    m.conv = b._CConv(C, H, W, kh, kw, stride, pad)
+    m.layer = b._CLayer(FAKE, 0, FAKE, 0, 0, C * kh * kw, d_out, 1, 0, FAKE, C * kh * kw, FAKE)
+    return m
+
+
+def _plan(b, layers, B, dtype):
+    arr = (b._CModelLayer * len(layers))(*layers)
+    return lambda: b.load_library().dpclip_model_workspace_bytes(arr, len(layers), B, dtype)
+
+
+# the plan of a step that is not recorded is made in every call: about as long as the launches of one kernel (3 us here; a search for bank
+# paddings at every size tried took 30 us)
+def test_planning_a_convolution_step_takes_microseconds(binding):
+    k3 = (3, 3)
+    plan = _plan(binding, [_conv(binding, 3, 32, 32, 64, k3, 1, 1), _conv(binding, 64, 32, 32, 128, k3, 2, 1),
+                           _conv(binding, 128, 16, 16, 256, k3, 2, 1), _conv(binding, 256, 8, 8, 256, k3, 1, 1)], 64, 1)
+    best = float("inf")
+    for _ in range(2000):
+        t = time.perf_counter()
+        plan()
+        best = min(best, time.perf_counter() - t)
+    assert best < 12e-6, best
