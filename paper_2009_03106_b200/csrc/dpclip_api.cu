@@ -2689,6 +2689,7 @@ static int ew_rows_grads(const dpclip_model_layer* other, float* const* rows, in
 // from the first launch of the step to its last.
 // ---------------------------------------------------------------------------
 constexpr int kStageMaxLayers = 64;
+constexpr int kLongRow = 64;
 // Copies of one step; a layer that no longer fits keeps its fp32-ALU form.
 constexpr size_t kStageCapBytes = (size_t)3 << 30;
 struct StagePlan {
@@ -2753,6 +2754,7 @@ static bool stage_plan(StagePlan& sp, const dpclip_layer* layers, const dpclip_m
             const bool narrow = dtype == DPCLIP_F32 && narrow_layer(T, p.d_in, p.d_out, 1, p.d_in, p.d_out);
             const long ldp = narrow ? p.d_in : (long)round_up(p.d_in, unit), ldz = narrow ? p.d_out : (long)round_up(p.d_out, unit);
             const int kk = g.kh * g.kw;
+            if ((double)B * T * ldp / unit > 4.0e9 || g.kh > 16 || g.kw > 16) continue;
             // A CTA: about 144 columns in whole channels whose columns are a multiple of 16 bytes, and 32 to 256 positions, about 18432
             // elements in all: rows of positions of one example, or whole examples (9216 and 36864 elements, 288 and 576 columns:
             // up to 15 % slower on the layers of two CNNs).  Odd rows of a narrow layer take one block of all channels.
@@ -2761,14 +2763,29 @@ static bool stage_plan(StagePlan& sp, const dpclip_layer* layers, const dpclip_m
             const int Ho = T / p.Wo;
             im.T = T; im.C = g.C; im.H = g.H; im.W = g.W; im.kh = g.kh; im.kw = g.kw; im.stride = g.stride; im.pad = g.pad; im.Wo = p.Wo;
             im.es = (int)es; im.dst_ld = (int)ldp; im.cols = p.d_in; im.rows = B * T;
+            bool short_of_room = false;
             auto cut = [&](int ct, int positions) {
                 im.ct = ct;
                 im.n_ex = positions / T > 1 ? positions / T : 1;
                 if (im.n_ex > B) im.n_ex = B;
                 im.r_out = positions / p.Wo < 1 ? 1 : positions / p.Wo > Ho ? Ho : positions / p.Wo;
                 im.tiles_a = ceil_div(Ho, (long)im.r_out); im.tiles_b = ceil_div(g.C, (long)ct);
-                im.pitch = g.W + 2 * g.pad;
-                im.plane = ((im.r_out - 1) * g.stride + g.kh) * im.pitch;
+                im.part = 0; im.w_out = p.Wo; im.tiles_x = 1; im.lead = 0; im.pitch = g.W + 2 * g.pad;
+                // loads start at a channel's first valid row: a multiple of W elements, or the channel's start when a CTA takes it whole
+                for (im.vec = unit; im.vec > 1; im.vec /= 2)
+                    if (aligned_to(y.A, im.vec * es) && (g.H * g.W) % im.vec == 0 && (im.tiles_a == 1 || g.W % im.vec == 0)) break;
+                if (p.Wo > kLongRow || (short_of_room && positions < p.Wo)) {
+                    im.part = 1; im.r_out = 1; im.tiles_a = Ho; im.n_ex = 1;
+                    im.w_out = ceil_div(p.Wo, ceil_div(p.Wo, (long)positions));
+                    if (im.w_out > 8) im.w_out = (int)round_up(im.w_out, 8);
+                    im.tiles_x = ceil_div(p.Wo, (long)im.w_out);
+                    for (im.vec = unit; im.vec > 1; im.vec /= 2)
+                        if (aligned_to(y.A, im.vec * es) && g.W % im.vec == 0 && (im.w_out * g.stride) % im.vec == 0) break;
+                    im.lead = (im.vec - g.pad % im.vec) % im.vec;
+                    im.pitch = (int)round_up(im.lead + (im.w_out - 1) * g.stride + g.kw, im.vec);
+                }
+                const double plane = ((im.r_out - 1.0) * g.stride + g.kh) * im.pitch;
+                im.plane = plane < 1 << 20 ? (int)plane : 1 << 20;            // far beyond any limit either way
             };
             // whether the window, its channels apart on the banks, takes more than so many bytes
             auto above = [&](size_t limit) {
@@ -2785,15 +2802,17 @@ static bool stage_plan(StagePlan& sp, const dpclip_layer* layers, const dpclip_m
             int positions = 18432 / (ct * kk);
             positions = positions < 32 ? 32 : positions > 256 ? 256 : positions;
             cut(ct, positions);
-            while (positions > 32 && (above(48 * 1024) || (long)ceil_div(B, (long)im.n_ex) * im.tiles_a * im.tiles_b < kNumSMs)) cut(ct, positions /= 2);
-            while (above(stage::SMEM_MAX) && ct > unit && ldp % unit == 0) cut(ct = (int)round_up((size_t)ct / 2, unit), positions);
-            if (above(stage::SMEM_MAX) || (double)B * T * ldp / unit > 4.0e9 || g.kh > 16 || g.kw > 16) continue;
-            if ((double)im.n_ex * g.C * g.H * g.W > 2.0e9) continue;
+            while (positions > 32 && (above(48 * 1024) || (long)ceil_div(B, (long)im.n_ex) * im.tiles_a * im.tiles_x * im.tiles_b < kNumSMs))
+                cut(ct, positions /= 2);
+            while (above(stage::SMEM_MAX)) {
+                if (ct > unit && ldp % unit == 0) ct = (int)round_up((size_t)ct / 2, unit);
+                else if (positions > 1) { short_of_room = true; positions /= 2; }
+                else break;
+                cut(ct, positions);
+            }
+            if (above(stage::SMEM_MAX) || (double)im.n_ex * g.C * g.H * g.W > 2.0e9) continue;
             im.plane += stage::im_bank_pad(im);
             const size_t im_bytes = stage::im_smem(im);
-            // loads start at a channel's first valid row: a multiple of W elements, or the channel's start when a CTA takes it whole
-            for (im.vec = unit; im.vec > 1; im.vec /= 2)
-                if (aligned_to(y.A, im.vec * es) && (g.H * g.W) % im.vec == 0 && (im.tiles_a == 1 || g.W % im.vec == 0)) break;
             {
                 stage::Job& j = add_job(l, false, stage::IM2COL, y.A, 0, (int)ldp, B * T, p.d_in, es);
                 im.kind = j.kind; im.src = j.src; im.src_ld = 0;
@@ -2924,17 +2943,20 @@ static int launch_stage(StagePlan& sp, float* sq, size_t n_sq, cudaStream_t st) 
         memset(&q, 0, sizeof(q));
         q.n = sp.n_jobs - i0 < stage::MAX_JOBS ? sp.n_jobs - i0 : stage::MAX_JOBS;
         if (i0 == 0) { q.clear = sq; q.n_clear = n_sq; }
+        bool parts = false;
         for (int i = 0; i < q.n; ++i) {
             stage::Job& j = q.job[i] = sp.job[i0 + i];
+            parts = parts || j.part;
             j.blk_begin = q.blocks;
-            if (j.kind == stage::IM2COL) q.blocks += ceil_div((long)j.rows / j.T, (long)j.n_ex) * j.tiles_a * j.tiles_b;
+            if (j.kind == stage::IM2COL) q.blocks += ceil_div((long)j.rows / j.T, (long)j.n_ex) * j.tiles_a * j.tiles_x * j.tiles_b;
             else if (j.kind == stage::TRANSPOSE) q.blocks += j.rows / j.T * j.tiles_a * j.tiles_b;
             else q.blocks += ceil_div((long)j.rows * (j.dst_ld / ((j.es == 4 || j.kind == stage::ROWS_TO_F32) ? 4 : 8)),
                                       (long)stage::ROWS_UNROLL * stage::THREADS);
         }
         // the limit is the kernel's, not the launch's: a smaller one would fail the launch another thread is about to make
-        if (sp.smem > 48 * 1024 && !enable_smem(stage_operands_kernel, stage::SMEM_MAX)) return DPCLIP_ERR_CUDA;
-        stage_operands_kernel<<<q.blocks, stage::THREADS, sp.smem, st>>>(q);
+        const auto kernel = parts ? stage_operands_kernel<true> : stage_operands_kernel<false>;
+        if (sp.smem > 48 * 1024 && !enable_smem(kernel, stage::SMEM_MAX)) return DPCLIP_ERR_CUDA;
+        kernel<<<q.blocks, stage::THREADS, sp.smem, st>>>(q);
         if (launch_status()) return DPCLIP_ERR_CUDA;
     }
     return DPCLIP_OK;

@@ -128,13 +128,18 @@ def test_elementwise_grads_of_many_examples(dp, B, d):
     ("bf16", 40, 32, (14, 14), 64, 3, 2, 0, True), ("bf16", 40, 32, (14, 14), 64, 3, 1, 1, True), ("f32", 80, 24, (6, 7), 64, 3, 2, 0, True),
     ("f32", 70, 36, (10, 5), 48, 2, 2, 0, True)])
 def test_convolutions_from_feature_maps(dp, dtype, B, C, size, d_out, k, stride, pad, cm):
+    _check_convolution(dp, dtype, B, C, size, d_out, (k, k), stride, pad, cm)
+
+
+def _check_convolution(dp, dtype, B, C, size, d_out, k, stride, pad, cm, offset=0):
     gen = torch.Generator(device="cuda"); gen.manual_seed(7)
     td = torch.float32 if dtype == "f32" else torch.bfloat16
-    X = torch.randn(B, C, *size, generator=gen, device="cuda").to(td)
-    T = ((size[0] + 2 * pad - k) // stride + 1) * ((size[1] + 2 * pad - k) // stride + 1)
-    Z = (torch.randn(B, T, d_out, generator=gen, device="cuda") / (T * d_out * C * k * k) ** 0.5).to(td)
+    n = B * C * size[0] * size[1]
+    X = torch.randn(n + offset, generator=gen, device="cuda").to(td)[offset:].view(B, C, *size)
+    T = ((size[0] + 2 * pad - k[0]) // stride + 1) * ((size[1] + 2 * pad - k[1]) // stride + 1)
+    Z = (torch.randn(B, T, d_out, generator=gen, device="cuda") * _spread(B)[:, None, None] / (T * d_out * C * k[0] * k[1]) ** 0.5).to(td)
     plan = dp.ModelPlan([dp.ModelLayer(dp.DPCLIP_KIND_CONV, X, Z.transpose(1, 2).contiguous() if cm else Z, True,
-                                       conv=(k, k, stride, pad), z_channel_major=cm)])
+                                       conv=(*k, stride, pad), z_channel_major=cm)])
     plan.run(1.0, 0.0, 0)
     torch.cuda.synchronize()
     assert dp.dpclip_read_status(plan.workspace) == 0
@@ -143,10 +148,27 @@ def test_convolutions_from_feature_maps(dp, dtype, B, C, size, d_out, k, stride,
     gb = Z.double().sum(1)
     norms = (G.pow(2).sum((1, 2)) + gb.pow(2).sum(1)).sqrt()
     clip = (1.0 / norms).clamp(max=1.0)
+    assert B < 3 or (clip.max().item() == 1.0 and clip.min().item() < 0.5)
     tol = TOL[dtype]
     assert ((plan.norms.double() - norms).abs() / norms).max().item() <= tol["norm"]
     assert _rel(plan.gW[0], (clip[:, None, None] * G).sum(0)) <= tol["grad"]
     assert _rel(plan.gb[0], (clip[:, None] * gb).sum(0)) <= tol["grad"]
+    return plan
+
+
+# rows of positions that a CTA takes in parts: windows that begin inside the padding, rows that are no multiple of a load or of a part,
+# strides, one window per position, inputs that begin off a 16-byte boundary
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("B,C,size,d_out,k,stride,pad,offset", [
+    (16, 24, (1, 300), 64, (1, 3), 1, 1, 0), (4, 24, (1, 301), 96, (1, 9), 1, 0, 0), (4, 64, (1, 4096), 64, (1, 3), 2, 0, 0), (4, 24, (1, 16000), 32, (1, 9), 1, 0, 0),
+    (3, 20, (9, 72), 64, (3, 3), 1, 1, 0), (3, 16, (12, 130), 64, (5, 5), 1, 2, 0), (3, 16, (20, 200), 64, (3, 3), 2, 1, 1), (4, 10, (7, 257), 64, (2, 7), 1, 9, 0),
+    (3, 16, (3, 2001), 64, (3, 2), 3, 3, 2), (3, 8, (40, 600), 64, (16, 16), 4, 0, 4), (16, 8, (64, 6000), 64, (16, 16), 64, 0, 0), (8, 3, (20, 1000), 32, (7, 7), 2, 3, 0)])
+def test_convolutions_of_long_rows(dp, dtype, B, C, size, d_out, k, stride, pad, offset):
+    plan = _check_convolution(dp, dtype, B, C, size, d_out, k, stride, pad, True, offset)
+    T = ((size[0] + 2 * pad - k[0]) // stride + 1) * ((size[1] + 2 * pad - k[1]) // stride + 1)
+    macs = B * T * C * k[0] * k[1] * d_out
+    if macs >= (4 if dtype == "bf16" else 32) << 20:              # from here on the patch matrix is copied
+        assert plan.workspace.numel() >= B * T * C * k[0] * k[1] * (2 if dtype == "bf16" else 4)
 
 
 # ---------------------------------------------------------------------------
