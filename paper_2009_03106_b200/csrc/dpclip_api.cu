@@ -1366,8 +1366,8 @@ int launch_group(const GroupLayer* ls, int n, int B, bool norm, const NoiseSpec*
         const int blocks = p.n_blocks < 8 * kNumSMs ? p.n_blocks : 8 * kNumSMs;
         // 48 CTAs of one 192 -> 256 layer stood on six SMs.  Steps, packed / spread (in order): 192 -> 256, 64 examples of 200 positions 60.0 /
         // 46.7 us (47.1); 256 -> 512, 32 of 300: 58.1 / 50.1 (51.0); 148 -> 412 with two of 148 -> 148, 61 of 48: 46.6 / 42.7 (42.8); seven
-        // layers of 512 and 2048 features, 32 of 128: the same.
-        const int spread = spread_smem(blocks, sizeof(float) * 32 * 33);
+        // layers of 512 and 2048 features, 32 of 128 (1184 CTAs): 421.2 / 423.5.
+        const int spread = blocks < 4 * kNumSMs ? spread_smem(blocks, sizeof(float) * 32 * 33) : 0;      // more fill the SMs anyway
         // one limit for all launches: a smaller one would fail the launch another thread is about to make
         if (!enable_smem(tc::reduce_group_kernel, spread_smem(1, sizeof(float) * 32 * 33))) return DPCLIP_ERR_CUDA;
         if ((rc = launch_behind(tc::reduce_group_kernel, dim3(blocks), 256, spread, st, p))) return rc;
