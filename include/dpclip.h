@@ -17,8 +17,10 @@
  *   factor  c_i = min(1, C / n_i)                                  (Eq. "per_example_weight")
  *   release sum_i c_i G_i (+ bias)  + N(0, sigma^2 C^2)            (Algorithm 1, last line, as a SUM)
  *
- * The library never writes a per-example gradient or a Gram matrix to global
- * memory.
+ * The library never writes a Gram matrix, nor the per-example gradient of a
+ * weight matrix, to global memory.  The 2 d numbers of an example's gradient of
+ * an element-wise layer do go through the workspace in dpclip_model_step* (see
+ * there); the workspace keeps them until a later call overwrites them.
  *
  * Conventions for every entry point
  *   - Pointers are DEVICE pointers unless the parameter comment says "host".
@@ -29,8 +31,9 @@
  *     What the process keeps between calls is bookkeeping only: an atomic
  *     launch counter (dpclip_launch_count), the path-switch mask read once
  *     from the environment (dpclip_reload_path_switches), per-device kernel
- *     attributes set at a kernel's first launch, and the device address of
- *     dpclip_clipped_grad_noalloc's fixed array.  Entry points may be called
+ *     attributes set at a kernel's first launch, per host thread the spacings
+ *     found for the shapes of the last few patch matrices, and the device
+ *     address of dpclip_clipped_grad_noalloc's fixed array.  Entry points may be called
  *     from several host threads.  A
  *     workspace holds scratch (partial tiles) and, in its header, a status
  *     word, the grid-barrier counter of the one-launch T = 1 step and the
@@ -501,7 +504,8 @@ int dpclip_read_status(const void* workspace, int* host_status /* host */, void*
 int dpclip_pick_method(int B, int T, int d_in, int d_out, long lda, long ldz, dpclip_dtype dtype);
 
 /* Number of kernels this library has launched in this process (a host-side
- * counter for benchmarks and tests; cudaMemset calls are not counted). */
+ * counter for benchmarks and tests; cudaMemset calls are not counted, nor is the
+ * kernel that stands for them in a step on several streams). */
 unsigned long long dpclip_launch_count(void);
 
 /* Launch floor, for benchmarks: enqueue one EMPTY kernel with the launch shape of the one-launch T = 1 step

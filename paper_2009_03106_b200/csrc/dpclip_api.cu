@@ -961,7 +961,7 @@ int launch_zta_stream(const StreamLayer* ls, int n, int B, int T, const NoiseSpe
     const auto kernel = any_split ? tc::zta_pair_kernel<true, true> : cut ? tc::zta_pair_kernel<false, true> : tc::zta_pair_kernel<false, false>;
     if (!enable_smem(kernel, zp::SMEM_BYTES)) return DPCLIP_ERR_CUDA;
     const int pairs = (int)ceil_div(p.total, U) * W;
-    DPCLIP_LOGF("clipped sum, CTA pairs: %d layer(s), B*T=%ld, %d tiles of 512x256 in %d super-layer(s) of %d, %d stages per tile, "
+    DPCLIP_LOGF("clipped sum, CTA pairs: %d layer(s), B*T=%ld, %d tiles of up to 512x256 in %d super-layer(s) of %d, %d stages per tile, "
                 "%d pairs in gangs of %d, runs of %ld stages, %ld segments, noise %s", n, R, G, n_super, W, p.S, pairs, W, U,
                 n_segments, fuse_noise ? "in the reduce" : "separate");
     int rc;
@@ -1489,7 +1489,7 @@ inline T1Planes t1_planes(int B, int d_in, int d_out, dpclip_dtype dtype) {
 }
 // Models of T = 1 layers that take the two launches of kernels_t1_planes.cuh: more than 16 output tiles of 128 x 128.  A step, one
 // cooperative launch / two launches: fp32, 784-1000-1000-10, B = 128: 14.4 / 13.0 us, 1000-2000-1000, B = 64: 20.6 / 15.4, 512-512-512-10,
-// B = 512: 30.8 / 23.2, 4096-4096-1000, B = 256: 121 / 78; bf16: the first 14.4 / 11.8, the last 72 / 46 (46 / 31 without noise).  784-256-10,
+// B = 512: 30.8 / 23.2, 4096-4096-1000, B = 256: 121 / 78; bf16: the first 12.5 / 10.7, the last 72 / 46 (46 / 31 without noise).  784-256-10,
 // B = 32 (16 tiles) would take 8.5 instead of 11.7, but up to there the one launch stays: it is the form whose barrier has its timeout
 // tested, on that model.
 inline bool t1_planes_pays(const dpclip_layer* layers, int L, int B, dpclip_dtype dtype) {
@@ -3230,6 +3230,8 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
         const int r = t1.active ? launch_fused_t1_tf32(t1.p, false, t1_dtype, lanes.ws[last], lanes.ws_bytes[last], lanes.st[last]) : 0;
         return r > 0 ? DPCLIP_ERR_UNSUPPORTED : r;           // prepare_t1_group checked the same conditions
     };
+    // fp32 on several streams: behind the other sums of its stream.  Steps of two CNNs, first / last: 132.8 / 129.9 and 162.2 / 160.2 us, with inputs
+    // from HBM 141.1 / 139.7 and 170.3 / 168.0.  (bf16 was measured first: a CNN's launch of 12 us beside three longer ones.)
     const bool t1_last = dtype == DPCLIP_F32 && lanes.n > 1;
     if (!t1_last && (rc = t1_grads())) return rc;
     int in_grad_group[64];

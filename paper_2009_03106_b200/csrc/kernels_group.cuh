@@ -33,9 +33,9 @@
 //
 // Measured (fp32): the loop of 256 x 256 tiles takes 1.15 us a stage, 1.6 PFLOP/s of bf16 products, the tensor core's rate
 // (two plane stages and four raw ones, or three and two: the same).  Seven layers of 512 and 2048 features, B = 32, T = 128:
-// norms 172 us, clipped sums 164 us, reduce 28 us, where one launch per layer took 305, 310 and 38.  Of those the loop is 127
-// us each (8192 stages on 74 pairs; tensor pipe active 56 and 54 % of a launch under ncu); the norms lose the rest to the
-// drain of 1.5 us behind the four stages of an example, the sums to fill, drains and partial tiles.
+// norms 159 us, clipped sums 171 us, reduce 28 us, where one launch per layer took 305, 310 and 38.  Of those the loop is 127
+// us each (8192 stages on 74 pairs; tensor pipe active 56 and 54 % of a launch under ncu, when the norms took 172); the norms lose the rest to
+// the drain behind the four stages of an example, the sums to fill, drains and partial tiles.
 //
 // Roles: warp 0 TMA (each CTA its own operands, plain loads), warp 1 MMA issuer (rank 0), 16 warps that prepare every
 // stage (factor, planes, bias column sums), 8 epilogue warps that take the finished accumulators.
@@ -294,7 +294,7 @@ zta_group_kernel(const __grid_constant__ zg::Maps maps, const __grid_constant__ 
                 }
                 u += w.units;
             }
-            griddep_launch_dependents();                        // the reduce may place CTAs beside the last drains
+            griddep_launch_dependents();                        // the launch that follows may place its CTAs as SMs fall idle
         }
     } else if (warp < 2 + PREP) {
         // ------------------------------------------------ preparation
