@@ -113,7 +113,7 @@ def test_reduces_beside_the_sums(dp, path_switch, dtype, B, T, d_in, d_out):
     behind, = _times(lambda: plan.run(1.0, 0.05, 1))
     path_switch("DPCLIP_NO_OVERLAP", "1")
     ordered, = _times(lambda: plan.run(1.0, 0.05, 1))
-    assert behind <= 1.03 * ordered, (behind, ordered)
+    assert behind <= 1.05 * ordered, (behind, ordered)
 
 
 # a long chain of few CTAs beside the shared fp32 norms, which fill every SM: on four streams the two run side by side
