@@ -342,19 +342,21 @@ void simt_noise(SimtParams& p, const NoiseSpec* noise, bool* noise_done) {
 
 // T = 1 layers of at most 16 outputs (kernels_t1_thin.cuh) while a warp's rows are few, or where the tile kernel has as many tiles
 // as there are SMs and gains nothing from its slices of rows.  Call with noise, thin / tile kernel, 10 outputs: bf16, 1024 inputs, B =
-// 192: 12.3 / 16.3 us, 256: 15.4 / 16.3 (301 inputs, odd rows: 17.8 / 16.8), 320: 19.0 / 16.6, 1024: 56 / 18; 4096 inputs, 1024: 56 / 31,
-// 16384: 59 / 97.  fp32, 1024 inputs, 320: 12.7 / 15.4, 384: 14.7 / 15.4 (odd rows: 16.4 / 15.7), 512: 18.9 / 15.4; 4096 inputs, 512: 18.8 / 27.7,
+// 192: 12.3 / 16.3 us, 256: 15.4 / 16.4 (301 inputs, element by element: 17.8 / 16.8), 320: 19.0 / 16.6, 1024: 56 / 18; 4096 inputs, 1024: 56 / 31,
+// 16384: 59 / 97.  fp32, 1024 inputs, 320: 12.7 / 15.4, 384: 14.7 / 15.4 (301 inputs: 16.4 / 15.7), 512: 18.9 / 15.4; 4096 inputs, 512: 18.8 / 27.7,
 // 1024: 35.7 / 37.6.
-inline bool t1_thin_ok(int B, int T, int d_in, int d_out, dpclip_dtype dtype) {
+inline bool t1_thin_pairs(const void* A, long lda, dpclip_dtype dtype) { return aligned_to(A, 2 * elt_size(dtype)) && lda % 2 == 0; }
+inline bool t1_thin_ok(const void* A, long lda, int B, int T, int d_in, int d_out, dpclip_dtype dtype) {
     if (T != 1 || d_out > THIN_OUT || B > 1024 || path_switch(SW_FORCE_SIMT)) return false;
-    return dtype == DPCLIP_F32 ? B <= 360 || d_in >= 4096 : B <= 240 || d_in >= 9216;
+    const bool pairs = t1_thin_pairs(A, lda, dtype);
+    return dtype == DPCLIP_F32 ? B <= (pairs ? 384 : 360) || d_in >= 4096 : B <= (pairs ? 256 : 240) || d_in >= 9216;
 }
 int launch_t1_thin_grad(const void* A, long lda, const void* Z, long ldz, int B, int d_in, int d_out, dpclip_dtype dtype,
                         const float* clip, float* gW, long ldg, float* gb, cudaStream_t st, const NoiseSpec* noise, bool* noise_done) {
     ThinParams p;
     memset(&p, 0, sizeof(p));
     p.A = A; p.lda = lda; p.Z = Z; p.ldz = ldz; p.B = B; p.d_in = d_in; p.d_out = d_out;
-    p.pairs_ok = aligned_to(A, 2 * elt_size(dtype)) && lda % 2 == 0;
+    p.pairs_ok = t1_thin_pairs(A, lda, dtype);
     p.clip = clip; p.gW = gW; p.ldg = ldg; p.gb = gb;
     if (noise && noise->scale > 0.f && ldg == d_in) {
         p.noise_scale = noise->scale;
@@ -417,7 +419,7 @@ int launch_simt_grad(const void* A, long lda, const void* Z, long ldz, int B, in
         if (gb && cudaMemsetAsync(gb, 0, sizeof(float) * (size_t)d_out, st) != cudaSuccess) return DPCLIP_ERR_CUDA;
         return launch_narrow<true>(q, grid, d_out, dtype, st);
     }
-    if (t1_thin_ok(B, T, d_in, d_out, dtype))
+    if (t1_thin_ok(A, lda, B, T, d_in, d_out, dtype))
         return launch_t1_thin_grad(A, lda, Z, ldz, B, d_in, d_out, dtype, clip, gW, ldg, gb, st, noise, noise_done);
     SimtParams p;
     fill_simt_params(p, A, lda, Z, ldz, T, d_in, d_out, gb != nullptr, dtype);
@@ -3267,7 +3269,7 @@ static int step_general(const dpclip_layer* layers_in, const dpclip_model_layer*
     k = (any_group ? 1 : 0) + (any_rest ? 1 : 0);
     // On several streams the small layers of one position go first, on the last one: a few microseconds in front of that stream's
     // larger layer, where at their place in the order they ended the stage.
-    auto first = [&](int l) { return lanes.n > 1 && !other_kind(l) && t1_thin_ok(B, layers[l].T, layers[l].d_in, layers[l].d_out, dtype); };
+    auto first = [&](int l) { return lanes.n > 1 && !other_kind(l) && t1_thin_ok(layers[l].A, layers[l].lda, B, layers[l].T, layers[l].d_in, layers[l].d_out, dtype); };
     if (ew_rows) {
         rc = ew_rows_grads(other, ew_rows, L, B, clip, C, sigma, seed, stream_id0, lanes.st[k % lanes.n]);
         if (rc) return rc;
